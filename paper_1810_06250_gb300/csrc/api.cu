@@ -68,6 +68,9 @@ void free_plan(rms_plan_s *p)
     cudaFree(p->d_w_all);
     if (p->d_bhi_raw != p->d_bhi) cudaFree(p->d_bhi_raw);
     if (p->d_blo_raw != p->d_blo) cudaFree(p->d_blo_raw);
+    cudaFree(p->d_dh);
+    cudaFree(p->fold.d_hi);
+    cudaFree(p->fold.d_lo);
     cudaFree(p->d_kbmask);
     cudaFree(p->d_stage);
     cudaFree(p->d_rexp);
@@ -294,7 +297,6 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
             return cst;
         }
     } else if (is_tensor(precision)) {
-        const int N = 2 * nphi;
         // RMS_MAX_TILE_N (16..208, multiple of 16) in the environment lowers the phase
         // rows per tensor-core tile (a tuning knob: smaller tiles leave shared memory
         // for more pipeline stages)
@@ -303,24 +305,26 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
             int t = std::atoi(v);
             if (t >= 16 && t <= max_tile_cap && t % 16 == 0) max_tile = t;
         }
-        // balanced tiles of at most max_tile rows, each a multiple of 16 (the last one
-        // rounded up to 16 as well)
-        auto tiling = [N](int cap, int32_t &ntiles, int32_t &tile, int32_t &last) {
+        // balanced tiles of at most cap rows, each a multiple of 16 (the last one
+        // rounded up to 16 as well); CTA pairs take tiles of up to 256 rows (plans for
+        // the single-CTA window kernel keep theirs)
+        auto tiling = [](int N, int cap, int32_t &ntiles, int32_t &tile, int32_t &last) {
             ntiles = (N + cap - 1) / cap;
             const int per = (N + ntiles - 1) / ntiles;
             tile = (per + 15) / 16 * 16;
             last = (N - (ntiles - 1) * tile + 15) / 16 * 16;
         };
-        tiling(max_tile, p->ntiles_n, p->tile_n, p->tile_n_last);
-        // CTA pairs take tiles of up to 256 rows (plans for the single-CTA window kernel keep theirs)
-        if (max_tile_cap == kMaxTileN) tiling(kMaxTileNPair, p->ntiles_n2, p->tile_n2, p->tile_n_last2);
-        else { p->ntiles_n2 = p->ntiles_n; p->tile_n2 = p->tile_n; p->tile_n_last2 = p->tile_n_last; }
-        p->npad = std::max(p->ntiles_n * p->tile_n, p->ntiles_n2 * p->tile_n2);
+        auto both_tilings = [&](int N, PhaseTiling &t) {
+            tiling(N, max_tile, t.ntiles_n, t.tile_n, t.tile_n_last);
+            tiling(N, max_tile_cap == kMaxTileN ? kMaxTileNPair : max_tile, t.ntiles_n2, t.tile_n2, t.tile_n_last2);
+            t.npad = std::max(t.ntiles_n * t.tile_n, t.ntiles_n2 * t.tile_n2);
+        };
+        both_tilings(2 * nphi, p->tiles);
         p->kblocks = (p->nact + kChanPerKBlock - 1) / kChanPerKBlock;
         p->kpad = p->kblocks * kKBlock;
         const bool fp16 = precision == RMS_FP16X3;
-        RMS_TRY(dalloc(&p->d_bhi, (size_t)p->npad * p->kpad));
-        RMS_TRY(dalloc(&p->d_blo, (size_t)p->npad * p->kpad));
+        RMS_TRY(dalloc(&p->d_bhi, (size_t)p->tiles.npad * p->kpad));
+        RMS_TRY(dalloc(&p->d_blo, (size_t)p->tiles.npad * p->kpad));
         RMS_TRY(launch_phase_bsplit(*p, p->d_dl2, p->d_wact, p->nact, p->kpad, p->d_bhi, p->d_blo, fp16, 0));
         // LOS-major cubes contract over every channel (zero rows where flagged)
         p->kblocks_raw = (nchan + kChanPerKBlock - 1) / kChanPerKBlock;
@@ -340,28 +344,59 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
             RMS_TRY(dalloc(&p->d_w_all, nchan));
             RMS_TRY(cudaMemcpy(p->d_dl2_all, dl2_all.data(), nchan * sizeof(double), cudaMemcpyHostToDevice));
             RMS_TRY(cudaMemcpy(p->d_w_all, w.data(), nchan * sizeof(double), cudaMemcpyHostToDevice));
-            RMS_TRY(dalloc(&p->d_bhi_raw, (size_t)p->npad * p->kpad_raw));
-            RMS_TRY(dalloc(&p->d_blo_raw, (size_t)p->npad * p->kpad_raw));
+            RMS_TRY(dalloc(&p->d_bhi_raw, (size_t)p->tiles.npad * p->kpad_raw));
+            RMS_TRY(dalloc(&p->d_blo_raw, (size_t)p->tiles.npad * p->kpad_raw));
             RMS_TRY(launch_phase_bsplit(*p, p->d_dl2_all, p->d_w_all, nchan, p->kpad_raw, p->d_bhi_raw,
                                         p->d_blo_raw, fp16, 0));
         }
         p->scratch_bytes = (size_t)p->num_sms * (size_t)std::max(p->kblocks, p->kblocks_raw) * kTileM * 128;
         RMS_TRY(cudaMalloc(&p->d_scratch, p->scratch_bytes));
-        if (!encode_b_map(&p->tmap_bhi, p->d_bhi, p->kpad, p->npad, p->tile_n) ||
-            !encode_b_map(&p->tmap_blo, p->d_blo, p->kpad, p->npad, p->tile_n) ||
-            !encode_b_map(&p->tmap_bhi_raw, p->d_bhi_raw, p->kpad_raw, p->npad, p->tile_n) ||
-            !encode_b_map(&p->tmap_blo_raw, p->d_blo_raw, p->kpad_raw, p->npad, p->tile_n)) {
+        if (!encode_b_map(&p->tmap_bhi, p->d_bhi, p->kpad, p->tiles.npad, p->tiles.tile_n) ||
+            !encode_b_map(&p->tmap_blo, p->d_blo, p->kpad, p->tiles.npad, p->tiles.tile_n) ||
+            !encode_b_map(&p->tmap_bhi_raw, p->d_bhi_raw, p->kpad_raw, p->tiles.npad, p->tiles.tile_n) ||
+            !encode_b_map(&p->tmap_blo_raw, p->d_blo_raw, p->kpad_raw, p->tiles.npad, p->tiles.tile_n)) {
             free_plan(p);
             return RMS_ERR_CUDA;
         }
         // half-tile boxes for the two-CTA contraction (tile_n a multiple of 16, so a
         // half is whole 8-row swizzle groups)
-        if (p->tile_n2 % 16 == 0 && p->tile_n_last2 % 16 == 0) {
-            const int h = p->tile_n2 / 2;
-            p->pair_maps = encode_b_map(&p->tmap2_bhi, p->d_bhi, p->kpad, p->npad, h) &&
-                           encode_b_map(&p->tmap2_blo, p->d_blo, p->kpad, p->npad, h) &&
-                           encode_b_map(&p->tmap2_bhi_raw, p->d_bhi_raw, p->kpad_raw, p->npad, h) &&
-                           encode_b_map(&p->tmap2_blo_raw, p->d_blo_raw, p->kpad_raw, p->npad, h);
+        if (p->tiles.tile_n2 % 16 == 0 && p->tiles.tile_n_last2 % 16 == 0) {
+            const int h = p->tiles.tile_n2 / 2;
+            p->pair_maps = encode_b_map(&p->tmap2_bhi, p->d_bhi, p->kpad, p->tiles.npad, h) &&
+                           encode_b_map(&p->tmap2_blo, p->d_blo, p->kpad, p->tiles.npad, h) &&
+                           encode_b_map(&p->tmap2_bhi_raw, p->d_bhi_raw, p->kpad_raw, p->tiles.npad, h) &&
+                           encode_b_map(&p->tmap2_blo_raw, p->d_blo_raw, p->kpad_raw, p->tiles.npad, h);
+        }
+        // A phi grid symmetric about zero folds: cos is even and sin odd in phi, so one
+        // column pair (c, s) serves phi and -phi.  Accepted when no phase moves by more
+        // than 1e-9 rad (the products' own FP64 rounding is of that order on wide bands).
+        double xmax = 0.0, off = 0.0;
+        for (double x : dl2) xmax = std::fmax(xmax, std::fabs(x));
+        for (int k = 0; 2 * k < nphi; ++k) off = std::fmax(off, std::fabs(phi[k] + phi[nphi - 1 - k]));
+        if (max_tile_cap == kMaxTileN && off * xmax <= 1e-9) {
+            FoldPlan &f = p->fold;
+            f.ncol = (nphi + 1) / 2;
+            f.kplus = nphi / 2;
+            f.kminus = (nphi - 1) / 2;
+            f.kblocks = (p->nact + kKBlock - 1) / kKBlock;
+            f.kpad = f.kblocks * kKBlock;
+            both_tilings(2 * f.ncol, f.tiles);
+            std::vector<double> dh(f.ncol);
+            for (int i = 0; i < f.ncol; ++i) dh[i] = 0.5 * (phi[f.kplus + i] - phi[f.kminus - i]);
+            RMS_TRY(dalloc(&p->d_dh, f.ncol));
+            RMS_TRY(cudaMemcpy(p->d_dh, dh.data(), f.ncol * sizeof(double), cudaMemcpyHostToDevice));
+            RMS_TRY(dalloc(&f.d_hi, (size_t)f.tiles.npad * f.kpad));
+            RMS_TRY(dalloc(&f.d_lo, (size_t)f.tiles.npad * f.kpad));
+            RMS_TRY(launch_phase_fold(*p, p->d_dh, fp16, 0));
+            const int h = f.tiles.tile_n2 / 2;
+            if (!encode_b_map(&f.tmap_bhi, f.d_hi, f.kpad, f.tiles.npad, f.tiles.tile_n) ||
+                !encode_b_map(&f.tmap_blo, f.d_lo, f.kpad, f.tiles.npad, f.tiles.tile_n)) {
+                free_plan(p);
+                return RMS_ERR_CUDA;
+            }
+            f.pair_maps = encode_b_map(&f.tmap2_bhi, f.d_hi, f.kpad, f.tiles.npad, h) &&
+                          encode_b_map(&f.tmap2_blo, f.d_lo, f.kpad, f.tiles.npad, h);
+            f.on = true;
         }
     }
     RMS_TRY(cudaEventCreateWithFlags(&p->last, cudaEventDisableTiming));
@@ -465,7 +500,7 @@ static rms_status synth_launch(rms_plan_t p, const float *Q, const float *U, int
     case RMS_FP16X3: {
         // the split operand (and FP16X3's per-LOS exponents): stream-ordered scratch
         // and 8 bytes of peak key per LOS (the contraction's split schedule)
-        const size_t abytes = split_operand_bytes(*p, nlos, layout);
+        const size_t abytes = p->fold.on ? fold_operand_bytes(*p, nlos) : split_operand_bytes(*p, nlos, layout);
         const size_t rbytes = p->precision == RMS_FP16X3 ? (size_t)((nlos + 255) & ~(int64_t)255) : 0;
         const size_t kbytes = (size_t)((nlos * 8 + 255) & ~(int64_t)255);
         uint8_t *scr = nullptr;
@@ -749,7 +784,7 @@ rms_status rms_plan_set_option(rms_plan_t p, int32_t option, int64_t value)
     switch (option) {
     case RMS_OPT_CONTRACTION:
         if (value < RMS_CONTRACT_AUTO || value > RMS_CONTRACT_PAIR) return RMS_ERR_INVALID_ARG;
-        if (value == RMS_CONTRACT_PAIR && !p->pair_maps) return RMS_ERR_UNSUPPORTED;
+        if (value == RMS_CONTRACT_PAIR && !(p->fold.on ? p->fold.pair_maps : p->pair_maps)) return RMS_ERR_UNSUPPORTED;
         p->contraction = (int32_t)value;
         return RMS_OK;
     case RMS_OPT_L2_BUDGET:
@@ -773,8 +808,8 @@ rms_status rms_plan_info(rms_plan_t p, int32_t what, int64_t *value)
     case RMS_INFO_NPHI: *value = p->nphi; break;
     case RMS_INFO_PRECISION: *value = p->precision; break;
     case RMS_INFO_KPAD: *value = p->kpad; break;
-    case RMS_INFO_NPAD: *value = p->npad; break;
-    case RMS_INFO_TILE_N: *value = p->tile_n; break;
+    case RMS_INFO_NPAD: *value = p->tiles.npad; break;
+    case RMS_INFO_TILE_N: *value = p->tiles.tile_n; break;
     case RMS_INFO_DEVICE: *value = p->device; break;
     case RMS_INFO_LAST_CTAS: *value = p->last_ctas; break;
     case RMS_INFO_LAST_PAIR: *value = p->last_pair; break;
@@ -795,8 +830,8 @@ rms_status rms_plan_get(rms_plan_t p, int32_t what, void *dst, int64_t bytes)
     case RMS_GET_LAMBDA2: src = p->lambda2.data(); n = p->lambda2.size() * sizeof(double); host = true; break;
     case RMS_GET_ACTIVE: src = p->active.data(); n = p->active.size() * sizeof(int32_t); host = true; break;
     case RMS_GET_TABLE: src = p->d_table; n = (size_t)p->nact * p->nphi * sizeof(float2); break;
-    case RMS_GET_B_HI: src = p->d_bhi; n = (size_t)p->npad * p->kpad * sizeof(uint16_t); break;
-    case RMS_GET_B_LO: src = p->d_blo; n = (size_t)p->npad * p->kpad * sizeof(uint16_t); break;
+    case RMS_GET_B_HI: src = p->d_bhi; n = (size_t)p->tiles.npad * p->kpad * sizeof(uint16_t); break;
+    case RMS_GET_B_LO: src = p->d_blo; n = (size_t)p->tiles.npad * p->kpad * sizeof(uint16_t); break;
     case RMS_GET_RMSF64: src = p->d_R64; n = (size_t)p->nphi * 2 * sizeof(double); break;
     default: return RMS_ERR_INVALID_ARG;
     }

@@ -1,4 +1,5 @@
-// Tensor-core RM synthesis in two kernels: a streaming split of the cube into
+// Tensor-core RM synthesis in two kernels (phi grids symmetric about zero run the
+// folded form of both, fold.cu, which halves the products): a streaming split of the cube into
 // 16-bit operands, then a tcgen05 contraction that only moves tiles.
 //
 // split_kernel (the layout stage): one CTA per 128-LOS M tile, one thread per
@@ -62,8 +63,6 @@ constexpr int kEpiCols = 8;                       // staging chunk: 8 columns x 
 constexpr int kEpiLd = kEpiCols + 1;
 constexpr int kEpiStageBytes = kNumEpiWarps * 32 * kEpiLd * 4;
 constexpr int kSmemLimit = 227 * 1024;
-
-enum { MODE_BF16 = 0, MODE_BF16X3 = 1, MODE_FP16X3 = 2 };
 
 // ----------------------------------------------------------------------------
 // split_kernel
@@ -286,6 +285,7 @@ struct GemmParams {
     const int64_t *rows;        // optional: results of row r go to output row rows[r]
     int32_t kblocks, group;
     int32_t nphi, ntiles_n, tile_n, tile_n_last;
+    int32_t ncol;               // column pairs (2 phase rows each) holding results: nphi, or ceil(nphi / 2) folded
     float *F;
     int32_t *pidx;
     float *pabs, *pphi;
@@ -307,6 +307,8 @@ struct GemmParams {
     // with a 64-bit atomicMax and peak_finalize_kernel writes the peak outputs
     int32_t jobs_split, npanels;
     unsigned long long *keys;
+    // folded grids (FOLD): phase column i serves the phi samples kplus + i and kminus - i
+    int32_t kplus, kminus;
     int32_t b_rows;             // phase rows of a B stage in this CTA's shared memory (tile_n, or tile_n / 2 in pairs)
     // window rotation (rotating kernel only): row r's operand is multiplied by
     // T[clamp(centre[r], cmin, cmax)][channel] before it enters the MMA
@@ -385,19 +387,23 @@ __device__ __forceinline__ void job_of(const GemmParams &P, int64_t nit, int64_t
 // HALF: columns of the tile per epilogue thread (tile_n <= 2 HALF).  ROT: the
 // window variant, 512 threads, whose converter warps rotate each stage's A
 // rows in shared memory before the MMA reads them.  PAIR: the two-CTA variant
-// (launched in clusters of two; not combined with ROT).
-template <int HALF, bool ROT, bool PAIR>
+// (launched in clusters of two; not combined with ROT).  FOLD: the phi grid is
+// symmetric and a tile holds 64 LOS (see fold.cu): P.nphi is then the number of
+// column pairs (i.e. of +-phi pairs).
+template <int HALF, bool ROT, bool PAIR, bool FOLD>
 __global__ void __launch_bounds__(ROT ? 512 : kThreads, 1)
 gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtensorMap tmB_hi,
             const __grid_constant__ CUtensorMap tmB_lo, const __grid_constant__ CUtensorMap tmA)
 {
     static_assert(!(ROT && PAIR), "the rotating variant is single-CTA");
+    static_assert(!(ROT && FOLD), "windows are not folded");
+    constexpr int kTileLos = FOLD ? kFoldTileLos : kTileM;   // lines of sight per M tile
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const GSmem S = gcarve(base, P);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nlos = P.count ? min(*P.count, P.nlos) : P.nlos;
-    const int64_t nmt = (nlos + kTileM - 1) / kTileM;
+    const int64_t nmt = (nlos + kTileLos - 1) / kTileLos;
     // work items: M tiles, or pairs of M tiles (even tile in the even CTA)
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
     const bool leader = rank == 0;
@@ -694,12 +700,15 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                 int nt0, nt1;
                 job_of(P, nit, j, it, nt0, nt1);
                 const int64_t mt = PAIR ? 2 * it + rank : it;
-                // the thread's rows i = 2 l + s: row0 + 16 l + 8 s
-                const int64_t row0 = mt * kTileM + 32 * q + rq;
+                // the thread's four result streams i = 2 l + s.  Plain: LOS row0 + 16 l + 8 s.
+                // FOLD: LOS row0 + 8 l (its Q and U rows sit 8 lanes apart), s = 0 the +phi
+                // samples and s = 1 the -phi ones.
+                const int64_t row0 = mt * kTileLos + (FOLD ? 16 : 32) * q + rq;
+                auto row_of = [&](int i) { return FOLD ? row0 + 8 * (i >> 1) : row0 + 16 * (i >> 1) + 8 * (i & 1); };
                 float scale[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const int64_t r = row0 + 16 * (i >> 1) + 8 * (i & 1);
+                    const int64_t r = row_of(i);
                     scale[i] = P.out_scale;
                     if (P.rexp != nullptr && r < nlos) scale[i] = ldexpf(scale[i], -(int)P.rexp[r]);
                 }
@@ -746,6 +755,60 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                     if (!ok) break;
                     const int ncols = ((nt == P.ntiles_n - 1) ? P.tile_n_last : P.tile_n) - h * HALF;
                     const int kbase = (nt * P.tile_n + h * HALF) >> 1;
+                    if constexpr (FOLD) {
+                        // The columns are (c, s) of +phi; rows Q and U give sum Q c, Q s, U c, U s:
+                        //   F(+phi) = (Qc + Us) + i (Uc - Qs),  F(-phi) = (Qc - Us) + i (Uc + Qs).
+                        // A row of F starts at any multiple of 8 bytes, so the four lanes of a row
+                        // group, which hold four consecutive samples, would straddle two 32-byte
+                        // sectors on three rows of four.  Lanes whose sample lies in the next sector
+                        // (late) store one step later, next to the following group's first lanes: every
+                        // store then fills one aligned sector (contraction of 262,144 LOS x 360 active
+                        // channels x 401 phi 0.449 -> 0.396 ms, plain BF16 of 400,000 x 800 x 1001 1.70 -> 1.48 ms).
+#pragma unroll
+                        for (int l = 0; l < 2; ++l) {
+                            const int64_t r = row_of(2 * l);
+                            const bool st = P.F != nullptr && r < nlos;
+                            const int64_t orow = st && P.rows ? P.rows[r] : r;
+                            float2 *dp = reinterpret_cast<float2 *>(P.F) + (orow * P.nphi + P.kplus + kbase);
+                            float2 *dm = reinterpret_cast<float2 *>(P.F) + (orow * P.nphi + P.kminus - kbase);
+                            const bool latep = (int)((reinterpret_cast<uintptr_t>(dp) >> 3) & 3) + cq >= 4;
+                            const bool latem = (int)((reinterpret_cast<uintptr_t>(dm) >> 3) & 3) < cq;
+                            dp += cq - (latep ? 4 : 0);
+                            dm -= cq - (latem ? 4 : 0);
+                            float2 prevp = make_float2(0.f, 0.f), prevm = prevp;
+                            bool okp1 = false, okm1 = false;
+#pragma unroll
+                            for (int gg = 0; gg <= NG; ++gg) {
+                                float2 vp = make_float2(0.f, 0.f), vm = vp;
+                                bool okp = false, okm = false;
+                                if (gg < NG) {
+                                    const int c = kbase + 4 * gg + cq;
+                                    okp = 2 * (4 * gg + cq) < ncols && c < P.ncol;
+                                    okm = okp && P.kminus - c != P.kplus + c;   // phi = 0 is its own partner
+                                    const float qc = master[l][gg][0], qs = master[l][gg][1];
+                                    const float uc = master[l][gg][2], us = master[l][gg][3];
+                                    vp = make_float2((qc + us) * scale[2 * l], (uc - qs) * scale[2 * l]);
+                                    vm = make_float2((qc - us) * scale[2 * l], (uc + qs) * scale[2 * l]);
+                                    const float mp = __fadd_rn(__fmul_rn(vp.x, vp.x), __fmul_rn(vp.y, vp.y));
+                                    const float mm = __fadd_rn(__fmul_rn(vm.x, vm.x), __fmul_rn(vm.y, vm.y));
+                                    // lowest index among equals: k ascends on the +phi side and descends on the other
+                                    if (okp && mp > bm[2 * l]) {
+                                        bm[2 * l] = mp; bi[2 * l] = P.kplus + c; br[2 * l] = vp.x; bim[2 * l] = vp.y;
+                                    }
+                                    if (okm && mm >= bm[2 * l + 1]) {
+                                        bm[2 * l + 1] = mm; bi[2 * l + 1] = P.kminus - c;
+                                        br[2 * l + 1] = vm.x; bim[2 * l + 1] = vm.y;
+                                    }
+                                }
+                                if (st) {
+                                    // streaming stores: F is written once and must not push the operands out of L2
+                                    if (latep ? okp1 : okp) __stcs(dp + 4 * gg, latep ? prevp : vp);
+                                    if (latem ? okm1 : okm) __stcs(dm - 4 * gg, latem ? prevm : vm);
+                                }
+                                prevp = vp; prevm = vm; okp1 = okp; okm1 = okm;
+                            }
+                        }
+                    } else {
 #pragma unroll
                     for (int l = 0; l < 2; ++l)
 #pragma unroll
@@ -771,12 +834,19 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                                 }
                             }
                         }
+                    }
                 }
                 if (!ok) break;
-                // the four lanes of a row group hold disjoint columns of the same four rows:
-                // a butterfly leaves every lane with all four rows' peaks (lowest index on ties)
+                // every -phi index is below every +phi one, so the -phi side wins ties
+                if constexpr (FOLD) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                    for (int i = 0; i < 4; i += 2)
+                        if (bm[i + 1] >= bm[i]) { bm[i] = bm[i + 1]; bi[i] = bi[i + 1]; br[i] = br[i + 1]; bim[i] = bim[i + 1]; }
+                }
+                // the four lanes of a row group hold disjoint columns of the same four (FOLD: two)
+                // rows: a butterfly leaves every lane with all their peaks (lowest index on ties)
+#pragma unroll
+                for (int i = 0; i < 4; i += FOLD ? 2 : 1)
 #pragma unroll
                     for (int off = 1; off <= 2; off <<= 1) {
                         const float om = __shfl_xor_sync(0xffffffffu, bm[i], off);
@@ -785,14 +855,15 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                         const float oim = __shfl_xor_sync(0xffffffffu, bim[i], off);
                         if (om > bm[i] || (om == bm[i] && oi < bi[i])) { bm[i] = om; bi[i] = oi; br[i] = ore; bim[i] = oim; }
                     }
-                // lane (rq, cq) now owns row i = cq of its group
+                // lane (rq, cq) now owns row i = cq of its group (FOLD: LOS l = cq, lanes cq > 1 none)
                 float pm = bm[0], pre = br[0], pim = bim[0];
                 int pi = bi[0];
+                const bool owner = !FOLD || cq < 2;
 #pragma unroll
                 for (int i = 1; i < 4; ++i)
-                    if (cq == i) { pm = bm[i]; pi = bi[i]; pre = br[i]; pim = bim[i]; }
-                const int rowq = 16 * (cq >> 1) + rq + 8 * (cq & 1);
-                const int64_t prow = mt * kTileM + 32 * q + rowq;
+                    if ((FOLD ? 2 * cq : cq) == i) { pm = bm[i]; pi = bi[i]; pre = br[i]; pim = bim[i]; }
+                const int rowq = FOLD ? 8 * (cq & 1) + rq : 16 * (cq >> 1) + rq + 8 * (cq & 1);
+                const int64_t prow = owner ? mt * kTileLos + (FOLD ? 16 : 32) * q + rowq : nlos;
                 // combine the two column halves of each row: half 1 publishes, half 0 writes
                 const int par = mt_count & 1;
                 const uint32_t pbar = smem_u32(&S.pkfull[par * 4 + q]);
@@ -800,10 +871,12 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                 const uint32_t use_par = (mt_count >> 1) & 1;
                 if (h == 1) {
                     if (!warp_wait(ebar, use_par ^ 1, S.abort_flag, P.err, P.timeout_ns)) { ok = false; break; }
-                    S.pk_m[(par * 4 + q) * 32 + rowq] = pm;
-                    S.pk_i[(par * 4 + q) * 32 + rowq] = pi;
-                    S.pk_re[(par * 4 + q) * 32 + rowq] = pre;
-                    S.pk_im[(par * 4 + q) * 32 + rowq] = pim;
+                    if (owner) {
+                        S.pk_m[(par * 4 + q) * 32 + rowq] = pm;
+                        S.pk_i[(par * 4 + q) * 32 + rowq] = pi;
+                        S.pk_re[(par * 4 + q) * 32 + rowq] = pre;
+                        S.pk_im[(par * 4 + q) * 32 + rowq] = pim;
+                    }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(pbar);
                 } else {
@@ -1072,11 +1145,6 @@ int gemm_stages(int b_rows, int mode)
 
 bool split_mode(int mode) { return mode != MODE_BF16; }
 
-int mode_of(int precision)
-{
-    return precision == RMS_BF16 ? MODE_BF16 : (precision == RMS_BF16X3 ? MODE_BF16X3 : MODE_FP16X3);
-}
-
 }  // namespace
 
 size_t split_operand_bytes(const rms_plan_s &p, int64_t nlos, int layout)
@@ -1086,6 +1154,11 @@ size_t split_operand_bytes(const rms_plan_s &p, int64_t nlos, int layout)
     const int kb = layout == RMS_CHAN_MAJOR ? p.kblocks : p.kblocks_raw;
     const int64_t nmt = (nlos + kTileM - 1) / kTileM;
     return (size_t)((nmt + 1) & ~(int64_t)1) * kb * (2 * kStageA);
+}
+
+size_t fold_operand_bytes(const rms_plan_s &p, int64_t nlos)
+{
+    return (size_t)((nlos + 2 * kFoldTileLos - 1) / (2 * kFoldTileLos)) * 2 * p.fold.kblocks * (2 * kStageA);
 }
 
 cudaError_t launch_split(const rms_plan_s &p, const SplitOpts &o, cudaStream_t s)
@@ -1137,16 +1210,20 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
 {
     const bool chan = o.layout == RMS_CHAN_MAJOR;
     const int mode = mode_of(p.precision);
-    const int64_t nmt = (o.nlos + kTileM - 1) / kTileM;
+    const bool fold = o.fold;
+    const int tile_los = fold ? kFoldTileLos : kTileM;
+    const int64_t nmt = (o.nlos + tile_los - 1) / tile_los;
     if (nmt < 1) return cudaSuccess;
     const bool rot = o.T != nullptr;
-    if (rot && (mode == MODE_FP16X3 || p.tile_n > 2 * kHalfRot || !o.centre)) return cudaErrorInvalidValue;
+    if (fold && (rot || !p.fold.on)) return cudaErrorInvalidValue;
+    const PhaseTiling &tl = fold ? p.fold.tiles : p.tiles;
+    if (rot && (mode == MODE_FP16X3 || tl.tile_n > 2 * kHalfRot || !o.centre)) return cudaErrorInvalidValue;
     GemmParams P;
     P.A = o.A;
     P.nlos = o.nlos;
     P.count = o.count;
     P.rows = o.rows;
-    P.kblocks = chan ? p.kblocks : p.kblocks_raw;
+    P.kblocks = fold ? p.fold.kblocks : chan ? p.kblocks : p.kblocks_raw;
     // K blocks chained into one TMEM partial before the round-to-nearest fold: the
     // tensor core's accumulation error grows ~4e-8 per chained MMA, which matters for
     // the split precisions only; plain BF16 (error ~1e-3) folds once per N tile.
@@ -1160,6 +1237,9 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
     int ngroups = (P.kblocks + group_max - 1) / group_max;
     P.group = (P.kblocks + ngroups - 1) / ngroups;
     P.nphi = p.nphi;
+    P.ncol = fold ? p.fold.ncol : p.nphi;
+    P.kplus = p.fold.kplus;
+    P.kminus = p.fold.kminus;
     P.F = o.F;
     P.pidx = o.pidx;
     P.pabs = o.pabs;
@@ -1192,15 +1272,18 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
     // one) only for split precisions under the job schedule, where the halved
     // shared-memory traffic wins (LOFAR cube, BF16x3: 0.68 against 0.70 ms
     // channel-major, 0.69 against 0.74 LOS-major; whole schedule 0.87 against 0.75;
-    // plain BF16 0.53 against 0.50).
+    // plain BF16 0.53 against 0.50).  A folded grid has half the phase rows: with three or
+    // more narrow tiles pairs win under the whole schedule too (1536 channels x 801 phi,
+    // BF16x3: 88.5 against 92.3 us for 3,000 LOS, 1.59 against 1.65 ms for 160,000).
     const bool f_at_peak = o.pq || o.pu || o.pchi;
     auto pair_for = [&](bool with_jobs) {
         const bool wanted =
             p.contraction == RMS_CONTRACT_PAIR ||
             (p.contraction == RMS_CONTRACT_AUTO &&
              (pair_default == 2 ||
-              (pair_default == 1 && (p.tile_n2 > 2 * kHalf || (with_jobs && split_mode(mode))))));
-        return !rot && wanted && p.pair_maps;
+              (pair_default == 1 && (tl.tile_n2 > 2 * kHalf ||
+                                     (split_mode(mode) && (with_jobs || (fold && tl.ntiles_n2 > 2)))))));
+        return !rot && wanted && (fold ? p.fold.pair_maps : p.pair_maps);
     };
     int ctas = p.num_sms;
     if (const char *v = std::getenv("RMS_GEMM_CTAS")) {   // tuning knob: persistent CTAs
@@ -1216,7 +1299,7 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
     }();
     const double budget = p.l2_budget > 0 ? (double)p.l2_budget : budget_default;
     const double a_tile = (double)P.kblocks * (split_mode(mode) ? 2 * kStageA : kStageA);
-    const double b_all = (double)p.npad * (chan ? p.kpad : p.kpad_raw) * 2.0 * (split_mode(mode) ? 2 : 1);
+    const double b_all = (double)tl.npad * P.kblocks * kKBlock * 2.0 * (split_mode(mode) ? 2 : 1);
     bool jobs = !rot && o.keys && p.schedule != RMS_SCHEDULE_WHOLE && (o.F || !f_at_peak);
     if (jobs && !o.F && p.schedule == RMS_SCHEDULE_AUTO) {
         // Peak map only: with no F to store, the whole schedule's longer jobs win wherever
@@ -1226,14 +1309,14 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
         const bool pr = pair_for(true);
         const int64_t nitp = pr ? (nmt + 1) / 2 : nmt;
         const int64_t u = std::min<int64_t>(nitp, pr ? std::max(1, ctas / 2) : ctas);
-        const int64_t nt = pr ? p.ntiles_n2 : p.ntiles_n;
+        const int64_t nt = pr ? tl.ntiles_n2 : tl.ntiles_n;
         const double live = (double)((u + nt - 1) / nt + 1) * (pr ? 2.0 : 1.0) * a_tile + b_all;
         if (live <= budget) jobs = false;
     }
     const bool pair = pair_for(jobs);
-    P.ntiles_n = pair ? p.ntiles_n2 : p.ntiles_n;
-    P.tile_n = pair ? p.tile_n2 : p.tile_n;
-    P.tile_n_last = pair ? p.tile_n_last2 : p.tile_n_last;
+    P.ntiles_n = pair ? tl.ntiles_n2 : tl.ntiles_n;
+    P.tile_n = pair ? tl.tile_n2 : tl.tile_n;
+    P.tile_n_last = pair ? tl.tile_n_last2 : tl.tile_n_last;
     const bool wide = pair && P.tile_n > 2 * kHalf;   // the pair kernel with 128 columns per epilogue thread
     P.b_rows = pair ? P.tile_n / 2 : P.tile_n;
     P.stages = gemm_stages(P.b_rows, mode);
@@ -1242,14 +1325,17 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
     const int64_t nit = pair ? (nmt + 1) / 2 : nmt;
     int maxunits = pair ? (ctas / 2 > 0 ? ctas / 2 : 1) : ctas;
     using KernelFn = void (*)(GemmParams, CUtensorMap, CUtensorMap, CUtensorMap);
-    const KernelFn pair_kern = wide ? gemm_kernel<kHalfWide, false, true> : gemm_kernel<kHalf, false, true>;
+    const KernelFn pair_kern =
+        fold ? (wide ? gemm_kernel<kHalfWide, false, true, true> : gemm_kernel<kHalf, false, true, true>)
+             : (wide ? gemm_kernel<kHalfWide, false, true, false> : gemm_kernel<kHalf, false, true, false>);
     if (!rot) {
         // the setmaxnreg shares of the non-window variants add up to 384 x 168 registers:
         // launching one with any other register count would leave its epilogue
         // warpgroups waiting for registers, so check the build once
         static const cudaError_t regs_ok = [] {
-            const KernelFn ks[3] = {gemm_kernel<kHalf, false, false>, gemm_kernel<kHalf, false, true>,
-                                    gemm_kernel<kHalfWide, false, true>};
+            const KernelFn ks[6] = {gemm_kernel<kHalf, false, false, false>,    gemm_kernel<kHalf, false, true, false>,
+                                    gemm_kernel<kHalfWide, false, true, false>, gemm_kernel<kHalf, false, false, true>,
+                                    gemm_kernel<kHalf, false, true, true>,      gemm_kernel<kHalfWide, false, true, true>};
             for (const KernelFn k : ks) {
                 cudaFuncAttributes fa;
                 cudaError_t e1 = cudaFuncGetAttributes(&fa, k);
@@ -1320,20 +1406,21 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
     }
     if (rot) {
         const CUtensorMap &bhi = chan ? p.tmap_bhi : p.tmap_bhi_raw, &blo = chan ? p.tmap_blo : p.tmap_blo_raw;
-        auto kern = gemm_kernel<kHalfRot, true, false>;
+        auto kern = gemm_kernel<kHalfRot, true, false, false>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         kern<<<units, 512, smem, s>>>(P, bhi, blo, bhi);   // (the last map is unused here)
     } else if (pair) {
         if (P.tile_n > 2 * kHalfWide || (P.tile_n & 15) || (P.tile_n_last & 15)) return cudaErrorInvalidValue;
-        const CUtensorMap &bhi = chan ? p.tmap2_bhi : p.tmap2_bhi_raw, &blo = chan ? p.tmap2_blo : p.tmap2_blo_raw;
+        const CUtensorMap &bhi = fold ? p.fold.tmap2_bhi : chan ? p.tmap2_bhi : p.tmap2_bhi_raw;
+        const CUtensorMap &blo = fold ? p.fold.tmap2_blo : chan ? p.tmap2_blo : p.tmap2_blo_raw;
         const int pairs = units;
         // the operand image as a 3-D tensor for the pair's TMA loads: 64-byte rows, 256
         // rows (hi then lo parts) per 16 KB block, one block per (M tile, K block); a
         // stage is one block's first a_rows rows
         CUtensorMap tmA;
         {
-            const int64_t nblocks = (((int64_t)o.nlos + 2 * kTileM - 1) / (2 * kTileM)) * 2 * P.kblocks;
+            const int64_t nblocks = ((nmt + 1) & ~(int64_t)1) * P.kblocks;
             const cuuint64_t dims[3] = {(cuuint64_t)kKBlock, (cuuint64_t)(2 * kTileM), (cuuint64_t)nblocks};
             const cuuint64_t strides[2] = {(cuuint64_t)kRowBytes, (cuuint64_t)(2 * kStageA)};
             const cuuint32_t box[3] = {(cuuint32_t)kKBlock, (cuuint32_t)(split_mode(mode) ? 2 * kTileM : kTileM), 1};
@@ -1358,9 +1445,10 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
         e = cudaLaunchKernelEx(&cfg, pair_kern, P, bhi, blo, tmA);
         if (e != cudaSuccess) return e;
     } else {
-        if (p.tile_n > 2 * kHalf) return cudaErrorInvalidValue;
-        const CUtensorMap &bhi = chan ? p.tmap_bhi : p.tmap_bhi_raw, &blo = chan ? p.tmap_blo : p.tmap_blo_raw;
-        auto kern = gemm_kernel<kHalf, false, false>;
+        if (P.tile_n > 2 * kHalf) return cudaErrorInvalidValue;
+        const CUtensorMap &bhi = fold ? p.fold.tmap_bhi : chan ? p.tmap_bhi : p.tmap_bhi_raw;
+        const CUtensorMap &blo = fold ? p.fold.tmap_blo : chan ? p.tmap_blo : p.tmap_blo_raw;
+        auto kern = fold ? gemm_kernel<kHalf, false, false, true> : gemm_kernel<kHalf, false, false, false>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         kern<<<units, kThreads, smem, s>>>(P, bhi, blo, bhi);   // (the last map is unused here)
@@ -1400,21 +1488,27 @@ cudaError_t launch_split_gemm(const rms_plan_s &p, const float *Q, const float *
                               cudaStream_t s, cudaEvent_t ev_mid, float *pq, float *pu, float *pchi,
                               unsigned long long *keys)
 {
-    SplitOpts so;
-    so.Q = Q;
-    so.U = U;
-    so.nlos_src = nlos;
-    so.nout = nlos;
-    so.layout = layout;
-    so.A = A;
-    so.rexp = rexp;
-    cudaError_t e = launch_split(p, so, s);
+    cudaError_t e;
+    if (p.fold.on) {
+        e = launch_fold_split(p, Q, U, nlos, layout, A, rexp, s);
+    } else {
+        SplitOpts so;
+        so.Q = Q;
+        so.U = U;
+        so.nlos_src = nlos;
+        so.nout = nlos;
+        so.layout = layout;
+        so.A = A;
+        so.rexp = rexp;
+        e = launch_split(p, so, s);
+    }
     if (e != cudaSuccess) return e;
     if (ev_mid && (e = cudaEventRecord(ev_mid, s)) != cudaSuccess) return e;
     GemmOpts go;
     go.A = A;
     go.nlos = nlos;
     go.layout = layout;
+    go.fold = p.fold.on;
     go.F = F;
     go.pidx = pidx;
     go.pabs = pabs;

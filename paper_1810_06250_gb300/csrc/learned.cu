@@ -288,8 +288,10 @@ rms_status rms_peakmap_learned(rms_window_t w, rms_net_t net, const float *Q, co
     const size_t ib = up(split_operand_bytes(p, nlos, layout));
     const size_t n4 = up((size_t)nlos * 4), n8 = up((size_t)nlos * 8);
     const size_t hb = up((size_t)nlos * net->hidden * 2);
+    // the fallback rows' image: folded like rms_synth's wherever the plan's grid folds
+    const size_t ib_fb = p.fold.on ? up(fold_operand_bytes(p, nlos)) : ib;
     // image | fallback image | h | rscale | bin | conf | centre | widx | wabs | rows | count | peak keys
-    const size_t total = 2 * ib + hb + 7 * n4 + 2 * n8 + 256;
+    const size_t total = ib + ib_fb + hb + 7 * n4 + 2 * n8 + 256;
     uint8_t *scr = nullptr;
     cudaError_t e = cudaStreamWaitEvent(s, net->last, 0);
     if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void **>(&scr), total, s);
@@ -298,7 +300,7 @@ rms_status rms_peakmap_learned(rms_window_t w, rms_net_t net, const float *Q, co
         return from_cuda(e);
     }
     uint8_t *img = scr, *img_fb = scr + ib;
-    uint8_t *q = scr + 2 * ib;
+    uint8_t *q = scr + ib + ib_fb;
     uint16_t *h = reinterpret_cast<uint16_t *>(q);
     q += hb;
     float *rs = reinterpret_cast<float *>(q);
@@ -363,7 +365,9 @@ rms_status rms_peakmap_learned(rms_window_t w, rms_net_t net, const float *Q, co
         merge_kernel<<<g256, 256, 0, s>>>(M);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = launch_image_gather(p, layout, img, rows, count, nlos, img_fb, s);
+    if (e == cudaSuccess)
+        e = p.fold.on ? launch_fold_split(p, Q, U, nlos, layout, img_fb, nullptr, s, rows, count)
+                      : launch_image_gather(p, layout, img, rows, count, nlos, img_fb, s);
     if (e == cudaSuccess) {
         GemmOpts go;
         go.A = img_fb;
@@ -371,6 +375,7 @@ rms_status rms_peakmap_learned(rms_window_t w, rms_net_t net, const float *Q, co
         go.count = count;
         go.rows = rows;
         go.layout = layout;
+        go.fold = p.fold.on;
         go.pabs = peak_abs;
         go.pphi = phi_peak;
         go.keys = keys;

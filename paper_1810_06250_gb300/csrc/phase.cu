@@ -122,6 +122,26 @@ __global__ void phase_bsplit_kernel(const double *__restrict__ dl2, const double
     }
 }
 
+// Folded operand, K-major [npad][kpad]: row 2i holds c and row 2i + 1 holds s of depth
+// dh[i], column a the a-th active channel, (c, s) = (w_a / w_max) (cos, sin)(theta).
+template <typename T>
+__global__ void phase_fold_kernel(const double *__restrict__ dl2, const double *__restrict__ w,
+                                  const double *__restrict__ dh, int32_t nact, int32_t ncol, double inv_wmax,
+                                  int32_t kpad, uint16_t *__restrict__ bhi, uint16_t *__restrict__ blo)
+{
+    const int64_t total = (int64_t)nact * ncol;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t i = (int32_t)(t / nact), a = (int32_t)(t % nact);
+        double s, c;
+        phase_sincos(dh[i], dl2[a], &s, &c);
+        const double wn = w[a] * inv_wmax;
+        const size_t r0 = (size_t)(2 * i) * kpad + a, r1 = r0 + kpad;
+        split16<T>(wn * c, bhi + r0, blo + r0);
+        split16<T>(wn * s, bhi + r1, blo + r1);
+    }
+}
+
 // R(phi_k) = K sum_j w_j exp(-i theta_jk), Eq. Rsum, accumulated in FP64.
 __global__ void rmsf_kernel(const double *__restrict__ dl2, const double *__restrict__ w,
                             int32_t nact, double K, const double *__restrict__ phi, int32_t n,
@@ -163,7 +183,7 @@ cudaError_t launch_phase_table(const rms_plan_s &p, cudaStream_t s)
 cudaError_t launch_phase_bsplit(const rms_plan_s &p, const double *dl2, const double *w, int32_t nk,
                                 int32_t kpad, uint16_t *bhi, uint16_t *blo, bool fp16, cudaStream_t s)
 {
-    size_t bytes = (size_t)p.npad * kpad * sizeof(uint16_t);
+    size_t bytes = (size_t)p.tiles.npad * kpad * sizeof(uint16_t);
     cudaError_t e = cudaMemsetAsync(bhi, 0, bytes, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(blo, 0, bytes, s);
     if (e != cudaSuccess) return e;
@@ -175,6 +195,23 @@ cudaError_t launch_phase_bsplit(const rms_plan_s &p, const double *dl2, const do
     else
         phase_bsplit_kernel<__nv_bfloat16><<<grid_for(total, 256), 256, 0, s>>>(dl2, w, p.d_phi, nk, p.nphi, inv,
                                                                                  kpad, bhi, blo);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_phase_fold(const rms_plan_s &p, const double *dh, bool fp16, cudaStream_t s)
+{
+    const FoldPlan &f = p.fold;
+    const size_t bytes = (size_t)f.tiles.npad * f.kpad * sizeof(uint16_t);
+    cudaError_t e = cudaMemsetAsync(f.d_hi, 0, bytes, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(f.d_lo, 0, bytes, s);
+    if (e != cudaSuccess) return e;
+    const int g = grid_for((int64_t)p.nact * f.ncol, 256);
+    const double inv = 1.0 / p.wmax;
+    if (fp16)
+        phase_fold_kernel<__half><<<g, 256, 0, s>>>(p.d_dl2, p.d_wact, dh, p.nact, f.ncol, inv, f.kpad, f.d_hi, f.d_lo);
+    else
+        phase_fold_kernel<__nv_bfloat16>
+            <<<g, 256, 0, s>>>(p.d_dl2, p.d_wact, dh, p.nact, f.ncol, inv, f.kpad, f.d_hi, f.d_lo);
     return cudaGetLastError();
 }
 

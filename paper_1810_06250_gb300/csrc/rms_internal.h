@@ -23,6 +23,34 @@ constexpr int kGroupKBlocks = 16;  // K blocks accumulated in TMEM before the FP
                                    // per-LOS error on the MWA cube 4.6e-6 (BF16x3) / 3.8e-6 (FP16x3) at 16,
                                    // 4.4e-6 / 1.8e-6 at 8, 6.1e-6 / 8.3e-6 at 32
 
+constexpr int kFoldTileLos = 64;   // folded grids: an M tile's 128 rows are the Q and U rows of 64 LOS
+
+// Operand arithmetic of the tensor-core precisions.
+enum { MODE_BF16 = 0, MODE_BF16X3 = 1, MODE_FP16X3 = 2 };
+inline int mode_of(int precision)
+{
+    return precision == RMS_BF16 ? MODE_BF16 : (precision == RMS_BF16X3 ? MODE_BF16X3 : MODE_FP16X3);
+}
+
+// Tiles of a phase matrix's rows: up to 208 rows for single CTAs, up to 256 (n2) for CTA pairs.
+struct PhaseTiling {
+    int32_t npad = 0, tile_n = 0, ntiles_n = 0, tile_n_last = 0;
+    int32_t tile_n2 = 0, ntiles_n2 = 0, tile_n_last2 = 0;
+};
+
+// The folded phase matrix of a symmetric phi grid (phi_k + phi_{nphi-1-k} = 0): rows
+// (c, s) = (w / w_max) (cos, sin)(theta) of the ncol depths phi >= 0, columns the active
+// channels, which the contraction multiplies with Q and U rows of their own (fold.cu).
+struct FoldPlan {
+    bool on = false, pair_maps = false;
+    int32_t ncol = 0;              // ceil(nphi / 2)
+    int32_t kplus = 0, kminus = 0; // column pair i holds phi samples kplus + i and kminus - i
+    int32_t kblocks = 0, kpad = 0; // K blocks of 32 active channels
+    PhaseTiling tiles;
+    uint16_t *d_hi = nullptr, *d_lo = nullptr;   // [tiles.npad][kpad]
+    CUtensorMap tmap_bhi, tmap_blo, tmap2_bhi, tmap2_blo;
+};
+
 struct rms_plan_s {
     int device = 0;
     int32_t nchan = 0, nact = 0, nphi = 0, precision = 0;
@@ -44,9 +72,10 @@ struct rms_plan_s {
     double *d_R64 = nullptr;       // [nphi][2]
     float2 *d_czt = nullptr;       // chirp-z constants: H [M], twiddles [2 M], g [nchan], v [nphi]
     int32_t czt_M = 0;             // chirp-z FFT length
-    int32_t kpad = 0, npad = 0, tile_n = 0, ntiles_n = 0, tile_n_last = 0, kblocks = 0;
-    // the tiling of the two-CTA contraction: up to 256 phase rows per tile (npad covers both)
-    int32_t tile_n2 = 0, ntiles_n2 = 0, tile_n_last2 = 0;
+    int32_t kpad = 0, kblocks = 0;
+    PhaseTiling tiles;      // npad covers both tilings
+    FoldPlan fold;
+    double *d_dh = nullptr;        // [fold.ncol] the folded grid's depths phi >= 0
     CUtensorMap tmap_bhi;   // CUtensorMap is 64-byte aligned by its own declaration
     CUtensorMap tmap_blo;
     // LOS-major cubes contract over all channels (flagged ones zeroed in the
@@ -104,6 +133,8 @@ struct rms_plan_s {
 cudaError_t launch_phase_table(const rms_plan_s &p, cudaStream_t s);
 cudaError_t launch_phase_bsplit(const rms_plan_s &p, const double *dl2, const double *w, int32_t nk,
                                 int32_t kpad, uint16_t *bhi, uint16_t *blo, bool fp16, cudaStream_t s);
+// the folded phase matrix: depths dh[ncol] (device), active channels
+cudaError_t launch_phase_fold(const rms_plan_s &p, const double *dh, bool fp16, cudaStream_t s);
 cudaError_t launch_rotation_table(const double *dl2, int32_t nk, int32_t ld, double phi0, double step,
                                   int32_t ncentre, float2 *T, cudaStream_t s);
 cudaError_t launch_rmsf(const rms_plan_s &p, const double *d_phi, int32_t n, double *d_R64,
@@ -136,6 +167,12 @@ rms_status check_synth_args(rms_plan_t p, const float *Q, const float *U, int64_
 // Split operand image: [ceil(rows / 128)][kblocks][16 KB], K blocks of 16 channels
 // (kblocks of the plan for channel-major cubes, kblocks_raw for LOS-major ones).
 size_t split_operand_bytes(const rms_plan_s &p, int64_t nlos, int layout);
+// Operand image of a folded grid: [ceil(nlos / 128) 2][fold.kblocks][16 KB], tiles of 64 LOS (fold.cu);
+// rows, count: optional gather of *count (<= nlos) LOS, as SplitOpts.
+size_t fold_operand_bytes(const rms_plan_s &p, int64_t nlos);
+cudaError_t launch_fold_split(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout,
+                              uint8_t *A, int8_t *rexp, cudaStream_t s, const int64_t *rows = nullptr,
+                              const int64_t *count = nullptr);
 struct SplitOpts {
     const float *Q = nullptr, *U = nullptr;
     int64_t nlos_src = 0;              // lines of sight in the cube
@@ -154,6 +191,7 @@ struct GemmOpts {
     const int64_t *count = nullptr;    // optional device count (<= nlos) of live rows
     const int64_t *rows = nullptr;     // optional scatter of results: row r -> rows[r]
     int layout = RMS_CHAN_MAJOR;
+    bool fold = false;                 // A is a folded image (plans with fold.on)
     float *F = nullptr;
     int32_t *pidx = nullptr;
     float *pabs = nullptr, *pphi = nullptr;

@@ -63,7 +63,6 @@ constexpr int kEpiStageBytes = kNumEpiWarps * 32 * kEpiLd * 4;
 constexpr int kSmemLimit = 227 * 1024;
 constexpr int kRegsLow = 96, kRegsHigh = 160;       // setmaxnreg split: 256*96 + 256*160 = 512*128
 
-enum { MODE_BF16 = 0, MODE_BF16X3 = 1, MODE_FP16X3 = 2 };
 
 struct UmmaParams {
     const float *Q, *U;
@@ -784,9 +783,9 @@ cudaError_t launch_umma(const rms_plan_s &p, const float *Q, const float *U, int
     int ngroups = (P.kblocks + kUmmaGroupKBlocks - 1) / kUmmaGroupKBlocks;
     P.group = (P.kblocks + ngroups - 1) / ngroups;
     P.nphi = p.nphi;
-    P.ntiles_n = p.ntiles_n;
-    P.tile_n = p.tile_n;
-    P.tile_n_last = p.tile_n_last;
+    P.ntiles_n = p.tiles.ntiles_n;
+    P.tile_n = p.tiles.tile_n;
+    P.tile_n_last = p.tiles.tile_n_last;
     P.F = F;
     P.pidx = pidx;
     P.pabs = pabs;
@@ -807,14 +806,14 @@ cudaError_t launch_umma(const rms_plan_s &p, const float *Q, const float *U, int
     P.use_tma = encode_data_map(&tq, Q, nlos, p.nchan, layout) && encode_data_map(&tu, U, nlos, p.nchan, layout);
     P.sd = P.use_tma ? 3 : 0;
     P.sa = 3;
-    P.sb = umma_bstages(p.tile_n, P.sd, P.sa);
+    P.sb = umma_bstages(p.tiles.tile_n, P.sd, P.sa);
     // Reloading from scratch is safe when a converter's write of K block kb for the
     // next M tile is ordered after the bulk copy that last read it: the converter
     // waits for the A slot used sa stages earlier, which is at or after that copy's
     // stage when kblocks >= sa.
-    P.reuse = (p.ntiles_n > 1 && P.kblocks >= P.sa && p.d_scratch != nullptr) ? 1 : 0;
+    P.reuse = (p.tiles.ntiles_n > 1 && P.kblocks >= P.sa && p.d_scratch != nullptr) ? 1 : 0;
     if (P.sb < 2) return cudaErrorInvalidConfiguration;
-    size_t smem = umma_smem_bytes(p.tile_n, P.sd, P.sa, P.sb);
+    size_t smem = umma_smem_bytes(p.tiles.tile_n, P.sd, P.sa, P.sb);
     cudaError_t e = cudaFuncSetAttribute(umma_synth_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int64_t nmt = (nlos + kTileM - 1) / kTileM;
