@@ -287,6 +287,26 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
     RMS_TRY(cudaMemcpy(p->d_l2x32, l2x32.data(), p->nact * sizeof(float), cudaMemcpyHostToDevice));
     RMS_TRY(cudaMemcpy(p->d_w32, w32.data(), p->nact * sizeof(float), cudaMemcpyHostToDevice));
 
+    // A phi grid symmetric about zero folds: cos is even and sin odd in phi, so one pair
+    // (c, s) serves phi and -phi.  Accepted when no phase moves by more than 1e-9 rad (the
+    // products' own FP64 rounding is of that order on wide bands); the on-the-fly path
+    // computes with FP32 depths, which then have to be exact negatives.
+    {
+        double xmax = 0.0, off = 0.0;
+        bool exact32 = true;
+        for (double x : dl2) xmax = std::fmax(xmax, std::fabs(x));
+        for (int k = 0; 2 * k < nphi; ++k) {
+            off = std::fmax(off, std::fabs(phi[k] + phi[nphi - 1 - k]));
+            if (2 * k + 1 != nphi && phi32[k] != -phi32[nphi - 1 - k]) exact32 = false;
+        }
+        p->fold.on = max_tile_cap == kMaxTileN && off * xmax <= 1e-9 &&
+                     (is_tensor(precision) || precision == RMS_FP32_SIMT_TABLE ||
+                      (precision == RMS_FP32_SIMT_FLY && exact32));
+        p->fold.ncol = (nphi + 1) / 2;
+        p->fold.kplus = nphi / 2;
+        p->fold.kminus = (nphi - 1) / 2;
+    }
+
     if (precision == RMS_FP32_SIMT_TABLE) {
         RMS_TRY(dalloc(&p->d_table, (size_t)p->nact * nphi));
         RMS_TRY(launch_phase_table(*p, 0));
@@ -367,17 +387,8 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
                            encode_b_map(&p->tmap2_bhi_raw, p->d_bhi_raw, p->kpad_raw, p->tiles.npad, h) &&
                            encode_b_map(&p->tmap2_blo_raw, p->d_blo_raw, p->kpad_raw, p->tiles.npad, h);
         }
-        // A phi grid symmetric about zero folds: cos is even and sin odd in phi, so one
-        // column pair (c, s) serves phi and -phi.  Accepted when no phase moves by more
-        // than 1e-9 rad (the products' own FP64 rounding is of that order on wide bands).
-        double xmax = 0.0, off = 0.0;
-        for (double x : dl2) xmax = std::fmax(xmax, std::fabs(x));
-        for (int k = 0; 2 * k < nphi; ++k) off = std::fmax(off, std::fabs(phi[k] + phi[nphi - 1 - k]));
-        if (max_tile_cap == kMaxTileN && off * xmax <= 1e-9) {
+        if (p->fold.on) {
             FoldPlan &f = p->fold;
-            f.ncol = (nphi + 1) / 2;
-            f.kplus = nphi / 2;
-            f.kminus = (nphi - 1) / 2;
             f.kblocks = (p->nact + kKBlock - 1) / kKBlock;
             f.kpad = f.kblocks * kKBlock;
             both_tilings(2 * f.ncol, f.tiles);
@@ -396,7 +407,6 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
             }
             f.pair_maps = encode_b_map(&f.tmap2_bhi, f.d_hi, f.kpad, f.tiles.npad, h) &&
                           encode_b_map(&f.tmap2_blo, f.d_lo, f.kpad, f.tiles.npad, h);
-            f.on = true;
         }
     }
     RMS_TRY(cudaEventCreateWithFlags(&p->last, cudaEventDisableTiming));

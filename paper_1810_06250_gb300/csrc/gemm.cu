@@ -700,9 +700,8 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                 int nt0, nt1;
                 job_of(P, nit, j, it, nt0, nt1);
                 const int64_t mt = PAIR ? 2 * it + rank : it;
-                // the thread's four result streams i = 2 l + s.  Plain: LOS row0 + 16 l + 8 s.
-                // FOLD: LOS row0 + 8 l (its Q and U rows sit 8 lanes apart), s = 0 the +phi
-                // samples and s = 1 the -phi ones.
+                // the thread's rows i = 2 l + s: LOS row0 + 16 l + 8 s, or FOLD: LOS row0 + 8 l
+                // (i = 2 l only), whose Q and U rows sit 8 lanes apart
                 const int64_t row0 = mt * kTileLos + (FOLD ? 16 : 32) * q + rq;
                 auto row_of = [&](int i) { return FOLD ? row0 + 8 * (i >> 1) : row0 + 16 * (i >> 1) + 8 * (i & 1); };
                 float scale[4];
@@ -791,13 +790,12 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                                     vm = make_float2((qc - us) * scale[2 * l], (uc + qs) * scale[2 * l]);
                                     const float mp = __fadd_rn(__fmul_rn(vp.x, vp.x), __fmul_rn(vp.y, vp.y));
                                     const float mm = __fadd_rn(__fmul_rn(vm.x, vm.x), __fmul_rn(vm.y, vm.y));
-                                    // lowest index among equals: k ascends on the +phi side and descends on the other
+                                    // lowest index among equals: a +phi index is above, a -phi one below all before it
                                     if (okp && mp > bm[2 * l]) {
                                         bm[2 * l] = mp; bi[2 * l] = P.kplus + c; br[2 * l] = vp.x; bim[2 * l] = vp.y;
                                     }
-                                    if (okm && mm >= bm[2 * l + 1]) {
-                                        bm[2 * l + 1] = mm; bi[2 * l + 1] = P.kminus - c;
-                                        br[2 * l + 1] = vm.x; bim[2 * l + 1] = vm.y;
+                                    if (okm && mm >= bm[2 * l]) {
+                                        bm[2 * l] = mm; bi[2 * l] = P.kminus - c; br[2 * l] = vm.x; bim[2 * l] = vm.y;
                                     }
                                 }
                                 if (st) {
@@ -837,12 +835,6 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                     }
                 }
                 if (!ok) break;
-                // every -phi index is below every +phi one, so the -phi side wins ties
-                if constexpr (FOLD) {
-#pragma unroll
-                    for (int i = 0; i < 4; i += 2)
-                        if (bm[i + 1] >= bm[i]) { bm[i] = bm[i + 1]; bi[i] = bi[i + 1]; br[i] = br[i + 1]; bim[i] = bim[i + 1]; }
-                }
                 // the four lanes of a row group hold disjoint columns of the same four (FOLD: two)
                 // rows: a butterfly leaves every lane with all their peaks (lowest index on ties)
 #pragma unroll

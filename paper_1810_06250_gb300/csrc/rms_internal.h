@@ -38,8 +38,8 @@ struct PhaseTiling {
     int32_t tile_n2 = 0, ntiles_n2 = 0, tile_n_last2 = 0;
 };
 
-// The folded phase matrix of a symmetric phi grid (phi_k + phi_{nphi-1-k} = 0): rows
-// (c, s) = (w / w_max) (cos, sin)(theta) of the ncol depths phi >= 0, columns the active
+// A symmetric phi grid (phi_k + phi_{nphi-1-k} = 0), and the tensor-core precisions'
+// folded phase matrix: rows (c, s) = (w / w_max) (cos, sin)(theta) of the ncol depths phi >= 0, columns the active
 // channels, which the contraction multiplies with Q and U rows of their own (fold.cu).
 struct FoldPlan {
     bool on = false, pair_maps = false;

@@ -11,6 +11,13 @@
 //   FLY   : (cos, sin) = sincosf(phi_k * 2(lambda_j^2 - lambda_0^2)) in FP32
 //           (the paper's method, argument and reduction in FP32);
 //   TABLE : (cos, sin) read from the plan's FP32 table built in FP64.
+// On a phi grid symmetric about zero (FOLD) cos is even and sin odd in phi, so
+// the four sums Qc, Qs, Uc, Us of a depth phi >= 0 give F at +phi and -phi:
+// 4 FMAs per (LOS, channel) for two outputs instead of 8.  The register tile is
+// then 8 LOS x 4 pairs, 128 FMAs per channel for 6 vector loads, and the copies
+// weigh twice as much: channel-major cubes whose rows start on 16 bytes copy 4 LOS
+// at a time.  262,144 LOS x 360 active channels x 401 phi: table 6.82 -> 3.61 ms,
+// on the fly 6.97 -> 3.70 ms (rows not aligned 4.58, LOS-major 7.05 -> 4.64 ms).
 // The peak of |F| (Sec. 2.2) is reduced in registers over the block's phi
 // tiles, so F never has to be re-read.
 #include <limits.h>
@@ -20,7 +27,8 @@
 namespace {
 
 constexpr int TL = 256;   // lines of sight per block (32 thread rows x 8)
-constexpr int TP = 64;    // phi per tile (8 thread columns x 8, as 4 pairs at stride 16)
+constexpr int TP = 64;    // phi per tile (8 thread columns x 8, as 4 pairs at stride 16);
+                          // folded: 32 phi columns, each a +-phi pair (8 thread columns x 4)
 constexpr int CH = 16;    // channels per chunk
 constexpr int LDQ = TL + 4;
 
@@ -42,6 +50,9 @@ struct SimtArgs {
     const float *phi32;    // [nphi]
     const float2 *table;   // [nact][nphi]
     float scale;           // K
+    int32_t ncol;          // phi columns: nphi, or folded the ceil(nphi / 2) depths phi >= 0
+    int32_t kplus, kminus; // column i is sample kplus + i (folded: and kminus - i)
+    int32_t vec4;          // channel-major rows start on 16 bytes: 4 LOS per copy
     float *F;
     int32_t *pidx;
     float *pabs, *pphi;
@@ -52,7 +63,7 @@ __device__ __forceinline__ bool better(float m, int i, float bm, int bi)
     return m > bm || (m == bm && i < bi);
 }
 
-// asynchronous global -> shared copy of 4 or 8 bytes; a false predicate
+// asynchronous global -> shared copy of 4, 8 or 16 bytes; a false predicate
 // writes zeros and reads nothing (the source is then any valid address)
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void *dst, const void *src, bool ok)
@@ -89,12 +100,24 @@ __device__ __forceinline__ int32_t load_active(const SimtArgs &a, int c0, int ti
 }
 
 // fill stage st with channel chunk c0 and phi tile p0 of the block's lines of sight
-template <bool FLY, int LAYOUT>
+template <bool FLY, bool FOLD, int LAYOUT>
 __device__ __forceinline__ void issue(const SimtArgs &a, Stage &st, int64_t l0, int c0, int p0, int32_t act,
                                       int tid)
 {
     const int c = issue_ch<LAYOUT>(tid);
-    if (LAYOUT == RMS_CHAN_MAJOR) {
+    constexpr int W = FOLD ? TP / 2 : TP;
+    if (LAYOUT == RMS_CHAN_MAJOR && a.vec4) {
+        // 16 threads per channel, each 4 x 4 LOS (256-byte runs along LOS; nlos is a
+        // multiple of 4, so a group of 4 is whole or beyond the end)
+#pragma unroll
+        for (int r = 0; r < TL / (256 / CH) / 4; ++r) {
+            const int m = 4 * (tid % (256 / CH) + r * (256 / CH));
+            const bool ok = act >= 0 && l0 + m < a.nlos;
+            const int64_t off = ok ? (int64_t)act * a.nlos + l0 + m : 0;
+            cp_async<16>(&st.q[c][m], a.Q + off, ok);
+            cp_async<16>(&st.u[c][m], a.U + off, ok);
+        }
+    } else if (LAYOUT == RMS_CHAN_MAJOR) {
         // 16 threads per channel, each 16 LOS at stride 16 (64-byte runs along LOS)
 #pragma unroll 4
         for (int r = 0; r < TL / (256 / CH); ++r) {
@@ -117,10 +140,10 @@ __device__ __forceinline__ void issue(const SimtArgs &a, Stage &st, int64_t l0, 
     }
     if (!FLY) {
 #pragma unroll
-        for (int i = tid; i < CH * TP; i += 256) {
-            const int c = i / TP, k = i % TP;
-            const bool ok = c0 + c < a.nact && p0 + k < a.nphi;
-            const int64_t off = ok ? (int64_t)(c0 + c) * a.nphi + p0 + k : 0;
+        for (int i = tid; i < CH * W; i += 256) {
+            const int c = i / W, k = i % W;
+            const bool ok = c0 + c < a.nact && p0 + k < a.ncol;
+            const int64_t off = ok ? (int64_t)(c0 + c) * a.nphi + a.kplus + p0 + k : 0;
             cp_async<8>(&st.cs[c][k], a.table + off, ok);
         }
     }
@@ -129,29 +152,32 @@ __device__ __forceinline__ void issue(const SimtArgs &a, Stage &st, int64_t l0, 
 // on-the-fly phases: the operands of a thread's CH * TP / 256 phase-tile
 // entries are loaded one chunk ahead and turned into (w cos, w sin) after the
 // current chunk's accumulation, so their load latency is hidden behind it
-constexpr int kFlyPer = CH * TP / 256;
+template <bool FOLD>
 struct FlyOps {
-    float ph[kFlyPer], l2[kFlyPer], w[kFlyPer];
+    static constexpr int W = FOLD ? TP / 2 : TP, kPer = CH * W / 256;
+    float ph[kPer], l2[kPer], w[kPer];
 };
 
-__device__ __forceinline__ void fly_load(const SimtArgs &a, FlyOps &o, int c0, int p0, int tid)
+template <bool FOLD>
+__device__ __forceinline__ void fly_load(const SimtArgs &a, FlyOps<FOLD> &o, int c0, int p0, int tid)
 {
 #pragma unroll
-    for (int r = 0; r < kFlyPer; ++r) {
-        const int i = tid + 256 * r, c = i / TP, k = i % TP;
-        const bool ok = c0 + c < a.nact && p0 + k < a.nphi;
+    for (int r = 0; r < FlyOps<FOLD>::kPer; ++r) {
+        const int i = tid + 256 * r, c = i / FlyOps<FOLD>::W, k = i % FlyOps<FOLD>::W;
+        const bool ok = c0 + c < a.nact && p0 + k < a.ncol;
         // a padded entry gets weight 0 (and phase 0), hence (0, 0)
-        o.ph[r] = ok ? __ldg(a.phi32 + p0 + k) : 0.f;
+        o.ph[r] = ok ? __ldg(a.phi32 + a.kplus + p0 + k) : 0.f;
         o.l2[r] = ok ? __ldg(a.l2x + c0 + c) : 0.f;
         o.w[r] = ok ? __ldg(a.w32 + c0 + c) : 0.f;
     }
 }
 
-__device__ __forceinline__ void fly_store(Stage &st, const FlyOps &o, int tid)
+template <bool FOLD>
+__device__ __forceinline__ void fly_store(Stage &st, const FlyOps<FOLD> &o, int tid)
 {
 #pragma unroll
-    for (int r = 0; r < kFlyPer; ++r) {
-        const int i = tid + 256 * r, c = i / TP, k = i % TP;
+    for (int r = 0; r < FlyOps<FOLD>::kPer; ++r) {
+        const int i = tid + 256 * r, c = i / FlyOps<FOLD>::W, k = i % FlyOps<FOLD>::W;
         float sn, cs;
         sincosf(o.ph[r] * o.l2[r], &sn, &cs);
         st.cs[c][k] = make_float2(o.w[r] * cs, o.w[r] * sn);
@@ -165,26 +191,30 @@ struct Pipe {
     int32_t act;    // active-channel index for the next copy
 };
 
-// One phi tile starting at p0: accumulate all channel chunks, then scale, store
-// and update the running peak.  JJ: phi pairs-of-16 of the tile that hold grid
-// points (4 for a full tile; the last, partial tile drops the columns beyond).
-template <int JJ, bool FLY, int LAYOUT>
-__device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_t l0, int p0, Pipe &pp, FlyOps &fo,
-                                         float (&bm)[8], int (&bi)[8])
+// One phi tile starting at column p0: accumulate all channel chunks, then scale,
+// store and update the running peak.  JJ: pairs-of-16 columns of the tile that hold
+// grid points (4, folded 2, for a full tile; the last, partial tile drops the columns
+// beyond).
+template <int JJ, bool FLY, bool FOLD, int LAYOUT>
+__device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_t l0, int p0, Pipe &pp,
+                                         FlyOps<FOLD> &fo, float (&bm)[8], int (&bi)[8])
 {
-    constexpr int NJ = 2 * JJ;
+    constexpr int NJ = 2 * JJ, W = FOLD ? TP / 2 : TP, NS = FOLD ? 4 : 2;
     const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
-    float re[8][NJ], im[8][NJ];
+    // sums of a (LOS, column): Re, Im of F, or folded Qc, Us, Uc, Qs
+    float acc[8][NJ][NS];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) { re[i][j] = 0.f; im[i][j] = 0.f; }
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+            for (int x = 0; x < NS; ++x) acc[i][j][x] = 0.f;
 
     for (int ck = 0; ck < pp.nck; ++ck, ++pp.t) {
         const int n = pp.t + 1;
         if (n < pp.total) {
-            issue<FLY, LAYOUT>(a, stage[n & 1], l0, (n % pp.nck) * CH, (n / pp.nck) * TP, pp.act, tid);
-            if (FLY) fly_load(a, fo, (n % pp.nck) * CH, (n / pp.nck) * TP, tid);
+            issue<FLY, FOLD, LAYOUT>(a, stage[n & 1], l0, (n % pp.nck) * CH, (n / pp.nck) * W, pp.act, tid);
+            if (FLY) fly_load<FOLD>(a, fo, (n % pp.nck) * CH, (n / pp.nck) * W, tid);
             if (n + 1 < pp.total) pp.act = load_active<LAYOUT>(a, ((n + 1) % pp.nck) * CH, tid);
         }
         cp_commit();
@@ -207,37 +237,57 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_
             for (int i = 0; i < 8; ++i)
 #pragma unroll
                 for (int j = 0; j < NJ; ++j) {
+                    float(&s)[NS] = acc[i][j];
                     // (q + iu)(c - is): Re += q c + u s, Im += u c - q s  (Eqs. qPhi, uPhi)
-                    re[i][j] = fmaf(qv[i], cv[j], re[i][j]);
-                    re[i][j] = fmaf(uv[i], sv[j], re[i][j]);
-                    im[i][j] = fmaf(uv[i], cv[j], im[i][j]);
-                    im[i][j] = fmaf(-qv[i], sv[j], im[i][j]);
+                    if constexpr (FOLD) {
+                        s[0] = fmaf(qv[i], cv[j], s[0]);
+                        s[1] = fmaf(uv[i], sv[j], s[1]);
+                        s[2] = fmaf(uv[i], cv[j], s[2]);
+                        s[3] = fmaf(qv[i], sv[j], s[3]);
+                    } else {
+                        s[0] = fmaf(qv[i], cv[j], s[0]);
+                        s[0] = fmaf(uv[i], sv[j], s[0]);
+                        s[1] = fmaf(uv[i], cv[j], s[1]);
+                        s[1] = fmaf(-qv[i], sv[j], s[1]);
+                    }
                 }
         }
         // stage n & 1 was last read before the previous trailing barrier
-        if (FLY && n < pp.total) fly_store(stage[n & 1], fo, tid);
+        if (FLY && n < pp.total) fly_store<FOLD>(stage[n & 1], fo, tid);
         __syncthreads();
     }
 
-    // epilogue for this phi tile: scale by K, store, update the running peak
+    // epilogue for this phi tile: scale by K, store, update the running peak (lowest
+    // index among equals: a +phi sample is above, a folded -phi one below all before it)
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int64_t l = l0 + 8 * ty + i;
+        float2 *row = reinterpret_cast<float2 *>(a.F) + l * a.nphi;
+        const bool st = a.F != nullptr && l < a.nlos;
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
-            const int k = p0 + 16 * (j >> 1) + 2 * tx + (j & 1);
-            const float fr = re[i][j] * a.scale, fi = im[i][j] * a.scale;
-            if (k < a.nphi) {
-                const float m2 = __fadd_rn(__fmul_rn(fr, fr), __fmul_rn(fi, fi));
-                if (m2 > bm[i]) { bm[i] = m2; bi[i] = k; }
-                if (a.F != nullptr && l < a.nlos)
-                    *reinterpret_cast<float2 *>(a.F + (l * a.nphi + k) * 2) = make_float2(fr, fi);
+            const int col = p0 + 16 * (j >> 1) + 2 * tx + (j & 1);
+            if (col >= a.ncol) continue;
+            const float(&s)[NS] = acc[i][j];
+            const int k = a.kplus + col;
+            const float fr = (FOLD ? s[0] + s[1] : s[0]) * a.scale;
+            const float fi = (FOLD ? s[2] - s[NS - 1] : s[1]) * a.scale;
+            const float m2 = __fadd_rn(__fmul_rn(fr, fr), __fmul_rn(fi, fi));
+            if (m2 > bm[i]) { bm[i] = m2; bi[i] = k; }
+            if (st) row[k] = make_float2(fr, fi);
+            if constexpr (FOLD) {
+                const int kn = a.kminus - col;
+                if (kn == k) continue;          // phi = 0 is its own partner
+                const float gr = (s[0] - s[1]) * a.scale, gi = (s[2] + s[3]) * a.scale;
+                const float g2 = __fadd_rn(__fmul_rn(gr, gr), __fmul_rn(gi, gi));
+                if (g2 >= bm[i]) { bm[i] = g2; bi[i] = kn; }
+                if (st) row[kn] = make_float2(gr, gi);
             }
         }
     }
 }
 
-template <bool FLY, int LAYOUT>
+template <bool FLY, bool FOLD, int LAYOUT>
 __global__ void __launch_bounds__(256, 1) simt_kernel(const SimtArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -247,7 +297,8 @@ __global__ void __launch_bounds__(256, 1) simt_kernel(const SimtArgs a)
     const int64_t l0 = (int64_t)blockIdx.x * TL;
     Pipe pp;
     pp.nck = (a.nact + CH - 1) / CH;
-    pp.total = pp.nck * ((a.nphi + TP - 1) / TP);
+    constexpr int W = FOLD ? TP / 2 : TP;
+    pp.total = pp.nck * ((a.ncol + W - 1) / W);
     pp.t = 0;
 
     float bm[8];
@@ -257,22 +308,22 @@ __global__ void __launch_bounds__(256, 1) simt_kernel(const SimtArgs a)
 
     // two-stage pipeline over (phi tile, channel chunk) pairs t: the copies of
     // pair t + 1 are in flight while pair t is accumulated
-    FlyOps fo;
-    issue<FLY, LAYOUT>(a, stage[0], l0, 0, 0, load_active<LAYOUT>(a, 0, tid), tid);
+    FlyOps<FOLD> fo;
+    issue<FLY, FOLD, LAYOUT>(a, stage[0], l0, 0, 0, load_active<LAYOUT>(a, 0, tid), tid);
     cp_commit();
     pp.act = pp.total > 1 ? load_active<LAYOUT>(a, (1 % pp.nck) * CH, tid) : -1;
     if (FLY) {
-        fly_load(a, fo, 0, 0, tid);
-        fly_store(stage[0], fo, tid);
+        fly_load<FOLD>(a, fo, 0, 0, tid);
+        fly_store<FOLD>(stage[0], fo, tid);
     }
-    const int full = a.nphi / TP, rem = a.nphi - full * TP;
-    for (int it = 0; it < full; ++it) phi_tile<4, FLY, LAYOUT>(a, stage, l0, it * TP, pp, fo, bm, bi);
+    const int full = a.ncol / W, rem = a.ncol - full * W;
+    for (int it = 0; it < full; ++it) phi_tile<W / 16, FLY, FOLD, LAYOUT>(a, stage, l0, it * W, pp, fo, bm, bi);
     // the last, partial tile computes only the pairs-of-16 that hold grid points
     switch ((rem + 15) / 16) {
-    case 1: phi_tile<1, FLY, LAYOUT>(a, stage, l0, full * TP, pp, fo, bm, bi); break;
-    case 2: phi_tile<2, FLY, LAYOUT>(a, stage, l0, full * TP, pp, fo, bm, bi); break;
-    case 3: phi_tile<3, FLY, LAYOUT>(a, stage, l0, full * TP, pp, fo, bm, bi); break;
-    case 4: phi_tile<4, FLY, LAYOUT>(a, stage, l0, full * TP, pp, fo, bm, bi); break;
+    case 1: phi_tile<1, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
+    case 2: phi_tile<2, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
+    case 3: if constexpr (!FOLD) phi_tile<3, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
+    case 4: if constexpr (!FOLD) phi_tile<4, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
     default: break;
     }
 
@@ -297,14 +348,21 @@ __global__ void __launch_bounds__(256, 1) simt_kernel(const SimtArgs a)
     }
 }
 
-template <bool FLY, int LAYOUT>
+template <bool FLY, bool FOLD, int LAYOUT>
 cudaError_t launch_one(const SimtArgs &a, dim3 g, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(simt_kernel<FLY, LAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSimtSmem);
+    auto kern = simt_kernel<FLY, FOLD, LAYOUT>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSimtSmem);
     if (e != cudaSuccess) return e;
-    simt_kernel<FLY, LAYOUT><<<g, 256, kSimtSmem, s>>>(a);
+    kern<<<g, 256, kSimtSmem, s>>>(a);
     return cudaGetLastError();
+}
+
+template <bool FLY, bool FOLD>
+cudaError_t launch_layout(const SimtArgs &a, int layout, dim3 g, cudaStream_t s)
+{
+    return layout == RMS_CHAN_MAJOR ? launch_one<FLY, FOLD, RMS_CHAN_MAJOR>(a, g, s)
+                                    : launch_one<FLY, FOLD, RMS_LOS_MAJOR>(a, g, s);
 }
 
 }  // namespace
@@ -330,12 +388,14 @@ cudaError_t launch_simt(const rms_plan_s &p, bool fly, const float *Q, const flo
     a.pidx = pidx;
     a.pabs = pabs;
     a.pphi = pphi;
+    const bool fold = p.fold.on;
+    a.ncol = fold ? p.fold.ncol : p.nphi;
+    a.kplus = fold ? p.fold.kplus : 0;
+    a.kminus = p.fold.kminus;
+    a.vec4 = nlos % 4 == 0 && !((reinterpret_cast<uintptr_t>(Q) | reinterpret_cast<uintptr_t>(U)) & 15);
     int64_t blocks = (nlos + TL - 1) / TL;
     if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
     dim3 g((unsigned)blocks);
-    if (fly)
-        return layout == RMS_CHAN_MAJOR ? launch_one<true, RMS_CHAN_MAJOR>(a, g, s)
-                                        : launch_one<true, RMS_LOS_MAJOR>(a, g, s);
-    return layout == RMS_CHAN_MAJOR ? launch_one<false, RMS_CHAN_MAJOR>(a, g, s)
-                                    : launch_one<false, RMS_LOS_MAJOR>(a, g, s);
+    if (fold) return fly ? launch_layout<true, true>(a, layout, g, s) : launch_layout<false, true>(a, layout, g, s);
+    return fly ? launch_layout<true, false>(a, layout, g, s) : launch_layout<false, false>(a, layout, g, s);
 }
