@@ -307,6 +307,7 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
         p->fold.kminus = (nphi - 1) / 2;
     }
 
+    if (precision == RMS_FP32_SIMT_FLY || precision == RMS_FP32_SIMT_TABLE) RMS_TRY(simt_prepare(p));
     if (precision == RMS_FP32_SIMT_TABLE) {
         RMS_TRY(dalloc(&p->d_table, (size_t)p->nact * nphi));
         RMS_TRY(launch_phase_table(*p, 0));

@@ -75,6 +75,7 @@ struct rms_plan_s {
     int32_t kpad = 0, kblocks = 0;
     PhaseTiling tiles;      // npad covers both tilings
     FoldPlan fold;
+    int32_t simt_clusters[8] = {};  // FP32 CUDA-core kernels: resident clusters of 1 .. 8 blocks
     double *d_dh = nullptr;        // [fold.ncol] the folded grid's depths phi >= 0
     CUtensorMap tmap_bhi;   // CUtensorMap is 64-byte aligned by its own declaration
     CUtensorMap tmap_blo;
@@ -144,6 +145,7 @@ cudaError_t launch_rmsf(const rms_plan_s &p, const double *d_phi, int32_t n, dou
 cudaError_t launch_simt(const rms_plan_s &p, bool fly, const float *Q, const float *U, int64_t nlos,
                         int layout, float *F, int32_t *pidx, float *pabs, float *pphi,
                         cudaStream_t s);
+cudaError_t simt_prepare(rms_plan_s *p);   // plan creation, FP32 CUDA-core precisions
 rms_status czt_plan_build(rms_plan_s *p);
 cudaError_t launch_czt(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout, float *F,
                        int32_t *pidx, float *pabs, float *pphi, float *pq, float *pu, float *pchi, cudaStream_t s);

@@ -20,9 +20,14 @@
 // on the fly 6.97 -> 3.70 ms (rows not aligned 4.58, LOS-major 7.05 -> 4.64 ms).
 // The peak of |F| (Sec. 2.2) is reduced in registers over the block's phi
 // tiles, so F never has to be re-read.
+#include <cooperative_groups.h>
 #include <limits.h>
 
+#include <algorithm>
+
 #include "rms_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -189,6 +194,9 @@ struct Pipe {
     int t;          // (phi tile, channel chunk) pair being accumulated
     int total, nck;
     int32_t act;    // active-channel index for the next copy
+    int rank, size; // this block's tiles: rank, rank + size, ... (its place in the cluster)
+    __device__ __forceinline__ int chunk(int n) const { return n % nck; }
+    __device__ __forceinline__ int tile(int n) const { return rank + (n / nck) * size; }
 };
 
 // One phi tile starting at column p0: accumulate all channel chunks, then scale,
@@ -213,9 +221,9 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_
     for (int ck = 0; ck < pp.nck; ++ck, ++pp.t) {
         const int n = pp.t + 1;
         if (n < pp.total) {
-            issue<FLY, FOLD, LAYOUT>(a, stage[n & 1], l0, (n % pp.nck) * CH, (n / pp.nck) * W, pp.act, tid);
-            if (FLY) fly_load<FOLD>(a, fo, (n % pp.nck) * CH, (n / pp.nck) * W, tid);
-            if (n + 1 < pp.total) pp.act = load_active<LAYOUT>(a, ((n + 1) % pp.nck) * CH, tid);
+            issue<FLY, FOLD, LAYOUT>(a, stage[n & 1], l0, pp.chunk(n) * CH, pp.tile(n) * W, pp.act, tid);
+            if (FLY) fly_load<FOLD>(a, fo, pp.chunk(n) * CH, pp.tile(n) * W, tid);
+            if (n + 1 < pp.total) pp.act = load_active<LAYOUT>(a, pp.chunk(n + 1) * CH, tid);
         }
         cp_commit();
         cp_wait_prev();
@@ -291,14 +299,20 @@ template <bool FLY, bool FOLD, int LAYOUT>
 __global__ void __launch_bounds__(256, 1) simt_kernel(const SimtArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ float pk_m[TL];
+    __shared__ int pk_k[TL];
     Stage *stage = reinterpret_cast<Stage *>(smem_raw);
 
     const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
-    const int64_t l0 = (int64_t)blockIdx.x * TL;
+    const cg::cluster_group cluster = cg::this_cluster();
     Pipe pp;
+    pp.rank = (int)cluster.block_rank();
+    pp.size = (int)cluster.num_blocks();
+    const int64_t l0 = (int64_t)(blockIdx.x / pp.size) * TL;
     pp.nck = (a.nact + CH - 1) / CH;
     constexpr int W = FOLD ? TP / 2 : TP;
-    pp.total = pp.nck * ((a.ncol + W - 1) / W);
+    const int ntiles = (a.ncol + W - 1) / W;        // the cluster has at most as many blocks
+    pp.total = pp.nck * ((ntiles - pp.rank + pp.size - 1) / pp.size);
     pp.t = 0;
 
     float bm[8];
@@ -309,22 +323,25 @@ __global__ void __launch_bounds__(256, 1) simt_kernel(const SimtArgs a)
     // two-stage pipeline over (phi tile, channel chunk) pairs t: the copies of
     // pair t + 1 are in flight while pair t is accumulated
     FlyOps<FOLD> fo;
-    issue<FLY, FOLD, LAYOUT>(a, stage[0], l0, 0, 0, load_active<LAYOUT>(a, 0, tid), tid);
+    issue<FLY, FOLD, LAYOUT>(a, stage[0], l0, 0, pp.rank * W, load_active<LAYOUT>(a, 0, tid), tid);
     cp_commit();
-    pp.act = pp.total > 1 ? load_active<LAYOUT>(a, (1 % pp.nck) * CH, tid) : -1;
+    pp.act = pp.total > 1 ? load_active<LAYOUT>(a, pp.chunk(1) * CH, tid) : -1;
     if (FLY) {
-        fly_load<FOLD>(a, fo, 0, 0, tid);
+        fly_load<FOLD>(a, fo, 0, pp.rank * W, tid);
         fly_store<FOLD>(stage[0], fo, tid);
     }
     const int full = a.ncol / W, rem = a.ncol - full * W;
-    for (int it = 0; it < full; ++it) phi_tile<W / 16, FLY, FOLD, LAYOUT>(a, stage, l0, it * W, pp, fo, bm, bi);
+    int it = pp.rank;
+    for (; it < full; it += pp.size) phi_tile<W / 16, FLY, FOLD, LAYOUT>(a, stage, l0, it * W, pp, fo, bm, bi);
     // the last, partial tile computes only the pairs-of-16 that hold grid points
-    switch ((rem + 15) / 16) {
-    case 1: phi_tile<1, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
-    case 2: phi_tile<2, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
-    case 3: if constexpr (!FOLD) phi_tile<3, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
-    case 4: if constexpr (!FOLD) phi_tile<4, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
-    default: break;
+    if (it == full) {
+        switch ((rem + 15) / 16) {
+        case 1: phi_tile<1, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
+        case 2: phi_tile<2, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
+        case 3: if constexpr (!FOLD) phi_tile<3, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
+        case 4: if constexpr (!FOLD) phi_tile<4, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
+        default: break;
+        }
     }
 
     // reduce the peak over the 8 threads (tx) that share each line of sight
@@ -338,34 +355,79 @@ __global__ void __launch_bounds__(256, 1) simt_kernel(const SimtArgs a)
             const int ko = __shfl_xor_sync(0xffffffffu, k, off);
             if (better(mo, ko, m, k)) { m = mo; k = ko; }
         }
-        const int64_t l = l0 + 8 * ty + i;
-        if (tx == 0 && l < a.nlos) {
+        if (tx == 0) { pk_m[8 * ty + i] = m; pk_k[8 * ty + i] = k; }
+    }
+    // the cluster's blocks hold disjoint phi of the same LOS: its first block merges them
+    if (pp.size > 1) cluster.sync();
+    else __syncthreads();
+    if (pp.rank == 0) {
+        float m = pk_m[tid];
+        int k = pk_k[tid];
+        for (int r = 1; r < pp.size; ++r) {
+            const float mo = cluster.map_shared_rank(pk_m, r)[tid];
+            const int ko = cluster.map_shared_rank(pk_k, r)[tid];
+            if (better(mo, ko, m, k)) { m = mo; k = ko; }
+        }
+        const int64_t l = l0 + tid;
+        if (l < a.nlos) {
             const bool ok = k != INT_MAX;
             if (a.pidx) a.pidx[l] = ok ? k : -1;
             if (a.pabs) a.pabs[l] = ok ? sqrtf(m) : __int_as_float(0x7fc00000);
             if (a.pphi) a.pphi[l] = ok ? a.phi32[k] : __int_as_float(0x7fc00000);
         }
     }
+    if (pp.size > 1) cluster.sync();    // no block leaves while another reads its shared memory
 }
 
-template <bool FLY, bool FOLD, int LAYOUT>
-cudaError_t launch_one(const SimtArgs &a, dim3 g, cudaStream_t s)
+cudaLaunchConfig_t launch_config(cudaLaunchAttribute *attr, unsigned grid, unsigned cluster, cudaStream_t s)
 {
-    auto kern = simt_kernel<FLY, FOLD, LAYOUT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSimtSmem);
-    if (e != cudaSuccess) return e;
-    kern<<<g, 256, kSimtSmem, s>>>(a);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(TL);
+    cfg.dynamicSmemBytes = kSimtSmem;
+    cfg.stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = cluster;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
 }
 
-template <bool FLY, bool FOLD>
-cudaError_t launch_layout(const SimtArgs &a, int layout, dim3 g, cudaStream_t s)
+using SimtKernel = void (*)(SimtArgs);
+SimtKernel kernel_of(bool fly, bool fold, int layout)
 {
-    return layout == RMS_CHAN_MAJOR ? launch_one<FLY, FOLD, RMS_CHAN_MAJOR>(a, g, s)
-                                    : launch_one<FLY, FOLD, RMS_LOS_MAJOR>(a, g, s);
+    const bool chan = layout == RMS_CHAN_MAJOR;
+    if (fly) {
+        if (fold) return chan ? simt_kernel<true, true, RMS_CHAN_MAJOR> : simt_kernel<true, true, RMS_LOS_MAJOR>;
+        return chan ? simt_kernel<true, false, RMS_CHAN_MAJOR> : simt_kernel<true, false, RMS_LOS_MAJOR>;
+    }
+    if (fold) return chan ? simt_kernel<false, true, RMS_CHAN_MAJOR> : simt_kernel<false, true, RMS_LOS_MAJOR>;
+    return chan ? simt_kernel<false, false, RMS_CHAN_MAJOR> : simt_kernel<false, false, RMS_LOS_MAJOR>;
 }
 
 }  // namespace
+
+// Clusters of 1 .. 8 blocks that the device holds at once (a cluster lives inside one
+// GPC, so sizes that do not divide a GPC's SMs leave some idle).
+cudaError_t simt_prepare(rms_plan_s *p)
+{
+    const bool fly = p->precision == RMS_FP32_SIMT_FLY;
+    for (int layout : {RMS_CHAN_MAJOR, RMS_LOS_MAJOR}) {
+        const SimtKernel kern = kernel_of(fly, p->fold.on, layout);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSimtSmem);
+        for (int c = 1; c <= 8 && e == cudaSuccess; ++c) {
+            cudaLaunchAttribute attr;
+            const cudaLaunchConfig_t cfg = launch_config(&attr, (unsigned)(c * p->num_sms), (unsigned)c, 0);
+            int n = 0;
+            e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+            p->simt_clusters[c - 1] = layout == RMS_CHAN_MAJOR ? n : std::min(n, p->simt_clusters[c - 1]);
+        }
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
 
 cudaError_t launch_simt(const rms_plan_s &p, bool fly, const float *Q, const float *U, int64_t nlos,
                         int layout, float *F, int32_t *pidx, float *pabs, float *pphi,
@@ -393,9 +455,21 @@ cudaError_t launch_simt(const rms_plan_s &p, bool fly, const float *Q, const flo
     a.kplus = fold ? p.fold.kplus : 0;
     a.kminus = p.fold.kminus;
     a.vec4 = nlos % 4 == 0 && !((reinterpret_cast<uintptr_t>(Q) | reinterpret_cast<uintptr_t>(U)) & 15);
-    int64_t blocks = (nlos + TL - 1) / TL;
-    if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-    dim3 g((unsigned)blocks);
-    if (fold) return fly ? launch_layout<true, true>(a, layout, g, s) : launch_layout<false, true>(a, layout, g, s);
-    return fly ? launch_layout<true, false>(a, layout, g, s) : launch_layout<false, false>(a, layout, g, s);
+    const int64_t blocks = (nlos + TL - 1) / TL;
+    // One block fits an SM, and its phi tiles re-read the block's data anyway, so a
+    // cluster of up to 8 blocks shares out the phi tiles of 256 LOS where that needs
+    // fewer rounds of tiles over the device (the smallest such cluster).  401 phi x 360
+    // channels: 3,000 LOS 522 -> 84 us, 10,000 LOS 520 -> 207, 100,000 unchanged (1.53 ms).
+    const int width = fold ? TP / 2 : TP, ntiles = (a.ncol + width - 1) / width;
+    int64_t best = INT64_MAX;
+    unsigned cluster = 1;
+    for (int c = 1; c <= std::min(8, ntiles); ++c) {
+        if (p.simt_clusters[c - 1] < 1) continue;
+        const int64_t rounds = (blocks + p.simt_clusters[c - 1] - 1) / p.simt_clusters[c - 1] * ((ntiles + c - 1) / c);
+        if (rounds < best) { best = rounds; cluster = (unsigned)c; }
+    }
+    if (blocks * cluster > 0x7fffffff) return cudaErrorInvalidValue;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = launch_config(&attr, (unsigned)blocks * cluster, cluster, s);
+    return cudaLaunchKernelEx(&cfg, kernel_of(fly, fold, layout), a);
 }
