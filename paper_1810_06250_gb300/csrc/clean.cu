@@ -6,8 +6,10 @@
 // on a uniform phi grid, then restore clean_k = res_k + sum_{|d|<=W} comp_{k-d} B(d)
 // with a real Gaussian beam B of the RMSF's FWHM, truncated at W = ceil(3 FWHM / dphi).
 //
-// One warp per LOS, residual and components in shared memory, R on the doubled
-// grid (2 N - 1 points) shared by the CTA.  The greedy choices must be the ones
+// One warp per LOS.  For N <= 1024 (clean_reg_kernel) the residual lives in
+// registers, the components in shared memory and R on the doubled grid
+// (2 N - 1 points) in L1; longer grids (clean_kernel) keep the residual and R in
+// shared memory too.  The greedy choices must be the ones
 // the FP64 definition makes, so the iteration runs in FP64 with every product
 // and sum rounded separately (no contraction into FMA): with the same R table
 // the device reproduces the definition bit for bit.
@@ -48,6 +50,134 @@ __device__ __forceinline__ double2 cmul_rn(double2 a, double2 b)
 {
     return make_double2(__dsub_rn(__dmul_rn(a.x, b.x), __dmul_rn(a.y, b.y)),
                         __dadd_rn(__dmul_rn(a.x, b.y), __dmul_rn(a.y, b.x)));
+}
+
+// A non-negative stand-in for |x|, low by less than 2^-20 of it, from the high word of
+// a double with magnitude below 2^60 (below 2^-126: 0): integer work only, because a
+// conversion would run at the FP64 rate.
+constexpr int kHiLo = (1023 - 50) << 20, kHiHi = (1023 + 60) << 20;
+__device__ __forceinline__ float trunc_abs(int hi) { return __int_as_float(max(hi - (896 << 20), 0) << 3); }
+
+// N <= 32 NR.  Bound by the FP64 pipe (2 lanes per clock and SM): the update's 8
+// separately rounded operations per sample are what the definition asks for.  The
+// search's 3 are not: an FP32 stand-in for |res|^2, low by at most 2^-18.9 of it and
+// high by at most 2^-22, rules out every sample below (1 - 2^-17) of its maximum, and
+// when one sample is left it is the argmax.  Anything else (ties, values outside
+// 2^-50 .. 2^60, NaN) takes the FP64 search.  One warp per block, so that the
+// scheduler evens out the LOS's different numbers of steps.  20,000 LOS x 401 phi, up
+// to 400 steps: 63.2 -> 39.4 ms (clean_kernel: 8 warps per SM, 11 FP64 operations per
+// sample and step); longer grids keep clean_kernel, whose residual does not need registers.
+template <int NR>
+__global__ void __launch_bounds__(32) clean_reg_kernel(const CleanParams P)
+{
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    double2 *comp = reinterpret_cast<double2 *>(smem_raw);
+    const int lane = threadIdx.x, N = P.N;
+    const int64_t l = blockIdx.x;
+    const unsigned all = 0xffffffffu;
+    const float2 *f = P.F + l * N;
+    double rx[NR], ry[NR];
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+        const int k = 32 * i + lane;
+        const float2 v = k < N ? f[k] : make_float2(0.f, 0.f);
+        rx[i] = (double)v.x;
+        ry[i] = (double)v.y;
+        if (k < N) comp[k] = make_double2(0.0, 0.0);
+    }
+    __syncwarp();
+    int it = 0;
+    for (; it < P.max_iter; ++it) {
+        float best = -1.f, second = -1.f;
+        double vx = 0.0, vy = 0.0;      // the candidate's residual
+        int bi = 0, raw = 0;
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const int hx = __double2hiint(rx[i]) & 0x7fffffff, hy = __double2hiint(ry[i]) & 0x7fffffff;
+            raw = max(raw, max(hx, hy));
+            const float fx = trunc_abs(hx), fy = trunc_abs(hy);
+            const float m = fmaf(fx, fx, fy * fy);
+            second = fmaxf(second, fminf(best, m));
+            if (m > best) { best = m; bi = i; vx = rx[i]; vy = ry[i]; }
+        }
+        raw = (int)__reduce_max_sync(all, (unsigned)raw);
+        const float top = __uint_as_float(__reduce_max_sync(all, __float_as_uint(best)));
+        const float cut = top * (1.f - 0x1p-17f);
+        const unsigned near = __ballot_sync(all, best >= cut), more = __ballot_sync(all, second >= cut);
+        int bj;
+        if (raw >= kHiLo && raw < kHiHi && __popc(near) == 1 && more == 0) {
+            const int who = __ffs(near) - 1;
+            bj = 32 * __shfl_sync(all, bi, who) + who;
+        } else {
+            double bm = -1.0;
+            bj = INT_MAX;
+#pragma unroll
+            for (int i = 0; i < NR; ++i) {
+                const int k = 32 * i + lane;
+                const double m2 = __dadd_rn(__dmul_rn(rx[i], rx[i]), __dmul_rn(ry[i], ry[i]));
+                if (k < N && m2 > bm) { bm = m2; bj = k; vx = rx[i]; vy = ry[i]; }   // the first maximum; NaN never
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double ob = __shfl_xor_sync(all, bm, o);
+                const int oj = __shfl_xor_sync(all, bj, o);
+                if (ob > bm || (ob == bm && oj < bj)) { bm = ob; bj = oj; }
+            }
+            if (bj == INT_MAX) break;
+        }
+        vx = __shfl_sync(all, vx, bj & 31);
+        vy = __shfl_sync(all, vy, bj & 31);
+        if (!(__dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy)) >= P.thr2)) break;
+        const double2 c = make_double2(__dmul_rn(P.gain, vx), __dmul_rn(P.gain, vy));
+        if (lane == 0) comp[bj] = make_double2(__dadd_rn(comp[bj].x, c.x), __dadd_rn(comp[bj].y, c.y));
+        const double2 *R = P.R2 + (lane - bj + N - 1);
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+            if (32 * i + lane < N) {
+                const double2 cr = cmul_rn(c, __ldg(R + 32 * i));
+                rx[i] = __dsub_rn(rx[i], cr.x);
+                ry[i] = __dsub_rn(ry[i], cr.y);
+            }
+        __syncwarp();
+    }
+    if (lane == 0 && P.niter) P.niter[l] = it;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+        const int k = 32 * i + lane;
+        if (P.clean) {
+            // sum over d = -W .. W in order; a tap without a component in any lane adds +0,
+            // which changes nothing but the sign of a zero: once, at the start
+            double sx = __dadd_rn(rx[i], 0.0), sy = __dadd_rn(ry[i], 0.0);
+            for (int d = -P.W; d <= P.W; ++d) {
+                const int kk = k - d;
+                const double2 cc = k < N && kk >= 0 && kk < N ? comp[kk] : make_double2(0.0, 0.0);
+                if (!__any_sync(all, cc.x != 0.0 || cc.y != 0.0)) continue;
+                const double b = __ldg(P.beam + P.W + d);
+                sx = __dadd_rn(sx, __dmul_rn(cc.x, b));
+                sy = __dadd_rn(sy, __dmul_rn(cc.y, b));
+            }
+            if (k < N) P.clean[l * N + k] = make_float2((float)sx, (float)sy);
+        }
+        if (k < N && P.res_out) P.res_out[l * N + k] = make_float2((float)rx[i], (float)ry[i]);
+        if (k < N && P.comp_out) P.comp_out[l * N + k] = make_float2((float)comp[k].x, (float)comp[k].y);
+    }
+}
+
+using CleanKernel = void (*)(CleanParams);
+// the register kernel with the fewest 32-sample rows that hold N (null above 1024)
+CleanKernel clean_kernel_for(int N)
+{
+    static const CleanKernel k[16] = {
+        clean_reg_kernel<1>, clean_reg_kernel<2>,  clean_reg_kernel<3>,  clean_reg_kernel<4>,  clean_reg_kernel<5>,  clean_reg_kernel<6>,
+        clean_reg_kernel<7>, clean_reg_kernel<8>,  clean_reg_kernel<9>,  clean_reg_kernel<10>, clean_reg_kernel<11>, clean_reg_kernel<12>,
+        clean_reg_kernel<13>, clean_reg_kernel<14>, clean_reg_kernel<15>, clean_reg_kernel<16>};
+    const int rows = (N + 31) / 32;
+    return rows <= 16 ? k[rows - 1]
+           : rows <= 20 ? clean_reg_kernel<20>
+           : rows <= 24 ? clean_reg_kernel<24>
+           : rows <= 28 ? clean_reg_kernel<28>
+           : rows <= 32 ? clean_reg_kernel<32> : nullptr;
 }
 
 __global__ void __launch_bounds__(256) clean_kernel(const CleanParams P)
@@ -232,6 +362,12 @@ rms_status rms_clean(rms_clean_t c, const float *F, int64_t nlos, float gain, in
     P.res_out = reinterpret_cast<float2 *>(residual);
     P.comp_out = reinterpret_cast<float2 *>(components);
     P.niter = niter;
+    if (const CleanKernel kern = clean_kernel_for(c->N); kern && nlos <= 0x7fffffff) {
+        kern<<<(unsigned)nlos, 32, (size_t)c->N * sizeof(double2), reinterpret_cast<cudaStream_t>(stream)>>>(P);
+        const cudaError_t e = cudaGetLastError();
+        if (prev >= 0 && prev != c->device) cudaSetDevice(prev);
+        return from_cuda(e);
+    }
     const size_t limit = 200 * 1024;
     int wpb = 8;
     while (wpb > 1 && clean_smem(c->N, c->W, wpb) > limit) --wpb;
