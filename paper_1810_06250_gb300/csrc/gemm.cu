@@ -17,7 +17,7 @@
 // tiles (whole schedule), or one (N panel, M tile, N tile) triple dealt
 // round-robin (job schedule, see GemmParams).
 //   warp 0      producer: the split A stage and TMA of the B hi/lo tiles  -> full
-//   warp 1      TMEM allocator, single-thread MMA issuer          -> empty, tfull
+//   warp 1      TMEM allocator, MMA issuer (one elected lane)     -> empty, tfull
 //   warps 4-11  epilogue: warp w owns TMEM lane quarter w % 4 and column half
 //               (w - 4) / 4; folds partials, scales, peak, stores F  -> tempty
 // The PAIR variant runs on clusters of two CTAs (two SMs) with tcgen05's
@@ -298,7 +298,7 @@ struct GemmParams {
     const int8_t *rexp;
     int *err;
     int64_t timeout_ns;
-    int32_t stages;
+    int32_t stages, kbs;        // pipeline stages of kbs K blocks each
     // schedule: jobs_split = 0: one job per M tile (or M-tile pair) covering every N
     // tile, peaks written directly; 1: one job per (N panel, M tile, N tile), ordered
     // panel by panel, M tile by M tile, and dealt round-robin to the persistent CTAs,
@@ -326,7 +326,7 @@ __host__ __device__ __forceinline__ uint32_t gemm_stage_bytes(int b_rows, int mo
 
 struct GSmem {
     uint8_t *ring;
-    uint32_t stage_bytes;
+    uint32_t stage_bytes, sub_bytes;
     float *epi, *pk_m, *pk_re, *pk_im;
     int *pk_i;
     uint64_t *full, *empty, *conv, *tfull, *tempty, *pkfull, *pkempty, *mma_done;   // conv: rotated stage (ROT)
@@ -337,7 +337,8 @@ struct GSmem {
 __device__ __forceinline__ GSmem gcarve(uint8_t *base, const GemmParams &P)
 {
     GSmem s;
-    s.stage_bytes = gemm_stage_bytes(P.b_rows, P.mode);
+    s.sub_bytes = gemm_stage_bytes(P.b_rows, P.mode);
+    s.stage_bytes = s.sub_bytes * (uint32_t)P.kbs;
     s.ring = base;
     s.epi = reinterpret_cast<float *>(s.ring + (size_t)P.stages * s.stage_bytes);
     s.pk_m = s.epi + kEpiStageBytes / 4;
@@ -478,28 +479,36 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                     // phase rows of this CTA's part of the tile: all of it, or the pair's half
                     int32_t y = nt * P.tile_n;
                     if (PAIR && !leader) y += ((nt == P.ntiles_n - 1) ? P.tile_n_last : P.tile_n) / 2;
-                    for (int kb = 0; kb < P.kblocks; ++kb) {
-                        if (!wait_bounded(smem_u32(&S.empty[s]), ph ^ 1, S.abort_flag, P.err, P.timeout_ns)) {
-                            ok = false;
-                            break;
+                    for (int g = 0; g < ngroups && ok; ++g) {
+                        const int g1 = min(P.kblocks, (g + 1) * P.group);
+                        for (int kb = g * P.group; kb < g1; kb += P.kbs) {
+                            const int n = min(P.kbs, g1 - kb);
+                            if (!wait_bounded(smem_u32(&S.empty[s]), ph ^ 1, S.abort_flag, P.err, P.timeout_ns)) {
+                                ok = false;
+                                break;
+                            }
+                            uint32_t st = smem_u32(S.ring + (size_t)s * S.stage_bytes);
+                            const uint32_t bar = smem_u32(&S.full[s]);
+                            if constexpr (PAIR) {
+                                const uint32_t bar0 = mapa_shared(bar, 0u);
+                                if (leader) mbar_arrive_expect_tx(bar, 2 * tx * (uint32_t)n);
+                                for (int i = 0; i < n; ++i, st += S.sub_bytes) {
+                                    tma_load_3d_pair(st, &tmA, 0, 0, (int32_t)(mt * P.kblocks + kb + i), bar0);
+                                    tma_load_2d_pair(st + a_bytes, &tmB_hi, (kb + i) * kKBlock, y, bar0);
+                                    if (split) tma_load_2d_pair(st + a_bytes + b_bytes, &tmB_lo, (kb + i) * kKBlock, y, bar0);
+                                }
+                            } else {
+                                mbar_arrive_expect_tx(bar, tx * (uint32_t)n);
+                                for (int i = 0; i < n; ++i, st += S.sub_bytes) {
+                                    bulk_load(st, a_mt + (size_t)(kb + i) * (2 * kStageA), a_bytes, bar);
+                                    tma_load_2d(st + a_bytes, &tmB_hi, (kb + i) * kKBlock, y, bar);
+                                    if (split) tma_load_2d(st + a_bytes + b_bytes, &tmB_lo, (kb + i) * kKBlock, y, bar);
+                                }
+                            }
+                            pending |= 1u << s;
+                            pend_par = (pend_par & ~(1u << s)) | (ph << s);
+                            if (++s == P.stages) { s = 0; ph ^= 1; }
                         }
-                        const uint32_t st = smem_u32(S.ring + (size_t)s * S.stage_bytes);
-                        const uint32_t bar = smem_u32(&S.full[s]);
-                        if constexpr (PAIR) {
-                            const uint32_t bar0 = mapa_shared(bar, 0u);
-                            if (leader) mbar_arrive_expect_tx(bar, 2 * tx);
-                            tma_load_3d_pair(st, &tmA, 0, 0, (int32_t)(mt * P.kblocks + kb), bar0);
-                            tma_load_2d_pair(st + a_bytes, &tmB_hi, kb * kKBlock, y, bar0);
-                            if (split) tma_load_2d_pair(st + a_bytes + b_bytes, &tmB_lo, kb * kKBlock, y, bar0);
-                        } else {
-                            mbar_arrive_expect_tx(bar, tx);
-                            bulk_load(st, a_mt + (size_t)kb * (2 * kStageA), a_bytes, bar);
-                            tma_load_2d(st + a_bytes, &tmB_hi, kb * kKBlock, y, bar);
-                            if (split) tma_load_2d(st + a_bytes + b_bytes, &tmB_lo, kb * kKBlock, y, bar);
-                        }
-                        pending |= 1u << s;
-                        pend_par = (pend_par & ~(1u << s)) | (ph << s);
-                        if (++s == P.stages) { s = 0; ph ^= 1; }
                     }
                 }
             }
@@ -532,8 +541,14 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
         if (PAIR && !leader) {
             // the even CTA's last commit: all MMAs that touch this CTA are complete
             if (lane == 0 && !wait_bounded(smem_u32(S.mma_done), 0, S.abort_flag, P.err, P.timeout_ns)) stop_peer();
-        } else if (lane == 0) {
+        } else {
             // -------------------------------------------------------- MMA issuer
+            // The warp runs convergent and one elected lane issues: its addresses and
+            // descriptors then stay in uniform registers.  With the loop on a single lane
+            // the issue, not the tensor pipe, set the pace (peak map only, pairs: 262,144
+            // LOS x 360 x 401 BF16x3 0.318 -> 0.303 ms; 400,000 x 800 x 1001 BF16 with
+            // four K blocks per stage 1.23 -> 1.00 ms).
+            const uint32_t one = elect_one();
             const bool bf = P.mode != MODE_FP16X3;
             const int mrows = PAIR ? 2 * kTileM : kTileM;
             const uint32_t id_full = idesc_f16_m(mrows, P.tile_n, bf), id_last = idesc_f16_m(mrows, P.tile_n_last, bf);
@@ -541,6 +556,11 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
             uint32_t ph = 0, tph = 0;
             int g_all = 0;
             bool ok = true, issued = false;
+            auto arrived = [&](const uint64_t *bar, uint32_t parity) {
+                const bool in = PAIR ? wait_bounded_cluster(smem_u32(bar), parity, S.abort_flag, P.err, P.timeout_ns)
+                                     : wait_bounded(smem_u32(bar), parity, S.abort_flag, P.err, P.timeout_ns);
+                return __all_sync(0xffffffffu, in) != 0;
+            };
             for (int64_t j = it0; j < njobs && ok; j += istride) {
                 int64_t it;
                 int nt0, nt1;
@@ -549,56 +569,51 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                     const uint32_t idesc = (nt == P.ntiles_n - 1) ? id_last : id_full;
                     for (int g = 0; g < ngroups && ok; ++g, ++g_all) {
                         const int b = g_all & 1;
-                        const bool got = PAIR ? wait_bounded_cluster(smem_u32(&S.tempty[b]), ((tph >> b) & 1) ^ 1,
-                                                                     S.abort_flag, P.err, P.timeout_ns)
-                                              : wait_bounded(smem_u32(&S.tempty[b]), ((tph >> b) & 1) ^ 1,
-                                                             S.abort_flag, P.err, P.timeout_ns);
-                        if (!got) {
+                        if (!arrived(&S.tempty[b], ((tph >> b) & 1) ^ 1)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
                         const uint32_t d = tmem_base + (uint32_t)(b * kAccStride);
                         const int kb0 = g * P.group, kb1 = min(P.kblocks, kb0 + P.group);
-                        for (int kb = kb0; kb < kb1; ++kb) {
-                            const uint64_t *ready = ROT ? &S.conv[s] : &S.full[s];
-                            const bool in = PAIR ? wait_bounded_cluster(smem_u32(ready), ph, S.abort_flag, P.err,
-                                                                        P.timeout_ns)
-                                                 : wait_bounded(smem_u32(ready), ph, S.abort_flag, P.err, P.timeout_ns);
-                            if (!in) {
+                        for (int kb = kb0; kb < kb1; kb += P.kbs) {
+                            const int n = min(P.kbs, kb1 - kb);
+                            if (!arrived(ROT ? &S.conv[s] : &S.full[s], ph)) {
                                 ok = false;
                                 break;
                             }
                             tc_fence_after();
-                            const uint32_t st = smem_u32(S.ring + (size_t)s * S.stage_bytes);
-                            const uint32_t a_hi = st, a_lo = st + kStageA;
-                            const uint32_t b_hi = st + a_bytes, b_lo = b_hi + b_bytes;
+                            uint32_t st = smem_u32(S.ring + (size_t)s * S.stage_bytes);
+                            for (int i = 0; i < n; ++i, st += S.sub_bytes) {
+                                const uint32_t a_hi = st, a_lo = st + kStageA;
+                                const uint32_t b_hi = st + a_bytes, b_lo = b_hi + b_bytes;
 #pragma unroll
-                            for (int kk = 0; kk < kKBlock / 16; ++kk) {
-                                const uint32_t ko = kk * 32;
-                                const uint32_t acc = (kb > kb0 || kk > 0) ? 1u : 0u;
-                                if constexpr (PAIR) {
-                                    mma_f16_pair(d, sdesc_k64(a_hi + ko), sdesc_k64(b_hi + ko), idesc, acc);
-                                    if (split) {
-                                        mma_f16_pair(d, sdesc_k64(a_hi + ko), sdesc_k64(b_lo + ko), idesc, 1u);
-                                        mma_f16_pair(d, sdesc_k64(a_lo + ko), sdesc_k64(b_hi + ko), idesc, 1u);
-                                    }
-                                } else {
-                                    mma_f16(d, sdesc_k64(a_hi + ko), sdesc_k64(b_hi + ko), idesc, acc);
-                                    if (split) {
-                                        mma_f16(d, sdesc_k64(a_hi + ko), sdesc_k64(b_lo + ko), idesc, 1u);
-                                        mma_f16(d, sdesc_k64(a_lo + ko), sdesc_k64(b_hi + ko), idesc, 1u);
+                                for (int kk = 0; kk < kKBlock / 16; ++kk) {
+                                    const uint32_t ko = kk * 32;
+                                    const uint32_t acc = (kb > kb0 || i > 0 || kk > 0) ? 1u : 0u;
+                                    if constexpr (PAIR) {
+                                        mma_f16_pair(d, sdesc_k64(a_hi + ko), sdesc_k64(b_hi + ko), idesc, acc, one);
+                                        if (split) {
+                                            mma_f16_pair(d, sdesc_k64(a_hi + ko), sdesc_k64(b_lo + ko), idesc, 1u, one);
+                                            mma_f16_pair(d, sdesc_k64(a_lo + ko), sdesc_k64(b_hi + ko), idesc, 1u, one);
+                                        }
+                                    } else {
+                                        mma_f16_one(d, sdesc_k64(a_hi + ko), sdesc_k64(b_hi + ko), idesc, acc, one);
+                                        if (split) {
+                                            mma_f16_one(d, sdesc_k64(a_hi + ko), sdesc_k64(b_lo + ko), idesc, 1u, one);
+                                            mma_f16_one(d, sdesc_k64(a_lo + ko), sdesc_k64(b_hi + ko), idesc, 1u, one);
+                                        }
                                     }
                                 }
                             }
                             issued = true;
-                            if constexpr (PAIR) mma_commit_pair_mc(smem_u32(&S.empty[s]), (uint16_t)3);
-                            else mma_commit(smem_u32(&S.empty[s]));
+                            if constexpr (PAIR) mma_commit_pair_mc(smem_u32(&S.empty[s]), (uint16_t)3, one);
+                            else mma_commit_one(smem_u32(&S.empty[s]), one);
                             if (++s == P.stages) { s = 0; ph ^= 1; }
                         }
                         if (!ok) break;
-                        if constexpr (PAIR) mma_commit_pair_mc(smem_u32(&S.tfull[b]), (uint16_t)3);
-                        else mma_commit(smem_u32(&S.tfull[b]));
+                        if constexpr (PAIR) mma_commit_pair_mc(smem_u32(&S.tfull[b]), (uint16_t)3, one);
+                        else mma_commit_one(smem_u32(&S.tfull[b]), one);
                         tph ^= 1u << b;
                     }
                 }
@@ -606,10 +621,10 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
             if (!ok) stop_peer();
             if constexpr (PAIR) {
                 // both CTAs wait for this commit before they leave (the odd CTA in its warp 1)
-                mma_commit_pair_mc(smem_u32(S.mma_done), (uint16_t)3);
+                mma_commit_pair_mc(smem_u32(S.mma_done), (uint16_t)3, one);
                 wait_bounded(smem_u32(S.mma_done), 0, S.abort_flag, P.err, P.timeout_ns, false);
             } else if (issued) {
-                mma_commit(smem_u32(S.mma_done));
+                mma_commit_one(smem_u32(S.mma_done), one);
                 wait_bounded(smem_u32(S.mma_done), 0, S.abort_flag, P.err, P.timeout_ns, false);
             }
         }
@@ -1128,9 +1143,9 @@ __global__ void peak_finalize_kernel(const unsigned long long *__restrict__ keys
 
 size_t gemm_fixed_smem() { return 1024 + kEpiStageBytes + 2 * 4 * 32 * 16 + 8 * 32 + 32; }
 
-int gemm_stages(int b_rows, int mode)
+int gemm_stages(int b_rows, int mode, int kbs)
 {
-    size_t st = gemm_stage_bytes(b_rows, mode);
+    size_t st = (size_t)kbs * gemm_stage_bytes(b_rows, mode);
     int s = (int)((kSmemLimit - gemm_fixed_smem()) / (st + 24));
     return s > 8 ? 8 : s;
 }
@@ -1311,9 +1326,19 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
     P.tile_n_last = pair ? tl.tile_n_last2 : tl.tile_n_last;
     const bool wide = pair && P.tile_n > 2 * kHalf;   // the pair kernel with 128 columns per epilogue thread
     P.b_rows = pair ? P.tile_n / 2 : P.tile_n;
-    P.stages = gemm_stages(P.b_rows, mode);
+    P.kbs = 1;
+    if (!rot) {
+        // Several K blocks per stage where at least three stages still fit: the waits and
+        // commits of a stage cost the issuing warp some 300 cycles, as much as a plain
+        // BF16 K block's MMAs (400,000 LOS x 800 x 1001, peak map only, pairs: 1.39 ms at
+        // one K block per stage, 1.02 at two, 1.00 at four).
+        for (int c = 4; c > 1; c /= 2)
+            if (gemm_stages(P.b_rows, mode, c) >= 3) { P.kbs = c; break; }
+        P.group = (P.group + P.kbs - 1) / P.kbs * P.kbs;
+    }
+    P.stages = gemm_stages(P.b_rows, mode, P.kbs);
     if (P.stages < 2) return cudaErrorInvalidConfiguration;
-    size_t smem = gemm_fixed_smem() + (size_t)P.stages * gemm_stage_bytes(P.b_rows, mode) + 24 * (size_t)P.stages;
+    size_t smem = gemm_fixed_smem() + (size_t)P.stages * P.kbs * gemm_stage_bytes(P.b_rows, mode) + 24 * (size_t)P.stages;
     const int64_t nit = pair ? (nmt + 1) / 2 : nmt;
     int maxunits = pair ? (ctas / 2 > 0 ? ctas / 2 : 1) : ctas;
     using KernelFn = void (*)(GemmParams, CUtensorMap, CUtensorMap, CUtensorMap);
