@@ -236,10 +236,13 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar_cluster)
         : "memory");
 }
-// Arrive (release, cluster scope) on an mbarrier given by its cluster address.
+// Arrive on an mbarrier given by its cluster address, to hand back TMEM columns that
+// this warp has read (tcgen05.wait::ld and the before_thread_sync fence order those
+// reads).  The release has CTA scope: one of cluster scope would also wait until every
+// F store the thread has in flight is acknowledged, and no other CTA reads F.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
 {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity)
 {
