@@ -52,6 +52,7 @@ void free_plan(rms_plan_s *p)
 {
     if (!p) return;
     cudaFree(p->d_active);
+    cudaFree(p->d_active_pad);
     cudaFree(p->d_dl2);
     cudaFree(p->d_wact);
     cudaFree(p->d_phi);
@@ -406,8 +407,13 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
                 free_plan(p);
                 return RMS_ERR_CUDA;
             }
+            std::vector<int32_t> padded(p->active);
+            padded.resize(f.kpad, p->active.back());
+            RMS_TRY(dalloc(&p->d_active_pad, f.kpad));
+            RMS_TRY(cudaMemcpy(p->d_active_pad, padded.data(), f.kpad * sizeof(int32_t), cudaMemcpyHostToDevice));
             f.pair_maps = encode_b_map(&f.tmap2_bhi, f.d_hi, f.kpad, f.tiles.npad, h) &&
                           encode_b_map(&f.tmap2_blo, f.d_lo, f.kpad, f.tiles.npad, h);
+            RMS_TRY(fused_prepare(p));
         }
     }
     RMS_TRY(cudaEventCreateWithFlags(&p->last, cudaEventDisableTiming));
@@ -511,9 +517,10 @@ static rms_status synth_launch(rms_plan_t p, const float *Q, const float *U, int
     case RMS_FP16X3: {
         // the split operand (and FP16X3's per-LOS exponents): stream-ordered scratch
         // and 8 bytes of peak key per LOS (the contraction's split schedule)
-        const size_t abytes = p->fold.on ? fold_operand_bytes(*p, nlos) : split_operand_bytes(*p, nlos, layout);
-        const size_t rbytes = p->precision == RMS_FP16X3 ? (size_t)((nlos + 255) & ~(int64_t)255) : 0;
-        const size_t kbytes = (size_t)((nlos * 8 + 255) & ~(int64_t)255);
+        const bool fused = fused_wanted(*p, Q, U, nlos, layout);
+        const size_t abytes = fused ? fused_ring_bytes(*p, nlos) : p->fold.on ? fold_operand_bytes(*p, nlos) : split_operand_bytes(*p, nlos, layout);
+        const size_t rbytes = p->precision == RMS_FP16X3 && !fused ? (size_t)((nlos + 255) & ~(int64_t)255) : 0;
+        const size_t kbytes = fused ? 0 : (size_t)((nlos * 8 + 255) & ~(int64_t)255);
         uint8_t *scr = nullptr;
         e = cudaMallocAsync(reinterpret_cast<void **>(&scr), abytes + rbytes + kbytes, s);
         if (e != cudaSuccess) {
@@ -533,9 +540,14 @@ static rms_status synth_launch(rms_plan_t p, const float *Q, const float *U, int
             }
             cudaGetLastError();
         }
-        e = launch_split_gemm(*p, Q, U, nlos, layout, F, pidx, pabs, pphi, scr,
+        if (fused) {
+            if (ev[1]) cudaEventRecord(ev[1], s);       // no layout stage of its own
+            e = launch_fused(*p, Q, U, nlos, layout, F, pidx, pabs, pphi, x.q, x.u, x.chi, scr, s);
+        } else {
+            e = launch_split_gemm(*p, Q, U, nlos, layout, F, pidx, pabs, pphi, scr,
                               rbytes ? reinterpret_cast<int8_t *>(scr + abytes) : nullptr, s, ev[1], x.q, x.u, x.chi,
                               reinterpret_cast<unsigned long long *>(scr + abytes + rbytes));
+        }
         if (ev[2]) {
             if (e == cudaSuccess) e = cudaEventRecord(ev[2], s);
             p->tev.insert(p->tev.end(), ev, ev + 3);

@@ -1,0 +1,898 @@
+// Folded synthesis in one kernel (see fold.cu for the folded form and gemm.cu for
+// the contraction): the layout stage runs inside the contraction's CTAs.
+//
+// As two kernels the operand image goes to HBM and back between them, 16 of the
+// 32 bytes per (LOS, active channel) that a call moves besides F.  Here each CTA
+// of a pair converts its own next 64 LOS while it contracts the current ones, into
+// one of two slots of a small image ring that stays in L2 (2 tiles per CTA: 58 MB
+// for 360 active channels), and the TMA producer reads the slot once per phase
+// tile.  The MMAs, their order and the scaling are gemm.cu's, so the results are
+// the same bits.
+//
+// CTA pairs (cta_group::2), 640 threads per CTA:
+//   warp 0      producer: TMA of the ring slot's operand and of the B hi/lo tiles -> full
+//   warp 1      TMEM allocator, MMA issuer (one elected lane)    -> empty, tfull, afree
+//   warp 2      loader (LOS-major): bulk copies of Q and U rows into staging slots -> sfull
+//   warps 4-11  epilogue: warp w owns TMEM lane quarter w % 4 and column half
+//               (w - 4) / 4; every phase tile is a single accumulation, so it goes
+//               from TMEM straight to F and the running peak       -> tempty
+//   warps 12-19 splitters: FP32 Q/U -> 16-bit hi/lo rows in the ring  -> sempty, ready
+// Channel-major cubes load straight into the splitters' registers (a warp reads 128
+// bytes of a channel row; bulk copies of 256-byte rows were slower, 0.83 against 0.43 ms
+// without F on 262,144 LOS x 360 x 401).  LOS-major cubes come through staging slots of
+// all channels of 8 LOS, one bulk copy per array, which leaves the channel gather to
+// shared memory and gives FP16X3 its row maxima without a second pass; where 8 rows do
+// not fit, the base is not on 16 bytes, or on a last, partial item, the splitters load
+// through registers.
+// 262,144 LOS x 360 x 401 with F: the epilogue (F stores and the peak search) is busy 65%
+// of the time and the splitters 90%; L2-evict-first loads and an evict-last ring keep the
+// ring on chip (0.507 -> 0.478 ms).
+// Every wait is bounded, as in gemm.cu.
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+#include <limits.h>
+
+#include <algorithm>
+
+#include "rms_internal.h"
+
+namespace {
+
+#include "tc_ptx.cuh"
+#include "fold_split.cuh"
+
+constexpr int kThreads = 640;
+constexpr int kEpiWarp0 = 4, kNumEpiWarps = 8, kSplitWarp0 = 12, kNumSplitWarps = 8;
+constexpr int kTmemCols = 512, kAccStride = 256;
+constexpr int kMaxSlots = 3;                    // staging slots
+constexpr int kSmemLimit = 227 * 1024;
+// 640 x 96 registers: the epilogue takes them from the control and splitter warpgroups
+constexpr int kRegsLaunch = 96, kRegsCtl = 48, kRegsEpi = 128, kRegsSplit = 88;
+static_assert(128 * kRegsCtl + 256 * kRegsEpi + 256 * kRegsSplit == kThreads * kRegsLaunch,
+              "register split must fill the launch");
+
+struct FusedParams {
+    FoldSource src;
+    int32_t kblocks, mode;
+    int32_t nphi, ncol, kplus, kminus;
+    int32_t ntiles_n, tile_n, tile_n_last;
+    uint8_t *ring;              // [CTAs][2][kblocks][parts x 8 KB]
+    float *F;
+    int32_t *pidx;
+    float *pabs, *pphi, *pq, *pu, *pchi;
+    const float *phi32;
+    const double *phi64;
+    double lambda0sq;
+    float out_scale;
+    int *err;
+    int64_t timeout_ns;
+    int32_t stages, kbs;        // pipeline stages of kbs K blocks each
+    int32_t sslots;             // staging slots; 0: direct loads
+    uint32_t sbytes;            // bytes of a staging slot
+};
+
+__host__ __device__ __forceinline__ uint32_t sub_stage_bytes(int tile_n, int mode)
+{
+    const uint32_t parts = mode == MODE_BF16 ? 1u : 2u;
+    return parts * (uint32_t)kFoldPart + parts * (uint32_t)(tile_n / 2) * kFoldRowBytes;
+}
+
+struct FSmem {
+    uint8_t *ring, *stage;
+    uint32_t stage_bytes, sub_bytes;
+    float *pk_m, *pk_re, *pk_im;
+    int *pk_i;
+    float *los_max;             // [2][8 warps][32] (FP16X3): partial maxima of the splitters' LOS
+    int *list;                  // [kblocks x 32]: the padded channel list (an index load from L2 before
+                                // every batch of data loads would double their latency)
+    int *los_exp;               // [4][64] (FP16X3): exponents of an item's LOS
+    uint64_t *full, *empty, *tfull, *tempty, *ready, *afree, *xmax, *sfull, *sempty, *pkfull, *pkempty, *mma_done;
+    uint32_t *tmem_slot;
+    volatile int *abort_flag;
+};
+constexpr int kExpSlots = 4;    // exponents outlive their ring slot until the epilogue has used them
+
+__device__ __forceinline__ FSmem fcarve(uint8_t *base, const FusedParams &P)
+{
+    FSmem s;
+    s.sub_bytes = sub_stage_bytes(P.tile_n, P.mode);
+    s.stage_bytes = s.sub_bytes * (uint32_t)P.kbs;
+    s.ring = base;
+    s.stage = base + (size_t)P.stages * s.stage_bytes;
+    s.pk_m = reinterpret_cast<float *>(s.stage + (size_t)P.sslots * P.sbytes);
+    s.pk_i = reinterpret_cast<int *>(s.pk_m + 2 * 64);
+    s.pk_re = reinterpret_cast<float *>(s.pk_i + 2 * 64);
+    s.pk_im = s.pk_re + 2 * 64;
+    s.los_max = s.pk_im + 2 * 64;
+    s.los_exp = reinterpret_cast<int *>(s.los_max + 2 * kNumSplitWarps * 32);
+    s.list = s.los_exp + kExpSlots * 64;
+    uint64_t *b = reinterpret_cast<uint64_t *>(s.list + P.kblocks * kKBlock);
+    s.full = b;
+    s.empty = s.full + P.stages;
+    s.tfull = s.empty + P.stages;
+    s.tempty = s.tfull + 2;
+    s.ready = s.tempty + 2;
+    s.afree = s.ready + 2;
+    s.xmax = s.afree + 2;
+    s.sfull = s.xmax + 1;
+    s.sempty = s.sfull + kMaxSlots;
+    s.pkfull = s.sempty + kMaxSlots;
+    s.pkempty = s.pkfull + 8;
+    s.mma_done = s.pkempty + 8;
+    s.tmem_slot = reinterpret_cast<uint32_t *>(s.mma_done + 1);
+    s.abort_flag = reinterpret_cast<volatile int *>(s.tmem_slot + 1);
+    return s;
+}
+constexpr size_t kFixedSmem = 1024 + 8 * 64 * 4 + (kNumSplitWarps + kExpSlots) * 64 * 4 + 8 * (2 * 4 + 1 + 2 * kMaxSlots + 16 + 1) + 16;
+
+// 16 lanes x 32 consecutive 32-bit columns, no wait: four tmem_ld16x256 side by side.
+__device__ __forceinline__ void tmem_ld16x256x4(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+
+// Untiled bulk copy of data that is read once.
+__device__ __forceinline__ void bulk_load_once(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(l2_evict_first())
+                 : "memory");
+}
+
+// Channel-major tile, one splitter warp: 32 LOS (half of the tile), one array (Q or U), every
+// other half K block of 16 channels, so that four warps share the work of a LOS.  f(h, v) gets
+// the 16 values of half K block h; the next ones are loaded ahead.
+template <bool LAST, typename F>
+__device__ __forceinline__ void chan_walk(const FoldSource &S, const int *list, int64_t los, int array, int h0, int nh,
+                                          F f)
+{
+    const float *const X = array ? S.U : S.Q;
+    const bool valid = los < S.nlos;
+    const int64_t at = min(los, S.nlos - 1);
+    auto load = [&](int h, float (&v)[16]) {
+        // unconditional loads (the channel list is padded with a valid channel), so that all
+        // 16 are in flight at once
+        int ch[16];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int4 c = *reinterpret_cast<const int4 *>(list + 16 * h + 4 * j);
+            ch[4 * j] = c.x; ch[4 * j + 1] = c.y; ch[4 * j + 2] = c.z; ch[4 * j + 3] = c.w;
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = load_here<LAST>(X + (int64_t)ch[j] * S.nlos + at);
+    };
+    auto masked = [&](int h, float (&v)[16]) {
+        if (16 * h + 16 > S.nact || !valid) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (16 * h + j >= S.nact || !valid) v[j] = 0.f;
+        }
+        f(h, v);
+    };
+    float a[16], b[16];
+    if (h0 < nh) load(h0, a);
+    for (int h = h0; h < nh; h += 4) {
+        if (h + 2 < nh) load(h + 2, b);
+        masked(h, a);
+        if (h + 4 < nh) load(h + 4, a);
+        if (h + 2 < nh) masked(h + 2, b);
+    }
+}
+
+template <int MODE, bool CHAN>
+__global__ void __launch_bounds__(kThreads, 1)
+fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUtensorMap tmB_hi,
+             const __grid_constant__ CUtensorMap tmB_lo, const __grid_constant__ CUtensorMap tmA)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const FSmem S = fcarve(base, P);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr bool kSplitPrec = MODE != MODE_BF16;
+    constexpr uint32_t kPartsBytes = (kSplitPrec ? 2 : 1) * kFoldPart;   // one K block of a ring slot
+    const int64_t nlos = P.src.nlos;
+    const uint32_t rank = cluster_ctarank();
+    const bool leader = rank == 0;
+    const int64_t nit = (nlos + 2 * kFoldTileLos - 1) / (2 * kFoldTileLos);   // items: 64 LOS in each CTA
+    const int64_t it0 = blockIdx.x >> 1, istride = gridDim.x >> 1;
+    const uint32_t b_bytes = (uint32_t)(P.tile_n / 2) * kFoldRowBytes;
+    const uint32_t peer_abort = mapa_shared(smem_u32((const void *)S.abort_flag), rank ^ 1u);
+    auto stop_peer = [&]() { st_cluster_u32(peer_abort, 1u); };
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < P.stages; ++s) {
+            mbar_init(smem_u32(&S.full[s]), 1);
+            mbar_init(smem_u32(&S.empty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&S.tfull[b]), 1);
+            mbar_init(smem_u32(&S.tempty[b]), 2 * kNumEpiWarps);
+            mbar_init(smem_u32(&S.ready[b]), kNumSplitWarps);
+            mbar_init(smem_u32(&S.afree[b]), 1);
+        }
+        for (int i = 0; i < 8; ++i) {
+            mbar_init(smem_u32(&S.pkfull[i]), 1);
+            mbar_init(smem_u32(&S.pkempty[i]), 1);
+        }
+        mbar_init(smem_u32(S.xmax), kNumSplitWarps);
+        for (int i = 0; i < kMaxSlots; ++i) {
+            mbar_init(smem_u32(&S.sfull[i]), 1);
+            mbar_init(smem_u32(&S.sempty[i]), kNumSplitWarps);
+        }
+        mbar_init(smem_u32(S.mma_done), 1);
+        *S.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    for (int i = threadIdx.x; i < P.kblocks * kKBlock; i += kThreads) S.list[i] = P.src.padded[i];
+    if (warp == 1) {
+        __syncwarp();
+        tmem_alloc_pair(smem_u32(S.tmem_slot), kTmemCols);
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    tc_fence_after();
+    const uint32_t tmem_base = *S.tmem_slot;
+
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCtl));
+        if (warp == 0) {
+            // ------------------------------------------------------------ producer
+            if (lane == 0) {
+                asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB_hi)) : "memory");
+                asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB_lo)) : "memory");
+                asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
+                const uint32_t tx = kPartsBytes + (kSplitPrec ? 2 : 1) * b_bytes;
+                int s = 0;
+                uint32_t ph = 0, pending = 0, pend_par = 0;
+                bool ok = true;
+                int n_item = 0;
+                for (int64_t it = it0; it < nit && ok; it += istride, ++n_item) {
+                    const int slot = n_item & 1;
+                    if (!wait_bounded(smem_u32(&S.ready[slot]), (n_item >> 1) & 1, S.abort_flag, P.err, P.timeout_ns)) {
+                        ok = false;
+                        break;
+                    }
+                    fence_proxy_async_global();
+                    const int32_t z0 = ((int32_t)blockIdx.x * 2 + slot) * P.kblocks;
+                    for (int nt = 0; nt < P.ntiles_n && ok; ++nt) {
+                        int32_t y = nt * P.tile_n;
+                        if (!leader) y += ((nt == P.ntiles_n - 1) ? P.tile_n_last : P.tile_n) / 2;
+                        for (int kb = 0; kb < P.kblocks; kb += P.kbs) {
+                            const int n = min(P.kbs, P.kblocks - kb);
+                            if (!wait_bounded(smem_u32(&S.empty[s]), ph ^ 1, S.abort_flag, P.err, P.timeout_ns)) {
+                                ok = false;
+                                break;
+                            }
+                            uint32_t st = smem_u32(S.ring + (size_t)s * S.stage_bytes);
+                            const uint32_t bar = smem_u32(&S.full[s]);
+                            const uint32_t bar0 = mapa_shared(bar, 0u);
+                            if (leader) mbar_arrive_expect_tx(bar, 2 * tx * (uint32_t)n);
+                            for (int i = 0; i < n; ++i, st += S.sub_bytes) {
+                                tma_load_3d_pair(st, &tmA, 0, 0, z0 + kb + i, bar0);
+                                tma_load_2d_pair(st + kPartsBytes, &tmB_hi, (kb + i) * kKBlock, y, bar0);
+                                if (kSplitPrec)
+                                    tma_load_2d_pair(st + kPartsBytes + b_bytes, &tmB_lo, (kb + i) * kKBlock, y, bar0);
+                            }
+                            pending |= 1u << s;
+                            pend_par = (pend_par & ~(1u << s)) | (ph << s);
+                            if (++s == P.stages) { s = 0; ph ^= 1; }
+                        }
+                    }
+                }
+                if (!ok) {
+                    stop_peer();
+                    if (leader) {
+                        for (int i = 0; i < P.stages; ++i)
+                            if (pending & (1u << i))
+                                wait_bounded(smem_u32(&S.full[i]), (pend_par >> i) & 1, S.abort_flag, P.err,
+                                             P.timeout_ns, false);
+                    } else {
+                        // the odd CTA's copies complete on the even CTA's barriers: give any still in
+                        // flight far longer than a copy takes before this CTA may leave
+                        const uint64_t t0 = global_ns();
+                        while (global_ns() - t0 < 200000ull) __nanosleep(1000);
+                    }
+                } else {
+                    // the MMAs' commits arrive on this CTA's barriers from the tensor core: wait for
+                    // the one that releases each slot's last fill before the CTA may exit
+                    for (int i = 0; i < P.stages; ++i)
+                        if ((pending & (1u << i)) &&
+                            !wait_bounded(smem_u32(&S.empty[i]), (pend_par >> i) & 1, S.abort_flag, P.err,
+                                          P.timeout_ns)) {
+                            stop_peer();
+                            break;
+                        }
+                }
+            }
+        } else if (warp == 1) {
+            if (!leader) {
+                // the even CTA's last commit: all MMAs that touch this CTA are complete
+                if (lane == 0 && !wait_bounded(smem_u32(S.mma_done), 0, S.abort_flag, P.err, P.timeout_ns)) stop_peer();
+            } else {
+                // -------------------------------------------------------- MMA issuer
+                const uint32_t one = elect_one();
+                constexpr bool bf = MODE != MODE_FP16X3;
+                const uint32_t id_full = idesc_f16_m(2 * kTileM, P.tile_n, bf);
+                const uint32_t id_last = idesc_f16_m(2 * kTileM, P.tile_n_last, bf);
+                int s = 0, g_all = 0, n_item = 0;
+                uint32_t ph = 0, tph = 0;
+                bool ok = true;
+                auto arrived = [&](const uint64_t *bar, uint32_t parity) {
+                    const bool in =
+                        wait_bounded_cluster(smem_u32(bar), parity, S.abort_flag, P.err, P.timeout_ns);
+                    return __all_sync(0xffffffffu, in) != 0;
+                };
+                for (int64_t it = it0; it < nit && ok; it += istride, ++n_item) {
+                    for (int nt = 0; nt < P.ntiles_n && ok; ++nt, ++g_all) {
+                        const uint32_t idesc = (nt == P.ntiles_n - 1) ? id_last : id_full;
+                        const int b = g_all & 1;
+                        if (!arrived(&S.tempty[b], ((tph >> b) & 1) ^ 1)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t d = tmem_base + (uint32_t)(b * kAccStride);
+                        for (int kb = 0; kb < P.kblocks; kb += P.kbs) {
+                            const int n = min(P.kbs, P.kblocks - kb);
+                            if (!arrived(&S.full[s], ph)) {
+                                ok = false;
+                                break;
+                            }
+                            tc_fence_after();
+                            uint32_t st = smem_u32(S.ring + (size_t)s * S.stage_bytes);
+                            for (int i = 0; i < n; ++i, st += S.sub_bytes) {
+                                const uint32_t a_hi = st, a_lo = st + kFoldPart;
+                                const uint32_t b_hi = st + kPartsBytes, b_lo = b_hi + b_bytes;
+#pragma unroll
+                                for (int kk = 0; kk < kKBlock / 16; ++kk) {
+                                    const uint32_t ko = kk * 32;
+                                    const uint32_t acc = (kb > 0 || i > 0 || kk > 0) ? 1u : 0u;
+                                    mma_f16_pair(d, sdesc_k64(a_hi + ko), sdesc_k64(b_hi + ko), idesc, acc, one);
+                                    if (kSplitPrec) {
+                                        mma_f16_pair(d, sdesc_k64(a_hi + ko), sdesc_k64(b_lo + ko), idesc, 1u, one);
+                                        mma_f16_pair(d, sdesc_k64(a_lo + ko), sdesc_k64(b_hi + ko), idesc, 1u, one);
+                                    }
+                                }
+                            }
+                            mma_commit_pair_mc(smem_u32(&S.empty[s]), (uint16_t)3, one);
+                            if (++s == P.stages) { s = 0; ph ^= 1; }
+                        }
+                        if (!ok) break;
+                        mma_commit_pair_mc(smem_u32(&S.tfull[b]), (uint16_t)3, one);
+                        tph ^= 1u << b;
+                    }
+                    // every load of the item's ring slot has arrived (in both CTAs): the splitters may refill it
+                    if (ok) mma_commit_pair_mc(smem_u32(&S.afree[n_item & 1]), (uint16_t)3, one);
+                }
+                if (!ok) stop_peer();
+                // both CTAs wait for this commit before they leave (the odd CTA in its warp 1)
+                mma_commit_pair_mc(smem_u32(S.mma_done), (uint16_t)3, one);
+                wait_bounded(smem_u32(S.mma_done), 0, S.abort_flag, P.err, P.timeout_ns, false);
+            }
+        } else if (!CHAN && warp == 2 && P.sslots > 0) {
+            // ------------------------------------------------------------ loader
+            // 8 whole rows of each array per slot: [array][8][nchan]
+            if (lane == 0) {
+                const uint32_t bytes = 8u * (uint32_t)P.src.nchan * 4u;
+                int s = 0;
+                uint32_t ph = 0, pending = 0, pend_par = 0;
+                bool ok = true;
+                for (int64_t it = it0; it < nit && ok; it += istride) {
+                    const int64_t los0 = (2 * it + rank) * kFoldTileLos;
+                    if (los0 + kFoldTileLos > nlos) continue;      // the splitters load a partial item
+                    for (int g = 0; g < kFoldTileLos / 8; ++g) {
+                        if (!wait_bounded(smem_u32(&S.sempty[s]), ph ^ 1, S.abort_flag, P.err, P.timeout_ns)) {
+                            ok = false;
+                            break;
+                        }
+                        const uint32_t dst = smem_u32(S.stage + (size_t)s * P.sbytes), bar = smem_u32(&S.sfull[s]);
+                        const int64_t at = (los0 + 8 * g) * P.src.nchan;
+                        mbar_arrive_expect_tx(bar, 2 * bytes);
+                        bulk_load_once(dst, P.src.Q + at, bytes, bar);
+                        bulk_load_once(dst + bytes, P.src.U + at, bytes, bar);
+                        pending |= 1u << s;
+                        pend_par = (pend_par & ~(1u << s)) | (ph << s);
+                        if (++s == P.sslots) { s = 0; ph ^= 1; }
+                    }
+                }
+                if (!ok) stop_peer();
+                // copies in flight land before the CTA may leave
+                for (int i = 0; i < P.sslots; ++i)
+                    if (pending & (1u << i))
+                        wait_bounded(smem_u32(&S.sfull[i]), (pend_par >> i) & 1, S.abort_flag, P.err, P.timeout_ns, false);
+            }
+        }
+    } else if (warp < kSplitWarp0) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
+        // ------------------------------------------------------------ epilogue
+        // TMEM lanes and F's sectors as in gemm.cu: thread (rq, cq) holds the Q and U rows
+        // of LOS 16 q + 8 l + rq, columns 4 g + cq; a lane whose sample lies in the next
+        // 32-byte sector stores one group later.  32 columns of both LOS are loaded ahead.
+        const int q = warp & 3, h = (warp - kEpiWarp0) >> 2;
+        const int rq = lane >> 2, cq = lane & 3;
+        uint32_t tph = 0;
+        int g_all = 0, n_item = 0;
+        bool ok = true;
+        uint32_t tempty_addr[2];
+        for (int b = 0; b < 2; ++b) tempty_addr[b] = mapa_shared(smem_u32(&S.tempty[b]), 0u);
+        const int half = (P.tile_n / 16) * 8;          // columns of half 0 (a multiple of 8)
+        for (int64_t it = it0; it < nit && ok; it += istride, ++n_item) {
+            const int64_t row0 = (2 * it + rank) * kFoldTileLos + 16 * q + rq;
+            float scale[2] = {P.out_scale, P.out_scale};
+            float bm[2] = {-1.f, -1.f}, br[2] = {0.f, 0.f}, bim[2] = {0.f, 0.f};
+            int bi[2] = {INT_MAX, INT_MAX};
+            for (int nt = 0; nt < P.ntiles_n; ++nt, ++g_all) {
+                const int b = g_all & 1;
+                if (!warp_wait(smem_u32(&S.tfull[b]), (tph >> b) & 1, S.abort_flag, P.err, P.timeout_ns)) {
+                    ok = false;
+                    break;
+                }
+                tph ^= 1u << b;
+                tc_fence_after();
+                if (MODE == MODE_FP16X3 && nt == 0) {
+                    // written by this CTA's splitters before they released the item
+#pragma unroll
+                    for (int l = 0; l < 2; ++l)
+                        scale[l] = ldexpf(P.out_scale, -S.los_exp[(n_item & (kExpSlots - 1)) * 64 + 16 * q + 8 * l + rq]);
+                }
+                const int ncols = ((nt == P.ntiles_n - 1) ? P.tile_n_last : P.tile_n) - h * half;
+                const int kbase = (nt * P.tile_n + h * half) >> 1;
+                const int mine = min(ncols, h ? P.tile_n - half : half);   // columns of this half with results
+                const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * kAccStride + h * half);
+                float2 *dp[2], *dm[2];
+                bool latep[2], latem[2], st[2];
+                float2 prevp[2], prevm[2];
+                bool okp1 = false, okm1 = false;
+#pragma unroll
+                for (int l = 0; l < 2; ++l) {
+                    const int64_t r = row0 + 8 * l;
+                    st[l] = P.F != nullptr && r < nlos;
+                    dp[l] = reinterpret_cast<float2 *>(P.F) + (r * P.nphi + P.kplus + kbase);
+                    dm[l] = reinterpret_cast<float2 *>(P.F) + (r * P.nphi + P.kminus - kbase);
+                    latep[l] = (int)((reinterpret_cast<uintptr_t>(dp[l]) >> 3) & 3) + cq >= 4;
+                    latem[l] = (int)((reinterpret_cast<uintptr_t>(dm[l]) >> 3) & 3) < cq;
+                    dp[l] += cq - (latep[l] ? 4 : 0);
+                    dm[l] -= cq - (latem[l] ? 4 : 0);
+                    prevp[l] = prevm[l] = make_float2(0.f, 0.f);
+                }
+                auto group = [&](int gg, const uint32_t (&v0)[4], const uint32_t (&v1)[4], bool last) {
+                    // last: no columns of its own, only the late lanes' stores of the group before
+                    const int c = kbase + 4 * gg + cq;
+                    const bool okp = !last && 2 * (4 * gg + cq) < mine && c < P.ncol;
+                    const bool okm = okp && P.kminus - c != P.kplus + c;   // phi = 0 is its own partner
+#pragma unroll
+                    for (int l = 0; l < 2; ++l) {
+                        const uint32_t(&v)[4] = l ? v1 : v0;
+                        const float qc = __uint_as_float(v[0]), qs = __uint_as_float(v[1]);
+                        const float uc = __uint_as_float(v[2]), us = __uint_as_float(v[3]);
+                        const float2 vp = make_float2((qc + us) * scale[l], (uc - qs) * scale[l]);
+                        const float2 vm = make_float2((qc - us) * scale[l], (uc + qs) * scale[l]);
+                        const float mp = __fadd_rn(__fmul_rn(vp.x, vp.x), __fmul_rn(vp.y, vp.y));
+                        const float mm = __fadd_rn(__fmul_rn(vm.x, vm.x), __fmul_rn(vm.y, vm.y));
+                        // lowest index among equals: a +phi index is above, a -phi one below all before it
+                        if (okp && mp > bm[l]) { bm[l] = mp; bi[l] = P.kplus + c; br[l] = vp.x; bim[l] = vp.y; }
+                        if (okm && mm >= bm[l]) { bm[l] = mm; bi[l] = P.kminus - c; br[l] = vm.x; bim[l] = vm.y; }
+                        if (st[l]) {
+                            // streaming stores: F is written once and must not push the operands out of L2
+                            if (latep[l] ? okp1 : okp) __stcs(dp[l] + 4 * gg, latep[l] ? prevp[l] : vp);
+                            if (latem[l] ? okm1 : okm) __stcs(dm[l] - 4 * gg, latem[l] ? prevm[l] : vm);
+                        }
+                        prevp[l] = vp;
+                        prevm[l] = vm;
+                    }
+                    okp1 = okp;
+                    okm1 = okm;
+                };
+                for (int c0 = 0; c0 < mine; c0 += 32) {
+                    uint32_t v[2][16];
+                    tmem_ld16x256x4(taddr + c0, v[0]);
+                    tmem_ld16x256x4(taddr + (16u << 16) + c0, v[1]);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (c0 + 8 * j >= mine) break;
+                        const uint32_t a0[4] = {v[0][4 * j], v[0][4 * j + 1], v[0][4 * j + 2], v[0][4 * j + 3]};
+                        const uint32_t a1[4] = {v[1][4 * j], v[1][4 * j + 1], v[1][4 * j + 2], v[1][4 * j + 3]};
+                        group((c0 >> 3) + j, a0, a1, false);
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(tempty_addr[b]);
+                const uint32_t none[4] = {0u, 0u, 0u, 0u};
+                if (mine > 0) group((mine + 7) >> 3, none, none, true);
+            }
+            if (!ok) break;
+            // the four lanes of a row group hold disjoint columns of the same two LOS: a butterfly
+            // leaves every lane with both peaks (lowest index on ties); lane cq owns LOS l = cq
+#pragma unroll
+            for (int l = 0; l < 2; ++l)
+#pragma unroll
+                for (int off = 1; off <= 2; off <<= 1) {
+                    const float om = __shfl_xor_sync(0xffffffffu, bm[l], off);
+                    const int oi = __shfl_xor_sync(0xffffffffu, bi[l], off);
+                    const float ore = __shfl_xor_sync(0xffffffffu, br[l], off);
+                    const float oim = __shfl_xor_sync(0xffffffffu, bim[l], off);
+                    if (om > bm[l] || (om == bm[l] && oi < bi[l])) { bm[l] = om; bi[l] = oi; br[l] = ore; bim[l] = oim; }
+                }
+            const bool owner = cq < 2;
+            float pm = cq ? bm[1] : bm[0], pre = cq ? br[1] : br[0], pim = cq ? bim[1] : bim[0];
+            int pi = cq ? bi[1] : bi[0];
+            // combine the two column halves: half 1 publishes, half 0 writes
+            const int par = n_item & 1, at = par * 64 + 16 * q + 8 * (cq & 1) + rq;
+            const uint32_t pbar = smem_u32(&S.pkfull[par * 4 + q]), ebar = smem_u32(&S.pkempty[par * 4 + q]);
+            const uint32_t use_par = (n_item >> 1) & 1;
+            if (h == 1) {
+                if (!warp_wait(ebar, use_par ^ 1, S.abort_flag, P.err, P.timeout_ns)) { ok = false; break; }
+                if (owner) {
+                    S.pk_m[at] = pm;
+                    S.pk_i[at] = pi;
+                    S.pk_re[at] = pre;
+                    S.pk_im[at] = pim;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(pbar);
+            } else {
+                if (!warp_wait(pbar, use_par, S.abort_flag, P.err, P.timeout_ns)) { ok = false; break; }
+                const float om = S.pk_m[at], ore = S.pk_re[at], oim = S.pk_im[at];
+                const int oi = S.pk_i[at];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(ebar);
+                if (om > pm || (om == pm && oi < pi)) { pm = om; pi = oi; pre = ore; pim = oim; }
+                const int64_t r = (2 * it + rank) * kFoldTileLos + 16 * q + 8 * (cq & 1) + rq;
+                if (owner && r < nlos) {
+                    const bool found = pi != INT_MAX;
+                    const float nan = __int_as_float(0x7fc00000);
+                    if (P.pidx) P.pidx[r] = found ? pi : -1;
+                    if (P.pabs) P.pabs[r] = found ? sqrtf(pm) : nan;
+                    if (P.pphi) P.pphi[r] = found ? P.phi32[pi] : nan;
+                    if (P.pq) P.pq[r] = found ? pre : nan;
+                    if (P.pu) P.pu[r] = found ? pim : nan;
+                    if (P.pchi) {
+                        // chi0 = arg F(phi_peak) / 2 - phi_peak lambda_0^2, reduced to [0, pi)
+                        float c = nan;
+                        if (found) {
+                            double x = 0.5 * atan2((double)pim, (double)pre) - P.phi64[pi] * P.lambda0sq;
+                            x -= M_PI * floor(x / M_PI);
+                            c = (float)x;
+                        }
+                        P.pchi[r] = c;
+                    }
+                }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsSplit));
+        // ------------------------------------------------------------ splitters
+        const int sw = warp - kSplitWarp0;
+        // channel-major: this warp's 32 LOS of the tile, its array and first half K block
+        const int i = 32 * (sw & 1) + lane, array = (sw >> 1) & 1, h0 = sw >> 2, nh = 2 * P.kblocks;
+        const int row = 16 * (i >> 3) + (i & 7) + 8 * array, swz = (row >> 1) & 3;
+        int n_item = 0, ss = 0, n_max = 0;
+        uint32_t sph = 0;
+        bool ok = true;
+        // FP16X3: publish this warp's maxima and wait for the other warps' (null: aborted)
+        auto join_max = [&](float mx) -> const float * {
+            float *x = S.los_max + (n_max & 1) * kNumSplitWarps * 32;
+            x[sw * 32 + lane] = mx;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(S.xmax));
+            if (!warp_wait(smem_u32(S.xmax), n_max & 1, S.abort_flag, P.err, P.timeout_ns)) return nullptr;
+            ++n_max;
+            return x;
+        };
+        for (int64_t it = it0; it < nit && ok; it += istride, ++n_item) {
+            const int slot = n_item & 1;
+            const int64_t los0 = (2 * it + rank) * kFoldTileLos;
+            const bool stg = !CHAN && P.sslots > 0 && los0 + kFoldTileLos <= nlos;
+            uint8_t *const tile = P.ring + ((size_t)blockIdx.x * 2 + slot) * P.kblocks * kPartsBytes;
+            int *const exps = S.los_exp + (n_item & (kExpSlots - 1)) * 64;
+            const int64_t los8 = los0 + 8 * sw;            // LOS-major, direct: this warp's 8 LOS
+            auto src_of = [&](int r) { return min(los8 + r, nlos - 1); };
+            const uint32_t dead = los8 + 8 <= nlos ? 0u : (0xffu << (int)max((int64_t)0, nlos - los8)) & 0xffu;
+            float scale[8] = {1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f};
+            int ex[8];
+            if constexpr (MODE == MODE_FP16X3) {
+                // the LOS's largest |value| sets its power-of-two scale: a first pass over the tile
+                // (staged LOS-major rows are complete in their slot and need none)
+                if constexpr (CHAN) {
+                    float mx = 0.f;
+                    chan_walk<false>(P.src, S.list, los0 + i, array, h0, nh, [&](int, const float (&v)[16]) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) mx = fmaxf(mx, fabsf(v[j]));
+                    });
+                    const float *x = join_max(mx);
+                    if (!x) {
+                        ok = false;
+                        break;
+                    }
+#pragma unroll
+                    for (int w = 0; w < kNumSplitWarps; w += 2) mx = fmaxf(mx, x[(w + (sw & 1)) * 32 + lane]);
+                    ex[0] = fold_exponent(mx);
+                    scale[0] = ldexpf(1.0f, ex[0]);
+                } else if (!stg) {
+                    fold_scales_los(P.src, S.list, P.kblocks, lane, src_of, dead, scale, ex);
+                }
+            }
+            // the slot's previous item has been read; and the epilogue is done with the item four
+            // before, whose exponents are replaced: its phase tiles are drained
+            if (!warp_wait(smem_u32(&S.afree[slot]), ((n_item >> 1) & 1) ^ 1, S.abort_flag, P.err, P.timeout_ns)) {
+                ok = false;
+                break;
+            }
+            if constexpr (CHAN) {
+                if (MODE == MODE_FP16X3 && sw < 2) exps[i] = ex[0];
+                uint8_t *const dst = tile + row * kFoldRowBytes;
+                chan_walk<true>(P.src, S.list, los0 + i, array, h0, nh, [&](int h, const float (&v)[16]) {
+                    emit16<MODE, true>(dst + (size_t)(h >> 1) * kPartsBytes, h & 1, swz, v, scale[0]);
+                });
+            } else if (stg) {
+                // 8 LOS per slot; units of (K block, array) go round the warps
+                for (int g = 0; g < kFoldTileLos / 8; ++g) {
+                    if (!warp_wait(smem_u32(&S.sfull[ss]), sph, S.abort_flag, P.err, P.timeout_ns)) {
+                        ok = false;
+                        break;
+                    }
+                    const float *rows = reinterpret_cast<const float *>(S.stage + (size_t)ss * P.sbytes);
+                    const int nchan = P.src.nchan;
+                    if constexpr (MODE == MODE_FP16X3) {
+                        // warp sw finds row sw's largest active |value|
+                        float mx = 0.f;
+                        for (int a = lane; a < P.src.nact; a += 32) {
+                            const int ch = S.list[a];
+                            mx = fmaxf(mx, fmaxf(fabsf(rows[sw * nchan + ch]), fabsf(rows[(8 + sw) * nchan + ch])));
+                        }
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                        const float *x = join_max(mx);
+                        if (!x) {
+                            ok = false;
+                            break;
+                        }
+#pragma unroll
+                        for (int r = 0; r < 8; ++r) {
+                            ex[r] = fold_exponent(x[r * 32]);
+                            scale[r] = ldexpf(1.0f, ex[r]);
+                            if (sw == 0 && lane == r) exps[8 * g + r] = ex[r];
+                        }
+                    }
+                    const int arr = sw & 1;
+                    for (int kb = sw >> 1; kb < P.kblocks; kb += kNumSplitWarps / 2) {
+                        const int ch = S.list[kb * kKBlock + lane];
+                        const bool live = kb * kKBlock + lane < P.src.nact;
+                        float v[8];
+#pragma unroll
+                        for (int r = 0; r < 8; ++r) v[r] = live ? rows[(8 * arr + r) * nchan + ch] : 0.f;
+                        fold_emit_rows<MODE, true>(tile + (size_t)kb * kPartsBytes + (16 * g + 8 * arr) * kFoldRowBytes, lane, v,
+                                             scale);
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&S.sempty[ss]));
+                    if (++ss == P.sslots) { ss = 0; sph ^= 1; }
+                }
+            } else {
+                if constexpr (MODE == MODE_FP16X3) {
+#pragma unroll
+                    for (int r = 0; r < 8; ++r)
+                        if (lane == r) exps[8 * sw + r] = ex[r];
+                }
+                uint8_t *const dst = tile + 16 * sw * kFoldRowBytes;
+                for (int kb = 0; kb < P.kblocks; ++kb) {
+                    float q[8], u[8];
+                    fold_load_los<true>(P.src, S.list, kb, lane, src_of, q, u);
+                    fold_mask_los(P.src, kb, lane, dead, q, u);
+                    fold_emit_rows<MODE, true>(dst + (size_t)kb * kPartsBytes, lane, q, scale);
+                    fold_emit_rows<MODE, true>(dst + (size_t)kb * kPartsBytes + 8 * kFoldRowBytes, lane, u, scale);
+                }
+            }
+            if (!ok) break;
+            // the TMA (async proxy) reads what these generic stores wrote
+            fence_proxy_async_global();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&S.ready[slot]));
+        }
+        // the commits that free the last slots arrive before the CTA leaves
+        for (int k = max(0, n_item - 2); k < n_item && ok; ++k)
+            ok = warp_wait(smem_u32(&S.afree[k & 1]), (k >> 1) & 1, S.abort_flag, P.err, P.timeout_ns);
+        if (!ok) stop_peer();
+    }
+
+    if (*S.abort_flag) stop_peer();
+    tc_fence_before();
+    __syncthreads();
+    // the ring's lines go back to normal priority: nobody else's working set should yield to them
+    {
+        uint8_t *const own = P.ring + (size_t)blockIdx.x * 2 * P.kblocks * kPartsBytes;
+        for (size_t at = (size_t)threadIdx.x * 128; at < (size_t)2 * P.kblocks * kPartsBytes; at += kThreads * 128)
+            asm volatile("applypriority.global.L2::evict_normal [%0], 128;" ::"l"(own + at) : "memory");
+    }
+    // neither CTA leaves (or frees TMEM) while the other may still use its shared memory,
+    // barriers or TMEM
+    cluster_sync_all();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, kTmemCols);
+    }
+}
+
+}  // namespace
+
+namespace {
+
+using FusedKernel = void (*)(FusedParams, CUtensorMap, CUtensorMap, CUtensorMap);
+
+FusedKernel fused_for(int mode, bool chan)
+{
+    if (mode == MODE_BF16) return chan ? fused_kernel<MODE_BF16, true> : fused_kernel<MODE_BF16, false>;
+    if (mode == MODE_BF16X3) return chan ? fused_kernel<MODE_BF16X3, true> : fused_kernel<MODE_BF16X3, false>;
+    return chan ? fused_kernel<MODE_FP16X3, true> : fused_kernel<MODE_FP16X3, false>;
+}
+
+// Pipeline shape beside `staging` bytes of staging slots and the channel list: K blocks per stage and stages, at
+// least three of them; stages = 0 if they do not fit.
+struct Shape {
+    int kbs = 0, stages = 0;
+    size_t smem = 0;
+};
+Shape shape_for(const rms_plan_s &p, size_t staging)
+{
+    Shape s;
+    const int tile_n = p.fold.tiles.tile_n2, mode = mode_of(p.precision);
+    staging += (size_t)p.fold.kpad * sizeof(int);
+    for (s.kbs = 4; s.kbs >= 1; s.kbs /= 2) {
+        const size_t per = s.kbs * (size_t)sub_stage_bytes(tile_n, mode) + 16;
+        if (kFixedSmem + staging + 3 * per > (size_t)kSmemLimit) continue;
+        s.stages = (int)std::min<size_t>(8, (kSmemLimit - kFixedSmem - staging) / per);
+        s.smem = kFixedSmem + staging + s.stages * per;
+        break;
+    }
+    return s;
+}
+
+// Staging slots of a LOS-major call: as many rows of 8 LOS as fit in 72 KB, two at least;
+// none where the bulk copies' 16-byte rule does not hold.
+constexpr size_t kStaging = 72 * 1024;
+int staging_slots(const rms_plan_s &p, const float *Q, const float *U, bool chan)
+{
+    if (chan || ((reinterpret_cast<uintptr_t>(Q) | reinterpret_cast<uintptr_t>(U)) & 15)) return 0;
+    const size_t slot = (size_t)2 * 8 * p.nchan * sizeof(float);
+    return 2 * slot > kStaging ? 0 : (int)std::min<size_t>(kMaxSlots, kStaging / slot);
+}
+
+cudaLaunchConfig_t launch_config(cudaLaunchAttribute *attr, unsigned grid, size_t smem, cudaStream_t s)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(kThreads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = 2;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    c.attrs = attr;
+    c.numAttrs = 1;
+    return c;
+}
+
+}  // namespace
+
+cudaError_t fused_prepare(rms_plan_s *p)
+{
+    FoldPlan &f = p->fold;
+    f.fused_pairs = 0;
+    const int mode = mode_of(p->precision);
+    if (!f.on || !f.pair_maps || (mode != MODE_BF16 && f.kblocks > kGroupKBlocks)) return cudaSuccess;
+    if (shape_for(*p, kStaging).stages < 3) return cudaSuccess;
+    for (bool chan : {true, false}) {
+        const FusedKernel k = fused_for(mode, chan);
+        cudaFuncAttributes fa;
+        cudaError_t e = cudaFuncGetAttributes(&fa, k);
+        if (e == cudaSuccess && fa.numRegs != kRegsLaunch) e = cudaErrorInvalidConfiguration;
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+        if (e != cudaSuccess) return e;
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t cfg = launch_config(&attr, 2 * (p->num_sms / 2), kSmemLimit, 0);
+        int n = 0;
+        e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
+        if (e != cudaSuccess) return e;
+        n = std::min(n, p->num_sms / 2);
+        f.fused_pairs = chan ? n : std::min(f.fused_pairs, n);
+    }
+    return cudaSuccess;
+}
+
+// One kernel unless the last round of items over the pairs is too empty (12,000 LOS are 94
+// items on 76 pairs: 69.9 against 64.2 us at 360 channels x 801 phi, but 161 items on two
+// thirds of three rounds 99.0 against 104) or there are few items with many phase tiles,
+// which the job schedule spreads over more SMs; FP16X3 only where its row maxima come with
+// the staged rows (channel-major it would walk each item twice: 0.92 against 0.81 ms on
+// 262,144 LOS x 360 x 401).  Measured with F and the peak map, one kernel against two:
+// 262,144 LOS x 360 x 401 BF16x3 0.474 / 0.636 ms (LOS-major 0.484 / 0.642), 200,003 x
+// 357 x 401 FP16x3 LOS-major 0.535 / 0.612, 400,000 x 800 x 1001 BF16 1.53 / 2.04 ms,
+// 5,000 LOS x 360 x 401 32.6 / 36.1 us.
+bool fused_wanted(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout)
+{
+    const FoldPlan &f = p.fold;
+    if (f.fused_pairs < 1 || p.contraction != RMS_CONTRACT_AUTO || p.schedule != RMS_SCHEDULE_AUTO || p.l2_budget != 0)
+        return false;
+    if (p.precision == RMS_FP16X3 && !staging_slots(p, Q, U, layout == RMS_CHAN_MAJOR)) return false;
+    const int64_t nit = (nlos + 2 * kFoldTileLos - 1) / (2 * kFoldTileLos);
+    const int64_t rounds = (nit + f.fused_pairs - 1) / f.fused_pairs;
+    if (rounds == 1) return 2 * nit >= f.fused_pairs || f.tiles.ntiles_n2 <= 2;
+    return 3 * nit >= 2 * rounds * f.fused_pairs;
+}
+
+size_t fused_ring_bytes(const rms_plan_s &p, int64_t nlos)
+{
+    const int64_t nit = (nlos + 2 * kFoldTileLos - 1) / (2 * kFoldTileLos);
+    const size_t parts = p.precision == RMS_BF16 ? 1 : 2;
+    return (size_t)(4 * std::min<int64_t>(nit, p.fold.fused_pairs)) * p.fold.kblocks * parts * kFoldPart;
+}
+
+cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout, float *F,
+                         int32_t *pidx, float *pabs, float *pphi, float *pq, float *pu, float *pchi, uint8_t *ring,
+                         cudaStream_t s)
+{
+    const FoldPlan &f = p.fold;
+    const bool chan = layout == RMS_CHAN_MAJOR;
+    const int mode = mode_of(p.precision);
+    const int64_t nit = (nlos + 2 * kFoldTileLos - 1) / (2 * kFoldTileLos);
+    const int pairs = (int)std::min<int64_t>(nit, f.fused_pairs);
+    FusedParams P;
+    P.src = {Q, U, nlos, p.nchan, p.nact, chan, p.d_active, p.d_active_pad};
+    P.kblocks = f.kblocks;
+    P.mode = mode;
+    P.nphi = p.nphi;
+    P.ncol = f.ncol;
+    P.kplus = f.kplus;
+    P.kminus = f.kminus;
+    P.ntiles_n = f.tiles.ntiles_n2;
+    P.tile_n = f.tiles.tile_n2;
+    P.tile_n_last = f.tiles.tile_n_last2;
+    P.ring = ring;
+    P.F = F;
+    P.pidx = pidx;
+    P.pabs = pabs;
+    P.pphi = pphi;
+    P.pq = pq;
+    P.pu = pu;
+    P.pchi = pchi;
+    P.phi32 = p.d_phi32;
+    P.phi64 = p.d_phi;
+    P.lambda0sq = p.lambda0sq;
+    P.out_scale = (float)(p.K * p.wmax);
+    P.err = p.d_err;
+    P.timeout_ns = p.timeout_ns;
+    P.sslots = staging_slots(p, Q, U, chan);
+    P.sbytes = (uint32_t)(2 * 8 * p.nchan * sizeof(float));
+    const Shape sh = shape_for(p, (size_t)P.sslots * P.sbytes);
+    if (sh.stages < 3) return cudaErrorInvalidConfiguration;
+    P.stages = sh.stages;
+    P.kbs = sh.kbs;
+    // the ring as a 3-D tensor: 64-byte rows, the hi (and lo) rows of a K block, K blocks
+    const int parts = mode == MODE_BF16 ? 1 : 2;
+    CUtensorMap tmA;
+    const cuuint64_t dims[3] = {(cuuint64_t)kKBlock, (cuuint64_t)(parts * kTileM), (cuuint64_t)(4 * pairs) * f.kblocks};
+    const cuuint64_t strides[2] = {(cuuint64_t)kFoldRowBytes, (cuuint64_t)(parts * kFoldPart)};
+    const cuuint32_t box[3] = {(cuuint32_t)kKBlock, (cuuint32_t)(parts * kTileM), 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    if (!encode_tensor_map(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT16, ring, dims, strides, box, estr,
+                           CU_TENSOR_MAP_SWIZZLE_NONE, 3))
+        return cudaErrorInvalidValue;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg =
+        launch_config(&attr, (unsigned)(2 * pairs), sh.smem, s);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_for(mode, chan), P, f.tmap2_bhi, f.tmap2_blo, tmA);
+    p.last_ctas = 2 * pairs;
+    p.last_pair = 1;
+    p.last_panels = 0;
+    p.last_kernels = 1;
+    return e;
+}

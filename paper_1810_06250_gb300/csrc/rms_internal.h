@@ -48,6 +48,7 @@ struct FoldPlan {
     int32_t kblocks = 0, kpad = 0; // K blocks of 32 active channels
     PhaseTiling tiles;
     uint16_t *d_hi = nullptr, *d_lo = nullptr;   // [tiles.npad][kpad]
+    int32_t fused_pairs = 0;       // the one-kernel form (fused.cu): resident CTA pairs (0: not for this plan)
     CUtensorMap tmap_bhi, tmap_blo, tmap2_bhi, tmap2_blo;
 };
 
@@ -60,6 +61,7 @@ struct rms_plan_s {
 
     // device arrays
     int32_t *d_active = nullptr;   // [nact] channel index of each active channel
+    int32_t *d_active_pad = nullptr;   // the same, padded to a multiple of 32 with the last active channel
     double *d_dl2 = nullptr;       // [nact] lambda_j^2 - lambda_0^2 (FP64)
     double *d_wact = nullptr;      // [nact] w_j
     double *d_phi = nullptr;       // [nphi]
@@ -175,6 +177,14 @@ size_t fold_operand_bytes(const rms_plan_s &p, int64_t nlos);
 cudaError_t launch_fold_split(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout,
                               uint8_t *A, int8_t *rexp, cudaStream_t s, const int64_t *rows = nullptr,
                               const int64_t *count = nullptr);
+// fused.cu: layout stage and contraction in one kernel, for plans whose K blocks form one
+// accumulation (fused_prepare, at plan creation) and calls of enough LOS (fused_wanted)
+cudaError_t fused_prepare(rms_plan_s *p);
+bool fused_wanted(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout);
+size_t fused_ring_bytes(const rms_plan_s &p, int64_t nlos);
+cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout, float *F,
+                         int32_t *pidx, float *pabs, float *pphi, float *pq, float *pu, float *pchi, uint8_t *ring,
+                         cudaStream_t s);
 struct SplitOpts {
     const float *Q = nullptr, *U = nullptr;
     int64_t nlos_src = 0;              // lines of sight in the cube

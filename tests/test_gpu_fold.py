@@ -82,3 +82,38 @@ def test_fold_edges(rms, oracle_mod, path, kind, nphi):
             gh.check_peaks_self(Fh, pi.cpu().numpy(), pa.cpu().numpy(), pp.cpu().numpy(), phi)
             if nlos > 3:
                 assert pi[2] == -1 and pi[3] == 0
+
+
+# several items per CTA pair with a ragged last one; three phase tiles; LOS-major rows too long for the staging
+# slots (75 channels otherwise); an odd number of LOS (channel-major rows off 16 bytes); data off 16 bytes
+@pytest.mark.parametrize("nlos,nchan,nphi,layout,shift", [(20011, 75, 103, "los", 0), (20011, 75, 401, "chan", 0),
+                                                         (29500, 75, 515, "los", 0), (20000, 75, 257, "chan", 1),
+                                                         (20011, 75, 64, "los", 1), (19999, 600, 33, "los", 0)])
+@pytest.mark.parametrize("path", ["bf16x3", "fp16x3", "bf16"])
+def test_one_kernel_matches_two(rms, path, nlos, nchan, nphi, layout, shift):
+    """The layout stage inside the contraction: the same bits as the split kernel and the contraction in turn."""
+    rng = np.random.default_rng(nlos + nphi)
+    freq = np.linspace(120e6, 168e6, nchan)
+    w = rng.uniform(0.5, 1.5, nchan)
+    w[rng.choice(nchan, 7, replace=False)] = 0.0
+    phi = grid("up", nphi)
+    data = torch.randn(2, nlos * nchan + 4, device="cuda", generator=torch.Generator("cuda").manual_seed(nphi))
+    data[0, 5 * nchan:6 * nchan] = float("nan")
+    data[:, 7 * nchan:9 * nchan] = 0.0
+    q, u = (data[i, shift:shift + nlos * nchan] for i in range(2))
+    got = []
+    with rms.Plan(freq, phi, path, weights=w) as plan:
+        for kind in (rms.RMS_CONTRACT_AUTO, rms.RMS_CONTRACT_PAIR):
+            rms.rms_plan_set_option(plan.handle, rms.RMS_OPT_CONTRACTION, kind)
+            for with_f in (True, False):
+                F = torch.full((nlos, nphi, 2), 3.0, device="cuda") if with_f else None
+                out = [torch.full((nlos,), -7, dtype=torch.int32, device="cuda")]
+                out += [torch.full((nlos,), -7.0, device="cuda") for _ in range(5)]
+                rms.rms_synth_peaks(plan.handle, q, u, nlos, layout, F, *out)
+                plan.sync()
+                got.append(([F] if with_f else []) + out)
+    for a, b in ((0, 2), (1, 3)):
+        for x, y in zip(got[a], got[b]):
+            assert torch.equal(x.view(torch.int32), y.view(torch.int32))
+    for x, y in zip(got[0][1:], got[1]):
+        assert torch.equal(x.view(torch.int32), y.view(torch.int32))
