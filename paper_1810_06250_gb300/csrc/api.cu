@@ -52,7 +52,6 @@ void free_plan(rms_plan_s *p)
 {
     if (!p) return;
     cudaFree(p->d_active);
-    cudaFree(p->d_active_pad);
     cudaFree(p->d_dl2);
     cudaFree(p->d_wact);
     cudaFree(p->d_phi);
@@ -69,7 +68,7 @@ void free_plan(rms_plan_s *p)
     cudaFree(p->d_w_all);
     if (p->d_bhi_raw != p->d_bhi) cudaFree(p->d_bhi_raw);
     if (p->d_blo_raw != p->d_blo) cudaFree(p->d_blo_raw);
-    cudaFree(p->d_dh);
+    cudaFree(p->fold.d_list);
     cudaFree(p->fold.d_hi);
     cudaFree(p->fold.d_lo);
     cudaFree(p->d_kbmask);
@@ -336,12 +335,10 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
             tile = (per + 15) / 16 * 16;
             last = (N - (ntiles - 1) * tile + 15) / 16 * 16;
         };
-        auto both_tilings = [&](int N, PhaseTiling &t) {
-            tiling(N, max_tile, t.ntiles_n, t.tile_n, t.tile_n_last);
-            tiling(N, max_tile_cap == kMaxTileN ? kMaxTileNPair : max_tile, t.ntiles_n2, t.tile_n2, t.tile_n_last2);
-            t.npad = std::max(t.ntiles_n * t.tile_n, t.ntiles_n2 * t.tile_n2);
-        };
-        both_tilings(2 * nphi, p->tiles);
+        PhaseTiling &t = p->tiles;
+        tiling(2 * nphi, max_tile, t.ntiles_n, t.tile_n, t.tile_n_last);
+        tiling(2 * nphi, max_tile_cap == kMaxTileN ? kMaxTileNPair : max_tile, t.ntiles_n2, t.tile_n2, t.tile_n_last2);
+        t.npad = std::max(t.ntiles_n * t.tile_n, t.ntiles_n2 * t.tile_n2);
         p->kblocks = (p->nact + kChanPerKBlock - 1) / kChanPerKBlock;
         p->kpad = p->kblocks * kKBlock;
         const bool fp16 = precision == RMS_FP16X3;
@@ -389,31 +386,44 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
                            encode_b_map(&p->tmap2_bhi_raw, p->d_bhi_raw, p->kpad_raw, p->tiles.npad, h) &&
                            encode_b_map(&p->tmap2_blo_raw, p->d_blo_raw, p->kpad_raw, p->tiles.npad, h);
         }
-        if (p->fold.on) {
+        const bool window = max_tile_cap != kMaxTileN;
+        if (p->fold.on || window) {
             FoldPlan &f = p->fold;
+            std::vector<double> dh;
+            if (window) {
+                // offsets -W/2 .. W/2 - 1 of a step: column pair i holds offsets +-i
+                f.ncol = nphi / 2 + 1;
+                f.kplus = f.kminus = nphi / 2;
+                for (int i = 0; i < f.ncol; ++i) dh.push_back(-phi[f.kminus - i]);
+            } else {
+                for (int i = 0; i < f.ncol; ++i) dh.push_back(0.5 * (phi[f.kplus + i] - phi[f.kminus - i]));
+            }
             f.kblocks = (p->nact + kKBlock - 1) / kKBlock;
             f.kpad = f.kblocks * kKBlock;
-            both_tilings(2 * f.ncol, f.tiles);
-            std::vector<double> dh(f.ncol);
-            for (int i = 0; i < f.ncol; ++i) dh[i] = 0.5 * (phi[f.kplus + i] - phi[f.kminus - i]);
-            RMS_TRY(dalloc(&p->d_dh, f.ncol));
-            RMS_TRY(cudaMemcpy(p->d_dh, dh.data(), f.ncol * sizeof(double), cudaMemcpyHostToDevice));
+            tiling(2 * f.ncol, max_tile, f.tiles.ntiles_n, f.tiles.tile_n, f.tiles.tile_n_last);
+            tiling(2 * f.ncol, kMaxTileNPair, f.tiles.ntiles_n2, f.tiles.tile_n2, f.tiles.tile_n_last2);
+            f.tiles.npad = std::max(f.tiles.ntiles_n * f.tiles.tile_n, f.tiles.ntiles_n2 * f.tiles.tile_n2);
+            std::vector<int32_t> list(p->active);
+            list.resize(f.kpad, p->active.back());
+            RMS_TRY(dalloc(&f.d_list, f.kpad));
+            RMS_TRY(cudaMemcpy(f.d_list, list.data(), f.kpad * sizeof(int32_t), cudaMemcpyHostToDevice));
             RMS_TRY(dalloc(&f.d_hi, (size_t)f.tiles.npad * f.kpad));
             RMS_TRY(dalloc(&f.d_lo, (size_t)f.tiles.npad * f.kpad));
-            RMS_TRY(launch_phase_fold(*p, p->d_dh, fp16, 0));
+            double *d_dh = nullptr;
+            RMS_TRY(dalloc(&d_dh, f.ncol));
+            e = cudaMemcpy(d_dh, dh.data(), f.ncol * sizeof(double), cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = launch_phase_fold(*p, f, d_dh, fp16, 0);
+            cudaFree(d_dh);         // after the launch's work: cudaFree synchronises
+            RMS_TRY(e);
             const int h = f.tiles.tile_n2 / 2;
             if (!encode_b_map(&f.tmap_bhi, f.d_hi, f.kpad, f.tiles.npad, f.tiles.tile_n) ||
                 !encode_b_map(&f.tmap_blo, f.d_lo, f.kpad, f.tiles.npad, f.tiles.tile_n)) {
                 free_plan(p);
                 return RMS_ERR_CUDA;
             }
-            std::vector<int32_t> padded(p->active);
-            padded.resize(f.kpad, p->active.back());
-            RMS_TRY(dalloc(&p->d_active_pad, f.kpad));
-            RMS_TRY(cudaMemcpy(p->d_active_pad, padded.data(), f.kpad * sizeof(int32_t), cudaMemcpyHostToDevice));
             f.pair_maps = encode_b_map(&f.tmap2_bhi, f.d_hi, f.kpad, f.tiles.npad, h) &&
                           encode_b_map(&f.tmap2_blo, f.d_lo, f.kpad, f.tiles.npad, h);
-            RMS_TRY(fused_prepare(p));
+            RMS_TRY(fused_prepare(p, window));
         }
     }
     RMS_TRY(cudaEventCreateWithFlags(&p->last, cudaEventDisableTiming));

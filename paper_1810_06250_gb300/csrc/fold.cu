@@ -125,8 +125,8 @@ __global__ void __launch_bounds__(256, MODE == MODE_FP16X3 ? 3 : 4) fold_split_l
         float q[8], u[8];
         fold_load_los<false>(P.src, P.src.padded, kb, lane, src_of, q, u);
         fold_mask_los(P.src, kb, lane, dead, q, u);
-        fold_emit_rows<MODE, false>(group + (size_t)kb * kBlock, lane, q, scale);
-        fold_emit_rows<MODE, false>(group + (size_t)kb * kBlock + 8 * kFoldRowBytes, lane, u, scale);
+        fold_emit_rows<MODE, false, 8>(group + (size_t)kb * kBlock, lane, 0, q, scale);
+        fold_emit_rows<MODE, false, 8>(group + (size_t)kb * kBlock + 8 * kFoldRowBytes, lane, 0, u, scale);
     }
 }
 
@@ -144,7 +144,7 @@ cudaError_t launch_fold_split(const rms_plan_s &p, const float *Q, const float *
     if (nb > 0x7fffffff) return cudaErrorInvalidValue;
     if (mode == MODE_FP16X3 && !rexp) return cudaErrorInvalidValue;
     FoldSplitParams P;
-    P.src = {Q, U, nlos, p.nchan, p.nact, chan, p.d_active, p.d_active_pad};
+    P.src = {Q, U, nlos, p.nchan, p.nact, chan, p.d_active, p.fold.d_list};
     P.rows = rows;
     P.count = count;
     P.kblocks = p.fold.kblocks;

@@ -151,15 +151,17 @@ __device__ __forceinline__ void fold_scales_los(const FoldSource &S, const int *
     }
 }
 
-// One K block of 8 LOS' Q or U; rows: the first of the 8 operand rows in K block kb of the image.
-template <int MODE, bool RING>
-__device__ __forceinline__ void fold_emit_rows(uint8_t *rows, int lane, const float (&v)[8], const float (&scale)[8])
+// One K block of LOS r0 .. r0 + N - 1 of a group of 8, Q or U; rows: the group's first
+// operand row in K block kb of the image.
+template <int MODE, bool RING, int N>
+__device__ __forceinline__ void fold_emit_rows(uint8_t *rows, int lane, int r0, const float (&v)[N], const float (&scale)[8])
 {
     uint8_t *const mine = rows + ((lane & 1) ? kFoldPart : 0) + 4 * ((lane >> 1) & 3);
     const int chunk = lane >> 3;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const uint32_t w = split_one<MODE>(MODE == MODE_FP16X3 ? v[r] * scale[r] : v[r]);
+    for (int j = 0; j < N; ++j) {
+        const int r = r0 + j;
+        const uint32_t w = split_one<MODE>(MODE == MODE_FP16X3 ? v[j] * scale[j] : v[j]);
         const uint32_t p = __shfl_xor_sync(0xffffffffu, w, 1);
         const uint32_t o = (lane & 1) ? __byte_perm(p, w, 0x7632) : __byte_perm(w, p, 0x5410);
         uint8_t *at = mine + r * kFoldRowBytes + ((chunk ^ ((r >> 1) & 3)) << 4);

@@ -69,6 +69,7 @@ struct FusedParams {
     int32_t stages, kbs;        // pipeline stages of kbs K blocks each
     int32_t sslots;             // staging slots; 0: direct loads
     uint32_t sbytes;            // bytes of a staging slot
+    FusedRotation rot;          // ROT
 };
 
 __host__ __device__ __forceinline__ uint32_t sub_stage_bytes(int tile_n, int mode)
@@ -183,7 +184,17 @@ __device__ __forceinline__ void chan_walk(const FoldSource &S, const int *list, 
     }
 }
 
-template <int MODE, bool CHAN>
+// (q + iu) t
+__device__ __forceinline__ void rotate(float &q, float &u, float2 t)
+{
+    const float qr = fmaf(q, t.x, -u * t.y), ur = fmaf(q, t.y, u * t.x);
+    q = qr;
+    u = ur;
+}
+
+// ROT: window synthesis (learned.cu): every LOS is multiplied by its own row of T on its
+// way into the ring, in FP32 like the data.
+template <int MODE, bool CHAN, bool ROT>
 __global__ void __launch_bounds__(kThreads, 1)
 fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUtensorMap tmB_hi,
              const __grid_constant__ CUtensorMap tmB_lo, const __grid_constant__ CUtensorMap tmA)
@@ -463,8 +474,9 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                 auto group = [&](int gg, const uint32_t (&v0)[4], const uint32_t (&v1)[4], bool last) {
                     // last: no columns of its own, only the late lanes' stores of the group before
                     const int c = kbase + 4 * gg + cq;
-                    const bool okp = !last && 2 * (4 * gg + cq) < mine && c < P.ncol;
-                    const bool okm = okp && P.kminus - c != P.kplus + c;   // phi = 0 is its own partner
+                    const bool ok2 = !last && 2 * (4 * gg + cq) < mine && c < P.ncol;
+                    const bool okp = ok2 && (!ROT || P.kplus + c < P.nphi);    // a window has one -phi sample more
+                    const bool okm = ok2 && P.kminus - c != P.kplus + c;       // phi = 0 is its own partner
 #pragma unroll
                     for (int l = 0; l < 2; ++l) {
                         const uint32_t(&v)[4] = l ? v1 : v0;
@@ -597,6 +609,19 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
             const uint32_t dead = los8 + 8 <= nlos ? 0u : (0xffu << (int)max((int64_t)0, nlos - los8)) & 0xffu;
             float scale[8] = {1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f};
             int ex[8];
+            // ROT: the T rows of the item's LOS, two LOS per lane, or the lane's own LOS (channel-major)
+            int32_t cen[2] = {0, 0};
+            if constexpr (ROT) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    cen[h] = max(P.rot.cmin, min(P.rot.cmax, __ldg(P.rot.centre + min(los0 + 32 * h + lane, nlos - 1))));
+                if constexpr (CHAN) cen[0] = (sw & 1) ? cen[1] : cen[0];
+            }
+            // T of LOS j of the item at this lane's channel of K block kb
+            auto t_of = [&](int j, int kb) {
+                const int c = __shfl_sync(0xffffffffu, j & 32 ? cen[1] : cen[0], j & 31);
+                return __ldg(P.rot.T + (size_t)c * P.rot.ldT + kb * kKBlock + lane);
+            };
             if constexpr (MODE == MODE_FP16X3) {
                 // the LOS's largest |value| sets its power-of-two scale: a first pass over the tile
                 // (staged LOS-major rows are complete in their slot and need none)
@@ -627,12 +652,55 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
             }
             if constexpr (CHAN) {
                 if (MODE == MODE_FP16X3 && sw < 2) exps[i] = ex[0];
+                if constexpr (ROT) {
+                    // both arrays of 8 channels at a time; four warps share a LOS
+                    const float2 *T = P.rot.T + (size_t)cen[0] * P.rot.ldT;
+                    const int64_t at = min(los0 + i, nlos - 1);
+                    const bool valid = los0 + i < nlos;
+                    const int r0 = 16 * (i >> 3) + (i & 7), sz = (r0 >> 1) & 3;
+                    for (int o = sw >> 1; o < 4 * P.kblocks; o += kNumSplitWarps / 2) {
+                        float q[8], u[8];
+                        float4 t[4];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const int64_t off = (int64_t)S.list[8 * o + j] * nlos + at;
+                            q[j] = load_here<true>(P.src.Q + off);
+                            u[j] = load_here<true>(P.src.U + off);
+                        }
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) t[j] = __ldg(reinterpret_cast<const float4 *>(T + 8 * o) + j);
+                        uint32_t qh[4], ql[4], uh[4], ul[4];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            if (8 * o + j >= P.src.nact || !valid) q[j] = u[j] = 0.f;
+                            rotate(q[j], u[j], j & 1 ? make_float2(t[j >> 1].z, t[j >> 1].w) : make_float2(t[j >> 1].x, t[j >> 1].y));
+                        }
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            split_pair_bf16(q[2 * j], q[2 * j + 1], qh[j], ql[j]);
+                            split_pair_bf16(u[2 * j], u[2 * j + 1], uh[j], ul[j]);
+                        }
+                        uint8_t *d = tile + (size_t)(o >> 2) * kPartsBytes + r0 * kFoldRowBytes + (((o & 3) ^ sz) << 4);
+                        *reinterpret_cast<uint4 *>(d) = make_uint4(qh[0], qh[1], qh[2], qh[3]);
+                        *reinterpret_cast<uint4 *>(d + 8 * kFoldRowBytes) = make_uint4(uh[0], uh[1], uh[2], uh[3]);
+                        if (kSplitPrec) {
+                            *reinterpret_cast<uint4 *>(d + kFoldPart) = make_uint4(ql[0], ql[1], ql[2], ql[3]);
+                            *reinterpret_cast<uint4 *>(d + kFoldPart + 8 * kFoldRowBytes) = make_uint4(ul[0], ul[1], ul[2], ul[3]);
+                        }
+                    }
+                } else {
                 uint8_t *const dst = tile + row * kFoldRowBytes;
                 chan_walk<true>(P.src, S.list, los0 + i, array, h0, nh, [&](int h, const float (&v)[16]) {
                     emit16<MODE, true>(dst + (size_t)(h >> 1) * kPartsBytes, h & 1, swz, v, scale[0]);
                 });
+                }
             } else if (stg) {
-                // 8 LOS per slot; units of (K block, array) go round the warps
+                // 8 LOS per slot; units of (K block, array), or ROT (K block, 4 LOS), go round the warps
+                float2 t[4];
+                if constexpr (ROT) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) t[j] = t_of(4 * (sw & 1) + j, min(sw >> 1, P.kblocks - 1));
+                }
                 for (int g = 0; g < kFoldTileLos / 8; ++g) {
                     if (!warp_wait(smem_u32(&S.sfull[ss]), sph, S.abort_flag, P.err, P.timeout_ns)) {
                         ok = false;
@@ -665,11 +733,32 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                     for (int kb = sw >> 1; kb < P.kblocks; kb += kNumSplitWarps / 2) {
                         const int ch = S.list[kb * kKBlock + lane];
                         const bool live = kb * kKBlock + lane < P.src.nact;
-                        float v[8];
+                        uint8_t *const blk = tile + (size_t)kb * kPartsBytes + 16 * g * kFoldRowBytes;
+                        if constexpr (ROT) {
+                            const int r0 = 4 * arr;
+                            float q[4], u[4];
+                            float2 tn[4];
+                            // T of the warp's next unit, here or in the next slot
+                            const bool more = kb + kNumSplitWarps / 2 < P.kblocks;
+                            const int gn = more ? g : min(g + 1, kFoldTileLos / 8 - 1);
+                            const int kn = more ? kb + kNumSplitWarps / 2 : sw >> 1;     // (kb itself is one: in range)
 #pragma unroll
-                        for (int r = 0; r < 8; ++r) v[r] = live ? rows[(8 * arr + r) * nchan + ch] : 0.f;
-                        fold_emit_rows<MODE, true>(tile + (size_t)kb * kPartsBytes + (16 * g + 8 * arr) * kFoldRowBytes, lane, v,
-                                             scale);
+                            for (int j = 0; j < 4; ++j) tn[j] = t_of(8 * gn + r0 + j, kn);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                q[j] = live ? rows[(r0 + j) * nchan + ch] : 0.f;
+                                u[j] = live ? rows[(8 + r0 + j) * nchan + ch] : 0.f;
+                                rotate(q[j], u[j], t[j]);
+                                t[j] = tn[j];
+                            }
+                            fold_emit_rows<MODE, true, 4>(blk, lane, r0, q, scale);
+                            fold_emit_rows<MODE, true, 4>(blk + 8 * kFoldRowBytes, lane, r0, u, scale);
+                        } else {
+                            float v[8];
+#pragma unroll
+                            for (int r = 0; r < 8; ++r) v[r] = live ? rows[(8 * arr + r) * nchan + ch] : 0.f;
+                            fold_emit_rows<MODE, true, 8>(blk + 8 * arr * kFoldRowBytes, lane, 0, v, scale);
+                        }
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&S.sempty[ss]));
@@ -686,8 +775,12 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                     float q[8], u[8];
                     fold_load_los<true>(P.src, S.list, kb, lane, src_of, q, u);
                     fold_mask_los(P.src, kb, lane, dead, q, u);
-                    fold_emit_rows<MODE, true>(dst + (size_t)kb * kPartsBytes, lane, q, scale);
-                    fold_emit_rows<MODE, true>(dst + (size_t)kb * kPartsBytes + 8 * kFoldRowBytes, lane, u, scale);
+                    if constexpr (ROT) {
+#pragma unroll
+                        for (int r = 0; r < 8; ++r) rotate(q[r], u[r], t_of(8 * sw + r, kb));
+                    }
+                    fold_emit_rows<MODE, true, 8>(dst + (size_t)kb * kPartsBytes, lane, 0, q, scale);
+                    fold_emit_rows<MODE, true, 8>(dst + (size_t)kb * kPartsBytes + 8 * kFoldRowBytes, lane, 0, u, scale);
                 }
             }
             if (!ok) break;
@@ -727,11 +820,15 @@ namespace {
 
 using FusedKernel = void (*)(FusedParams, CUtensorMap, CUtensorMap, CUtensorMap);
 
-FusedKernel fused_for(int mode, bool chan)
+FusedKernel fused_for(int mode, bool chan, bool rot)
 {
-    if (mode == MODE_BF16) return chan ? fused_kernel<MODE_BF16, true> : fused_kernel<MODE_BF16, false>;
-    if (mode == MODE_BF16X3) return chan ? fused_kernel<MODE_BF16X3, true> : fused_kernel<MODE_BF16X3, false>;
-    return chan ? fused_kernel<MODE_FP16X3, true> : fused_kernel<MODE_FP16X3, false>;
+    if (rot) {      // window plans are BF16 or BF16X3
+        if (mode == MODE_BF16) return chan ? fused_kernel<MODE_BF16, true, true> : fused_kernel<MODE_BF16, false, true>;
+        return chan ? fused_kernel<MODE_BF16X3, true, true> : fused_kernel<MODE_BF16X3, false, true>;
+    }
+    if (mode == MODE_BF16) return chan ? fused_kernel<MODE_BF16, true, false> : fused_kernel<MODE_BF16, false, false>;
+    if (mode == MODE_BF16X3) return chan ? fused_kernel<MODE_BF16X3, true, false> : fused_kernel<MODE_BF16X3, false, false>;
+    return chan ? fused_kernel<MODE_FP16X3, true, false> : fused_kernel<MODE_FP16X3, false, false>;
 }
 
 // Pipeline shape beside `staging` bytes of staging slots and the channel list: K blocks per stage and stages, at
@@ -783,15 +880,15 @@ cudaLaunchConfig_t launch_config(cudaLaunchAttribute *attr, unsigned grid, size_
 
 }  // namespace
 
-cudaError_t fused_prepare(rms_plan_s *p)
+cudaError_t fused_prepare(rms_plan_s *p, bool window)
 {
     FoldPlan &f = p->fold;
     f.fused_pairs = 0;
     const int mode = mode_of(p->precision);
-    if (!f.on || !f.pair_maps || (mode != MODE_BF16 && f.kblocks > kGroupKBlocks)) return cudaSuccess;
+    if (!f.pair_maps || (window && mode == MODE_FP16X3) || (mode != MODE_BF16 && f.kblocks > kGroupKBlocks)) return cudaSuccess;
     if (shape_for(*p, kStaging).stages < 3) return cudaSuccess;
     for (bool chan : {true, false}) {
-        const FusedKernel k = fused_for(mode, chan);
+        const FusedKernel k = fused_for(mode, chan, window);
         cudaFuncAttributes fa;
         cudaError_t e = cudaFuncGetAttributes(&fa, k);
         if (e == cudaSuccess && fa.numRegs != kRegsLaunch) e = cudaErrorInvalidConfiguration;
@@ -838,7 +935,7 @@ size_t fused_ring_bytes(const rms_plan_s &p, int64_t nlos)
 
 cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout, float *F,
                          int32_t *pidx, float *pabs, float *pphi, float *pq, float *pu, float *pchi, uint8_t *ring,
-                         cudaStream_t s)
+                         cudaStream_t s, const FusedRotation *rot)
 {
     const FoldPlan &f = p.fold;
     const bool chan = layout == RMS_CHAN_MAJOR;
@@ -846,9 +943,10 @@ cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, in
     const int64_t nit = (nlos + 2 * kFoldTileLos - 1) / (2 * kFoldTileLos);
     const int pairs = (int)std::min<int64_t>(nit, f.fused_pairs);
     FusedParams P;
-    P.src = {Q, U, nlos, p.nchan, p.nact, chan, p.d_active, p.d_active_pad};
+    P.src = {Q, U, nlos, p.nchan, p.nact, chan, p.d_active, f.d_list};
     P.kblocks = f.kblocks;
     P.mode = mode;
+    if (rot) P.rot = *rot;
     P.nphi = p.nphi;
     P.ncol = f.ncol;
     P.kplus = f.kplus;
@@ -889,7 +987,7 @@ cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, in
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg =
         launch_config(&attr, (unsigned)(2 * pairs), sh.smem, s);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_for(mode, chan), P, f.tmap2_bhi, f.tmap2_blo, tmA);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_for(mode, chan, rot != nullptr), P, f.tmap2_bhi, f.tmap2_blo, tmA);
     p.last_ctas = 2 * pairs;
     p.last_pair = 1;
     p.last_panels = 0;

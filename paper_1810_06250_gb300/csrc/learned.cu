@@ -7,15 +7,16 @@
 //     T[n][j] = exp(-2i phi_n (lambda_j^2 - lambda_0^2)),
 // so every LOS shares one phase matrix (a plan whose phi grid is the W offsets
 // m D/2) once its data has been multiplied by its own row of T.  T is built in
-// FP64 and stored in FP32; the multiplication happens in shared memory inside
-// the contraction kernel (its rotating variant), so the split operand is read
-// from HBM once.
+// FP64 and stored in FP32.  BF16, and BF16X3 up to 512 channels, multiply on the way
+// into the one-kernel form's ring (fused.cu), whose phase matrix folds the offsets
+// +-m: one pass over the cube and half the products (262,144 LOS x 360 channels x 64:
+// 0.69 -> 0.37 ms against the split and the rotating contraction, which multiplies in
+// shared memory and serves the longer BF16X3 channel lists).
 //
-// Learned peak map: one split of the cube feeds (1) the network (hi parts of
-// the operand image, scaled by 1/RMS per row), (2) the window contraction
-// around 2 * proposed bin, (3) for the LOS that fall back (confidence below tau
-// or NaN, window maximum on the window edge or absent) a compacted copy of
-// their operand rows and the full-grid contraction on those rows only.
+// Learned peak map: (1) the network on a BF16 image of the cube, scaled by 1/RMS per
+// row, (2) window synthesis around 2 * proposed bin, (3) for the LOS that fall back
+// (confidence below tau or NaN, window maximum on the window edge or absent) the
+// layout stage and the full-grid contraction on those rows only.
 #include <math.h>
 
 #include <algorithm>
@@ -132,6 +133,33 @@ __global__ void merge_kernel(const MergeParams P)
     if (fb) P.rows[base + __popc(mask & ((1u << lane) - 1u))] = i;
 }
 
+// Window synthesis of the cube in one kernel (BF16, or BF16X3 up to 512 channels).
+cudaError_t window_fused(const rms_window_s &w, const float *Q, const float *U, int64_t nlos, int32_t layout,
+                         const int32_t *centre, float *F, int32_t *widx, float *wabs, uint8_t *ring, cudaStream_t s)
+{
+    const FusedRotation rot = {centre, w.d_Tc, w.ldc, w.cmin, w.cmax};
+    return launch_fused(*w.sub, Q, U, nlos, layout, F, widx, wabs, nullptr, nullptr, nullptr, nullptr, ring, s, &rot);
+}
+
+// The rotating contraction of a split image.
+cudaError_t window_contract(const rms_window_s &w, const uint8_t *img, int64_t nlos, int32_t layout,
+                            const int32_t *centre, float *F, int32_t *widx, float *wabs, cudaStream_t s)
+{
+    GemmOpts go;
+    go.A = img;
+    go.nlos = nlos;
+    go.layout = layout;
+    go.F = F;
+    go.pidx = widx;
+    go.pabs = wabs;
+    go.centre = centre;
+    go.T = layout == RMS_CHAN_MAJOR ? w.d_Tc : w.d_Tr;
+    go.ldT = layout == RMS_CHAN_MAJOR ? w.ldc : w.ldr;
+    go.cmin = w.cmin;
+    go.cmax = w.cmax;
+    return launch_gemm(*w.sub, go, s);
+}
+
 }  // namespace
 
 extern "C" {
@@ -170,7 +198,7 @@ rms_status rms_window_create(rms_window_t *out, rms_plan_t plan, int32_t width)
         free_window(w);
         return st;
     }
-    w->ldc = p.kblocks * kChanPerKBlock;
+    w->ldc = (p.nact + kKBlock - 1) / kKBlock * kKBlock;   // whole K blocks of either contraction
     w->ldr = p.kblocks_raw * kChanPerKBlock;
     std::vector<double> dl2c(p.nact), dl2r(p.nchan);
     for (int a = 0; a < p.nact; ++a) dl2c[a] = p.lambda2[p.active[a]] - p.lambda0sq;
@@ -230,7 +258,8 @@ rms_status rms_synth_window(rms_window_t w, const float *Q, const float *U, int6
     if (!guard.ok) return RMS_ERR_CUDA;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t ib = split_operand_bytes(p, nlos, layout), xb = (size_t)nlos * 4;
+    const bool one = w->sub->fold.fused_pairs > 0;      // one kernel (fused.cu), or split and rotating contraction
+    const size_t ib = one ? fused_ring_bytes(*w->sub, nlos) : split_operand_bytes(p, nlos, layout), xb = (size_t)nlos * 4;
     uint8_t *scr = nullptr;
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&scr), up(ib) + (widx ? 0 : up(xb)), s);
     if (e != cudaSuccess) {
@@ -238,28 +267,18 @@ rms_status rms_synth_window(rms_window_t w, const float *Q, const float *U, int6
         return from_cuda(e);
     }
     int32_t *k = widx ? widx : reinterpret_cast<int32_t *>(scr + up(ib));
-    SplitOpts so;
-    so.Q = Q;
-    so.U = U;
-    so.nlos_src = nlos;
-    so.layout = layout;
-    so.nout = nlos;
-    so.A = scr;
-    e = launch_split(p, so, s);
-    if (e == cudaSuccess) {
-        GemmOpts go;
-        go.A = scr;
-        go.nlos = nlos;
-        go.layout = layout;
-        go.F = F_out;
-        go.pidx = k;
-        go.pabs = wabs;
-        go.centre = centre;
-        go.T = layout == RMS_CHAN_MAJOR ? w->d_Tc : w->d_Tr;
-        go.ldT = layout == RMS_CHAN_MAJOR ? w->ldc : w->ldr;
-        go.cmin = w->cmin;
-        go.cmax = w->cmax;
-        e = launch_gemm(*w->sub, go, s);
+    if (one) {
+        e = window_fused(*w, Q, U, nlos, layout, centre, F_out, k, wabs, scr, s);
+    } else {
+        SplitOpts so;
+        so.Q = Q;
+        so.U = U;
+        so.nlos_src = nlos;
+        so.layout = layout;
+        so.nout = nlos;
+        so.A = scr;
+        e = launch_split(p, so, s);
+        if (e == cudaSuccess) e = window_contract(*w, scr, nlos, layout, centre, F_out, k, wabs, s);
     }
     if (e == cudaSuccess && wphi) {
         window_phi_kernel<<<(unsigned)((nlos + 255) / 256), 256, 0, s>>>(centre, k, nlos, w->width / 2, w->cmin,
@@ -291,7 +310,9 @@ rms_status rms_peakmap_learned(rms_window_t w, rms_net_t net, const float *Q, co
     // the fallback rows' image: folded like rms_synth's wherever the plan's grid folds
     const size_t ib_fb = p.fold.on ? up(fold_operand_bytes(p, nlos)) : ib;
     // image | fallback image | h | rscale | bin | conf | centre | widx | wabs | rows | count | peak keys
-    const size_t total = ib + ib_fb + hb + 7 * n4 + 2 * n8 + 256;
+    const bool one = w->sub->fold.fused_pairs > 0;
+    const size_t rb = one ? up(fused_ring_bytes(*w->sub, nlos)) : 0;
+    const size_t total = ib + ib_fb + hb + 7 * n4 + 2 * n8 + 256 + rb;
     uint8_t *scr = nullptr;
     cudaError_t e = cudaStreamWaitEvent(s, net->last, 0);
     if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void **>(&scr), total, s);
@@ -313,6 +334,7 @@ rms_status rms_peakmap_learned(rms_window_t w, rms_net_t net, const float *Q, co
     int64_t *count = reinterpret_cast<int64_t *>(q + 7 * n4 + n8);
     // the fallback contraction's peak keys (its job schedule and CTA pairs)
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(q + 7 * n4 + n8 + 256);
+    uint8_t *const ring = scr + total - rb;
     const unsigned g256 = (unsigned)((nlos + 255) / 256);
 
     SplitOpts so;
@@ -323,6 +345,7 @@ rms_status rms_peakmap_learned(rms_window_t w, rms_net_t net, const float *Q, co
     so.nout = nlos;
     so.A = img;
     so.rscale = rs;
+    if (one && p.fold.on) so.mode = 0;      // only the network reads this image: hi parts
     e = launch_split(p, so, s);
     if (e == cudaSuccess)
         e = net_forward_image(*net, img, layout, rs, nlos, h, nullptr, bin, conf, w->width / 4 - 2, s);
@@ -330,20 +353,9 @@ rms_status rms_peakmap_learned(rms_window_t w, rms_net_t net, const float *Q, co
         centre_kernel<<<g256, 256, 0, s>>>(bin, nlos, w->cmin, w->cmax, centre);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) {
-        GemmOpts go;
-        go.A = img;
-        go.nlos = nlos;
-        go.layout = layout;
-        go.pidx = widx;
-        go.pabs = wabs;
-        go.centre = centre;
-        go.T = layout == RMS_CHAN_MAJOR ? w->d_Tc : w->d_Tr;
-        go.ldT = layout == RMS_CHAN_MAJOR ? w->ldc : w->ldr;
-        go.cmin = w->cmin;
-        go.cmax = w->cmax;
-        e = launch_gemm(*w->sub, go, s);
-    }
+    if (e == cudaSuccess)
+        e = one ? window_fused(*w, Q, U, nlos, layout, centre, nullptr, widx, wabs, ring, s)
+                : window_contract(*w, img, nlos, layout, centre, nullptr, widx, wabs, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(count, 0, sizeof(int64_t), s);
     if (e == cudaSuccess) {
         MergeParams M;

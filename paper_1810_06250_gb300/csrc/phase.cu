@@ -198,9 +198,8 @@ cudaError_t launch_phase_bsplit(const rms_plan_s &p, const double *dl2, const do
     return cudaGetLastError();
 }
 
-cudaError_t launch_phase_fold(const rms_plan_s &p, const double *dh, bool fp16, cudaStream_t s)
+cudaError_t launch_phase_fold(const rms_plan_s &p, const FoldPlan &f, const double *dh, bool fp16, cudaStream_t s)
 {
-    const FoldPlan &f = p.fold;
     const size_t bytes = (size_t)f.tiles.npad * f.kpad * sizeof(uint16_t);
     cudaError_t e = cudaMemsetAsync(f.d_hi, 0, bytes, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(f.d_lo, 0, bytes, s);

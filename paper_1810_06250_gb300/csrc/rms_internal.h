@@ -39,7 +39,7 @@ struct PhaseTiling {
 };
 
 // A symmetric phi grid (phi_k + phi_{nphi-1-k} = 0), and the tensor-core precisions'
-// folded phase matrix: rows (c, s) = (w / w_max) (cos, sin)(theta) of the ncol depths phi >= 0, columns the active
+// folded phase matrix (window plans: the W offsets -W/2 .. W/2 - 1, one -phi sample more): rows (c, s) = (w / w_max) (cos, sin)(theta) of the ncol depths phi >= 0, columns the active
 // channels, which the contraction multiplies with Q and U rows of their own (fold.cu).
 struct FoldPlan {
     bool on = false, pair_maps = false;
@@ -48,6 +48,7 @@ struct FoldPlan {
     int32_t kblocks = 0, kpad = 0; // K blocks of 32 active channels
     PhaseTiling tiles;
     uint16_t *d_hi = nullptr, *d_lo = nullptr;   // [tiles.npad][kpad]
+    int32_t *d_list = nullptr;     // [kpad] the active channels, padded with the last one
     int32_t fused_pairs = 0;       // the one-kernel form (fused.cu): resident CTA pairs (0: not for this plan)
     CUtensorMap tmap_bhi, tmap_blo, tmap2_bhi, tmap2_blo;
 };
@@ -61,7 +62,6 @@ struct rms_plan_s {
 
     // device arrays
     int32_t *d_active = nullptr;   // [nact] channel index of each active channel
-    int32_t *d_active_pad = nullptr;   // the same, padded to a multiple of 32 with the last active channel
     double *d_dl2 = nullptr;       // [nact] lambda_j^2 - lambda_0^2 (FP64)
     double *d_wact = nullptr;      // [nact] w_j
     double *d_phi = nullptr;       // [nphi]
@@ -78,7 +78,6 @@ struct rms_plan_s {
     PhaseTiling tiles;      // npad covers both tilings
     FoldPlan fold;
     int32_t simt_clusters[8] = {};  // FP32 CUDA-core kernels: resident clusters of 1 .. 8 blocks
-    double *d_dh = nullptr;        // [fold.ncol] the folded grid's depths phi >= 0
     CUtensorMap tmap_bhi;   // CUtensorMap is 64-byte aligned by its own declaration
     CUtensorMap tmap_blo;
     // LOS-major cubes contract over all channels (flagged ones zeroed in the
@@ -137,7 +136,7 @@ cudaError_t launch_phase_table(const rms_plan_s &p, cudaStream_t s);
 cudaError_t launch_phase_bsplit(const rms_plan_s &p, const double *dl2, const double *w, int32_t nk,
                                 int32_t kpad, uint16_t *bhi, uint16_t *blo, bool fp16, cudaStream_t s);
 // the folded phase matrix: depths dh[ncol] (device), active channels
-cudaError_t launch_phase_fold(const rms_plan_s &p, const double *dh, bool fp16, cudaStream_t s);
+cudaError_t launch_phase_fold(const rms_plan_s &p, const FoldPlan &f, const double *dh, bool fp16, cudaStream_t s);
 cudaError_t launch_rotation_table(const double *dl2, int32_t nk, int32_t ld, double phi0, double step,
                                   int32_t ncentre, float2 *T, cudaStream_t s);
 cudaError_t launch_rmsf(const rms_plan_s &p, const double *d_phi, int32_t n, double *d_R64,
@@ -179,12 +178,17 @@ cudaError_t launch_fold_split(const rms_plan_s &p, const float *Q, const float *
                               const int64_t *count = nullptr);
 // fused.cu: layout stage and contraction in one kernel, for plans whose K blocks form one
 // accumulation (fused_prepare, at plan creation) and calls of enough LOS (fused_wanted)
-cudaError_t fused_prepare(rms_plan_s *p);
+struct FusedRotation {             // window plans: LOS l is multiplied by T[clamp(centre[l], cmin, cmax)][active channel]
+    const int32_t *centre = nullptr;
+    const float2 *T = nullptr;
+    int32_t ldT = 0, cmin = 0, cmax = 0;
+};
+cudaError_t fused_prepare(rms_plan_s *p, bool window);
 bool fused_wanted(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout);
 size_t fused_ring_bytes(const rms_plan_s &p, int64_t nlos);
 cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout, float *F,
                          int32_t *pidx, float *pabs, float *pphi, float *pq, float *pu, float *pchi, uint8_t *ring,
-                         cudaStream_t s);
+                         cudaStream_t s, const FusedRotation *rot = nullptr);
 struct SplitOpts {
     const float *Q = nullptr, *U = nullptr;
     int64_t nlos_src = 0;              // lines of sight in the cube
