@@ -14,14 +14,20 @@
 //   SOFTMAX  z = acc + b over the whole row (<= 512 bins in one tile): argmax,
 //            softmax, confidence = mass within a window of bins; with labels the
 //            cross-entropy and dz = (softmax - onehot) / batch in BF16 (row- and
-//            column-major) and FP32
-//   DRELU    da = acc * [h > 0] -> BF16 (da * rowscale)^T and FP32 da
+//            column-major), its FP32 column sums added into the bias gradient
+//   DRELU    da = acc * [h > 0] -> BF16 (da * rowscale)^T, column sums likewise
 //   ACC      split-K partial sums added into FP32 gradients (optionally through a
 //            column map from image columns to weight columns)
 //   warp 0      TMA / bulk producer                        -> full
 //   warp 1      TMEM allocator, single-thread MMA issuer   -> empty, tfull
-//   warps 4-11  epilogue: warp w owns TMEM lane quarter w % 4 and column half
+//   warps 4-19  epilogue: warp w owns TMEM lane quarter w % 4 and column quarter
 //               (w - 4) / 4 of each accumulator row          -> tempty
+// The products are small (K <= 1600 or so); the epilogues, serial per row, set the pace,
+// which is why 16 warps share a tile's rows and every store is a whole sector.
+// 262,144 LOS x 256 x 401: softmax and confidence 0.225 -> 0.184 ms against 8 warps.  A
+// 4,096-LOS gradient (720 x 256 x 401): softmax loss 102 -> 48 us, hidden gradient 64 ->
+// 17, the two split-K products 32 + 28 -> 12 + 12 with vector reductions of whole
+// sectors, and no FP32 copies of dz and da to sum for the bias gradients (37 us).
 // Every wait is bounded (abort flag, device error word, drain, TMEM freed).
 #include <cuda_bf16.h>
 #include <math.h>
@@ -39,16 +45,21 @@ namespace {
 
 typedef __nv_bfloat16 bf16;
 
-enum { EPI_RELU = 0, EPI_SOFTMAX = 1, EPI_DRELU = 2, EPI_ACC = 3 };
-constexpr int kNetThreads = 384;
-constexpr int kNetEpiWarp0 = 4;    // warps 4-11: two per TMEM lane quarter, one per column half
+enum { EPI_RELU = 0, EPI_SOFTMAX = 1, EPI_DRELU = 2, EPI_ACC = 3, EPI_LOSS = 4 };   // LOSS: SOFTMAX with labels
+constexpr int kNetThreads = 640;
+constexpr int kNetEpiWarp0 = 4, kNetEpiWarps = 16;   // four per TMEM lane quarter, one per column quarter
+constexpr int kNetParts = kNetEpiWarps / 4;
+// 640 x 96 registers: the epilogue warpgroups take some from the control warpgroup
+constexpr int kNetRegsLaunch = 96, kNetRegsCtl = 64, kNetRegsEpi = 104;
+static_assert(128 * kNetRegsCtl + 512 * kNetRegsEpi == kNetThreads * kNetRegsLaunch, "register split must fill the launch");
 constexpr int kNetTmemCols = 512;
 constexpr int kNetStageA = kTileM * 64;       // 8 KB: 128 rows x 32 BF16
 constexpr int kImageKBlockBytes = 2 * kNetStageA;   // split image: hi then lo per K block
 constexpr int kNetSmemLimit = 227 * 1024;
-constexpr int kNetXchFloats = 4 * kTileM;     // (max, sum, argmax, z_label) per row
-constexpr int kNetBiasMax = 512;               // bias staged in shared memory (N <= 512 when a bias is used)
-constexpr int kNetFixedSmem = 1024 + 256 + (kNetXchFloats + kNetBiasMax) * 4;
+constexpr int kNetXchFloats = 5 * kNetParts * kTileM;   // (max, sum, argmax, z_label, window mass) per part and row
+constexpr int kNetBiasMax = 512;               // bias staged in shared memory (N <= 512 when a bias is used), read in
+                                               // chunks of 32
+constexpr int kNetFixedSmem = 1024 + 256 + (kNetXchFloats + kNetBiasMax + 32) * 4;
 
 struct NetGemmParams {
     int32_t M, N, kblocks, kb_per_split, ksplit, mtiles, ntiles;
@@ -63,6 +74,7 @@ struct NetGemmParams {
     int64_t ldt;
     float *outf;
     int64_t ldf;
+    float *colsum;              // bias gradient: the epilogue's FP32 columns summed over the rows
     const bf16 *hmask;
     int64_t ldh;
     const int32_t *colmap;
@@ -82,7 +94,7 @@ struct NSmem {
     uint64_t *full, *empty, *tfull, *tempty, *mma_done;
     uint32_t *tmem_slot;
     volatile int *abort_flag;
-    float *xch;                 // softmax: per-row values exchanged between the two column halves
+    float *xch;                 // softmax: per-row values exchanged between the column quarters
 };
 
 __device__ __forceinline__ NSmem ncarve(uint8_t *base, const NetGemmParams &P)
@@ -98,7 +110,8 @@ __device__ __forceinline__ NSmem ncarve(uint8_t *base, const NetGemmParams &P)
     s.mma_done = s.tempty + 2;
     s.tmem_slot = reinterpret_cast<uint32_t *>(s.mma_done + 1);
     s.abort_flag = reinterpret_cast<volatile int *>(s.tmem_slot + 1);
-    s.xch = reinterpret_cast<float *>(const_cast<int *>(s.abort_flag) + 2);
+    // 16-byte aligned: the bias behind it is read in vectors
+    s.xch = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(const_cast<int *>(s.abort_flag) + 1) + 15) & ~(uintptr_t)15);
     return s;
 }
 
@@ -126,8 +139,8 @@ __device__ __forceinline__ void load32(uint32_t taddr, int c0, int end, float (&
         for (int e = 0; e < 8; ++e) v[8 * j + e] = (c0 + 8 * j < end) ? __uint_as_float(r[j][e]) : 0.f;
 }
 
-// The two warps that share a TMEM lane quarter (64 threads, named barrier 1 + q).
-__device__ __forceinline__ void pair_sync(int q) { asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory"); }
+// The four warps that share a TMEM lane quarter (128 threads, named barrier 1 + q).
+__device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory"); }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
@@ -135,8 +148,31 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
-// One accumulator row per thread; the warp pair of a lane quarter splits the
-// columns in halves [c_lo, c_hi).  bias_s: the bias in shared memory.
+// Next row of a transposed output; opaque, so that the compiler does not keep the
+// addresses of all rows of a chunk in registers.
+__device__ __forceinline__ void next_row(bf16 *&t, int64_t ld)
+{
+    t += ld;
+    asm volatile("" : "+l"(t));
+}
+
+// Sum of 32 values over the warp's 32 lanes, value j's total in lane j (31 shuffles).
+__device__ __forceinline__ float transpose_sum(float (&v)[32], int lane)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int j = 0; j < off; ++j) {
+            const float give = up ? v[j] : v[j + off], keep = up ? v[j + off] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
+    }
+    return v[0];
+}
+
+// One accumulator row per thread (ACC: 8 rows of a quarter per load); the four warps of a
+// lane quarter split the columns.  bias_s: the bias in shared memory.
 template <int EPI>
 __device__ void epilogue(const NetGemmParams &P, const NSmem &SM, const float *bias_s, uint32_t tacc, int mt, int nt,
                          int q, int h, int lane)
@@ -144,90 +180,104 @@ __device__ void epilogue(const NetGemmParams &P, const NSmem &SM, const float *b
     const int r = 32 * q + lane;
     const int64_t m = (int64_t)mt * kTileM + r;
     const bool valid = m < P.M;
-    const float rs = (P.row_scale && valid) ? P.row_scale[m] : 1.0f;
     const int n_base = nt * P.BN;
-    const int half = P.BN / 2;
-    const int c_lo = h * half, c_hi = c_lo + half;
-    float v[32];
-    if constexpr (EPI != EPI_SOFTMAX) {
+    const int width = ((P.BN + kNetParts - 1) / kNetParts + 7) / 8 * 8;
+    const int c_lo = min(P.BN, h * width), c_hi = min(P.BN, c_lo + width);
+    if constexpr (EPI == EPI_ACC) {
+        // 16-lane loads: thread (rq, cq) holds columns 2 cq, 2 cq + 1 of rows rq and rq + 8, so
+        // four lanes add 32 contiguous bytes of a gradient row in one vector reduction
+        const int rq = lane >> 2, cq = lane & 3;
+        for (int c0 = c_lo; c0 < c_hi; c0 += 8) {
+            uint32_t v[2][4];
+            tmem_ld16x256(tacc + c0, v[0]);
+            tmem_ld16x256(tacc + (16u << 16) + c0, v[1]);
+            tmem_wait_ld();
+            const int n = n_base + c0 + 2 * cq;
+            if (n >= P.N) continue;                 // N is even, and so are the mapped pairs
+            const int col = P.colmap ? P.colmap[n] : n;
+            if (col < 0) continue;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int64_t row = (int64_t)mt * kTileM + 32 * q + 16 * (i >> 1) + 8 * (i & 1) + rq;
+                if (row < P.M)
+                    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(P.outf + row * P.ldf + col),
+                                 "f"(__uint_as_float(v[i >> 1][2 * (i & 1)])), "f"(__uint_as_float(v[i >> 1][2 * (i & 1) + 1]))
+                                 : "memory");
+            }
+        }
+        return;
+    } else if constexpr (EPI == EPI_RELU || EPI == EPI_DRELU) {
+        const float rs = (P.row_scale && valid) ? P.row_scale[m] : 1.0f;
+        float v[32];
         for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
             load32(tacc, c0, c_hi, v);
-            if (!valid) continue;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int n0 = n_base + c0 + 8 * j;
-                if (c0 + 8 * j >= c_hi || n0 >= P.N) continue;
+                const bool live = valid && c0 + 8 * j < c_hi && n0 < P.N;      // N is a multiple of 16
                 if constexpr (EPI == EPI_RELU) {
+                    if (!live) continue;
                     float o[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int n = n0 + e;
-                        o[e] = n < P.N ? fmaxf(fmaf(v[8 * j + e], rs, bias_s ? bias_s[n] : 0.f), 0.f) : 0.f;
-                    }
-                    if (n0 + 8 <= P.N) {
-                        *reinterpret_cast<uint4 *>(P.out + m * P.ldo + n0) =
-                            make_uint4(pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]), pack_bf16(o[4], o[5]),
-                                       pack_bf16(o[6], o[7]));
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (n0 + e < P.N) P.out[m * P.ldo + n0 + e] = __float2bfloat16_rn(o[e]);
-                    }
+                    for (int e = 0; e < 8; ++e) o[e] = fmaxf(fmaf(v[8 * j + e], rs, bias_s[n0 + e]), 0.f);
+                    *reinterpret_cast<uint4 *>(P.out + m * P.ldo + n0) =
+                        make_uint4(pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]), pack_bf16(o[4], o[5]), pack_bf16(o[6], o[7]));
                     if (P.outT) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (n0 + e < P.N) P.outT[(int64_t)(n0 + e) * P.ldt + m] = __float2bfloat16_rn(o[e]);
-                    }
-                } else if constexpr (EPI == EPI_DRELU) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int n = n0 + e;
-                        if (n >= P.N) continue;
-                        const float hv = __bfloat162float(P.hmask[m * P.ldh + n]);
-                        const float da = hv > 0.f ? v[8 * j + e] : 0.f;
-                        P.outT[(int64_t)n * P.ldt + m] = __float2bfloat16_rn(da * rs);
-                        P.outf[m * P.ldf + n] = da;
+                        for (int e = 0; e < 8; ++e) P.outT[(int64_t)(n0 + e) * P.ldt + m] = __float2bfloat16_rn(o[e]);
                     }
                 } else {
+                    uint4 hv = make_uint4(0u, 0u, 0u, 0u);
+                    if (live) hv = *reinterpret_cast<const uint4 *>(P.hmask + m * P.ldh + n0);
+                    const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w};
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        const int n = n0 + e;
-                        if (n >= P.N) continue;
-                        const int col = P.colmap ? P.colmap[n] : n;
-                        if (col >= 0) atomicAdd(P.outf + m * P.ldf + col, v[8 * j + e]);
+                        const float hx = __uint_as_float((e & 1) ? hw[e >> 1] & 0xffff0000u : hw[e >> 1] << 16);
+                        const float da = hx > 0.f ? v[8 * j + e] : 0.f;
+                        if (live) P.outT[(int64_t)(n0 + e) * P.ldt + m] = __float2bfloat16_rn(da * rs);
+                        v[8 * j + e] = da;
                     }
                 }
+            }
+            if constexpr (EPI == EPI_DRELU) {
+                const float s = transpose_sum(v, lane);
+                const int n = n_base + c0 + lane;
+                if (c0 + lane < c_hi && n < P.N) atomicAdd(P.colsum + n, s);
             }
         }
         return;
     } else {
-        // One pass per half: running max, argmax (lowest index on ties) and the sum
-        // of exp(z - max), rescaled once per 32-column chunk; the halves then combine
-        // through shared memory.  Missing columns read as -inf (exp gives 0).
-        const bool train = P.label != nullptr;
+        // One pass per part: running max, argmax (lowest index on ties) and the sum of
+        // exp(z - max), rescaled once per 32-column chunk; the parts then combine through
+        // shared memory.  Missing columns read as -inf (exp gives 0).
+        float v[32];
+        constexpr bool train = EPI == EPI_LOSS;
         const int y = (train && valid) ? P.label[m] : -1;
         const int lim = min(c_hi, P.N);
         float mx = -INFINITY, S = 0.f, zy = 0.f;
         int bi = -1;
-        for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
-            load32(tacc, c0, c_hi, v);
-            float cm = -INFINITY;
-            int ci = -1;
-            if (c0 + 32 <= lim) {
+        // The training sum is one chain per half row (a rounding of it moves dz by an ulp of
+        // BF16 here and there), so two warps of a quarter take it and four the rest.
+        constexpr int kSumParts = train ? 2 : kNetParts;
+        const int s_width = train ? P.BN / 2 : width;
+        const int s_lo = h < kSumParts ? min(P.BN, h * s_width) : P.BN, s_hi = h < kSumParts ? min(P.BN, s_lo + s_width) : P.BN;
+        const int s_lim = min(s_hi, P.N);
+#pragma unroll 1
+        for (int c0 = s_lo; c0 < s_hi; c0 += 32) {
+            load32(tacc, c0, s_hi, v);
+            float top[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    const float z = v[e] + bias_s[c0 + e];
-                    v[e] = z;
-                    if (z > cm) { cm = z; ci = c0 + e; }
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    const float z = c0 + e < lim ? v[e] + bias_s[c0 + e] : -INFINITY;
-                    v[e] = z;
-                    if (z > cm) { cm = z; ci = c0 + e; }
-                }
+            for (int e = 0; e < 32; e += 4) {
+                const float4 b = *reinterpret_cast<const float4 *>(bias_s + c0 + e);    // padded past N
+                v[e] += b.x; v[e + 1] += b.y; v[e + 2] += b.z; v[e + 3] += b.w;
             }
+            if (c0 + 32 > s_lim) {
+#pragma unroll
+                for (int e = 0; e < 32; ++e)
+                    if (c0 + e >= s_lim) v[e] = -INFINITY;
+            }
+#pragma unroll
+            for (int e = 0; e < 32; ++e) top[e & 3] = fmaxf(top[e & 3], v[e]);          // NaN is never the larger
             if (train) {
 #pragma unroll
                 for (int e = 0; e < 32; ++e)
@@ -235,47 +285,56 @@ __device__ void epilogue(const NetGemmParams &P, const NSmem &SM, const float *b
             } else if (P.outf && valid) {
 #pragma unroll
                 for (int e = 0; e < 32; ++e)
-                    if (c0 + e < lim) P.outf[m * P.ldf + c0 + e] = v[e];
+                    if (c0 + e < s_lim) P.outf[m * P.ldf + c0 + e] = v[e];
             }
+            const float cm = fmaxf(fmaxf(top[0], top[1]), fmaxf(top[2], top[3]));
             if (cm > mx) {
                 S *= __expf(mx - cm);
                 mx = cm;
-                bi = ci;
+                int at = 31;
+#pragma unroll
+                for (int e = 30; e >= 0; --e) at = v[e] == cm ? e : at;
+                bi = c0 + at;
             }
-            if (mx > -INFINITY) {
+            if (train && mx > -INFINITY) {
 #pragma unroll
                 for (int e = 0; e < 32; ++e) S += __expf(v[e] - mx);
+            } else if (mx > -INFINITY) {
+                float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int e = 0; e < 32; ++e) sum[e & 3] += __expf(v[e] - mx);
+                S += (sum[0] + sum[1]) + (sum[2] + sum[3]);
             }
         }
-        float *X = SM.xch;   // [4][128]: max, sum, argmax, z_label
-        if (h == 1) {
-            X[r] = mx;
-            X[kTileM + r] = S;
-            X[2 * kTileM + r] = __int_as_float(bi);
-            X[3 * kTileM + r] = zy;
+        // [part][max, sum, argmax, z_label][row], then [part][row] of the window mass
+        float *const X = SM.xch, *const W = X + 4 * kNetParts * kTileM;
+        {
+            float *x = X + 4 * kTileM * h + r;
+            x[0] = mx;
+            x[kTileM] = S;
+            x[2 * kTileM] = __int_as_float(bi);
+            x[3 * kTileM] = zy;
         }
-        pair_sync(q);
-        if (h == 0) {
-            const float m1 = X[r], s1 = X[kTileM + r], z1 = X[3 * kTileM + r];
-            const int b1 = __float_as_int(X[2 * kTileM + r]);
-            const float M = fmaxf(mx, m1);
-            const float St =
-                (mx > -INFINITY ? S * __expf(mx - M) : 0.f) + (m1 > -INFINITY ? s1 * __expf(m1 - M) : 0.f);
-            if (m1 > mx) bi = b1;
-            if (y >= c_hi) zy = z1;
-            mx = M;
-            S = St;
-            X[r] = mx;
-            X[kTileM + r] = S;
-            X[2 * kTileM + r] = __int_as_float(bi);
+        quarter_sync(q);
+        {
+            // every warp merges all four parts of its rows (lowest index on ties: parts ascend)
+            mx = -INFINITY;
+            bi = -1;
+            zy = 0.f;
+#pragma unroll
+            for (int p = 0; p < kSumParts; ++p) {
+                const float *x = X + 4 * kTileM * p + r;
+                if (x[0] > mx) { mx = x[0]; bi = __float_as_int(x[2 * kTileM]); }
+                if (y >= p * s_width) zy = x[3 * kTileM];
+            }
+            S = 0.f;
+#pragma unroll
+            for (int p = 0; p < kSumParts; ++p) {
+                const float *x = X + 4 * kTileM * p + r;
+                S = __fadd_rn(S, x[0] > -INFINITY ? __fmul_rn(x[kTileM], __expf(x[0] - mx)) : 0.f);
+            }
         }
-        pair_sync(q);
-        if (h == 1) {
-            mx = X[r];
-            S = X[kTileM + r];
-            bi = __float_as_int(X[2 * kTileM + r]);
-        }
-        // window mass: columns within halfwin of the argmax that lie in this half.  The
+        // window mass: columns within halfwin of the argmax that lie in this part.  The
         // TMEM loads are warp-collective (.sync.aligned), so every lane walks the same
         // 8-column groups -- those that meet any lane's window -- and masks its own.
         float Sw = 0.f;
@@ -283,28 +342,24 @@ __device__ void epilogue(const NetGemmParams &P, const NSmem &SM, const float *b
             const bool has = bi >= 0;
             const int w0 = has ? max(c_lo, bi - P.halfwin) : c_hi;
             const int w1 = has ? min(lim, bi + P.halfwin + 1) : c_lo;
-            int g0 = w0, g1 = w1;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                g0 = min(g0, __shfl_xor_sync(0xffffffffu, g0, o));
-                g1 = max(g1, __shfl_xor_sync(0xffffffffu, g1, o));
-            }
-            for (int c0 = g0 & ~7; c0 < g1; c0 += 8) {
-                uint32_t rr[8];
-                tmem_ld8(tacc + c0, rr);
+            const int g0 = __reduce_min_sync(0xffffffffu, w0), g1 = __reduce_max_sync(0xffffffffu, w1);
+            const unsigned span = (unsigned)max(0, w1 - w0);
+#pragma unroll 1
+            for (int c0 = g0 & ~7; c0 < g1; c0 += 16) {
+                uint32_t rr[2][8];
+                tmem_ld8(tacc + c0, rr[0]);
+                if (c0 + 8 < c_hi) tmem_ld8(tacc + c0 + 8, rr[1]);
                 tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int n = c0 + e;
-                    if (n >= w0 && n < w1) Sw += __expf(__uint_as_float(rr[e]) + bias_s[n] - mx);
-                }
+                for (int e = 0; e < 16; ++e)
+                    if ((unsigned)(c0 + e - w0) < span) Sw += __expf(__uint_as_float(rr[e >> 3][e & 7]) + bias_s[c0 + e] - mx);
             }
         }
-        pair_sync(q);
-        if (h == 1) X[r] = Sw;
-        pair_sync(q);
+        W[kTileM * h + r] = Sw;
+        quarter_sync(q);
         if (h == 0) {
-            Sw += X[r];
+            // (the next tile's first exchange comes after its first barrier, this read before it)
+            Sw = (W[r] + W[kTileM + r]) + (W[2 * kTileM + r] + W[3 * kTileM + r]);
             if (valid) {
                 if (P.bin) P.bin[m] = max(bi, 0);
                 if (P.conf) P.conf[m] = P.halfwin >= 0 ? Sw / S : 1.0f / S;
@@ -316,23 +371,36 @@ __device__ void epilogue(const NetGemmParams &P, const NSmem &SM, const float *b
                 if (lane == 0 && P.loss) atomicAdd(P.loss, lrow * P.inv_batch);
             }
         }
-        pair_sync(q);   // the exchange buffer is reused by the next tile
         if (!train) return;
         const float invS = 1.0f / S;
+#pragma unroll 1
         for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
             load32(tacc, c0, c_hi, v);
-            if (!valid) continue;
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
                 const int n = c0 + e;
-                if (n < lim) {
-                    const float z = v[e] + bias_s[n];
-                    const float d = (__expf(z - mx) * invS - (n == y ? 1.f : 0.f)) * P.inv_batch;
-                    P.out[m * P.ldo + n] = __float2bfloat16_rn(d);
-                    P.outT[(int64_t)n * P.ldt + m] = __float2bfloat16_rn(d);
-                    P.outf[m * P.ldf + n] = d;
+                float d = 0.f;
+                if (valid && n < lim) d = (__expf(v[e] + bias_s[n] - mx) * invS - (n == y ? 1.f : 0.f)) * P.inv_batch;
+                v[e] = d;
+            }
+            if (valid) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int n0 = c0 + 8 * j;
+                    if (n0 < lim)                       // rows are padded to 8 columns
+                        *reinterpret_cast<uint4 *>(P.out + m * P.ldo + n0) =
+                            make_uint4(pack_bf16(v[8 * j], v[8 * j + 1]), pack_bf16(v[8 * j + 2], v[8 * j + 3]),
+                                       pack_bf16(v[8 * j + 4], v[8 * j + 5]), pack_bf16(v[8 * j + 6], v[8 * j + 7]));
+                }
+                bf16 *t = P.outT + (int64_t)c0 * P.ldt + m;
+#pragma unroll
+                for (int e = 0; e < 32; ++e) {
+                    if (c0 + e < lim) *t = __float2bfloat16_rn(v[e]);
+                    next_row(t, P.ldt);
                 }
             }
+            const float s = transpose_sum(v, lane);
+            if (c0 + lane < lim) atomicAdd(P.colsum + c0 + lane, s);
         }
     }
 }
@@ -355,7 +423,7 @@ net_gemm_kernel(const __grid_constant__ NetGemmParams P, const __grid_constant__
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&S.tfull[b]), 1);
-            mbar_init(smem_u32(&S.tempty[b]), 8);
+            mbar_init(smem_u32(&S.tempty[b]), kNetEpiWarps);
         }
         mbar_init(smem_u32(S.mma_done), 1);
         *S.abort_flag = 0;
@@ -368,7 +436,7 @@ net_gemm_kernel(const __grid_constant__ NetGemmParams P, const __grid_constant__
     float *bias_s = nullptr;
     if (P.bias && P.N <= kNetBiasMax) {
         bias_s = S.xch + kNetXchFloats;
-        for (int i = threadIdx.x; i < P.N; i += blockDim.x) bias_s[i] = P.bias[i];
+        for (int i = threadIdx.x; i < kNetBiasMax + 32; i += blockDim.x) bias_s[i] = i < P.N ? P.bias[i] : 0.f;
     }
     tc_fence_before();
     __syncthreads();
@@ -376,6 +444,8 @@ net_gemm_kernel(const __grid_constant__ NetGemmParams P, const __grid_constant__
     const uint32_t tmem_base = *S.tmem_slot;
     const uint32_t b_bytes = (uint32_t)P.tile_n * 64;
 
+    if (warp < kNetEpiWarp0) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kNetRegsCtl));
     if (warp == 0) {
         if (lane == 0) {
             if (!P.a_image) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
@@ -457,7 +527,9 @@ net_gemm_kernel(const __grid_constant__ NetGemmParams P, const __grid_constant__
                 wait_bounded(smem_u32(S.mma_done), 0, S.abort_flag, P.err, P.timeout_ns, false);
             }
         }
-    } else if (warp >= kNetEpiWarp0) {
+    }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kNetRegsEpi));
         const int q = warp & 3, h = (warp - kNetEpiWarp0) >> 2;
         uint32_t tph = 0;
         int t = 0;
@@ -503,18 +575,6 @@ __global__ void __launch_bounds__(128) image_transpose_kernel(const uint8_t *img
     uint16_t *dst = reinterpret_cast<uint16_t *>(XT);
 #pragma unroll
     for (int e = 0; e < 8; ++e) dst[(int64_t)(kb * kKBlock + c * 8 + e) * ldt + m] = h[e];
-}
-
-// out[n] += sum over rows of X[r][n] (FP32), a column chunk per thread, rows split over blockIdx.y.
-__global__ void __launch_bounds__(128) colsum_kernel(const float *X, int64_t ld, int64_t rows, int32_t cols,
-                                                     int64_t rows_per, float *out)
-{
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= cols) return;
-    const int64_t r0 = (int64_t)blockIdx.y * rows_per, r1 = min(rows, r0 + rows_per);
-    float s = 0.f;
-    for (int64_t r = r0; r < r1; ++r) s += X[r * ld + n];
-    atomicAdd(out + n, s);
 }
 
 struct AdamParams {
@@ -579,6 +639,7 @@ struct NetGemm {
     int64_t ldt = 0;
     float *outf = nullptr;
     int64_t ldf = 0;
+    float *colsum = nullptr;
     const bf16 *hmask = nullptr;
     int64_t ldh = 0;
     const int32_t *colmap = nullptr, *label = nullptr;
@@ -591,7 +652,7 @@ struct NetGemm {
 
 void tile_shape(int N, int epi, int &ntiles, int &tile_n, int &nsub)
 {
-    if (epi == EPI_SOFTMAX) {
+    if (epi == EPI_SOFTMAX || epi == EPI_LOSS) {
         ntiles = 1;
         nsub = N > 256 ? 2 : 1;
         tile_n = ((N + nsub - 1) / nsub + 15) / 16 * 16;
@@ -650,6 +711,7 @@ cudaError_t net_gemm(const rms_plan_s &p, const NetGemm &g, cudaStream_t s)
     P.ldt = g.ldt;
     P.outf = g.outf;
     P.ldf = g.ldf;
+    P.colsum = g.colsum;
     P.hmask = g.hmask;
     P.ldh = g.ldh;
     P.colmap = g.colmap;
@@ -679,7 +741,21 @@ cudaError_t net_gemm(const rms_plan_s &p, const NetGemm &g, cudaStream_t s)
     const int grid = (int)std::min<int64_t>(items, p.num_sms);
     auto kern = g.epi == EPI_RELU ? net_gemm_kernel<EPI_RELU>
               : g.epi == EPI_SOFTMAX ? net_gemm_kernel<EPI_SOFTMAX>
+              : g.epi == EPI_LOSS ? net_gemm_kernel<EPI_LOSS>
               : g.epi == EPI_DRELU ? net_gemm_kernel<EPI_DRELU> : net_gemm_kernel<EPI_ACC>;
+    // the setmaxnreg shares add up to 640 x 96 registers: another register count at launch
+    // would leave the epilogue warpgroups waiting, so the build is checked once
+    static const cudaError_t regs_ok = [] {
+        for (const auto k : {net_gemm_kernel<EPI_RELU>, net_gemm_kernel<EPI_SOFTMAX>, net_gemm_kernel<EPI_LOSS>,
+                             net_gemm_kernel<EPI_DRELU>, net_gemm_kernel<EPI_ACC>}) {
+            cudaFuncAttributes fa;
+            const cudaError_t e1 = cudaFuncGetAttributes(&fa, k);
+            if (e1 != cudaSuccess) return e1;
+            if (fa.numRegs != kNetRegsLaunch) return cudaErrorInvalidConfiguration;
+        }
+        return cudaSuccess;
+    }();
+    if (regs_ok != cudaSuccess) return regs_ok;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, kNetThreads, smem, s>>>(P, tmA, tmB);
@@ -719,16 +795,6 @@ cudaError_t publish(rms_net_s &n, bool update, float lr, float b1, float b2, flo
     return cudaGetLastError();
 }
 
-cudaError_t colsum(const float *X, int64_t ld, int64_t rows, int32_t cols, float *out, cudaStream_t s)
-{
-    const int64_t per = 256;
-    const int64_t gy = (rows + per - 1) / per;
-    if (gy < 1) return cudaSuccess;
-    dim3 grid((unsigned)((cols + 127) / 128), (unsigned)gy);
-    colsum_kernel<<<grid, 128, 0, s>>>(X, ld, rows, cols, per, out);
-    return cudaGetLastError();
-}
-
 rms_status from_cuda(cudaError_t e)
 {
     if (e == cudaSuccess) return RMS_OK;
@@ -740,7 +806,7 @@ void free_net(rms_net_s *n)
 {
     if (!n) return;
     void *ptrs[] = {n->d_p, n->d_g, n->d_m, n->d_v, n->d_W1c, n->d_W1r, n->d_W2, n->d_W2T, n->d_colmap_c,
-                    n->d_colmap_r, n->d_img, n->d_rs, n->d_dz32, n->d_da32, n->d_loss, n->d_h, n->d_hT,
+                    n->d_colmap_r, n->d_img, n->d_rs, n->d_loss, n->d_h, n->d_hT,
                     n->d_dz, n->d_dzT, n->d_da1T, n->d_XT};
     for (void *q : ptrs) cudaFree(q);
     if (n->last) cudaEventDestroy(n->last);
@@ -830,7 +896,7 @@ cudaError_t net_grad(rms_net_s &n, const float *Q, const float *U, int64_t B, in
         g.ldt = n.ldb;
         if ((e = net_gemm(p, g, s)) != cudaSuccess) return e;
     }
-    {   // softmax cross-entropy: loss, dz, dz^T, dz (FP32)
+    {   // softmax cross-entropy: loss, dz, dz^T, db2
         NetGemm g;
         g.A = h;
         g.lda = n.hidden;
@@ -838,7 +904,7 @@ cudaError_t net_grad(rms_net_s &n, const float *Q, const float *U, int64_t B, in
         g.M = (int32_t)B;
         g.N = n.nbins;
         g.K = n.hidden;
-        g.epi = EPI_SOFTMAX;
+        g.epi = EPI_LOSS;
         g.bias = n.d_p + n.ob2;
         g.label = label;
         g.loss = n.d_loss;
@@ -847,8 +913,7 @@ cudaError_t net_grad(rms_net_s &n, const float *Q, const float *U, int64_t B, in
         g.ldo = n.nbp;
         g.outT = dzT;
         g.ldt = n.ldb;
-        g.outf = n.d_dz32;
-        g.ldf = n.nbp;
+        g.colsum = n.d_g + n.ob2;
         if ((e = net_gemm(p, g, s)) != cudaSuccess) return e;
     }
     {   // dW2 = dz^T h
@@ -865,8 +930,7 @@ cudaError_t net_grad(rms_net_s &n, const float *Q, const float *U, int64_t B, in
         g.ldf = n.hidden;
         if ((e = net_gemm(p, g, s)) != cudaSuccess) return e;
     }
-    if ((e = colsum(n.d_dz32, n.nbp, B, n.nbins, n.d_g + n.ob2, s)) != cudaSuccess) return e;
-    {   // da1 = (dz W2) * [h > 0]: (da1 / s)^T for dW1, da1 for db1
+    {   // da1 = (dz W2) * [h > 0]: (da1 / s)^T for dW1, db1
         NetGemm g;
         g.A = dz;
         g.lda = n.nbp;
@@ -880,11 +944,9 @@ cudaError_t net_grad(rms_net_s &n, const float *Q, const float *U, int64_t B, in
         g.ldh = n.hidden;
         g.outT = da1T;
         g.ldt = n.ldb;
-        g.outf = n.d_da32;
-        g.ldf = n.hidden;
+        g.colsum = n.d_g + n.ob1;
         if ((e = net_gemm(p, g, s)) != cudaSuccess) return e;
     }
-    if ((e = colsum(n.d_da32, n.hidden, B, n.hidden, n.d_g + n.ob1, s)) != cudaSuccess) return e;
     {   // X^T from the image, then dW1 = (da1 / s)^T X_raw in W1's column order
         dim3 grid((unsigned)((B + kTileM - 1) / kTileM), (unsigned)(kb * 4));
         image_transpose_kernel<<<grid, 128, 0, s>>>(n.d_img, kb, B, XT, n.ldb);
@@ -997,8 +1059,6 @@ rms_status rms_net_create(rms_net_t *out, rms_plan_t plan, int32_t hidden, int32
     NET_TRY(cudaMalloc(&n->d_colmap_r, p.kpad_raw * sizeof(int32_t)));
     NET_TRY(cudaMalloc(&n->d_img, img));
     NET_TRY(cudaMalloc(&n->d_rs, B * sizeof(float)));
-    NET_TRY(cudaMalloc(&n->d_dz32, B * n->nbp * sizeof(float)));
-    NET_TRY(cudaMalloc(&n->d_da32, B * hidden * sizeof(float)));
     NET_TRY(cudaMalloc(&n->d_loss, sizeof(float)));
     NET_TRY(cudaMalloc(&n->d_h, B * hidden * 2));
     NET_TRY(cudaMalloc(&n->d_hT, (size_t)hidden * L * 2));

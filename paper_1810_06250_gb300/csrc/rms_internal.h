@@ -249,7 +249,7 @@ struct rms_net_s {
     CUtensorMap tm_W1c, tm_W1r, tm_W2, tm_W2T;
     // training scratch for max_batch lines of sight
     uint8_t *d_img = nullptr;
-    float *d_rs = nullptr, *d_dz32 = nullptr, *d_da32 = nullptr, *d_loss = nullptr;
+    float *d_rs = nullptr, *d_loss = nullptr;
     uint16_t *d_h = nullptr, *d_hT = nullptr, *d_dz = nullptr, *d_dzT = nullptr, *d_da1T = nullptr, *d_XT = nullptr;
     cudaEvent_t last = nullptr;
 };
