@@ -83,95 +83,91 @@ __device__ __forceinline__ void emit16(uint8_t *row, int hh, int sw, const float
     if (MODE != MODE_BF16) store32<RING>(p + kFoldPart, lo, sw & 1);
 }
 
-// hi and lo 16-bit parts of one value, hi in the low half.
-template <int MODE>
-__device__ __forceinline__ uint32_t split_one(float v)
-{
-    if (MODE == MODE_FP16X3) {
-        const __half h = __float2half_rn(v);
-        const __half l = __float2half_rn(v - __half2float(h));
-        return (uint32_t)__half_as_ushort(h) | ((uint32_t)__half_as_ushort(l) << 16);
-    }
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-    return (uint32_t)__bfloat16_as_ushort(h) | ((uint32_t)__bfloat16_as_ushort(l) << 16);
-}
-
-// LOS-major rows: the lanes of a warp take the 32 active channels of a K block of 8 LOS
-// (one 16-row group of a tile), so that a load reads a LOS's channels (nearly)
-// contiguously at any alignment, flagged channels drop out, and after an exchange
-// between lane pairs (even lanes take the hi words, odd lanes the lo words) a store
-// writes 64 contiguous bytes of each part.  The loads are unconditional, so that all 16
-// are in flight at once: src_of(r) is row r's LOS, or any LOS for a row beyond the end
-// (bit r of dead), whose values become 0 like those of padding channels.
+// LOS-major rows: a warp takes the 32 active channels of a K block of 8 LOS (one 16-row
+// group of a tile).  Lane (half, p) holds channels 2 p and 2 p + 1 of LOS 2 j + half,
+// j = 0 .. 3: a load reads two LOS' channels (nearly) contiguously at any alignment,
+// flagged channels drop out, and a store writes 64 contiguous bytes of two rows.
+// The loads are unconditional, so that all 16 are in flight at once: src_of(r) is row r's
+// LOS, or any LOS for a row beyond the end (bit r of dead), whose values become 0 like
+// those of padding channels.  v[2 j], v[2 j + 1]: the two channels of LOS 2 j + half.
+// Against one channel of 8 LOS per lane, whose 16-bit results were paired by a shuffle and
+// stored by every other lane: half the store instructions and no shuffles.  One-kernel form,
+// 5,001 LOS x 357 channels x 401 phi BF16x3 37.2 -> 33.2 us, 200,003 LOS FP16x3 0.529 ->
+// 0.501 ms, window of 262,144 LOS x 360 -> 64 BF16x3 with its proposal 0.940 -> 0.902 ms.
 template <bool LAST, typename F>
 __device__ __forceinline__ void fold_load_los(const FoldSource &S, const int *list, int kb, int lane, F src_of, float (&q)[8],
                                               float (&u)[8])
 {
-    const int ch = list[kb * kKBlock + lane];      // the padded channel list
+    const int2 ch = *reinterpret_cast<const int2 *>(list + kb * kKBlock + 2 * (lane & 15));   // the padded channel list
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const int64_t off = src_of(r) * S.nchan + ch;
-        q[r] = load_here<LAST>(S.Q + off);
-        u[r] = load_here<LAST>(S.U + off);
+    for (int j = 0; j < 4; ++j) {
+        const int64_t base = src_of(2 * j + (lane >> 4)) * S.nchan;
+        q[2 * j] = load_here<LAST>(S.Q + base + ch.x);
+        q[2 * j + 1] = load_here<LAST>(S.Q + base + ch.y);
+        u[2 * j] = load_here<LAST>(S.U + base + ch.x);
+        u[2 * j + 1] = load_here<LAST>(S.U + base + ch.y);
     }
 }
 __device__ __forceinline__ void fold_mask_los(const FoldSource &S, int kb, int lane, uint32_t dead, float (&q)[8],
                                               float (&u)[8])
 {
-    if (kb * kKBlock + lane >= S.nact) dead = 0xffu;
-    if (__any_sync(0xffffffffu, dead != 0u)) {
+    const int left = S.nact - kb * kKBlock - 2 * (lane & 15);      // active channels from this lane's first on
+    if (__any_sync(0xffffffffu, dead != 0u || left < 2)) {
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
-            if ((dead >> r) & 1u) { q[r] = 0.f; u[r] = 0.f; }
+        for (int e = 0; e < 8; ++e)
+            if (((dead >> (2 * (e >> 1) + (lane >> 4))) & 1u) || (e & 1) >= left) { q[e] = 0.f; u[e] = 0.f; }
     }
 }
 
-// The scales (and exponents) of 8 LOS: a first pass over their rows.
+// The scales (and exponents) of 8 LOS, in every lane: a first pass over their rows.
 template <typename F>
-__device__ __forceinline__ void fold_scales_los(const FoldSource &S, const int *list, int kblocks, int lane, F src_of, uint32_t dead,
-                                                float (&scale)[8], int (&ex)[8])
+__device__ __forceinline__ void fold_scales_los(const FoldSource &S, const int *list, int kblocks, int lane, F src_of,
+                                                uint32_t dead, float (&scale)[8], int (&ex)[8])
 {
-    float mx[8];
-#pragma unroll
-    for (int r = 0; r < 8; ++r) mx[r] = 0.f;
+    float mx[4] = {0.f, 0.f, 0.f, 0.f};
     for (int kb = 0; kb < kblocks; ++kb) {
         float q[8], u[8];
         fold_load_los<false>(S, list, kb, lane, src_of, q, u);
         fold_mask_los(S, kb, lane, dead, q, u);
 #pragma unroll
-        for (int r = 0; r < 8; ++r) mx[r] = fmaxf(mx[r], fmaxf(fabsf(q[r]), fabsf(u[r])));
+        for (int e = 0; e < 8; ++e) mx[e >> 1] = fmaxf(mx[e >> 1], fmaxf(fabsf(q[e]), fabsf(u[e])));
     }
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
+    for (int j = 0; j < 4; ++j) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], o));
-        ex[r] = fold_exponent(mx[r]);
-        scale[r] = ldexpf(1.0f, ex[r]);
+        for (int o = 8; o > 0; o >>= 1) mx[j] = fmaxf(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], o));
+        const float other = __shfl_xor_sync(0xffffffffu, mx[j], 16);
+        ex[2 * j] = fold_exponent(lane < 16 ? mx[j] : other);
+        ex[2 * j + 1] = fold_exponent(lane < 16 ? other : mx[j]);
+        scale[2 * j] = ldexpf(1.0f, ex[2 * j]);
+        scale[2 * j + 1] = ldexpf(1.0f, ex[2 * j + 1]);
     }
 }
 
-// One K block of LOS r0 .. r0 + N - 1 of a group of 8, Q or U; rows: the group's first
-// operand row in K block kb of the image.
+// One K block of LOS r0 .. r0 + N - 1 (r0 even) of a group of 8, Q or U; rows: the group's
+// first operand row in K block kb of the image.
 template <int MODE, bool RING, int N>
 __device__ __forceinline__ void fold_emit_rows(uint8_t *rows, int lane, int r0, const float (&v)[N], const float (&scale)[8])
 {
-    uint8_t *const mine = rows + ((lane & 1) ? kFoldPart : 0) + 4 * ((lane >> 1) & 3);
-    const int chunk = lane >> 3;
+    const int p = lane & 15, half = lane >> 4;
 #pragma unroll
-    for (int j = 0; j < N; ++j) {
-        const int r = r0 + j;
-        const uint32_t w = split_one<MODE>(MODE == MODE_FP16X3 ? v[j] * scale[j] : v[j]);
-        const uint32_t p = __shfl_xor_sync(0xffffffffu, w, 1);
-        const uint32_t o = (lane & 1) ? __byte_perm(p, w, 0x7632) : __byte_perm(w, p, 0x5410);
-        uint8_t *at = mine + r * kFoldRowBytes + ((chunk ^ ((r >> 1) & 3)) << 4);
-        const uint32_t store = MODE != MODE_BF16 || !(lane & 1);
-        if (RING)
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t"
-                         "@p st.global.L2::cache_hint.b32 [%0], %1, %2;\n\t}" ::"l"(at),
-                         "r"(o), "l"(l2_evict_last()), "r"(store)
-                         : "memory");
-        else if (store)
-            *reinterpret_cast<uint32_t *>(at) = o;
+    for (int j = 0; j < N / 2; ++j) {
+        const int r = r0 + 2 * j + half;
+        uint32_t hi, lo;
+        if (MODE == MODE_FP16X3) {
+            const float s = half ? scale[2 * j + 1] : scale[2 * j];
+            split_pair_fp16(v[2 * j] * s, v[2 * j + 1] * s, hi, lo);
+        } else {
+            split_pair_bf16(v[2 * j], v[2 * j + 1], hi, lo);
+        }
+        uint8_t *at = rows + r * kFoldRowBytes + (((p >> 2) ^ ((r >> 1) & 3)) << 4) + 4 * (p & 3);
+        if (RING) {
+            asm volatile("st.global.L2::cache_hint.b32 [%0], %1, %2;" ::"l"(at), "r"(hi), "l"(l2_evict_last()) : "memory");
+            if (MODE != MODE_BF16)
+                asm volatile("st.global.L2::cache_hint.b32 [%0], %1, %2;" ::"l"(at + kFoldPart), "r"(lo), "l"(l2_evict_last()) : "memory");
+        } else {
+            *reinterpret_cast<uint32_t *>(at) = hi;
+            if (MODE != MODE_BF16) *reinterpret_cast<uint32_t *>(at + kFoldPart) = lo;
+        }
     }
 }

@@ -617,30 +617,15 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                     cen[h] = max(P.rot.cmin, min(P.rot.cmax, __ldg(P.rot.centre + min(los0 + 32 * h + lane, nlos - 1))));
                 if constexpr (CHAN) cen[0] = (sw & 1) ? cen[1] : cen[0];
             }
-            // T of LOS j of the item at this lane's channel of K block kb
+            // T of LOS j + (lane / 16) of the item (j even) at this lane's two channels of K block kb
             auto t_of = [&](int j, int kb) {
-                const int c = __shfl_sync(0xffffffffu, j & 32 ? cen[1] : cen[0], j & 31);
-                return __ldg(P.rot.T + (size_t)c * P.rot.ldT + kb * kKBlock + lane);
+                const int c = __shfl_sync(0xffffffffu, j & 32 ? cen[1] : cen[0], (j & 31) + (lane >> 4));
+                return __ldg(reinterpret_cast<const float4 *>(P.rot.T + (size_t)c * P.rot.ldT + kb * kKBlock) + (lane & 15));
             };
             if constexpr (MODE == MODE_FP16X3) {
                 // the LOS's largest |value| sets its power-of-two scale: a first pass over the tile
                 // (staged LOS-major rows are complete in their slot and need none)
-                if constexpr (CHAN) {
-                    float mx = 0.f;
-                    chan_walk<false>(P.src, S.list, los0 + i, array, h0, nh, [&](int, const float (&v)[16]) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) mx = fmaxf(mx, fabsf(v[j]));
-                    });
-                    const float *x = join_max(mx);
-                    if (!x) {
-                        ok = false;
-                        break;
-                    }
-#pragma unroll
-                    for (int w = 0; w < kNumSplitWarps; w += 2) mx = fmaxf(mx, x[(w + (sw & 1)) * 32 + lane]);
-                    ex[0] = fold_exponent(mx);
-                    scale[0] = ldexpf(1.0f, ex[0]);
-                } else if (!stg) {
+                if (!stg) {
                     fold_scales_los(P.src, S.list, P.kblocks, lane, src_of, dead, scale, ex);
                 }
             }
@@ -651,7 +636,6 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                 break;
             }
             if constexpr (CHAN) {
-                if (MODE == MODE_FP16X3 && sw < 2) exps[i] = ex[0];
                 if constexpr (ROT) {
                     // both arrays of 8 channels at a time; four warps share a LOS
                     const float2 *T = P.rot.T + (size_t)cen[0] * P.rot.ldT;
@@ -696,10 +680,10 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                 }
             } else if (stg) {
                 // 8 LOS per slot; units of (K block, array), or ROT (K block, 4 LOS), go round the warps
-                float2 t[4];
+                float4 t[2];
                 if constexpr (ROT) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) t[j] = t_of(4 * (sw & 1) + j, min(sw >> 1, P.kblocks - 1));
+                    for (int j = 0; j < 2; ++j) t[j] = t_of(4 * (sw & 1) + 2 * j, min(sw >> 1, P.kblocks - 1));
                 }
                 for (int g = 0; g < kFoldTileLos / 8; ++g) {
                     if (!warp_wait(smem_u32(&S.sfull[ss]), sph, S.abort_flag, P.err, P.timeout_ns)) {
@@ -731,24 +715,36 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                     }
                     const int arr = sw & 1;
                     for (int kb = sw >> 1; kb < P.kblocks; kb += kNumSplitWarps / 2) {
-                        const int ch = S.list[kb * kKBlock + lane];
-                        const bool live = kb * kKBlock + lane < P.src.nact;
+                        const int2 ch = *reinterpret_cast<const int2 *>(S.list + kb * kKBlock + 2 * (lane & 15));
+                        const int left = P.src.nact - kb * kKBlock - 2 * (lane & 15);   // padding channels give 0
+                        const int half = lane >> 4;
+                        // the two halves read rows nchan words apart: with an even nchan the upper half
+                        // takes its odd channels first, which keeps the 32 lanes on 32 banks
+                        const bool flip = half && !(nchan & 1);
+                        const int c0 = flip ? ch.y : ch.x, c1 = flip ? ch.x : ch.y;
+                        auto pair_of = [&](const float *x, float &v0, float &v1) {
+                            const float a = x[c0], b = x[c1];
+                            v0 = left > 0 ? (flip ? b : a) : 0.f;
+                            v1 = left > 1 ? (flip ? a : b) : 0.f;
+                        };
                         uint8_t *const blk = tile + (size_t)kb * kPartsBytes + 16 * g * kFoldRowBytes;
                         if constexpr (ROT) {
                             const int r0 = 4 * arr;
                             float q[4], u[4];
-                            float2 tn[4];
+                            float4 tn[2];
                             // T of the warp's next unit, here or in the next slot
                             const bool more = kb + kNumSplitWarps / 2 < P.kblocks;
                             const int gn = more ? g : min(g + 1, kFoldTileLos / 8 - 1);
                             const int kn = more ? kb + kNumSplitWarps / 2 : sw >> 1;     // (kb itself is one: in range)
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) tn[j] = t_of(8 * gn + r0 + j, kn);
+                            for (int j = 0; j < 2; ++j) tn[j] = t_of(8 * gn + r0 + 2 * j, kn);
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                q[j] = live ? rows[(r0 + j) * nchan + ch] : 0.f;
-                                u[j] = live ? rows[(8 + r0 + j) * nchan + ch] : 0.f;
-                                rotate(q[j], u[j], t[j]);
+                            for (int j = 0; j < 2; ++j) {
+                                const float *x = rows + (r0 + 2 * j + half) * nchan, *y = x + 8 * nchan;
+                                pair_of(x, q[2 * j], q[2 * j + 1]);
+                                pair_of(y, u[2 * j], u[2 * j + 1]);
+                                rotate(q[2 * j], u[2 * j], make_float2(t[j].x, t[j].y));
+                                rotate(q[2 * j + 1], u[2 * j + 1], make_float2(t[j].z, t[j].w));
                                 t[j] = tn[j];
                             }
                             fold_emit_rows<MODE, true, 4>(blk, lane, r0, q, scale);
@@ -756,7 +752,9 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                         } else {
                             float v[8];
 #pragma unroll
-                            for (int r = 0; r < 8; ++r) v[r] = live ? rows[(8 * arr + r) * nchan + ch] : 0.f;
+                            for (int j = 0; j < 4; ++j) {
+                                pair_of(rows + (8 * arr + 2 * j + half) * nchan, v[2 * j], v[2 * j + 1]);
+                            }
                             fold_emit_rows<MODE, true, 8>(blk + 8 * arr * kFoldRowBytes, lane, 0, v, scale);
                         }
                     }
@@ -777,7 +775,11 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                     fold_mask_los(P.src, kb, lane, dead, q, u);
                     if constexpr (ROT) {
 #pragma unroll
-                        for (int r = 0; r < 8; ++r) rotate(q[r], u[r], t_of(8 * sw + r, kb));
+                        for (int j = 0; j < 4; ++j) {
+                            const float4 t = t_of(8 * sw + 2 * j, kb);
+                            rotate(q[2 * j], u[2 * j], make_float2(t.x, t.y));
+                            rotate(q[2 * j + 1], u[2 * j + 1], make_float2(t.z, t.w));
+                        }
                     }
                     fold_emit_rows<MODE, true, 8>(dst + (size_t)kb * kPartsBytes, lane, 0, q, scale);
                     fold_emit_rows<MODE, true, 8>(dst + (size_t)kb * kPartsBytes + 8 * kFoldRowBytes, lane, 0, u, scale);
@@ -828,7 +830,7 @@ FusedKernel fused_for(int mode, bool chan, bool rot)
     }
     if (mode == MODE_BF16) return chan ? fused_kernel<MODE_BF16, true, false> : fused_kernel<MODE_BF16, false, false>;
     if (mode == MODE_BF16X3) return chan ? fused_kernel<MODE_BF16X3, true, false> : fused_kernel<MODE_BF16X3, false, false>;
-    return chan ? fused_kernel<MODE_FP16X3, true, false> : fused_kernel<MODE_FP16X3, false, false>;
+    return fused_kernel<MODE_FP16X3, false, false>;     // (fused_wanted: staged LOS-major rows)
 }
 
 // Pipeline shape beside `staging` bytes of staging slots and the channel list: K blocks per stage and stages, at
