@@ -55,7 +55,7 @@ struct FusedParams {
     FoldSource src;
     int32_t kblocks, mode;
     int32_t nphi, ncol, kplus, kminus;
-    int32_t ntiles_n, tile_n, tile_n_last;
+    int32_t ntiles_n, tile_n, tile_n_last, npad;
     uint8_t *ring;              // [CTAs][2][kblocks][parts x 8 KB]
     float *F;
     int32_t *pidx;
@@ -285,9 +285,9 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                             if (leader) mbar_arrive_expect_tx(bar, 2 * tx * (uint32_t)n);
                             for (int i = 0; i < n; ++i, st += S.sub_bytes) {
                                 tma_load_3d_pair(st, &tmA, 0, 0, z0 + kb + i, bar0);
-                                tma_load_2d_pair(st + kPartsBytes, &tmB_hi, (kb + i) * kKBlock, y, bar0);
-                                if (kSplitPrec)
-                                    tma_load_2d_pair(st + kPartsBytes + b_bytes, &tmB_lo, (kb + i) * kKBlock, y, bar0);
+                                const int32_t yb = ((kb + i) * P.npad + y) / kFoldMapRows;
+                                tma_load_2d_pair(st + kPartsBytes, &tmB_hi, 0, yb, bar0);
+                                if (kSplitPrec) tma_load_2d_pair(st + kPartsBytes + b_bytes, &tmB_lo, 0, yb, bar0);
                             }
                             pending |= 1u << s;
                             pend_par = (pend_par & ~(1u << s)) | (ph << s);
@@ -956,6 +956,7 @@ cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, in
     P.ntiles_n = f.tiles.ntiles_n2;
     P.tile_n = f.tiles.tile_n2;
     P.tile_n_last = f.tiles.tile_n_last2;
+    P.npad = f.tiles.npad;
     P.ring = ring;
     P.F = F;
     P.pidx = pidx;
@@ -976,12 +977,14 @@ cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, in
     if (sh.stages < 3) return cudaErrorInvalidConfiguration;
     P.stages = sh.stages;
     P.kbs = sh.kbs;
-    // the ring as a 3-D tensor: 64-byte rows, the hi (and lo) rows of a K block, K blocks
+    // the ring as a 3-D tensor: 8 of the image's 64-byte rows to a row (whole lines per request), the
+    // hi (and lo) rows of a K block, K blocks
     const int parts = mode == MODE_BF16 ? 1 : 2;
+    constexpr int kRow = kFoldMapRows * kKBlock;
     CUtensorMap tmA;
-    const cuuint64_t dims[3] = {(cuuint64_t)kKBlock, (cuuint64_t)(parts * kTileM), (cuuint64_t)(4 * pairs) * f.kblocks};
-    const cuuint64_t strides[2] = {(cuuint64_t)kFoldRowBytes, (cuuint64_t)(parts * kFoldPart)};
-    const cuuint32_t box[3] = {(cuuint32_t)kKBlock, (cuuint32_t)(parts * kTileM), 1};
+    const cuuint64_t dims[3] = {(cuuint64_t)kRow, (cuuint64_t)(parts * kTileM / kFoldMapRows), (cuuint64_t)(4 * pairs) * f.kblocks};
+    const cuuint64_t strides[2] = {(cuuint64_t)kRow * 2, (cuuint64_t)(parts * kFoldPart)};
+    const cuuint32_t box[3] = {(cuuint32_t)kRow, (cuuint32_t)(parts * kTileM / kFoldMapRows), 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     if (!encode_tensor_map(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT16, ring, dims, strides, box, estr,
                            CU_TENSOR_MAP_SWIZZLE_NONE, 3))

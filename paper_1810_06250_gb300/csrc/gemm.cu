@@ -285,6 +285,7 @@ struct GemmParams {
     const int64_t *rows;        // optional: results of row r go to output row rows[r]
     int32_t kblocks, group;
     int32_t nphi, ntiles_n, tile_n, tile_n_last;
+    int32_t npad;               // FOLD: rows per K block of the phase matrix
     int32_t ncol;               // column pairs (2 phase rows each) holding results: nphi, or ceil(nphi / 2) folded
     float *F;
     int32_t *pidx;
@@ -494,15 +495,19 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                                 if (leader) mbar_arrive_expect_tx(bar, 2 * tx * (uint32_t)n);
                                 for (int i = 0; i < n; ++i, st += S.sub_bytes) {
                                     tma_load_3d_pair(st, &tmA, 0, 0, (int32_t)(mt * P.kblocks + kb + i), bar0);
-                                    tma_load_2d_pair(st + a_bytes, &tmB_hi, (kb + i) * kKBlock, y, bar0);
-                                    if (split) tma_load_2d_pair(st + a_bytes + b_bytes, &tmB_lo, (kb + i) * kKBlock, y, bar0);
+                                    const int32_t bx = FOLD ? 0 : (kb + i) * kKBlock;
+                                    const int32_t by = FOLD ? ((kb + i) * P.npad + y) / kFoldMapRows : y;
+                                    tma_load_2d_pair(st + a_bytes, &tmB_hi, bx, by, bar0);
+                                    if (split) tma_load_2d_pair(st + a_bytes + b_bytes, &tmB_lo, bx, by, bar0);
                                 }
                             } else {
                                 mbar_arrive_expect_tx(bar, tx * (uint32_t)n);
                                 for (int i = 0; i < n; ++i, st += S.sub_bytes) {
                                     bulk_load(st, a_mt + (size_t)(kb + i) * (2 * kStageA), a_bytes, bar);
-                                    tma_load_2d(st + a_bytes, &tmB_hi, (kb + i) * kKBlock, y, bar);
-                                    if (split) tma_load_2d(st + a_bytes + b_bytes, &tmB_lo, (kb + i) * kKBlock, y, bar);
+                                    const int32_t bx = FOLD ? 0 : (kb + i) * kKBlock;
+                                    const int32_t by = FOLD ? ((kb + i) * P.npad + y) / kFoldMapRows : y;
+                                    tma_load_2d(st + a_bytes, &tmB_hi, bx, by, bar);
+                                    if (split) tma_load_2d(st + a_bytes + b_bytes, &tmB_lo, bx, by, bar);
                                 }
                             }
                             pending |= 1u << s;
@@ -1324,6 +1329,7 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
     P.ntiles_n = pair ? tl.ntiles_n2 : tl.ntiles_n;
     P.tile_n = pair ? tl.tile_n2 : tl.tile_n;
     P.tile_n_last = pair ? tl.tile_n_last2 : tl.tile_n_last;
+    P.npad = tl.npad;
     const bool wide = pair && P.tile_n > 2 * kHalf;   // the pair kernel with 128 columns per epilogue thread
     P.b_rows = pair ? P.tile_n / 2 : P.tile_n;
     P.kbs = 1;
@@ -1432,15 +1438,16 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
         const CUtensorMap &bhi = fold ? p.fold.tmap2_bhi : chan ? p.tmap2_bhi : p.tmap2_bhi_raw;
         const CUtensorMap &blo = fold ? p.fold.tmap2_blo : chan ? p.tmap2_blo : p.tmap2_blo_raw;
         const int pairs = units;
-        // the operand image as a 3-D tensor for the pair's TMA loads: 64-byte rows, 256
-        // rows (hi then lo parts) per 16 KB block, one block per (M tile, K block); a
-        // stage is one block's first a_rows rows
+        // the operand image as a 3-D tensor for the pair's TMA loads: 256 rows of 64 bytes (hi
+        // then lo parts) per 16 KB block, taken eight to a row of the map (whole lines per
+        // request), one block per (M tile, K block); a stage is one block's first part or both
         CUtensorMap tmA;
         {
             const int64_t nblocks = ((nmt + 1) & ~(int64_t)1) * P.kblocks;
-            const cuuint64_t dims[3] = {(cuuint64_t)kKBlock, (cuuint64_t)(2 * kTileM), (cuuint64_t)nblocks};
-            const cuuint64_t strides[2] = {(cuuint64_t)kRowBytes, (cuuint64_t)(2 * kStageA)};
-            const cuuint32_t box[3] = {(cuuint32_t)kKBlock, (cuuint32_t)(split_mode(mode) ? 2 * kTileM : kTileM), 1};
+            constexpr int kRow = 8 * kKBlock;
+            const cuuint64_t dims[3] = {(cuuint64_t)kRow, (cuuint64_t)(2 * kTileM / 8), (cuuint64_t)nblocks};
+            const cuuint64_t strides[2] = {(cuuint64_t)kRow * 2, (cuuint64_t)(2 * kStageA)};
+            const cuuint32_t box[3] = {(cuuint32_t)kRow, (cuuint32_t)((split_mode(mode) ? 2 * kTileM : kTileM) / 8), 1};
             const cuuint32_t estr[3] = {1, 1, 1};
             if (nblocks > 0x7fffffff ||
                 !encode_tensor_map(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT16, const_cast<uint8_t *>(o.A), dims, strides,

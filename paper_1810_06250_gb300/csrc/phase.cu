@@ -122,12 +122,14 @@ __global__ void phase_bsplit_kernel(const double *__restrict__ dl2, const double
     }
 }
 
-// Folded operand, K-major [npad][kpad]: row 2i holds c and row 2i + 1 holds s of depth
-// dh[i], column a the a-th active channel, (c, s) = (w_a / w_max) (cos, sin)(theta).
+// Folded operand: row 2i holds c and row 2i + 1 holds s of depth dh[i], column a the a-th
+// active channel, (c, s) = (w_a / w_max) (cos, sin)(theta).  K blocks of 32 columns, each
+// [npad] rows of 64 bytes in the order in which a tile stands in shared memory
+// (SWIZZLE_64B), so that a tile of one K block is one contiguous piece of memory.
 template <typename T>
 __global__ void phase_fold_kernel(const double *__restrict__ dl2, const double *__restrict__ w,
                                   const double *__restrict__ dh, int32_t nact, int32_t ncol, double inv_wmax,
-                                  int32_t kpad, uint16_t *__restrict__ bhi, uint16_t *__restrict__ blo)
+                                  int32_t npad, uint16_t *__restrict__ bhi, uint16_t *__restrict__ blo)
 {
     const int64_t total = (int64_t)nact * ncol;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
@@ -136,7 +138,8 @@ __global__ void phase_fold_kernel(const double *__restrict__ dl2, const double *
         double s, c;
         phase_sincos(dh[i], dl2[a], &s, &c);
         const double wn = w[a] * inv_wmax;
-        const size_t r0 = (size_t)(2 * i) * kpad + a, r1 = r0 + kpad;
+        // rows 2 i and 2 i + 1 swizzle alike: the pattern changes every second row
+        const size_t r0 = ((size_t)(a >> 5) * npad + 2 * i) * 32 + ((((a >> 3) ^ i) & 3) << 3) + (a & 7), r1 = r0 + 32;
         split16<T>(wn * c, bhi + r0, blo + r0);
         split16<T>(wn * s, bhi + r1, blo + r1);
     }
@@ -207,10 +210,10 @@ cudaError_t launch_phase_fold(const rms_plan_s &p, const FoldPlan &f, const doub
     const int g = grid_for((int64_t)p.nact * f.ncol, 256);
     const double inv = 1.0 / p.wmax;
     if (fp16)
-        phase_fold_kernel<__half><<<g, 256, 0, s>>>(p.d_dl2, p.d_wact, dh, p.nact, f.ncol, inv, f.kpad, f.d_hi, f.d_lo);
+        phase_fold_kernel<__half><<<g, 256, 0, s>>>(p.d_dl2, p.d_wact, dh, p.nact, f.ncol, inv, f.tiles.npad, f.d_hi, f.d_lo);
     else
         phase_fold_kernel<__nv_bfloat16>
-            <<<g, 256, 0, s>>>(p.d_dl2, p.d_wact, dh, p.nact, f.ncol, inv, f.kpad, f.d_hi, f.d_lo);
+            <<<g, 256, 0, s>>>(p.d_dl2, p.d_wact, dh, p.nact, f.ncol, inv, f.tiles.npad, f.d_hi, f.d_lo);
     return cudaGetLastError();
 }
 

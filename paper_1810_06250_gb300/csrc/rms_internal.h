@@ -41,13 +41,14 @@ struct PhaseTiling {
 // A symmetric phi grid (phi_k + phi_{nphi-1-k} = 0), and the tensor-core precisions'
 // folded phase matrix (window plans: the W offsets -W/2 .. W/2 - 1, one -phi sample more): rows (c, s) = (w / w_max) (cos, sin)(theta) of the ncol depths phi >= 0, columns the active
 // channels, which the contraction multiplies with Q and U rows of their own (fold.cu).
+constexpr int kFoldMapRows = 8;    // rows of a K block of the folded phase matrix per row of its tensor maps
 struct FoldPlan {
     bool on = false, pair_maps = false;
     int32_t ncol = 0;              // ceil(nphi / 2)
     int32_t kplus = 0, kminus = 0; // column pair i holds phi samples kplus + i and kminus - i
     int32_t kblocks = 0, kpad = 0; // K blocks of 32 active channels
     PhaseTiling tiles;
-    uint16_t *d_hi = nullptr, *d_lo = nullptr;   // [tiles.npad][kpad]
+    uint16_t *d_hi = nullptr, *d_lo = nullptr;   // [kblocks][tiles.npad][32], 16-byte pieces in SWIZZLE_64B order
     int32_t *d_list = nullptr;     // [kpad] the active channels, padded with the last one
     int32_t fused_pairs = 0;       // the one-kernel form (fused.cu): resident CTA pairs (0: not for this plan)
     CUtensorMap tmap_bhi, tmap_blo, tmap2_bhi, tmap2_blo;
