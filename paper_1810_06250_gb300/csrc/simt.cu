@@ -18,6 +18,9 @@
 // weigh twice as much: channel-major cubes whose rows start on 16 bytes copy 4 LOS
 // at a time.  262,144 LOS x 360 active channels x 401 phi: table 6.82 -> 3.61 ms,
 // on the fly 6.97 -> 3.70 ms (rows not aligned 4.58, LOS-major 7.05 -> 4.64 ms).
+// The FMAs are packed over two LOS (one instruction, the rounding of two): the issue slots
+// were the bound, now the FMA pipe is busy 67 % of the time.  Table 3.56 -> 3.33 ms, on the
+// fly 3.66 -> 3.32 ms, rows not aligned 4.53 -> 4.31 ms, LOS-major 4.61 -> 4.40 ms.
 // The peak of |F| (Sec. 2.2) is reduced in registers over the block's phi
 // tiles, so F never has to be re-read.
 #include <cooperative_groups.h>
@@ -81,11 +84,11 @@ __device__ __forceinline__ void cp_async(void *dst, const void *src, bool ok)
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-__device__ __forceinline__ void load8(const float *p, float (&v)[8])
+__device__ __forceinline__ void load8(const float *p, float2 (&v)[4])
 {
     const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w);
+    v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
 }
 
 // Each thread copies one channel of every chunk: ISSUE_CH(tid) is that channel's
@@ -210,13 +213,14 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_
     constexpr int NJ = 2 * JJ, W = FOLD ? TP / 2 : TP, NS = FOLD ? 4 : 2;
     const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
     // sums of a (LOS, column): Re, Im of F, or folded Qc, Us, Uc, Qs
-    float acc[8][NJ][NS];
+    // of LOS 2 i and 2 i + 1: one packed FMA feeds both
+    float2 acc[4][NJ][NS];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < NJ; ++j)
 #pragma unroll
-            for (int x = 0; x < NS; ++x) acc[i][j][x] = 0.f;
+            for (int x = 0; x < NS; ++x) acc[i][j][x] = make_float2(0.f, 0.f);
 
     for (int ck = 0; ck < pp.nck; ++ck, ++pp.t) {
         const int n = pp.t + 1;
@@ -231,7 +235,8 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_
         const Stage &st = stage[pp.t & 1];
 #pragma unroll 2
         for (int c = 0; c < CH; ++c) {
-            float qv[8], uv[8], cv[NJ], sv[NJ];
+            float2 qv[4], uv[4];
+            float cv[NJ], sv[NJ];
             load8(&st.q[c][8 * ty], qv);
             load8(&st.u[c][8 * ty], uv);
             // thread tx owns phi pairs 16 jj + 2 tx + {0, 1}: the 8 threads of a
@@ -242,23 +247,26 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_
                 cv[j] = v.x; sv[j] = v.y; cv[j + 1] = v.z; sv[j + 1] = v.w;
             }
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int j = 0; j < NJ; ++j) {
+                const float2 c2 = make_float2(cv[j], cv[j]), s2 = make_float2(sv[j], sv[j]);
+                const float2 n2 = make_float2(-sv[j], -sv[j]);
 #pragma unroll
-                for (int j = 0; j < NJ; ++j) {
-                    float(&s)[NS] = acc[i][j];
+                for (int i = 0; i < 4; ++i) {
+                    float2(&s)[NS] = acc[i][j];
                     // (q + iu)(c - is): Re += q c + u s, Im += u c - q s  (Eqs. qPhi, uPhi)
                     if constexpr (FOLD) {
-                        s[0] = fmaf(qv[i], cv[j], s[0]);
-                        s[1] = fmaf(uv[i], sv[j], s[1]);
-                        s[2] = fmaf(uv[i], cv[j], s[2]);
-                        s[3] = fmaf(qv[i], sv[j], s[3]);
+                        s[0] = __ffma2_rn(qv[i], c2, s[0]);
+                        s[1] = __ffma2_rn(uv[i], s2, s[1]);
+                        s[2] = __ffma2_rn(uv[i], c2, s[2]);
+                        s[3] = __ffma2_rn(qv[i], s2, s[3]);
                     } else {
-                        s[0] = fmaf(qv[i], cv[j], s[0]);
-                        s[0] = fmaf(uv[i], sv[j], s[0]);
-                        s[1] = fmaf(uv[i], cv[j], s[1]);
-                        s[1] = fmaf(-qv[i], sv[j], s[1]);
+                        s[0] = __ffma2_rn(qv[i], c2, s[0]);
+                        s[0] = __ffma2_rn(uv[i], s2, s[0]);
+                        s[1] = __ffma2_rn(uv[i], c2, s[1]);
+                        s[1] = __ffma2_rn(qv[i], n2, s[1]);
                     }
                 }
+            }
         }
         // stage n & 1 was last read before the previous trailing barrier
         if (FLY && n < pp.total) fly_store<FOLD>(stage[n & 1], fo, tid);
@@ -276,7 +284,9 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_
         for (int j = 0; j < NJ; ++j) {
             const int col = p0 + 16 * (j >> 1) + 2 * tx + (j & 1);
             if (col >= a.ncol) continue;
-            const float(&s)[NS] = acc[i][j];
+            float s[NS];
+#pragma unroll
+            for (int x = 0; x < NS; ++x) s[x] = i & 1 ? acc[i >> 1][j][x].y : acc[i >> 1][j][x].x;
             const int k = a.kplus + col;
             const float fr = (FOLD ? s[0] + s[1] : s[0]) * a.scale;
             const float fi = (FOLD ? s[2] - s[NS - 1] : s[1]) * a.scale;
