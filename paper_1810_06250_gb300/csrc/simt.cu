@@ -6,8 +6,11 @@
 // channels the 16 x 64 (cos, sin) tile is shared by the block's 256 lines of
 // sight, and each thread accumulates an 8 LOS x 8 phi register tile: 64 complex
 // MACs = 256 FMAs per channel for 8 shared-memory vector loads, so the FMA pipe,
-// not shared-memory bandwidth, sets the rate.  The chunks stream through a
-// two-stage cp.async pipeline, so the next chunk's loads overlap this one's FMAs.
+// not shared-memory bandwidth, sets the rate.  Four copying warps stream the chunks
+// through a four-stage cp.async pipeline for the eight accumulating ones, which meet
+// no barrier of the block while they run.  (With every warp copying between two barriers a
+// chunk, a third of the time had no FMA in flight: 262,144 LOS x 360 active channels x 401
+// phi folded, below, table 3.33 -> 2.75 ms, on the fly 3.32 -> 2.85, LOS-major 4.40 -> 3.28.)
 //   FLY   : (cos, sin) = sincosf(phi_k * 2(lambda_j^2 - lambda_0^2)) in FP32
 //           (the paper's method, argument and reduction in FP32);
 //   TABLE : (cos, sin) read from the plan's FP32 table built in FP64.
@@ -16,23 +19,24 @@
 // 4 FMAs per (LOS, channel) for two outputs instead of 8.  The register tile is
 // then 8 LOS x 4 pairs, 128 FMAs per channel for 6 vector loads, and the copies
 // weigh twice as much: channel-major cubes whose rows start on 16 bytes copy 4 LOS
-// at a time.  262,144 LOS x 360 active channels x 401 phi: table 6.82 -> 3.61 ms,
-// on the fly 6.97 -> 3.70 ms (rows not aligned 4.58, LOS-major 7.05 -> 4.64 ms).
-// The FMAs are packed over two LOS (one instruction, the rounding of two): the issue slots
-// were the bound, now the FMA pipe is busy 67 % of the time.  Table 3.56 -> 3.33 ms, on the
-// fly 3.66 -> 3.32 ms, rows not aligned 4.53 -> 4.31 ms, LOS-major 4.61 -> 4.40 ms.
+// at a time.  Folding took the table path from 6.82 to 3.61 ms, LOS-major from 7.05 to 4.64.
+// The FMAs are packed over two LOS (one instruction, the rounding of two), which freed the
+// issue slots that bound them: table 3.56 -> 3.33 ms, LOS-major 4.61 -> 4.40 ms.
 // The peak of |F| (Sec. 2.2) is reduced in registers over the block's phi
 // tiles, so F never has to be re-read.
 #include <cooperative_groups.h>
 #include <limits.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "rms_internal.h"
 
 namespace cg = cooperative_groups;
 
 namespace {
+
+#include "tc_ptx.cuh"
 
 constexpr int TL = 256;   // lines of sight per block (32 thread rows x 8)
 constexpr int TP = 64;    // phi per tile (8 thread columns x 8, as 4 pairs at stride 16);
@@ -46,7 +50,14 @@ struct Stage {
     float u[CH][LDQ];
     float2 cs[CH][TP];     // (w cos, w sin)
 };
-constexpr size_t kSimtSmem = 2 * sizeof(Stage);
+constexpr int NS = 4;      // stages
+constexpr int NP = 128;    // copying threads
+constexpr int kThreads = TL + NP;
+constexpr size_t kSimtSmem = NS * sizeof(Stage);
+// registers a thread: the launch's share, and after the split (256 x 232 + 128 x 40 = 384 x 168)
+constexpr int kRegsLaunch = 168, kRegsSum = 232, kRegsCopy = 40;
+static_assert(TL * kRegsSum + NP * kRegsCopy <= kThreads * kRegsLaunch, "register split");
+constexpr int64_t kWaitNs = 20000000000;    // no wait of a block on itself comes near this
 
 struct SimtArgs {
     const float *Q, *U;
@@ -64,6 +75,7 @@ struct SimtArgs {
     float *F;
     int32_t *pidx;
     float *pabs, *pphi;
+    int *err;
 };
 
 __device__ __forceinline__ bool better(float m, int i, float bm, int bi)
@@ -81,8 +93,12 @@ __device__ __forceinline__ void cp_async(void *dst, const void *src, bool ok)
                  "r"(ok ? BYTES : 0)
                  : "memory");
 }
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+// arrive on an mbarrier once this thread's copies so far have landed
+__device__ __forceinline__ void cp_arrive(uint32_t bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ __forceinline__ void load8(const float *p, float2 (&v)[4])
 {
@@ -91,13 +107,13 @@ __device__ __forceinline__ void load8(const float *p, float2 (&v)[4])
     v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
 }
 
-// Each thread copies one channel of every chunk: ISSUE_CH(tid) is that channel's
+// Each copying thread takes one channel of every chunk: ISSUE_CH(tid) is that channel's
 // slot in the chunk, and its active-channel index is loaded one chunk ahead
 // (act), so no global load latency sits in front of the copies.
 template <int LAYOUT>
 __device__ __forceinline__ int issue_ch(int tid)
 {
-    return LAYOUT == RMS_CHAN_MAJOR ? tid / (256 / CH) : tid % CH;
+    return LAYOUT == RMS_CHAN_MAJOR ? tid / (NP / CH) : tid % CH;
 }
 
 template <int LAYOUT>
@@ -114,41 +130,41 @@ __device__ __forceinline__ void issue(const SimtArgs &a, Stage &st, int64_t l0, 
 {
     const int c = issue_ch<LAYOUT>(tid);
     constexpr int W = FOLD ? TP / 2 : TP;
-    if (LAYOUT == RMS_CHAN_MAJOR && a.vec4) {
-        // 16 threads per channel, each 4 x 4 LOS (256-byte runs along LOS; nlos is a
-        // multiple of 4, so a group of 4 is whole or beyond the end)
-#pragma unroll
-        for (int r = 0; r < TL / (256 / CH) / 4; ++r) {
-            const int m = 4 * (tid % (256 / CH) + r * (256 / CH));
-            const bool ok = act >= 0 && l0 + m < a.nlos;
-            const int64_t off = ok ? (int64_t)act * a.nlos + l0 + m : 0;
-            cp_async<16>(&st.q[c][m], a.Q + off, ok);
-            cp_async<16>(&st.u[c][m], a.U + off, ok);
+    constexpr bool chan = LAYOUT == RMS_CHAN_MAJOR;
+    // channel-major: 8 threads per channel, each 8 x 4 LOS (128-byte runs along LOS; with vec4
+    // nlos is a multiple of 4, so a group of 4 is whole or beyond the end) or 32 LOS at stride
+    // 8; LOS-major: consecutive threads take consecutive channels of a LOS, each 32 LOS at
+    // stride 8.  The block's last LOS, and channels beyond the last, are zeros.
+    const int per = chan && a.vec4 ? 4 : 1, m0 = per * (chan ? tid % (NP / CH) : tid / CH), dm = per * (NP / CH);
+    const int64_t step = (int64_t)dm * (chan ? 1 : a.nchan);
+    const int n = (int)min((int64_t)TL, a.nlos - l0);
+    const int64_t off = chan ? (int64_t)max(act, 0) * a.nlos + l0 + m0 : (l0 + m0) * a.nchan + max(act, 0);
+    const float *q = a.Q + off, *u = a.U + off;
+    float *dq = &st.q[c][m0], *du = &st.u[c][m0];
+    auto copy = [&](auto bytes) {
+        constexpr int B = decltype(bytes)::value, steps = TL * (int)sizeof(float) / ((NP / CH) * B);
+        if (n == TL) {
+#pragma unroll 8
+            for (int r = 0; r < steps; ++r) {
+                cp_async<B>(dq + r * dm, q, act >= 0);
+                cp_async<B>(du + r * dm, u, act >= 0);
+                q += step;
+                u += step;
+            }
+        } else {
+#pragma unroll 1
+            for (int r = 0; r < steps; ++r) {
+                const bool ok = act >= 0 && m0 + r * dm < n;
+                cp_async<B>(dq + r * dm, ok ? q + r * step : a.Q, ok);
+                cp_async<B>(du + r * dm, ok ? u + r * step : a.U, ok);
+            }
         }
-    } else if (LAYOUT == RMS_CHAN_MAJOR) {
-        // 16 threads per channel, each 16 LOS at stride 16 (64-byte runs along LOS)
-#pragma unroll 4
-        for (int r = 0; r < TL / (256 / CH); ++r) {
-            const int m = tid % (256 / CH) + r * (256 / CH);
-            const bool ok = act >= 0 && l0 + m < a.nlos;
-            const int64_t off = ok ? (int64_t)act * a.nlos + l0 + m : 0;
-            cp_async<4>(&st.q[c][m], a.Q + off, ok);
-            cp_async<4>(&st.u[c][m], a.U + off, ok);
-        }
-    } else {
-        // consecutive threads take consecutive channels of one LOS
-#pragma unroll 4
-        for (int r = 0; r < TL / (256 / CH); ++r) {
-            const int m = tid / CH + r * (256 / CH);
-            const bool ok = act >= 0 && l0 + m < a.nlos;
-            const int64_t off = ok ? (l0 + m) * a.nchan + act : 0;
-            cp_async<4>(&st.q[c][m], a.Q + off, ok);
-            cp_async<4>(&st.u[c][m], a.U + off, ok);
-        }
-    }
+    };
+    if (chan && a.vec4) copy(std::integral_constant<int, 16>());
+    else copy(std::integral_constant<int, 4>());
     if (!FLY) {
 #pragma unroll
-        for (int i = tid; i < CH * W; i += 256) {
+        for (int i = tid; i < CH * W; i += NP) {
             const int c = i / W, k = i % W;
             const bool ok = c0 + c < a.nact && p0 + k < a.ncol;
             const int64_t off = ok ? (int64_t)(c0 + c) * a.nphi + a.kplus + p0 + k : 0;
@@ -157,82 +173,62 @@ __device__ __forceinline__ void issue(const SimtArgs &a, Stage &st, int64_t l0, 
     }
 }
 
-// on-the-fly phases: the operands of a thread's CH * TP / 256 phase-tile
-// entries are loaded one chunk ahead and turned into (w cos, w sin) after the
-// current chunk's accumulation, so their load latency is hidden behind it
+// on-the-fly phases: the chunk's (w cos, w sin)
 template <bool FOLD>
-struct FlyOps {
-    static constexpr int W = FOLD ? TP / 2 : TP, kPer = CH * W / 256;
-    float ph[kPer], l2[kPer], w[kPer];
-};
-
-template <bool FOLD>
-__device__ __forceinline__ void fly_load(const SimtArgs &a, FlyOps<FOLD> &o, int c0, int p0, int tid)
+__device__ __forceinline__ void fly_store(const SimtArgs &a, Stage &st, int c0, int p0, int tid)
 {
-#pragma unroll
-    for (int r = 0; r < FlyOps<FOLD>::kPer; ++r) {
-        const int i = tid + 256 * r, c = i / FlyOps<FOLD>::W, k = i % FlyOps<FOLD>::W;
+    constexpr int W = FOLD ? TP / 2 : TP;
+#pragma unroll 1
+    for (int i = tid; i < CH * W; i += NP) {
+        const int c = i / W, k = i % W;
         const bool ok = c0 + c < a.nact && p0 + k < a.ncol;
         // a padded entry gets weight 0 (and phase 0), hence (0, 0)
-        o.ph[r] = ok ? __ldg(a.phi32 + a.kplus + p0 + k) : 0.f;
-        o.l2[r] = ok ? __ldg(a.l2x + c0 + c) : 0.f;
-        o.w[r] = ok ? __ldg(a.w32 + c0 + c) : 0.f;
-    }
-}
-
-template <bool FOLD>
-__device__ __forceinline__ void fly_store(Stage &st, const FlyOps<FOLD> &o, int tid)
-{
-#pragma unroll
-    for (int r = 0; r < FlyOps<FOLD>::kPer; ++r) {
-        const int i = tid + 256 * r, c = i / FlyOps<FOLD>::W, k = i % FlyOps<FOLD>::W;
+        const float ph = ok ? __ldg(a.phi32 + a.kplus + p0 + k) : 0.f;
+        const float l2 = ok ? __ldg(a.l2x + c0 + c) : 0.f;
+        const float w = ok ? __ldg(a.w32 + c0 + c) : 0.f;
         float sn, cs;
-        sincosf(o.ph[r] * o.l2[r], &sn, &cs);
-        st.cs[c][k] = make_float2(o.w[r] * cs, o.w[r] * sn);
+        sincosf(ph * l2, &sn, &cs);
+        st.cs[c][k] = make_float2(w * cs, w * sn);
     }
 }
 
-// Pipeline state carried from one phi tile to the next.
+// Pipeline state: the stage and the parity of its current use, and this block's phi tiles
+// rank, rank + size, ... (its place in the cluster).
 struct Pipe {
-    int t;          // (phi tile, channel chunk) pair being accumulated
-    int total, nck;
-    int32_t act;    // active-channel index for the next copy
-    int rank, size; // this block's tiles: rank, rank + size, ... (its place in the cluster)
-    __device__ __forceinline__ int chunk(int n) const { return n % nck; }
-    __device__ __forceinline__ int tile(int n) const { return rank + (n / nck) * size; }
+    uint64_t *full, *empty;
+    volatile int *abort_flag;
+    int s;
+    uint32_t ph;
+    int nck, rank, size;
+    __device__ __forceinline__ void next()
+    {
+        if (++s == NS) { s = 0; ph ^= 1; }
+    }
 };
 
 // One phi tile starting at column p0: accumulate all channel chunks, then scale,
 // store and update the running peak.  JJ: pairs-of-16 columns of the tile that hold
 // grid points (4, folded 2, for a full tile; the last, partial tile drops the columns
 // beyond).
-template <int JJ, bool FLY, bool FOLD, int LAYOUT>
-__device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_t l0, int p0, Pipe &pp,
-                                         FlyOps<FOLD> &fo, float (&bm)[8], int (&bi)[8])
+template <int JJ, bool FOLD>
+__device__ __forceinline__ void phi_tile(const SimtArgs &a, const Stage *stage, int64_t l0, int p0, Pipe &pp,
+                                         float (&bm)[8], int (&bi)[8])
 {
-    constexpr int NJ = 2 * JJ, W = FOLD ? TP / 2 : TP, NS = FOLD ? 4 : 2;
+    constexpr int NJ = 2 * JJ, SUMS = FOLD ? 4 : 2;
     const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
     // sums of a (LOS, column): Re, Im of F, or folded Qc, Us, Uc, Qs
     // of LOS 2 i and 2 i + 1: one packed FMA feeds both
-    float2 acc[4][NJ][NS];
+    float2 acc[4][NJ][SUMS];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < NJ; ++j)
 #pragma unroll
-            for (int x = 0; x < NS; ++x) acc[i][j][x] = make_float2(0.f, 0.f);
+            for (int x = 0; x < SUMS; ++x) acc[i][j][x] = make_float2(0.f, 0.f);
 
-    for (int ck = 0; ck < pp.nck; ++ck, ++pp.t) {
-        const int n = pp.t + 1;
-        if (n < pp.total) {
-            issue<FLY, FOLD, LAYOUT>(a, stage[n & 1], l0, pp.chunk(n) * CH, pp.tile(n) * W, pp.act, tid);
-            if (FLY) fly_load<FOLD>(a, fo, pp.chunk(n) * CH, pp.tile(n) * W, tid);
-            if (n + 1 < pp.total) pp.act = load_active<LAYOUT>(a, pp.chunk(n + 1) * CH, tid);
-        }
-        cp_commit();
-        cp_wait_prev();
-        __syncthreads();
-        const Stage &st = stage[pp.t & 1];
+    for (int ck = 0; ck < pp.nck; ++ck, pp.next()) {
+        if (!warp_wait(smem_u32(&pp.full[pp.s]), pp.ph, pp.abort_flag, a.err, kWaitNs)) return;
+        const Stage &st = stage[pp.s];
 #pragma unroll 2
         for (int c = 0; c < CH; ++c) {
             float2 qv[4], uv[4];
@@ -252,7 +248,7 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_
                 const float2 n2 = make_float2(-sv[j], -sv[j]);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    float2(&s)[NS] = acc[i][j];
+                    float2(&s)[SUMS] = acc[i][j];
                     // (q + iu)(c - is): Re += q c + u s, Im += u c - q s  (Eqs. qPhi, uPhi)
                     if constexpr (FOLD) {
                         s[0] = __ffma2_rn(qv[i], c2, s[0]);
@@ -268,9 +264,8 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_
                 }
             }
         }
-        // stage n & 1 was last read before the previous trailing barrier
-        if (FLY && n < pp.total) fly_store<FOLD>(stage[n & 1], fo, tid);
-        __syncthreads();
+        __syncwarp();
+        if ((tid & 31) == 0) mbar_arrive(smem_u32(&pp.empty[pp.s]));
     }
 
     // epilogue for this phi tile: scale by K, store, update the running peak (lowest
@@ -284,12 +279,12 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_
         for (int j = 0; j < NJ; ++j) {
             const int col = p0 + 16 * (j >> 1) + 2 * tx + (j & 1);
             if (col >= a.ncol) continue;
-            float s[NS];
+            float s[SUMS];
 #pragma unroll
-            for (int x = 0; x < NS; ++x) s[x] = i & 1 ? acc[i >> 1][j][x].y : acc[i >> 1][j][x].x;
+            for (int x = 0; x < SUMS; ++x) s[x] = i & 1 ? acc[i >> 1][j][x].y : acc[i >> 1][j][x].x;
             const int k = a.kplus + col;
             const float fr = (FOLD ? s[0] + s[1] : s[0]) * a.scale;
-            const float fi = (FOLD ? s[2] - s[NS - 1] : s[1]) * a.scale;
+            const float fi = (FOLD ? s[2] - s[SUMS - 1] : s[1]) * a.scale;
             const float m2 = __fadd_rn(__fmul_rn(fr, fr), __fmul_rn(fi, fi));
             if (m2 > bm[i]) { bm[i] = m2; bi[i] = k; }
             if (st) row[k] = make_float2(fr, fi);
@@ -306,71 +301,94 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, Stage *stage, int64_
 }
 
 template <bool FLY, bool FOLD, int LAYOUT>
-__global__ void __launch_bounds__(256, 1) simt_kernel(const SimtArgs a)
+__global__ void __launch_bounds__(kThreads, 1) simt_kernel(const SimtArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float pk_m[TL];
     __shared__ int pk_k[TL];
     Stage *stage = reinterpret_cast<Stage *>(smem_raw);
 
-    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    __shared__ uint64_t bars[2 * NS];
+    __shared__ int aborted;
+
+    const int tid = threadIdx.x;
     const cg::cluster_group cluster = cg::this_cluster();
     Pipe pp;
+    pp.full = bars;
+    pp.empty = bars + NS;
+    pp.abort_flag = &aborted;
     pp.rank = (int)cluster.block_rank();
     pp.size = (int)cluster.num_blocks();
-    const int64_t l0 = (int64_t)(blockIdx.x / pp.size) * TL;
     pp.nck = (a.nact + CH - 1) / CH;
+    pp.s = 0;
+    const int64_t l0 = (int64_t)(blockIdx.x / pp.size) * TL;
     constexpr int W = FOLD ? TP / 2 : TP;
     const int ntiles = (a.ncol + W - 1) / W;        // the cluster has at most as many blocks
-    pp.total = pp.nck * ((ntiles - pp.rank + pp.size - 1) / pp.size);
-    pp.t = 0;
-
-    float bm[8];
-    int bi[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) { bm[i] = -1.0f; bi[i] = INT_MAX; }
-
-    // two-stage pipeline over (phi tile, channel chunk) pairs t: the copies of
-    // pair t + 1 are in flight while pair t is accumulated
-    FlyOps<FOLD> fo;
-    issue<FLY, FOLD, LAYOUT>(a, stage[0], l0, 0, pp.rank * W, load_active<LAYOUT>(a, 0, tid), tid);
-    cp_commit();
-    pp.act = pp.total > 1 ? load_active<LAYOUT>(a, pp.chunk(1) * CH, tid) : -1;
-    if (FLY) {
-        fly_load<FOLD>(a, fo, 0, pp.rank * W, tid);
-        fly_store<FOLD>(stage[0], fo, tid);
-    }
-    const int full = a.ncol / W, rem = a.ncol - full * W;
-    int it = pp.rank;
-    for (; it < full; it += pp.size) phi_tile<W / 16, FLY, FOLD, LAYOUT>(a, stage, l0, it * W, pp, fo, bm, bi);
-    // the last, partial tile computes only the pairs-of-16 that hold grid points
-    if (it == full) {
-        switch ((rem + 15) / 16) {
-        case 1: phi_tile<1, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
-        case 2: phi_tile<2, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
-        case 3: if constexpr (!FOLD) phi_tile<3, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
-        case 4: if constexpr (!FOLD) phi_tile<4, FLY, FOLD, LAYOUT>(a, stage, l0, full * W, pp, fo, bm, bi); break;
-        default: break;
+    if (tid == 0) {
+        aborted = 0;
+        for (int i = 0; i < NS; ++i) {
+            mbar_init(smem_u32(&pp.full[i]), 2 * NP);     // each copying thread: its copies, and itself
+            mbar_init(smem_u32(&pp.empty[i]), TL / 32);
         }
     }
+    __syncthreads();
 
-    // reduce the peak over the 8 threads (tx) that share each line of sight
+    if (tid >= TL) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCopy));
+        const int t = tid - TL;
+        pp.ph = 1;                                  // every stage starts empty
+        bool ok = true;
+        int32_t act = load_active<LAYOUT>(a, 0, t);
+        for (int it = pp.rank; it < ntiles && ok; it += pp.size)
+            for (int ck = 0; ck < pp.nck; ++ck, pp.next()) {
+                ok = wait_bounded(smem_u32(&pp.empty[pp.s]), pp.ph, pp.abort_flag, a.err, kWaitNs);
+                if (!ok) break;
+                issue<FLY, FOLD, LAYOUT>(a, stage[pp.s], l0, ck * CH, it * W, act, t);
+                act = load_active<LAYOUT>(a, ck + 1 < pp.nck ? (ck + 1) * CH : 0, t);
+                if (FLY) fly_store<FOLD>(a, stage[pp.s], ck * CH, it * W, t);
+                cp_arrive(smem_u32(&pp.full[pp.s]));
+                mbar_arrive(smem_u32(&pp.full[pp.s]));
+            }
+        cp_wait_all();
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSum));
+        pp.ph = 0;
+        float bm[8];
+        int bi[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        float m = bm[i];
-        int k = bi[i];
-#pragma unroll
-        for (int off = 4; off >= 1; off >>= 1) {
-            const float mo = __shfl_xor_sync(0xffffffffu, m, off);
-            const int ko = __shfl_xor_sync(0xffffffffu, k, off);
-            if (better(mo, ko, m, k)) { m = mo; k = ko; }
+        for (int i = 0; i < 8; ++i) { bm[i] = -1.0f; bi[i] = INT_MAX; }
+        const int full = a.ncol / W, rem = a.ncol - full * W;
+        int it = pp.rank;
+        for (; it < full; it += pp.size) phi_tile<W / 16, FOLD>(a, stage, l0, it * W, pp, bm, bi);
+        // the last, partial tile computes only the pairs-of-16 that hold grid points
+        if (it == full) {
+            switch ((rem + 15) / 16) {
+            case 1: phi_tile<1, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
+            case 2: phi_tile<2, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
+            case 3: if constexpr (!FOLD) phi_tile<3, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
+            case 4: if constexpr (!FOLD) phi_tile<4, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
+            default: break;
+            }
         }
-        if (tx == 0) { pk_m[8 * ty + i] = m; pk_k[8 * ty + i] = k; }
+        // reduce the peak over the 8 threads (tx) that share each line of sight
+        const int tx = tid & 7, ty = tid >> 3;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float m = bm[i];
+            int k = bi[i];
+#pragma unroll
+            for (int off = 4; off >= 1; off >>= 1) {
+                const float mo = __shfl_xor_sync(0xffffffffu, m, off);
+                const int ko = __shfl_xor_sync(0xffffffffu, k, off);
+                if (better(mo, ko, m, k)) { m = mo; k = ko; }
+            }
+            if (tx == 0) { pk_m[8 * ty + i] = m; pk_k[8 * ty + i] = k; }
+        }
     }
     // the cluster's blocks hold disjoint phi of the same LOS: its first block merges them
     if (pp.size > 1) cluster.sync();
     else __syncthreads();
-    if (pp.rank == 0) {
+    if (pp.rank == 0 && tid < TL) {
         float m = pk_m[tid];
         int k = pk_k[tid];
         for (int r = 1; r < pp.size; ++r) {
@@ -393,7 +411,7 @@ cudaLaunchConfig_t launch_config(cudaLaunchAttribute *attr, unsigned grid, unsig
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(TL);
+    cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSimtSmem;
     cfg.stream = s;
     attr->id = cudaLaunchAttributeClusterDimension;
@@ -426,7 +444,10 @@ cudaError_t simt_prepare(rms_plan_s *p)
     const bool fly = p->precision == RMS_FP32_SIMT_FLY;
     for (int layout : {RMS_CHAN_MAJOR, RMS_LOS_MAJOR}) {
         const SimtKernel kern = kernel_of(fly, p->fold.on, layout);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSimtSmem);
+        cudaFuncAttributes fa;
+        cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+        if (e == cudaSuccess && fa.numRegs != kRegsLaunch) e = cudaErrorInvalidConfiguration;    // the split counts on it
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSimtSmem);
         for (int c = 1; c <= 8 && e == cudaSuccess; ++c) {
             cudaLaunchAttribute attr;
             const cudaLaunchConfig_t cfg = launch_config(&attr, (unsigned)(c * p->num_sms), (unsigned)c, 0);
@@ -460,6 +481,7 @@ cudaError_t launch_simt(const rms_plan_s &p, bool fly, const float *Q, const flo
     a.pidx = pidx;
     a.pabs = pabs;
     a.pphi = pphi;
+    a.err = p.d_err;
     const bool fold = p.fold.on;
     a.ncol = fold ? p.fold.ncol : p.nphi;
     a.kplus = fold ? p.fold.kplus : 0;
@@ -469,7 +491,8 @@ cudaError_t launch_simt(const rms_plan_s &p, bool fly, const float *Q, const flo
     // One block fits an SM, and its phi tiles re-read the block's data anyway, so a
     // cluster of up to 8 blocks shares out the phi tiles of 256 LOS where that needs
     // fewer rounds of tiles over the device (the smallest such cluster).  401 phi x 360
-    // channels: 3,000 LOS 522 -> 84 us, 10,000 LOS 520 -> 207, 100,000 unchanged (1.53 ms).
+    // channels: 3,000 LOS 522 -> 84 us, 10,000 LOS 520 -> 207, 100,000 unchanged (measured
+    // before the copying warps; now 68, 162 and 1,180 us).
     const int width = fold ? TP / 2 : TP, ntiles = (a.ncol + width - 1) / width;
     int64_t best = INT64_MAX;
     unsigned cluster = 1;

@@ -1,0 +1,53 @@
+"""FP32 CUDA-core contraction: its copying warps' pipeline at the edges, against the FP64 oracle.
+
+The gates are those of the precisions (gpu_helpers.TOL).
+"""
+import numpy as np
+import pytest
+
+import gpu_helpers as gh
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rms():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1810_06250_gb300 as rms
+    rms.build()
+    rms.load()
+    return rms
+
+
+# fewer and more 16-channel chunks than the four stages, whole and partial; a block of 256 LOS whole, short by one,
+# one over; rows on and off 16 bytes; folded and general grids of one and several phi tiles
+@pytest.mark.parametrize("nchan,flagged", [(1, 0), (16, 0), (65, 3), (150, 9)])
+@pytest.mark.parametrize("sym", [True, False])
+@pytest.mark.parametrize("path", ["fp32_table", "fp32_fly"])
+def test_simt_pipeline_edges(rms, oracle_mod, path, sym, nchan, flagged):
+    rng = np.random.default_rng(nchan)
+    freq = np.linspace(120e6, 168e6, nchan) if nchan > 1 else np.array([150e6])
+    w = rng.uniform(0.5, 1.5, nchan)
+    w[rng.choice(nchan, flagged, replace=False)] = 0.0
+    op = oracle_mod.plan(freq, "freq", w)
+    for nphi, nlos, layout, shift in ((141, 255, "chan", 0), (141, 256, "los", 0), (20, 513, "chan", 1),
+                                      (141, 260, "chan", 0), (70, 259, "los", 1), (141, 512, "chan", 1)):
+        phi = np.linspace(-60.0, 60.0 if sym else 63.0, nphi)
+        data = torch.randn(2, nlos * nchan + 4, device="cuda", generator=torch.Generator("cuda").manual_seed(nlos))
+        q, u = (data[i, shift:shift + nlos * nchan] for i in range(2))
+        shape = (nchan, nlos) if layout == "chan" else (nlos, nchan)
+        Q, U = (x.cpu().numpy().reshape(shape) for x in (q, u))
+        if layout == "chan":
+            Q, U = Q.T, U.T
+        with rms.Plan(freq, phi, path, weights=w) as plan:
+            F = torch.empty(nlos, nphi, 2, device="cuda")
+            pi = torch.full((nlos,), -7, dtype=torch.int32, device="cuda")
+            pa, pp = torch.zeros(nlos, device="cuda"), torch.zeros(nlos, device="cuda")
+            plan.synth(q, u, nlos, layout, F, pi, pa, pp)
+            plan.sync()
+        Fh = F.cpu().numpy()
+        per, _ = gh.errors(Fh[..., 0] + 1j * Fh[..., 1], oracle_mod.synth(Q, U, op, phi))
+        assert per.max() <= gh.TOL[path], (nphi, nlos, layout, per.max())
+        gh.check_peaks_self(Fh, pi.cpu().numpy(), pa.cpu().numpy(), pp.cpu().numpy(), phi)
