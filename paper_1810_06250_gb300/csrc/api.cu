@@ -542,9 +542,9 @@ static rms_status synth_launch(rms_plan_t p, const float *Q, const float *U, int
     case RMS_FP16X3: {
         // the split operand (and FP16X3's per-LOS exponents): stream-ordered scratch
         // and 8 bytes of peak key per LOS (the contraction's split schedule)
-        const bool fused = fused_wanted(*p, Q, U, nlos, layout);
+        const bool fused = fused_wanted(*p, nlos);
         const size_t abytes = fused ? fused_ring_bytes(*p, nlos) : p->fold.on ? fold_operand_bytes(*p, nlos) : split_operand_bytes(*p, nlos, layout);
-        const size_t rbytes = p->precision == RMS_FP16X3 && !fused ? (size_t)((nlos + 255) & ~(int64_t)255) : 0;
+        const size_t rbytes = p->precision == RMS_FP16X3 ? (size_t)((nlos + 255) & ~(int64_t)255) : 0;
         const size_t kbytes = fused ? 0 : (size_t)((nlos * 8 + 255) & ~(int64_t)255);
         uint8_t *scr = nullptr;
         e = cudaMallocAsync(reinterpret_cast<void **>(&scr), abytes + rbytes + kbytes, s);
@@ -566,8 +566,12 @@ static rms_status synth_launch(rms_plan_t p, const float *Q, const float *U, int
             cudaGetLastError();
         }
         if (fused) {
-            if (ev[1]) cudaEventRecord(ev[1], s);       // no layout stage of its own
-            e = launch_fused(*p, Q, U, nlos, layout, F, pidx, pabs, pphi, x.q, x.u, x.chi, scr, s);
+            // no layout stage of its own but FP16X3's exponents
+            int8_t *rexp = rbytes ? reinterpret_cast<int8_t *>(scr + abytes) : nullptr;
+            if (rexp) e = launch_fold_exponents(*p, Q, U, nlos, layout, rexp, s);
+            if (ev[1]) cudaEventRecord(ev[1], s);
+            if (e == cudaSuccess)
+                e = launch_fused(*p, Q, U, nlos, layout, F, pidx, pabs, pphi, x.q, x.u, x.chi, scr, rexp, s);
         } else {
             e = launch_split_gemm(*p, Q, U, nlos, layout, F, pidx, pabs, pphi, scr,
                               rbytes ? reinterpret_cast<int8_t *>(scr + abytes) : nullptr, s, ev[1], x.q, x.u, x.chi,

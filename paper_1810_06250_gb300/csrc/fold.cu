@@ -47,8 +47,87 @@ struct FoldSplitParams {
     int32_t kblocks;
     int32_t kpg;                // K blocks per CTA: blockIdx.y covers K blocks [y kpg, (y + 1) kpg)
     uint8_t *A;                 // [ceil(nlos / 128) 2][kblocks][16 KB]
-    int8_t *rexp;               // [nlos] (FP16X3): the LOS's exponent
+    const int8_t *rexp;         // [nlos] (FP16X3): the LOS's exponent
 };
+
+// FP16X3: the exponent of every LOS's scale, from its largest active |value|, in a pass of its
+// own at copy bandwidth, so that what follows (the split, or the one-kernel form) can take a
+// LOS's channels in any order and by any number of CTAs.  It took the place of passes inside
+// the split (one thread walked a LOS's channels twice) and inside the one-kernel form (whose
+// warps waited for each other's maxima, LOS-major only).  Whole call, channel-major:
+// 262,144 LOS x 360 x 401 0.808 -> 0.597 ms, 60,000 x 1350 x 301 0.804 -> 0.544, 8,506 x 416 x
+// 497 121 -> 56 us, 3,000 x 360 x 401 96 -> 43 us; LOS-major 0.631 -> 0.610, 0.623 -> 0.555 ms,
+// 54 -> 54, 48 -> 45 us.
+// Channel-major: 128 LOS per CTA, four per lane, the channels dealt out to 16 warps; VEC:
+// rows start on 16 bytes.  0.127 ms for the first cube: 5.9 TB/s.
+constexpr int kExpWarps = 16, kExpBatch = 8;
+template <bool VEC>
+__global__ void __launch_bounds__(32 * kExpWarps) fold_exp_chan_kernel(const FoldSource S, int8_t *rexp)
+{
+    __shared__ float part[kExpWarps][kLosPerCta];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t los0 = (int64_t)blockIdx.x * kLosPerCta;
+    auto at = [&](int k) { return min(los0 + lane + 32 * k, S.nlos - 1); };          // beyond the end: any LOS
+    const int64_t at4 = min(los0 + 4 * lane, S.nlos - 4);
+    float mx[4] = {0.f, 0.f, 0.f, 0.f};
+    // the warp's channels warp, warp + 16, ..: their numbers first, one per lane, so that all of a
+    // batch's loads are in flight at once (a number beyond the last is the last channel's again)
+    for (int a0 = warp; a0 < S.nact; a0 += 32 * kExpWarps) {
+        const int mine = __ldg(S.active + min(a0 + kExpWarps * lane, S.nact - 1));
+        const int nj = min(32, (S.nact - a0 + kExpWarps - 1) / kExpWarps);
+        for (int j0 = 0; j0 < nj; j0 += kExpBatch) {
+            float q[kExpBatch][4], u[kExpBatch][4];
+#pragma unroll
+            for (int j = 0; j < kExpBatch; ++j) {
+                const int64_t row = (int64_t)__shfl_sync(0xffffffffu, mine, j0 + j) * S.nlos;
+                if (VEC) {
+                    const float4 x = __ldg(reinterpret_cast<const float4 *>(S.Q + row + at4));
+                    const float4 y = __ldg(reinterpret_cast<const float4 *>(S.U + row + at4));
+                    q[j][0] = x.x; q[j][1] = x.y; q[j][2] = x.z; q[j][3] = x.w;
+                    u[j][0] = y.x; u[j][1] = y.y; u[j][2] = y.z; u[j][3] = y.w;
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        q[j][k] = __ldg(S.Q + row + at(k));
+                        u[j][k] = __ldg(S.U + row + at(k));
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < kExpBatch; ++j)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) mx[k] = fmaxf(mx[k], fmaxf(fabsf(q[j][k]), fabsf(u[j][k])));
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) part[warp][VEC ? 4 * lane + k : lane + 32 * k] = mx[k];
+    __syncthreads();
+    const int64_t los = los0 + threadIdx.x;
+    if (threadIdx.x < kLosPerCta && los < S.nlos) {
+        float m = part[0][threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < kExpWarps; ++w) m = fmaxf(m, part[w][threadIdx.x]);
+        rexp[los] = (int8_t)fold_exponent(m);
+    }
+}
+
+// LOS-major: a warp per LOS (the list's padding repeats an active channel).
+__global__ void __launch_bounds__(256) fold_exp_los_kernel(const FoldSource S, int32_t kblocks, int8_t *rexp)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t los = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (los >= S.nlos) return;
+    const float *q = S.Q + los * S.nchan, *u = S.U + los * S.nchan;
+    float mx = 0.f;
+#pragma unroll 4
+    for (int kb = 0; kb < kblocks; ++kb) {
+        const int c = __ldg(S.padded + kb * kKBlock + lane);
+        mx = fmaxf(mx, fmaxf(fabsf(__ldg(q + c)), fabsf(__ldg(u + c))));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) rexp[los] = (int8_t)fold_exponent(mx);
+}
 
 // Channel-major cubes: one thread per LOS, 128 LOS (two tiles) per CTA; a warp
 // reads 128 contiguous bytes of a channel row.
@@ -76,19 +155,7 @@ __global__ void __launch_bounds__(kLosPerCta) fold_split_chan_kernel(const FoldS
             }
         }
     };
-    float scale = 1.0f;
-    if (MODE == MODE_FP16X3) {
-        float mx = 0.f;
-        for (int c0 = 0; c0 < P.src.nact; c0 += 16) {
-            float q[16], u[16];
-            load(c0, q, u);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) mx = fmaxf(mx, fmaxf(fabsf(q[j]), fabsf(u[j])));
-        }
-        const int e = fold_exponent(mx);
-        scale = ldexpf(1.0f, e);
-        if (valid) P.rexp[los] = (int8_t)e;
-    }
+    const float scale = MODE == MODE_FP16X3 ? ldexpf(1.0f, __ldg(P.rexp + min(los, n - 1))) : 1.0f;
     for (int h = 2 * kb0; h < 2 * kb1; ++h) {
         float q[16], u[16];
         load(16 * h, q, u);
@@ -100,7 +167,7 @@ __global__ void __launch_bounds__(kLosPerCta) fold_split_chan_kernel(const FoldS
 
 // LOS-major cubes: one tile of 64 LOS per CTA, 8 LOS per warp.
 template <int MODE>
-__global__ void __launch_bounds__(256, MODE == MODE_FP16X3 ? 3 : 4) fold_split_los_kernel(const FoldSplitParams P)
+__global__ void __launch_bounds__(256, 4) fold_split_los_kernel(const FoldSplitParams P)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t n = P.count ? min(*P.count, P.src.nlos) : P.src.nlos;
@@ -113,13 +180,10 @@ __global__ void __launch_bounds__(256, MODE == MODE_FP16X3 ? 3 : 4) fold_split_l
         return P.rows ? __ldg(P.rows + los) : los;
     };
     const uint32_t dead = los0 + 8 <= n ? 0u : (0xffu << max(0, (int)(n - los0))) & 0xffu;
-    float scale[8];
+    float scale[4];
     if constexpr (MODE == MODE_FP16X3) {
-        int ex[8];
-        fold_scales_los(P.src, P.src.padded, P.kblocks, lane, src_of, dead, scale, ex);
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
-            if (lane == r && los0 + r < n) P.rexp[los0 + r] = (int8_t)ex[r];
+        for (int j = 0; j < 4; ++j) scale[j] = ldexpf(1.0f, __ldg(P.rexp + min(los0 + 2 * j + (lane >> 4), n - 1)));
     }
     for (int kb = kb0; kb < kb1; ++kb) {
         float q[8], u[8];
@@ -132,6 +196,21 @@ __global__ void __launch_bounds__(256, MODE == MODE_FP16X3 ? 3 : 4) fold_split_l
 
 }  // namespace
 
+cudaError_t launch_fold_exponents(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout,
+                                  int8_t *rexp, cudaStream_t s)
+{
+    const bool chan = layout == RMS_CHAN_MAJOR;
+    const FoldSource src = {Q, U, nlos, p.nchan, p.nact, chan, p.d_active, p.fold.d_list};
+    const int64_t nb = chan ? (nlos + kLosPerCta - 1) / kLosPerCta : (nlos + 7) / 8;
+    if (nb < 1) return cudaSuccess;
+    if (nb > 0x7fffffff) return cudaErrorInvalidValue;
+    const bool vec = nlos % 4 == 0 && !((reinterpret_cast<uintptr_t>(Q) | reinterpret_cast<uintptr_t>(U)) & 15);
+    if (!chan) fold_exp_los_kernel<<<(unsigned)nb, 256, 0, s>>>(src, p.fold.kblocks, rexp);
+    else if (vec) fold_exp_chan_kernel<true><<<(unsigned)nb, 32 * kExpWarps, 0, s>>>(src, rexp);
+    else fold_exp_chan_kernel<false><<<(unsigned)nb, 32 * kExpWarps, 0, s>>>(src, rexp);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_fold_split(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout,
                               uint8_t *A, int8_t *rexp, cudaStream_t s, const int64_t *rows, const int64_t *count)
 {
@@ -142,7 +221,11 @@ cudaError_t launch_fold_split(const rms_plan_s &p, const float *Q, const float *
     const int64_t nb = chan ? pairs : 2 * pairs;
     if (nb < 1) return cudaSuccess;
     if (nb > 0x7fffffff) return cudaErrorInvalidValue;
-    if (mode == MODE_FP16X3 && !rexp) return cudaErrorInvalidValue;
+    if (mode == MODE_FP16X3) {
+        if (!rexp || rows || count) return cudaErrorInvalidValue;      // (only BF16 plans gather)
+        const cudaError_t e = launch_fold_exponents(p, Q, U, nlos, layout, rexp, s);
+        if (e != cudaSuccess) return e;
+    }
     FoldSplitParams P;
     P.src = {Q, U, nlos, p.nchan, p.nact, chan, p.d_active, p.fold.d_list};
     P.rows = rows;
@@ -151,12 +234,9 @@ cudaError_t launch_fold_split(const rms_plan_s &p, const float *Q, const float *
     P.A = A;
     P.rexp = rexp;
     // K blocks of a tile are shared out over blockIdx.y until the grid is about 8 waves
-    // (8-9 CTAs of 128 threads per SM, 4 of 256); FP16X3 needs a LOS's whole row
-    int64_t groups = 1;
-    if (mode != MODE_FP16X3) {
-        const int64_t target = (int64_t)8 * (chan ? 9 : 4) * p.num_sms;
-        groups = std::min<int64_t>(P.kblocks, std::max<int64_t>(1, (target + nb - 1) / nb));
-    }
+    // (8-9 CTAs of 128 threads per SM, 4 of 256)
+    const int64_t target = (int64_t)8 * (chan ? 9 : 4) * p.num_sms;
+    const int64_t groups = std::min<int64_t>(P.kblocks, std::max<int64_t>(1, (target + nb - 1) / nb));
     P.kpg = (int32_t)((P.kblocks + groups - 1) / groups);
     const dim3 grid((unsigned)nb, (unsigned)((P.kblocks + P.kpg - 1) / P.kpg));
     if (chan) {

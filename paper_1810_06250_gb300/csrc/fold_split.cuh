@@ -119,35 +119,11 @@ __device__ __forceinline__ void fold_mask_los(const FoldSource &S, int kb, int l
     }
 }
 
-// The scales (and exponents) of 8 LOS, in every lane: a first pass over their rows.
-template <typename F>
-__device__ __forceinline__ void fold_scales_los(const FoldSource &S, const int *list, int kblocks, int lane, F src_of,
-                                                uint32_t dead, float (&scale)[8], int (&ex)[8])
-{
-    float mx[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int kb = 0; kb < kblocks; ++kb) {
-        float q[8], u[8];
-        fold_load_los<false>(S, list, kb, lane, src_of, q, u);
-        fold_mask_los(S, kb, lane, dead, q, u);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) mx[e >> 1] = fmaxf(mx[e >> 1], fmaxf(fabsf(q[e]), fabsf(u[e])));
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) mx[j] = fmaxf(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], o));
-        const float other = __shfl_xor_sync(0xffffffffu, mx[j], 16);
-        ex[2 * j] = fold_exponent(lane < 16 ? mx[j] : other);
-        ex[2 * j + 1] = fold_exponent(lane < 16 ? other : mx[j]);
-        scale[2 * j] = ldexpf(1.0f, ex[2 * j]);
-        scale[2 * j + 1] = ldexpf(1.0f, ex[2 * j + 1]);
-    }
-}
-
 // One K block of LOS r0 .. r0 + N - 1 (r0 even) of a group of 8, Q or U; rows: the group's
-// first operand row in K block kb of the image.
+// first operand row in K block kb of the image; scale[j]: that of LOS r0 + 2 j + half.
 template <int MODE, bool RING, int N>
-__device__ __forceinline__ void fold_emit_rows(uint8_t *rows, int lane, int r0, const float (&v)[N], const float (&scale)[8])
+__device__ __forceinline__ void fold_emit_rows(uint8_t *rows, int lane, int r0, const float (&v)[N],
+                                               const float (&scale)[N / 2])
 {
     const int p = lane & 15, half = lane >> 4;
 #pragma unroll
@@ -155,8 +131,7 @@ __device__ __forceinline__ void fold_emit_rows(uint8_t *rows, int lane, int r0, 
         const int r = r0 + 2 * j + half;
         uint32_t hi, lo;
         if (MODE == MODE_FP16X3) {
-            const float s = half ? scale[2 * j + 1] : scale[2 * j];
-            split_pair_fp16(v[2 * j] * s, v[2 * j + 1] * s, hi, lo);
+            split_pair_fp16(v[2 * j] * scale[j], v[2 * j + 1] * scale[j], hi, lo);
         } else {
             split_pair_bf16(v[2 * j], v[2 * j + 1], hi, lo);
         }

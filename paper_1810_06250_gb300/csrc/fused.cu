@@ -64,6 +64,7 @@ struct FusedParams {
     const double *phi64;
     double lambda0sq;
     float out_scale;
+    const int8_t *rexp;         // FP16X3: [nlos] exponents
     int *err;
     int64_t timeout_ns;
     int32_t stages, kbs;        // pipeline stages of kbs K blocks each
@@ -83,15 +84,12 @@ struct FSmem {
     uint32_t stage_bytes, sub_bytes;
     float *pk_m, *pk_re, *pk_im;
     int *pk_i;
-    float *los_max;             // [2][8 warps][32] (FP16X3): partial maxima of the splitters' LOS
     int *list;                  // [kblocks x 32]: the padded channel list (an index load from L2 before
                                 // every batch of data loads would double their latency)
-    int *los_exp;               // [4][64] (FP16X3): exponents of an item's LOS
-    uint64_t *full, *empty, *tfull, *tempty, *ready, *afree, *xmax, *sfull, *sempty, *pkfull, *pkempty, *mma_done;
+    uint64_t *full, *empty, *tfull, *tempty, *ready, *afree, *sfull, *sempty, *pkfull, *pkempty, *mma_done;
     uint32_t *tmem_slot;
     volatile int *abort_flag;
 };
-constexpr int kExpSlots = 4;    // exponents outlive their ring slot until the epilogue has used them
 
 __device__ __forceinline__ FSmem fcarve(uint8_t *base, const FusedParams &P)
 {
@@ -104,9 +102,7 @@ __device__ __forceinline__ FSmem fcarve(uint8_t *base, const FusedParams &P)
     s.pk_i = reinterpret_cast<int *>(s.pk_m + 2 * 64);
     s.pk_re = reinterpret_cast<float *>(s.pk_i + 2 * 64);
     s.pk_im = s.pk_re + 2 * 64;
-    s.los_max = s.pk_im + 2 * 64;
-    s.los_exp = reinterpret_cast<int *>(s.los_max + 2 * kNumSplitWarps * 32);
-    s.list = s.los_exp + kExpSlots * 64;
+    s.list = reinterpret_cast<int *>(s.pk_im + 2 * 64);
     uint64_t *b = reinterpret_cast<uint64_t *>(s.list + P.kblocks * kKBlock);
     s.full = b;
     s.empty = s.full + P.stages;
@@ -114,8 +110,7 @@ __device__ __forceinline__ FSmem fcarve(uint8_t *base, const FusedParams &P)
     s.tempty = s.tfull + 2;
     s.ready = s.tempty + 2;
     s.afree = s.ready + 2;
-    s.xmax = s.afree + 2;
-    s.sfull = s.xmax + 1;
+    s.sfull = s.afree + 2;
     s.sempty = s.sfull + kMaxSlots;
     s.pkfull = s.sempty + kMaxSlots;
     s.pkempty = s.pkfull + 8;
@@ -124,7 +119,7 @@ __device__ __forceinline__ FSmem fcarve(uint8_t *base, const FusedParams &P)
     s.abort_flag = reinterpret_cast<volatile int *>(s.tmem_slot + 1);
     return s;
 }
-constexpr size_t kFixedSmem = 1024 + 8 * 64 * 4 + (kNumSplitWarps + kExpSlots) * 64 * 4 + 8 * (2 * 4 + 1 + 2 * kMaxSlots + 16 + 1) + 16;
+constexpr size_t kFixedSmem = 1024 + 8 * 64 * 4 + 8 * (2 * 4 + 2 * kMaxSlots + 16 + 1) + 16;
 
 // 16 lanes x 32 consecutive 32-bit columns, no wait: four tmem_ld16x256 side by side.
 __device__ __forceinline__ void tmem_ld16x256x4(uint32_t taddr, uint32_t (&r)[16])
@@ -229,7 +224,6 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
             mbar_init(smem_u32(&S.pkfull[i]), 1);
             mbar_init(smem_u32(&S.pkempty[i]), 1);
         }
-        mbar_init(smem_u32(S.xmax), kNumSplitWarps);
         for (int i = 0; i < kMaxSlots; ++i) {
             mbar_init(smem_u32(&S.sfull[i]), 1);
             mbar_init(smem_u32(&S.sempty[i]), kNumSplitWarps);
@@ -434,7 +428,11 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
         const int half = (P.tile_n / 16) * 8;          // columns of half 0 (a multiple of 8)
         for (int64_t it = it0; it < nit && ok; it += istride, ++n_item) {
             const int64_t row0 = (2 * it + rank) * kFoldTileLos + 16 * q + rq;
-            float scale[2] = {P.out_scale, P.out_scale};
+            float scale[2];
+#pragma unroll
+            for (int l = 0; l < 2; ++l)
+                scale[l] = MODE == MODE_FP16X3 ? ldexpf(P.out_scale, -(int)__ldg(P.rexp + min(row0 + 8 * l, nlos - 1)))
+                                               : P.out_scale;
             float bm[2] = {-1.f, -1.f}, br[2] = {0.f, 0.f}, bim[2] = {0.f, 0.f};
             int bi[2] = {INT_MAX, INT_MAX};
             for (int nt = 0; nt < P.ntiles_n; ++nt, ++g_all) {
@@ -445,12 +443,6 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                 }
                 tph ^= 1u << b;
                 tc_fence_after();
-                if (MODE == MODE_FP16X3 && nt == 0) {
-                    // written by this CTA's splitters before they released the item
-#pragma unroll
-                    for (int l = 0; l < 2; ++l)
-                        scale[l] = ldexpf(P.out_scale, -S.los_exp[(n_item & (kExpSlots - 1)) * 64 + 16 * q + 8 * l + rq]);
-                }
                 const int ncols = ((nt == P.ntiles_n - 1) ? P.tile_n_last : P.tile_n) - h * half;
                 const int kbase = (nt * P.tile_n + h * half) >> 1;
                 const int mine = min(ncols, h ? P.tile_n - half : half);   // columns of this half with results
@@ -585,30 +577,31 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
         // channel-major: this warp's 32 LOS of the tile, its array and first half K block
         const int i = 32 * (sw & 1) + lane, array = (sw >> 1) & 1, h0 = sw >> 2, nh = 2 * P.kblocks;
         const int row = 16 * (i >> 3) + (i & 7) + 8 * array, swz = (row >> 1) & 3;
-        int n_item = 0, ss = 0, n_max = 0;
+        int n_item = 0, ss = 0;
         uint32_t sph = 0;
         bool ok = true;
-        // FP16X3: publish this warp's maxima and wait for the other warps' (null: aborted)
-        auto join_max = [&](float mx) -> const float * {
-            float *x = S.los_max + (n_max & 1) * kNumSplitWarps * 32;
-            x[sw * 32 + lane] = mx;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(S.xmax));
-            if (!warp_wait(smem_u32(S.xmax), n_max & 1, S.abort_flag, P.err, P.timeout_ns)) return nullptr;
-            ++n_max;
-            return x;
-        };
         for (int64_t it = it0; it < nit && ok; it += istride, ++n_item) {
             const int slot = n_item & 1;
             const int64_t los0 = (2 * it + rank) * kFoldTileLos;
             const bool stg = !CHAN && P.sslots > 0 && los0 + kFoldTileLos <= nlos;
             uint8_t *const tile = P.ring + ((size_t)blockIdx.x * 2 + slot) * P.kblocks * kPartsBytes;
-            int *const exps = S.los_exp + (n_item & (kExpSlots - 1)) * 64;
             const int64_t los8 = los0 + 8 * sw;            // LOS-major, direct: this warp's 8 LOS
             auto src_of = [&](int r) { return min(los8 + r, nlos - 1); };
             const uint32_t dead = los8 + 8 <= nlos ? 0u : (0xffu << (int)max((int64_t)0, nlos - los8)) & 0xffu;
-            float scale[8] = {1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f};
-            int ex[8];
+            // FP16X3: the exponents of the item's LOS, two per lane
+            int e64[2] = {0, 0};
+            if constexpr (MODE == MODE_FP16X3) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) e64[h] = __ldg(P.rexp + min(los0 + 32 * h + lane, nlos - 1));
+            }
+            // the scales of LOS j + 2 k + (lane / 16) of the item (j a multiple of 8)
+            auto scales_of = [&](int j, float (&scale)[4]) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    scale[k] = MODE != MODE_FP16X3 ? 1.f
+                               : ldexpf(1.0f, __shfl_sync(0xffffffffu, j & 32 ? e64[1] : e64[0], (j & 31) + 2 * k + (lane >> 4)));
+            };
+            float scale[4];
             // ROT: the T rows of the item's LOS, two LOS per lane, or the lane's own LOS (channel-major)
             int32_t cen[2] = {0, 0};
             if constexpr (ROT) {
@@ -622,15 +615,7 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                 const int c = __shfl_sync(0xffffffffu, j & 32 ? cen[1] : cen[0], (j & 31) + (lane >> 4));
                 return __ldg(reinterpret_cast<const float4 *>(P.rot.T + (size_t)c * P.rot.ldT + kb * kKBlock) + (lane & 15));
             };
-            if constexpr (MODE == MODE_FP16X3) {
-                // the LOS's largest |value| sets its power-of-two scale: a first pass over the tile
-                // (staged LOS-major rows are complete in their slot and need none)
-                if (!stg) {
-                    fold_scales_los(P.src, S.list, P.kblocks, lane, src_of, dead, scale, ex);
-                }
-            }
-            // the slot's previous item has been read; and the epilogue is done with the item four
-            // before, whose exponents are replaced: its phase tiles are drained
+            // the slot's previous item has been read
             if (!warp_wait(smem_u32(&S.afree[slot]), ((n_item >> 1) & 1) ^ 1, S.abort_flag, P.err, P.timeout_ns)) {
                 ok = false;
                 break;
@@ -674,8 +659,9 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                     }
                 } else {
                 uint8_t *const dst = tile + row * kFoldRowBytes;
+                const float sc = MODE == MODE_FP16X3 ? ldexpf(1.0f, sw & 1 ? e64[1] : e64[0]) : 1.f;
                 chan_walk<true>(P.src, S.list, los0 + i, array, h0, nh, [&](int h, const float (&v)[16]) {
-                    emit16<MODE, true>(dst + (size_t)(h >> 1) * kPartsBytes, h & 1, swz, v, scale[0]);
+                    emit16<MODE, true>(dst + (size_t)(h >> 1) * kPartsBytes, h & 1, swz, v, sc);
                 });
                 }
             } else if (stg) {
@@ -692,27 +678,7 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                     }
                     const float *rows = reinterpret_cast<const float *>(S.stage + (size_t)ss * P.sbytes);
                     const int nchan = P.src.nchan;
-                    if constexpr (MODE == MODE_FP16X3) {
-                        // warp sw finds row sw's largest active |value|
-                        float mx = 0.f;
-                        for (int a = lane; a < P.src.nact; a += 32) {
-                            const int ch = S.list[a];
-                            mx = fmaxf(mx, fmaxf(fabsf(rows[sw * nchan + ch]), fabsf(rows[(8 + sw) * nchan + ch])));
-                        }
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                        const float *x = join_max(mx);
-                        if (!x) {
-                            ok = false;
-                            break;
-                        }
-#pragma unroll
-                        for (int r = 0; r < 8; ++r) {
-                            ex[r] = fold_exponent(x[r * 32]);
-                            scale[r] = ldexpf(1.0f, ex[r]);
-                            if (sw == 0 && lane == r) exps[8 * g + r] = ex[r];
-                        }
-                    }
+                    if constexpr (MODE == MODE_FP16X3) scales_of(8 * g, scale);
                     const int arr = sw & 1;
                     for (int kb = sw >> 1; kb < P.kblocks; kb += kNumSplitWarps / 2) {
                         const int2 ch = *reinterpret_cast<const int2 *>(S.list + kb * kKBlock + 2 * (lane & 15));
@@ -730,6 +696,7 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                         uint8_t *const blk = tile + (size_t)kb * kPartsBytes + 16 * g * kFoldRowBytes;
                         if constexpr (ROT) {
                             const int r0 = 4 * arr;
+                            const float one2[2] = {1.f, 1.f};       // (never FP16X3)
                             float q[4], u[4];
                             float4 tn[2];
                             // T of the warp's next unit, here or in the next slot
@@ -747,8 +714,8 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                                 rotate(q[2 * j + 1], u[2 * j + 1], make_float2(t[j].z, t[j].w));
                                 t[j] = tn[j];
                             }
-                            fold_emit_rows<MODE, true, 4>(blk, lane, r0, q, scale);
-                            fold_emit_rows<MODE, true, 4>(blk + 8 * kFoldRowBytes, lane, r0, u, scale);
+                            fold_emit_rows<MODE, true, 4>(blk, lane, r0, q, one2);
+                            fold_emit_rows<MODE, true, 4>(blk + 8 * kFoldRowBytes, lane, r0, u, one2);
                         } else {
                             float v[8];
 #pragma unroll
@@ -763,11 +730,7 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                     if (++ss == P.sslots) { ss = 0; sph ^= 1; }
                 }
             } else {
-                if constexpr (MODE == MODE_FP16X3) {
-#pragma unroll
-                    for (int r = 0; r < 8; ++r)
-                        if (lane == r) exps[8 * sw + r] = ex[r];
-                }
+                if constexpr (MODE == MODE_FP16X3) scales_of(8 * sw, scale);
                 uint8_t *const dst = tile + 16 * sw * kFoldRowBytes;
                 for (int kb = 0; kb < P.kblocks; ++kb) {
                     float q[8], u[8];
@@ -830,7 +793,7 @@ FusedKernel fused_for(int mode, bool chan, bool rot)
     }
     if (mode == MODE_BF16) return chan ? fused_kernel<MODE_BF16, true, false> : fused_kernel<MODE_BF16, false, false>;
     if (mode == MODE_BF16X3) return chan ? fused_kernel<MODE_BF16X3, true, false> : fused_kernel<MODE_BF16X3, false, false>;
-    return fused_kernel<MODE_FP16X3, false, false>;     // (fused_wanted: staged LOS-major rows)
+    return chan ? fused_kernel<MODE_FP16X3, true, false> : fused_kernel<MODE_FP16X3, false, false>;
 }
 
 // Pipeline shape beside `staging` bytes of staging slots and the channel list: K blocks per stage and stages, at
@@ -910,18 +873,16 @@ cudaError_t fused_prepare(rms_plan_s *p, bool window)
 // One kernel unless the last round of items over the pairs is too empty (12,000 LOS are 94
 // items on 76 pairs: 69.9 against 64.2 us at 360 channels x 801 phi, but 161 items on two
 // thirds of three rounds 99.0 against 104) or there are few items with many phase tiles,
-// which the job schedule spreads over more SMs; FP16X3 only where its row maxima come with
-// the staged rows (channel-major it would walk each item twice: 0.92 against 0.81 ms on
-// 262,144 LOS x 360 x 401).  Measured with F and the peak map, one kernel against two:
+// which the job schedule spreads over more SMs.  Measured with F and the peak map, one
+// kernel against two:
 // 262,144 LOS x 360 x 401 BF16x3 0.474 / 0.636 ms (LOS-major 0.484 / 0.642), 200,003 x
 // 357 x 401 FP16x3 LOS-major 0.535 / 0.612, 400,000 x 800 x 1001 BF16 1.53 / 2.04 ms,
 // 5,000 LOS x 360 x 401 32.6 / 36.1 us.
-bool fused_wanted(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout)
+bool fused_wanted(const rms_plan_s &p, int64_t nlos)
 {
     const FoldPlan &f = p.fold;
     if (f.fused_pairs < 1 || p.contraction != RMS_CONTRACT_AUTO || p.schedule != RMS_SCHEDULE_AUTO || p.l2_budget != 0)
         return false;
-    if (p.precision == RMS_FP16X3 && !staging_slots(p, Q, U, layout == RMS_CHAN_MAJOR)) return false;
     const int64_t nit = (nlos + 2 * kFoldTileLos - 1) / (2 * kFoldTileLos);
     const int64_t rounds = (nit + f.fused_pairs - 1) / f.fused_pairs;
     if (rounds == 1) return 2 * nit >= f.fused_pairs || f.tiles.ntiles_n2 <= 2;
@@ -937,7 +898,7 @@ size_t fused_ring_bytes(const rms_plan_s &p, int64_t nlos)
 
 cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout, float *F,
                          int32_t *pidx, float *pabs, float *pphi, float *pq, float *pu, float *pchi, uint8_t *ring,
-                         cudaStream_t s, const FusedRotation *rot)
+                         const int8_t *rexp, cudaStream_t s, const FusedRotation *rot)
 {
     const FoldPlan &f = p.fold;
     const bool chan = layout == RMS_CHAN_MAJOR;
@@ -969,6 +930,7 @@ cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, in
     P.phi64 = p.d_phi;
     P.lambda0sq = p.lambda0sq;
     P.out_scale = (float)(p.K * p.wmax);
+    P.rexp = rexp;
     P.err = p.d_err;
     P.timeout_ns = p.timeout_ns;
     P.sslots = staging_slots(p, Q, U, chan);

@@ -138,7 +138,7 @@ cudaError_t window_fused(const rms_window_s &w, const float *Q, const float *U, 
                          const int32_t *centre, float *F, int32_t *widx, float *wabs, uint8_t *ring, cudaStream_t s)
 {
     const FusedRotation rot = {centre, w.d_Tc, w.ldc, w.cmin, w.cmax};
-    return launch_fused(*w.sub, Q, U, nlos, layout, F, widx, wabs, nullptr, nullptr, nullptr, nullptr, ring, s, &rot);
+    return launch_fused(*w.sub, Q, U, nlos, layout, F, widx, wabs, nullptr, nullptr, nullptr, nullptr, ring, nullptr, s, &rot);
 }
 
 // The rotating contraction of a split image.

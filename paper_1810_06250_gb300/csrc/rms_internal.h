@@ -174,6 +174,9 @@ size_t split_operand_bytes(const rms_plan_s &p, int64_t nlos, int layout);
 // Operand image of a folded grid: [ceil(nlos / 128) 2][fold.kblocks][16 KB], tiles of 64 LOS (fold.cu);
 // rows, count: optional gather of *count (<= nlos) LOS, as SplitOpts.
 size_t fold_operand_bytes(const rms_plan_s &p, int64_t nlos);
+// FP16X3 on folded grids: the exponent of each LOS's scale (launch_fold_split calls it itself)
+cudaError_t launch_fold_exponents(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout,
+                                  int8_t *rexp, cudaStream_t s);
 cudaError_t launch_fold_split(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout,
                               uint8_t *A, int8_t *rexp, cudaStream_t s, const int64_t *rows = nullptr,
                               const int64_t *count = nullptr);
@@ -185,11 +188,11 @@ struct FusedRotation {             // window plans: LOS l is multiplied by T[cla
     int32_t ldT = 0, cmin = 0, cmax = 0;
 };
 cudaError_t fused_prepare(rms_plan_s *p, bool window);
-bool fused_wanted(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout);
+bool fused_wanted(const rms_plan_s &p, int64_t nlos);
 size_t fused_ring_bytes(const rms_plan_s &p, int64_t nlos);
 cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout, float *F,
                          int32_t *pidx, float *pabs, float *pphi, float *pq, float *pu, float *pchi, uint8_t *ring,
-                         cudaStream_t s, const FusedRotation *rot = nullptr);
+                         const int8_t *rexp, cudaStream_t s, const FusedRotation *rot = nullptr);
 struct SplitOpts {
     const float *Q = nullptr, *U = nullptr;
     int64_t nlos_src = 0;              // lines of sight in the cube
