@@ -41,6 +41,7 @@
 
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "rms_internal.h"
 
@@ -240,6 +241,113 @@ __global__ void __launch_bounds__(128) split_kernel(const SplitParams P)
     if (P.rscale && valid) {
         const float rms = sqrtf(ss / (float)P.nact_norm);
         P.rscale[row] = rms > 0.f ? 1.0f / rms : 1.0f;
+    }
+}
+
+// The same image and row scales for calls of few rows: 32 rows per CTA, staged in shared
+// memory by copies that are all in flight at once.  A row's sum of squares is one chain of
+// additions in channel order (another order moves roundings of what is computed from it), so
+// one warp walks the 32 rows' chains while the others split.  Latency-bound: 4,096 rows x 400
+// channels LOS-major 30 -> 10 us, 222 rows 38 -> 9 us.
+constexpr int kTileRows = 32;
+// staged row of a LOS-major tile: whole K blocks, an odd number of 16-byte pieces (a column of
+// 16-byte reads takes all banks)
+__host__ __device__ constexpr int tile_ld(int kblocks) { return (kblocks * kChanPerKBlock / 4 | 1) * 4; }
+
+template <bool CHAN>
+__global__ void __launch_bounds__(256) split_tile_kernel(const SplitParams P)
+{
+    extern __shared__ __align__(16) unsigned char tile_raw[];
+    float *const tq = reinterpret_cast<float *>(tile_raw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t row0 = (int64_t)blockIdx.x * kTileRows, mt = row0 / kTileM;
+    const int64_t n_eff = P.count ? min(*P.count, P.nout) : P.nout;
+    if (mt * kTileM >= n_eff) return;          // tiles past a device-side count stay untouched
+    const bool valid = row0 + lane < n_eff;
+    const int64_t src = valid ? (P.rows ? P.rows[row0 + lane] : row0 + lane) : 0;     // the lane's row
+    const int ld = CHAN ? kTileRows + 1 : tile_ld(P.kblocks);
+    float *const tu = tq + (size_t)(CHAN ? P.nk : kTileRows) * ld;
+    auto copy = [](float *dst, const float *from, auto bytes) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(from),
+                     "n"(decltype(bytes)::value)
+                     : "memory");
+    };
+    if (CHAN) {
+        for (int a = warp; a < P.nk; a += 8) {
+            const int64_t off = (int64_t)__ldg(P.active + a) * P.nlos_src + src;
+            copy(tq + a * ld + lane, P.Q + off, std::integral_constant<int, 4>());
+            copy(tu + a * ld + lane, P.U + off, std::integral_constant<int, 4>());
+        }
+    } else {
+        for (int r = warp; r < kTileRows; r += 8) {
+            const int64_t from = __shfl_sync(0xffffffffu, src, r) * P.nchan;
+            if (P.vec4) {
+                for (int c = 4 * lane; c < P.nchan; c += 128) {
+                    copy(tq + r * ld + c, P.Q + from + c, std::integral_constant<int, 16>());
+                    copy(tu + r * ld + c, P.U + from + c, std::integral_constant<int, 16>());
+                }
+            } else {
+                for (int c = lane; c < P.nchan; c += 32) {
+                    copy(tq + r * ld + c, P.Q + from + c, std::integral_constant<int, 4>());
+                    copy(tu + r * ld + c, P.U + from + c, std::integral_constant<int, 4>());
+                }
+            }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    // 16 channels of the lane's row; flagged and padding ones are 0, whatever stands there
+    auto block = [&](int kb, float (&q)[16], float (&u)[16]) {
+        const int c0 = kb * kChanPerKBlock;
+        if (CHAN) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const bool live = valid && c0 + i < P.nk;
+                q[i] = live ? tq[(c0 + i) * ld + lane] : 0.f;
+                u[i] = live ? tu[(c0 + i) * ld + lane] : 0.f;
+            }
+        } else {
+            const uint32_t live = valid ? __ldg(P.kbmask + kb) : 0u;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const float4 x = *reinterpret_cast<const float4 *>(tq + lane * ld + c0 + 4 * v);
+                const float4 y = *reinterpret_cast<const float4 *>(tu + lane * ld + c0 + 4 * v);
+                q[4 * v] = x.x; q[4 * v + 1] = x.y; q[4 * v + 2] = x.z; q[4 * v + 3] = x.w;
+                u[4 * v] = y.x; u[4 * v + 1] = y.y; u[4 * v + 2] = y.z; u[4 * v + 3] = y.w;
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (!((live >> i) & 1u)) { q[i] = 0.f; u[i] = 0.f; }
+        }
+    };
+    if (warp == 0) {
+        float ss = 0.f;
+        for (int kb = 0; kb < P.kblocks; ++kb) {
+            float q[16], u[16];
+            block(kb, q, u);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) ss = fmaf(q[i], q[i], fmaf(u[i], u[i], ss));
+        }
+        if (valid) {
+            const float rms = sqrtf(ss / (float)P.nact_norm);
+            P.rscale[row0 + lane] = rms > 0.f ? 1.0f / rms : 1.0f;
+        }
+    } else {
+        const int m = (int)(row0 % kTileM) + lane, sw = (m >> 1) & 3;
+        for (int kb = warp - 1; kb < P.kblocks; kb += 7) {
+            float q[16], u[16];
+            block(kb, q, u);
+            uint8_t *const dst = P.A + ((size_t)mt * P.kblocks + kb) * (2 * kStageA) + (uint32_t)m * kRowBytes;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                uint32_t hi[4], lo[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) split_pair_bf16(q[4 * c + j], u[4 * c + j], hi[j], lo[j]);
+                const uint32_t off = (uint32_t)(c ^ sw) << 4;
+                *reinterpret_cast<uint4 *>(dst + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                if (P.mode != MODE_BF16) *reinterpret_cast<uint4 *>(dst + kStageA + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            }
+        }
     }
 }
 
@@ -1200,6 +1308,19 @@ cudaError_t launch_split(const rms_plan_s &p, const SplitOpts &o, cudaStream_t s
     sp.vec4 = !chan && (p.nchan % 4 == 0) && !(reinterpret_cast<uintptr_t>(o.Q) & 15) &&
               !(reinterpret_cast<uintptr_t>(o.U) & 15);
     if (sp.mode == MODE_FP16X3 && !o.rexp) return cudaErrorInvalidValue;
+    const size_t tile_bytes = 2 * sizeof(float) * (chan ? (size_t)p.nact * (kTileRows + 1) : (size_t)kTileRows * tile_ld(sp.kblocks));
+    // few rows: one thread per row walks it in a latency-bound chain (30 us whatever the row count), while
+    // 32-row tiles take about 7 us a wave of two CTAs per SM.  Proposal and window, 360 channels x 401 phi,
+    // tiles against threads: 222 LOS 74 / 97 us, 4,000 76 / 95, 20,000 152 / 159, 40,000 225 / 222 us
+    // (channel-major 267 / 251), 262,144 0.975 / 0.905 ms
+    if (o.rscale && sp.mode != MODE_FP16X3 && o.nout <= (int64_t)5 * kTileRows * p.num_sms && tile_bytes <= (size_t)kSmemLimit) {
+        const auto kern = chan ? split_tile_kernel<true> : split_tile_kernel<false>;
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+        if (e != cudaSuccess) return e;
+        sp.kpg = sp.kblocks;
+        kern<<<(unsigned)(nmt * (kTileM / kTileRows)), 256, tile_bytes, s>>>(sp);
+        return cudaGetLastError();
+    }
     // A grid of one CTA per M tile leaves a partial last wave (the LOFAR cube's 2,048
     // tiles are 1.5 waves at 9 CTAs per SM), so the K blocks of a tile are shared out
     // over blockIdx.y until the grid is about 8 waves; FP16X3 (a row's largest value
