@@ -51,6 +51,8 @@ constexpr int kRegsLaunch = 96, kRegsCtl = 48, kRegsEpi = 128, kRegsSplit = 88;
 static_assert(128 * kRegsCtl + 256 * kRegsEpi + 256 * kRegsSplit == kThreads * kRegsLaunch,
               "register split must fill the launch");
 
+constexpr int kMaxChunks = 4;
+
 struct FusedParams {
     FoldSource src;
     int32_t kblocks, mode;
@@ -69,6 +71,7 @@ struct FusedParams {
     int64_t timeout_ns;
     int32_t stages, kbs;        // pipeline stages of kbs K blocks each
     int32_t sslots;             // staging slots; 0: direct loads
+    int32_t chunk_log;          // the splitters release an item's K blocks by parts of 2^chunk_log (>= kbs)
     uint32_t sbytes;            // bytes of a staging slot
     FusedRotation rot;          // ROT
 };
@@ -109,7 +112,7 @@ __device__ __forceinline__ FSmem fcarve(uint8_t *base, const FusedParams &P)
     s.tfull = s.empty + P.stages;
     s.tempty = s.tfull + 2;
     s.ready = s.tempty + 2;
-    s.afree = s.ready + 2;
+    s.afree = s.ready + 2 * kMaxChunks;
     s.sfull = s.afree + 2;
     s.sempty = s.sfull + kMaxSlots;
     s.pkfull = s.sempty + kMaxSlots;
@@ -119,7 +122,7 @@ __device__ __forceinline__ FSmem fcarve(uint8_t *base, const FusedParams &P)
     s.abort_flag = reinterpret_cast<volatile int *>(s.tmem_slot + 1);
     return s;
 }
-constexpr size_t kFixedSmem = 1024 + 8 * 64 * 4 + 8 * (2 * 4 + 2 * kMaxSlots + 16 + 1) + 16;
+constexpr size_t kFixedSmem = 1024 + 8 * 64 * 4 + 8 * (2 * 3 + 2 * kMaxChunks + 2 * kMaxSlots + 16 + 1) + 16;
 
 // 16 lanes x 32 consecutive 32-bit columns, no wait: four tmem_ld16x256 side by side.
 __device__ __forceinline__ void tmem_ld16x256x4(uint32_t taddr, uint32_t (&r)[16])
@@ -217,7 +220,7 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&S.tfull[b]), 1);
             mbar_init(smem_u32(&S.tempty[b]), 2 * kNumEpiWarps);
-            mbar_init(smem_u32(&S.ready[b]), kNumSplitWarps);
+            for (int c = 0; c < kMaxChunks; ++c) mbar_init(smem_u32(&S.ready[b * kMaxChunks + c]), kNumSplitWarps);
             mbar_init(smem_u32(&S.afree[b]), 1);
         }
         for (int i = 0; i < 8; ++i) {
@@ -258,17 +261,21 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                 int n_item = 0;
                 for (int64_t it = it0; it < nit && ok; it += istride, ++n_item) {
                     const int slot = n_item & 1;
-                    if (!wait_bounded(smem_u32(&S.ready[slot]), (n_item >> 1) & 1, S.abort_flag, P.err, P.timeout_ns)) {
-                        ok = false;
-                        break;
-                    }
-                    fence_proxy_async_global();
                     const int32_t z0 = ((int32_t)blockIdx.x * 2 + slot) * P.kblocks;
                     for (int nt = 0; nt < P.ntiles_n && ok; ++nt) {
                         int32_t y = nt * P.tile_n;
                         if (!leader) y += ((nt == P.ntiles_n - 1) ? P.tile_n_last : P.tile_n) / 2;
                         for (int kb = 0; kb < P.kblocks; kb += P.kbs) {
                             const int n = min(P.kbs, P.kblocks - kb);
+                            if (nt == 0 && (kb & ((1 << P.chunk_log) - 1)) == 0) {
+                                // the item's next K blocks are in the ring
+                                if (!wait_bounded(smem_u32(&S.ready[slot * kMaxChunks + (kb >> P.chunk_log)]), (n_item >> 1) & 1,
+                                                  S.abort_flag, P.err, P.timeout_ns)) {
+                                    ok = false;
+                                    break;
+                                }
+                                fence_proxy_async_global();
+                            }
                             if (!wait_bounded(smem_u32(&S.empty[s]), ph ^ 1, S.abort_flag, P.err, P.timeout_ns)) {
                                 ok = false;
                                 break;
@@ -575,7 +582,7 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
         // ------------------------------------------------------------ splitters
         const int sw = warp - kSplitWarp0;
         // channel-major: this warp's 32 LOS of the tile, its array and first half K block
-        const int i = 32 * (sw & 1) + lane, array = (sw >> 1) & 1, h0 = sw >> 2, nh = 2 * P.kblocks;
+        const int i = 32 * (sw & 1) + lane, array = (sw >> 1) & 1, h0 = sw >> 2;
         const int row = 16 * (i >> 3) + (i & 7) + 8 * array, swz = (row >> 1) & 3;
         int n_item = 0, ss = 0;
         uint32_t sph = 0;
@@ -620,6 +627,13 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                 ok = false;
                 break;
             }
+            // release part c of the item's K blocks, as far as this warp goes
+            auto release = [&](int c) {
+                // the TMA (async proxy) reads what these generic stores wrote
+                fence_proxy_async_global();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&S.ready[slot * kMaxChunks + c]));
+            };
             if constexpr (CHAN) {
                 if constexpr (ROT) {
                     // both arrays of 8 channels at a time; four warps share a LOS
@@ -627,7 +641,9 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                     const int64_t at = min(los0 + i, nlos - 1);
                     const bool valid = los0 + i < nlos;
                     const int r0 = 16 * (i >> 3) + (i & 7), sz = (r0 >> 1) & 3;
-                    for (int o = sw >> 1; o < 4 * P.kblocks; o += kNumSplitWarps / 2) {
+                    for (int c = 0; c << P.chunk_log < P.kblocks; ++c) {
+                    const int o_end = 4 * min(P.kblocks, (c + 1) << P.chunk_log);
+                    for (int o = (4 * c << P.chunk_log) + (sw >> 1); o < o_end; o += kNumSplitWarps / 2) {
                         float q[8], u[8];
                         float4 t[4];
 #pragma unroll
@@ -657,12 +673,18 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                             *reinterpret_cast<uint4 *>(d + kFoldPart + 8 * kFoldRowBytes) = make_uint4(ul[0], ul[1], ul[2], ul[3]);
                         }
                     }
+                    release(c);
+                    }
                 } else {
                 uint8_t *const dst = tile + row * kFoldRowBytes;
                 const float sc = MODE == MODE_FP16X3 ? ldexpf(1.0f, sw & 1 ? e64[1] : e64[0]) : 1.f;
-                chan_walk<true>(P.src, S.list, los0 + i, array, h0, nh, [&](int h, const float (&v)[16]) {
-                    emit16<MODE, true>(dst + (size_t)(h >> 1) * kPartsBytes, h & 1, swz, v, sc);
-                });
+                for (int c = 0; c << P.chunk_log < P.kblocks; ++c) {
+                    const int h1 = 2 * min(P.kblocks, (c + 1) << P.chunk_log);
+                    chan_walk<true>(P.src, S.list, los0 + i, array, (2 * c << P.chunk_log) + h0, h1, [&](int h, const float (&v)[16]) {
+                        emit16<MODE, true>(dst + (size_t)(h >> 1) * kPartsBytes, h & 1, swz, v, sc);
+                    });
+                    release(c);
+                }
                 }
             } else if (stg) {
                 // 8 LOS per slot; units of (K block, array), or ROT (K block, 4 LOS), go round the warps
@@ -732,43 +754,71 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
             } else {
                 if constexpr (MODE == MODE_FP16X3) scales_of(8 * sw, scale);
                 uint8_t *const dst = tile + 16 * sw * kFoldRowBytes;
-                for (int kb = 0; kb < P.kblocks; ++kb) {
-                    float q[8], u[8];
-                    fold_load_los<true>(P.src, S.list, kb, lane, src_of, q, u);
-                    fold_mask_los(P.src, kb, lane, dead, q, u);
-                    if constexpr (ROT) {
+                if constexpr (ROT || MODE == MODE_FP16X3) {
+                    // one K block at a time: with the next one's values the registers run out here
+                    for (int c = 0; ROT ? c < 1 : c << P.chunk_log < P.kblocks; ++c) {      // (ROT: one part)
+                        const int kb1 = ROT ? P.kblocks : min(P.kblocks, (c + 1) << P.chunk_log);
+#pragma unroll (ROT ? 1 : 2)
+                        for (int kb = ROT ? 0 : c << P.chunk_log; kb < kb1; ++kb) {
+                            float q[8], u[8];
+                            fold_load_los<true>(P.src, S.list, kb, lane, src_of, q, u);
+                            fold_mask_los(P.src, kb, lane, dead, q, u);
+                            if constexpr (ROT) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const float4 t = t_of(8 * sw + 2 * j, kb);
-                            rotate(q[2 * j], u[2 * j], make_float2(t.x, t.y));
-                            rotate(q[2 * j + 1], u[2 * j + 1], make_float2(t.z, t.w));
+                                for (int j = 0; j < 4; ++j) {
+                                    const float4 t = t_of(8 * sw + 2 * j, kb);
+                                    rotate(q[2 * j], u[2 * j], make_float2(t.x, t.y));
+                                    rotate(q[2 * j + 1], u[2 * j + 1], make_float2(t.z, t.w));
+                                }
+                            }
+                            fold_emit_rows<MODE, true, 8>(dst + (size_t)kb * kPartsBytes, lane, 0, q, scale);
+                            fold_emit_rows<MODE, true, 8>(dst + (size_t)kb * kPartsBytes + 8 * kFoldRowBytes, lane, 0, u, scale);
                         }
+                        release(c);
                     }
-                    fold_emit_rows<MODE, true, 8>(dst + (size_t)kb * kPartsBytes, lane, 0, q, scale);
-                    fold_emit_rows<MODE, true, 8>(dst + (size_t)kb * kPartsBytes + 8 * kFoldRowBytes, lane, 0, u, scale);
+                } else {
+                    auto load = [&](int kb, float (&q)[8], float (&u)[8]) {
+                        fold_load_los<true>(P.src, S.list, kb, lane, src_of, q, u);
+                    };
+                    auto emit = [&](int kb, float (&q)[8], float (&u)[8]) {
+                        fold_mask_los(P.src, kb, lane, dead, q, u);
+                        fold_emit_rows<MODE, true, 8>(dst + (size_t)kb * kPartsBytes, lane, 0, q, scale);
+                        fold_emit_rows<MODE, true, 8>(dst + (size_t)kb * kPartsBytes + 8 * kFoldRowBytes, lane, 0, u, scale);
+                    };
+                    for (int c = 0; c << P.chunk_log < P.kblocks; ++c) {
+                        const int kb1 = min(P.kblocks, (c + 1) << P.chunk_log);
+                        float qa[8], ua[8], qb[8], ub[8];
+                        int kb = c << P.chunk_log;
+                        load(kb, qa, ua);
+                        // the next K block's loads are in flight while one is split
+                        for (; kb < kb1; kb += 2) {
+                            if (kb + 1 < kb1) load(kb + 1, qb, ub);
+                            emit(kb, qa, ua);
+                            if (kb + 2 < kb1) load(kb + 2, qa, ua);
+                            if (kb + 1 < kb1) emit(kb + 1, qb, ub);
+                        }
+                        release(c);
+                    }
                 }
             }
             if (!ok) break;
-            // the TMA (async proxy) reads what these generic stores wrote
-            fence_proxy_async_global();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&S.ready[slot]));
+            if (stg) release(0);            // (one part)
         }
         // the commits that free the last slots arrive before the CTA leaves
         for (int k = max(0, n_item - 2); k < n_item && ok; ++k)
             ok = warp_wait(smem_u32(&S.afree[k & 1]), (k >> 1) & 1, S.abort_flag, P.err, P.timeout_ns);
         if (!ok) stop_peer();
+        // the ring's lines go back to normal priority: nobody else's working set should yield to them.
+        // (Here, beside the last epilogue: after it, it took 1.4 us of a 27 us call.)
+        uint8_t *const own = P.ring + (size_t)blockIdx.x * 2 * P.kblocks * kPartsBytes;
+        const uint32_t used = (uint32_t)min(n_item, 2) * P.kblocks * kPartsBytes;
+        for (uint32_t at = (uint32_t)(32 * sw + lane) * 128; at < used; at += kNumSplitWarps * 32 * 128)
+            asm volatile("applypriority.global.L2::evict_normal [%0], 128;" ::"l"(own + at) : "memory");
     }
 
     if (*S.abort_flag) stop_peer();
     tc_fence_before();
     __syncthreads();
-    // the ring's lines go back to normal priority: nobody else's working set should yield to them
-    {
-        uint8_t *const own = P.ring + (size_t)blockIdx.x * 2 * P.kblocks * kPartsBytes;
-        for (size_t at = (size_t)threadIdx.x * 128; at < (size_t)2 * P.kblocks * kPartsBytes; at += kThreads * 128)
-            asm volatile("applypriority.global.L2::evict_normal [%0], 128;" ::"l"(own + at) : "memory");
-    }
     // neither CTA leaves (or frees TMEM) while the other may still use its shared memory,
     // barriers or TMEM
     cluster_sync_all();
@@ -933,12 +983,19 @@ cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, in
     P.rexp = rexp;
     P.err = p.d_err;
     P.timeout_ns = p.timeout_ns;
-    P.sslots = staging_slots(p, Q, U, chan);
+    // One item per pair: its K blocks are released in up to four parts, so that the MMAs start while it
+    // is being split; LOS-major it is then loaded K block by K block, not by whole staged rows (the
+    // window's rows stay staged: its rotation leaves no registers for the loads ahead).  5,001 LOS x 357 x
+    // 401 BF16x3 32.5 -> 27.1 us (channel-major 30.8 -> 26.7), 2,000 LOS 28.8 -> 24.7, 9,728 33.0 -> 28.8.
+    // Fewer than five K blocks are one part: a part costs a fence and its loads' latency.
+    const bool once = nit <= f.fused_pairs && (chan || !rot);
+    P.sslots = once ? 0 : staging_slots(p, Q, U, chan);
     P.sbytes = (uint32_t)(2 * 8 * p.nchan * sizeof(float));
     const Shape sh = shape_for(p, (size_t)P.sslots * P.sbytes);
     if (sh.stages < 3) return cudaErrorInvalidConfiguration;
     P.stages = sh.stages;
     P.kbs = sh.kbs;
+    for (P.chunk_log = 2; f.kblocks > (once ? kMaxChunks : 1) << P.chunk_log;) ++P.chunk_log;   // (4 >= kbs)
     // the ring as a 3-D tensor: 8 of the image's 64-byte rows to a row (whole lines per request), the
     // hi (and lo) rows of a K block, K blocks
     const int parts = mode == MODE_BF16 ? 1 : 2;
