@@ -74,6 +74,7 @@ void free_plan(rms_plan_s *p)
     cudaFree(p->d_kbmask);
     cudaFree(p->d_stage);
     cudaFree(p->d_rexp);
+    cudaFree(p->d_simt_part);
     cudaFree(p->d_scratch);
     for (cudaEvent_t x : p->tev) cudaEventDestroy(x);
     for (cudaEvent_t x : p->hev)

@@ -78,6 +78,7 @@ struct rms_plan_s {
     int32_t kpad = 0, kblocks = 0;
     PhaseTiling tiles;      // npad covers both tilings
     FoldPlan fold;
+    float *d_simt_part = nullptr;   // FP32 CUDA-core kernels: peaks of blocks shared by two CTAs, and arrivals
     int32_t simt_clusters[8] = {};  // FP32 CUDA-core kernels: resident clusters of 1 .. 8 blocks
     CUtensorMap tmap_bhi;   // CUtensorMap is 64-byte aligned by its own declaration
     CUtensorMap tmap_blo;

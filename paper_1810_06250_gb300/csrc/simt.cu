@@ -76,6 +76,13 @@ struct SimtArgs {
     int32_t *pidx;
     float *pabs, *pphi;
     int *err;
+    // balanced form (one CTA per SM): the cost of a block's phi tiles, in 16-column pieces, and
+    // what two CTAs that share a block exchange: [CTA][2][TL] peaks, [CTA] arrivals (0 at launch)
+    int32_t balanced, block_cost;
+    int64_t blocks;
+    float *part_m;
+    int32_t *part_k;
+    int32_t *arrived;
 };
 
 __device__ __forceinline__ bool better(float m, int i, float bm, int bi)
@@ -300,12 +307,25 @@ __device__ __forceinline__ void phi_tile(const SimtArgs &a, const Stage *stage, 
     }
 }
 
+__device__ __forceinline__ void write_peak(const SimtArgs &a, int64_t l, float m, int k)
+{
+    if (l >= a.nlos) return;
+    const bool ok = k != INT_MAX;
+    if (a.pidx) a.pidx[l] = ok ? k : -1;
+    if (a.pabs) a.pabs[l] = ok ? sqrtf(m) : __int_as_float(0x7fc00000);
+    if (a.pphi) a.pphi[l] = ok ? a.phi32[k] : __int_as_float(0x7fc00000);
+}
+
+// the accumulating warps
+__device__ __forceinline__ void sum_sync() { asm volatile("bar.sync 1, %0;" ::"n"(TL) : "memory"); }
+
 template <bool FLY, bool FOLD, int LAYOUT>
 __global__ void __launch_bounds__(kThreads, 1) simt_kernel(const SimtArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ float pk_m[TL];
-    __shared__ int pk_k[TL];
+    __shared__ float pk_m[2 * TL];
+    __shared__ int pk_k[2 * TL];
+    __shared__ int second;
     Stage *stage = reinterpret_cast<Stage *>(smem_raw);
 
     __shared__ uint64_t bars[2 * NS];
@@ -321,7 +341,6 @@ __global__ void __launch_bounds__(kThreads, 1) simt_kernel(const SimtArgs a)
     pp.size = (int)cluster.num_blocks();
     pp.nck = (a.nact + CH - 1) / CH;
     pp.s = 0;
-    const int64_t l0 = (int64_t)(blockIdx.x / pp.size) * TL;
     constexpr int W = FOLD ? TP / 2 : TP;
     const int ntiles = (a.ncol + W - 1) / W;        // the cluster has at most as many blocks
     if (tid == 0) {
@@ -333,76 +352,123 @@ __global__ void __launch_bounds__(kThreads, 1) simt_kernel(const SimtArgs a)
     }
     __syncthreads();
 
+    // This CTA's share: phi tiles t0, t0 + size, .. of one block; or balanced, the run of
+    // (block, tile) units whose costs start in its part of the total.
+    const int piece = W / 16;
+    int64_t b0 = blockIdx.x / pp.size, b1 = b0;        // first and last block
+    int t0 = pp.rank, t1 = ntiles;                      // first tile of b0, end of b1's tiles
+    if (a.balanced) {
+        auto bound = [&](int64_t i, int64_t &b, int &t) {
+            const int64_t c = (i * a.blocks * a.block_cost + gridDim.x - 1) / gridDim.x;
+            b = c / a.block_cost;
+            t = (int)(c - b * a.block_cost + piece - 1) / piece;
+            if (t == ntiles) { t = 0; ++b; }
+        };
+        bound(blockIdx.x, b0, t0);
+        bound(blockIdx.x + 1, b1, t1);
+        if (t1 == 0) { t1 = ntiles; --b1; }
+    }
+
     if (tid >= TL) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCopy));
         const int t = tid - TL;
         pp.ph = 1;                                  // every stage starts empty
         bool ok = true;
         int32_t act = load_active<LAYOUT>(a, 0, t);
-        for (int it = pp.rank; it < ntiles && ok; it += pp.size)
-            for (int ck = 0; ck < pp.nck; ++ck, pp.next()) {
-                ok = wait_bounded(smem_u32(&pp.empty[pp.s]), pp.ph, pp.abort_flag, a.err, kWaitNs);
-                if (!ok) break;
-                issue<FLY, FOLD, LAYOUT>(a, stage[pp.s], l0, ck * CH, it * W, act, t);
-                act = load_active<LAYOUT>(a, ck + 1 < pp.nck ? (ck + 1) * CH : 0, t);
-                if (FLY) fly_store<FOLD>(a, stage[pp.s], ck * CH, it * W, t);
-                cp_arrive(smem_u32(&pp.full[pp.s]));
-                mbar_arrive(smem_u32(&pp.full[pp.s]));
-            }
+        for (int64_t b = b0; b <= b1 && ok; ++b) {
+            const int end = b == b1 ? t1 : ntiles;
+            for (int it = b == b0 ? t0 : 0; it < end && ok; it += pp.size)
+                for (int ck = 0; ck < pp.nck; ++ck, pp.next()) {
+                    ok = wait_bounded(smem_u32(&pp.empty[pp.s]), pp.ph, pp.abort_flag, a.err, kWaitNs);
+                    if (!ok) break;
+                    issue<FLY, FOLD, LAYOUT>(a, stage[pp.s], b * TL, ck * CH, it * W, act, t);
+                    act = load_active<LAYOUT>(a, ck + 1 < pp.nck ? (ck + 1) * CH : 0, t);
+                    if (FLY) fly_store<FOLD>(a, stage[pp.s], ck * CH, it * W, t);
+                    cp_arrive(smem_u32(&pp.full[pp.s]));
+                    mbar_arrive(smem_u32(&pp.full[pp.s]));
+                }
+        }
         cp_wait_all();
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSum));
         pp.ph = 0;
-        float bm[8];
-        int bi[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { bm[i] = -1.0f; bi[i] = INT_MAX; }
         const int full = a.ncol / W, rem = a.ncol - full * W;
-        int it = pp.rank;
-        for (; it < full; it += pp.size) phi_tile<W / 16, FOLD>(a, stage, l0, it * W, pp, bm, bi);
-        // the last, partial tile computes only the pairs-of-16 that hold grid points
-        if (it == full) {
-            switch ((rem + 15) / 16) {
-            case 1: phi_tile<1, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
-            case 2: phi_tile<2, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
-            case 3: if constexpr (!FOLD) phi_tile<3, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
-            case 4: if constexpr (!FOLD) phi_tile<4, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
-            default: break;
-            }
-        }
-        // reduce the peak over the 8 threads (tx) that share each line of sight
-        const int tx = tid & 7, ty = tid >> 3;
+        for (int64_t b = b0; b <= b1; ++b) {
+            const int64_t l0 = b * TL;
+            const int first = b == b0 ? t0 : 0, end = b == b1 ? t1 : ntiles;
+            float bm[8];
+            int bi[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float m = bm[i];
-            int k = bi[i];
-#pragma unroll
-            for (int off = 4; off >= 1; off >>= 1) {
-                const float mo = __shfl_xor_sync(0xffffffffu, m, off);
-                const int ko = __shfl_xor_sync(0xffffffffu, k, off);
-                if (better(mo, ko, m, k)) { m = mo; k = ko; }
+            for (int i = 0; i < 8; ++i) { bm[i] = -1.0f; bi[i] = INT_MAX; }
+            int it = first;
+            for (; it < min(full, end); it += pp.size) phi_tile<W / 16, FOLD>(a, stage, l0, it * W, pp, bm, bi);
+            // the last, partial tile computes only the pairs-of-16 that hold grid points
+            if (it == full && it < end) {
+                switch ((rem + 15) / 16) {
+                case 1: phi_tile<1, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
+                case 2: phi_tile<2, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
+                case 3: if constexpr (!FOLD) phi_tile<3, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
+                case 4: if constexpr (!FOLD) phi_tile<4, FOLD>(a, stage, l0, full * W, pp, bm, bi); break;
+                default: break;
+                }
             }
-            if (tx == 0) { pk_m[8 * ty + i] = m; pk_k[8 * ty + i] = k; }
+            // reduce the peak over the 8 threads (tx) that share each line of sight
+            const int tx = tid & 7, ty = tid >> 3;
+            float *const pm = pk_m + (b & 1) * TL;
+            int *const pk = pk_k + (b & 1) * TL;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                float m = bm[i];
+                int k = bi[i];
+#pragma unroll
+                for (int off = 4; off >= 1; off >>= 1) {
+                    const float mo = __shfl_xor_sync(0xffffffffu, m, off);
+                    const int ko = __shfl_xor_sync(0xffffffffu, k, off);
+                    if (better(mo, ko, m, k)) { m = mo; k = ko; }
+                }
+                if (tx == 0) { pm[8 * ty + i] = m; pk[8 * ty + i] = k; }
+            }
+            if (!a.balanced) break;
+            sum_sync();
+            float m = pm[tid];
+            int k = pk[tid];
+            bool mine = true;
+            if (first > 0 || end < ntiles) {
+                // the block's other tiles are the neighbour CTA's: whoever comes second merges
+                const int64_t slot = blockIdx.x - (first > 0 ? 1 : 0);
+                const int side = first > 0;
+                a.part_m[(2 * slot + side) * TL + tid] = m;
+                a.part_k[(2 * slot + side) * TL + tid] = k;
+                __threadfence();
+                sum_sync();
+                if (tid == 0) second = atomicAdd(a.arrived + slot, 1);
+                sum_sync();
+                mine = second != 0;
+                if (mine) {
+                    __threadfence();
+                    const float mo = __ldcg(a.part_m + (2 * slot + 1 - side) * TL + tid);
+                    const int ko = __ldcg(a.part_k + (2 * slot + 1 - side) * TL + tid);
+                    if (better(mo, ko, m, k)) { m = mo; k = ko; }
+                }
+            }
+            if (mine) write_peak(a, l0 + tid, m, k);
         }
     }
+    if (a.balanced) return;
     // the cluster's blocks hold disjoint phi of the same LOS: its first block merges them
+    float *const pm = pk_m + (b0 & 1) * TL;
+    int *const pk = pk_k + (b0 & 1) * TL;
     if (pp.size > 1) cluster.sync();
     else __syncthreads();
     if (pp.rank == 0 && tid < TL) {
-        float m = pk_m[tid];
-        int k = pk_k[tid];
+        float m = pm[tid];
+        int k = pk[tid];
         for (int r = 1; r < pp.size; ++r) {
-            const float mo = cluster.map_shared_rank(pk_m, r)[tid];
-            const int ko = cluster.map_shared_rank(pk_k, r)[tid];
+            const float mo = cluster.map_shared_rank(pm, r)[tid];
+            const int ko = cluster.map_shared_rank(pk, r)[tid];
             if (better(mo, ko, m, k)) { m = mo; k = ko; }
         }
-        const int64_t l = l0 + tid;
-        if (l < a.nlos) {
-            const bool ok = k != INT_MAX;
-            if (a.pidx) a.pidx[l] = ok ? k : -1;
-            if (a.pabs) a.pabs[l] = ok ? sqrtf(m) : __int_as_float(0x7fc00000);
-            if (a.pphi) a.pphi[l] = ok ? a.phi32[k] : __int_as_float(0x7fc00000);
-        }
+        write_peak(a, b0 * TL + tid, m, k);
     }
     if (pp.size > 1) cluster.sync();    // no block leaves while another reads its shared memory
 }
@@ -457,7 +523,7 @@ cudaError_t simt_prepare(rms_plan_s *p)
         }
         if (e != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    return cudaMalloc(reinterpret_cast<void **>(&p->d_simt_part), ((size_t)4 * TL + 1) * p->num_sms * sizeof(float));
 }
 
 cudaError_t launch_simt(const rms_plan_s &p, bool fly, const float *Q, const float *U, int64_t nlos,
@@ -491,18 +557,37 @@ cudaError_t launch_simt(const rms_plan_s &p, bool fly, const float *Q, const flo
     // One block fits an SM, and its phi tiles re-read the block's data anyway, so a
     // cluster of up to 8 blocks shares out the phi tiles of 256 LOS where that needs
     // fewer rounds of tiles over the device (the smallest such cluster).  401 phi x 360
-    // channels: 3,000 LOS 522 -> 84 us, 10,000 LOS 520 -> 207, 100,000 unchanged (measured
-    // before the copying warps; now 68, 162 and 1,180 us).
+    // channels: 3,000 LOS 522 -> 84 us, 10,000 LOS 520 -> 207 (before the copying warps;
+    // now 68 and 162 us).
     const int width = fold ? TP / 2 : TP, ntiles = (a.ncol + width - 1) / width;
-    int64_t best = INT64_MAX;
     unsigned cluster = 1;
-    for (int c = 1; c <= std::min(8, ntiles); ++c) {
-        if (p.simt_clusters[c - 1] < 1) continue;
-        const int64_t rounds = (blocks + p.simt_clusters[c - 1] - 1) / p.simt_clusters[c - 1] * ((ntiles + c - 1) / c);
-        if (rounds < best) { best = rounds; cluster = (unsigned)c; }
+    int64_t grid = blocks;
+    // More blocks than SMs: one CTA per SM takes an equal run of all blocks' phi tiles, where whole blocks
+    // in rounds would leave the last round partly empty; a run's first and last block may be shared with
+    // the neighbour CTA, whose peaks are merged by the later of the two.  401 phi x 360 channels: 60,000
+    // LOS (1.5 blocks per SM) 793 -> 674 us, 100,000 (2.6) 1,185 -> 1,066, 262,144 (6.7) 2.75 -> 2.68 ms.
+    a.balanced = blocks > p.num_sms;
+    a.blocks = blocks;
+    a.block_cost = a.ncol / width * (width / 16) + (a.ncol % width + 15) / 16;
+    if (a.balanced) {
+        grid = p.num_sms;
+        const size_t n = (size_t)2 * p.num_sms * TL;
+        a.part_m = p.d_simt_part;
+        a.part_k = reinterpret_cast<int32_t *>(p.d_simt_part + n);
+        a.arrived = a.part_k + n;
+        const cudaError_t e = cudaMemsetAsync(a.arrived, 0, p.num_sms * sizeof(int32_t), s);
+        if (e != cudaSuccess) return e;
+    } else {
+        int64_t best = INT64_MAX;
+        for (int c = 1; c <= std::min(8, ntiles); ++c) {
+            if (p.simt_clusters[c - 1] < 1) continue;
+            const int64_t rounds = (blocks + p.simt_clusters[c - 1] - 1) / p.simt_clusters[c - 1] * ((ntiles + c - 1) / c);
+            if (rounds < best) { best = rounds; cluster = (unsigned)c; }
+        }
+        grid = blocks * cluster;
     }
-    if (blocks * cluster > 0x7fffffff) return cudaErrorInvalidValue;
+    if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
     cudaLaunchAttribute attr;
-    const cudaLaunchConfig_t cfg = launch_config(&attr, (unsigned)blocks * cluster, cluster, s);
+    const cudaLaunchConfig_t cfg = launch_config(&attr, (unsigned)grid, cluster, s);
     return cudaLaunchKernelEx(&cfg, kernel_of(fly, fold, layout), a);
 }

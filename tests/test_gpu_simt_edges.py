@@ -51,3 +51,38 @@ def test_simt_pipeline_edges(rms, oracle_mod, path, sym, nchan, flagged):
         per, _ = gh.errors(Fh[..., 0] + 1j * Fh[..., 1], oracle_mod.synth(Q, U, op, phi))
         assert per.max() <= gh.TOL[path], (nphi, nlos, layout, per.max())
         gh.check_peaks_self(Fh, pi.cpu().numpy(), pa.cpu().numpy(), pp.cpu().numpy(), phi)
+
+
+# a few LOS more than one block per SM, and 1.5 to 3.1 blocks per SM with a ragged last one; one, two and several phi
+# tiles, with a whole and a partial last one
+@pytest.mark.parametrize("per_sm,extra,layout", [(1.0, 1, "chan"), (1.5, 77, "los"), (3.1, 130, "chan")])
+@pytest.mark.parametrize("nphi", [20, 64, 128, 141, 211])
+@pytest.mark.parametrize("path,sym", [("fp32_table", True), ("fp32_table", False), ("fp32_fly", True)])
+def test_simt_balanced_runs(rms, path, sym, nphi, per_sm, extra, layout):
+    """The same bits as calls of at most one block per SM, whose blocks are each one CTA's or one cluster's."""
+    nchan = 20
+    nsm = torch.cuda.get_device_properties(0).multi_processor_count
+    nlos = int(256 * nsm * per_sm) + extra
+    freq = np.linspace(120e6, 168e6, nchan)
+    phi = np.linspace(-60.0, 60.0 if sym else 63.0, nphi)
+    X = torch.randn(2, nlos, nchan, device="cuda", generator=torch.Generator("cuda").manual_seed(nphi))
+    X[:, 7] = 0.0
+    X[0, 300, 2] = float("nan")
+
+    def synth(plan, a, b):
+        n = b - a
+        q, u = ((X[i, a:b].t() if layout == "chan" else X[i, a:b]).contiguous() for i in range(2))
+        F = torch.empty(n, nphi, 2, device="cuda")
+        out = [torch.full((n,), -7, dtype=torch.int32, device="cuda")] + [torch.zeros(n, device="cuda") for _ in range(2)]
+        plan.synth(q, u, n, layout, F, *out)
+        return [F] + out
+
+    with rms.Plan(freq, phi, path) as plan:
+        got = [synth(plan, 0, nlos) for _ in range(2)]
+        step = 256 * nsm
+        parts = [synth(plan, a, min(a + step, nlos)) for a in range(0, nlos, step)]
+        plan.sync()
+    for k in range(4):
+        want = torch.cat([p[k] for p in parts]).view(torch.int32)
+        for g in got:
+            assert torch.equal(g[k].view(torch.int32), want), k
