@@ -73,6 +73,8 @@ _i32, _i64 = ctypes.c_int32, ctypes.c_int64
 def load(path: str = LIB_PATH):
     """Load librms.so (once).  Raises if it has not been built."""
     global _lib
+    if _lib is not None:        # set once, complete: no lock on the way of every call
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -169,6 +171,10 @@ def _hptr(a, dtype=None, name="array"):
 def _stream(stream):
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():
+            # the current device's current stream as a number: torch.cuda.current_stream() builds an
+            # object around it, 2.7 us of a 13 us call
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
