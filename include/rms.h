@@ -36,8 +36,10 @@
  *                                  MWA cube, BF16X3 4.6e-6 at 16 and 6.1e-6 at 32);
  *      RMS_GEMM_CTAS (1..SMs)      persistent CTAs of the contraction;
  *      RMS_HOST_CHUNK (>= 1024)    LOS per chunk of rms_synth_host.
- *  - A plan may be used from several streams.  The tensor-core precisions keep
- *    a per-plan scratch for split operands, so every synthesis call on a plan
+ *    Any of the contraction's five knobs set, a call takes the two-kernel form
+ *    (rms_synth below).
+ *  - A plan may be used from several streams and host threads.  Its scratch (device
+ *    work areas owned by the plan) is shared, so every synthesis call on a plan
  *    waits on the device for the previous call on that plan (an event recorded
  *    by each call); use one plan per stream for concurrent work.
  *    rms_synth_host owns per-plan staging buffers and must not run
@@ -157,11 +159,25 @@ rms_status rms_rmsf(rms_plan_t plan, float *R_out, double *lambda0sq, double *K,
  *  stream    cudaStream_t as void*.
  * |F| is sqrt(re*re + im*im) of the stored FP32 values, each product and the sum
  * rounded to FP32 separately, so the peak index can be recomputed bit-exactly
- * from F_out.  Asynchronous, no host sync.  The tensor-core precisions take a
+ * from F_out.
+ *
+ * On a phi grid symmetric about zero (phi_k = -phi_{nphi-1-k}, up to 1e-9 rad of
+ * phase) cos is even and sin odd in phi, and the tensor-core and FP32 SIMT
+ * precisions evaluate each depth once for both signs: half the products.  The sums
+ * are the same terms added in another order.  The tensor-core precisions then also
+ * have a one-kernel form, in which each SM pair splits its next lines of sight while
+ * it contracts the current ones; it is taken where the plan allows it (for the split
+ * precisions at most 16 K blocks of 32 active channels) and the call fills the
+ * device's pairs well enough, unless an option or knob of the contraction is set.
+ * Both forms give the same bits.
+ *
+ * Asynchronous, no host sync.  The tensor-core precisions take a
  * per-call scratch from the device's default stream-ordered memory pool on
  * `stream` (cudaMallocAsync / cudaFreeAsync): the cube split into 16-bit hi and
  * lo operands, 8 bytes per (LOS, contraction channel slot; the channels are
- * padded to a multiple of 16 per 128 LOS), and for RMS_FP16X3 one exponent
+ * padded to a multiple of 16 per 128 LOS, or 32 per 64 LOS on a symmetric grid),
+ * in the one-kernel form only those of the lines of sight in flight (at most 256
+ * per SM), and for RMS_FP16X3 one exponent
  * byte per LOS; creating a tensor-core plan sets that pool to keep freed
  * memory reserved.  The FP32 precisions allocate nothing.
  */
@@ -285,7 +301,9 @@ rms_status rms_plan_sync(rms_plan_t plan, void *stream);
 /* Plan facts for callers and tests. */
 enum {
     RMS_INFO_NCHAN = 0, RMS_INFO_NCHAN_ACTIVE = 1, RMS_INFO_NPHI = 2, RMS_INFO_PRECISION = 3,
-    RMS_INFO_KPAD = 4,        /* padded contraction length of the tensor-core operand */
+    RMS_INFO_KPAD = 4,        /* padded contraction length of the tensor-core operand
+                                 (KPAD, NPAD, TILE_N and RMS_GET_B_*: of the form for any
+                                 grid, which a symmetric one does not use) */
     RMS_INFO_NPAD = 5,        /* padded rows (2 * nphi rounded up) of the phase matrix */
     RMS_INFO_TILE_N = 6,      /* phase-matrix rows per tensor-core tile */
     RMS_INFO_DEVICE = 7,
@@ -327,9 +345,11 @@ rms_status rms_plan_set_timeout(rms_plan_t plan, int64_t ns);
 /*
  * How the tensor-core contraction of a plan is scheduled (no paper counterpart;
  * for measurement and tuning -- none of these changes a result):
- *   RMS_OPT_CONTRACTION  RMS_CONTRACT_AUTO (default): CTA pairs when the plan's pair
- *                        tiles are wider than 208 phase rows (2 nphi > 832 or so),
- *                        single CTAs otherwise; RMS_CONTRACT_SINGLE: one CTA per
+ *   RMS_OPT_CONTRACTION  RMS_CONTRACT_AUTO (default): the one-kernel form where it is
+ *                        taken (rms_synth); otherwise CTA pairs when the plan's pair
+ *                        tiles are wider than 208 phase rows (2 nphi > 832 or so, on
+ *                        a symmetric grid nphi), and for the split precisions
+ *                        with single-tile jobs, single CTAs otherwise; RMS_CONTRACT_SINGLE: one CTA per
  *                        128-row MMA with tiles of up to 208 phase rows;
  *                        RMS_CONTRACT_PAIR: CTA pairs (256-row MMAs on two SMs, each
  *                        SM holding half of a tile of up to 256 phase rows), or
@@ -357,8 +377,9 @@ rms_status rms_plan_set_option(rms_plan_t plan, int32_t option, int64_t value);
 /*
  * Kernel timing for measurement (the paper has no counterpart).  While enabled,
  * every tensor-core synthesis call on the plan records CUDA events on its
- * stream around its two kernels (the layout stage that splits the cube into
- * 16-bit operands, and the tensor-core contraction).  rms_plan_kernel_times
+ * stream around its two stages (the layout stage that splits the cube into
+ * 16-bit operands, and the tensor-core contraction; in the one-kernel form the
+ * first is empty, or RMS_FP16X3's exponents).  rms_plan_kernel_times
  * waits for the recorded events, returns the summed milliseconds of each kernel
  * and the number of calls timed (host outputs, each may be NULL), and forgets
  * them.  FP32 plans and calls made while disabled record nothing.  Timing adds

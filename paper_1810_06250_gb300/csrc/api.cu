@@ -516,7 +516,9 @@ static rms_status synth_device(rms_plan_t p, const float *Q, const float *U, int
                                float *F, int32_t *pidx, float *pabs, float *pphi, cudaStream_t s,
                                const PeakExtras &x = PeakExtras())
 {
-    // the plan's scratch is shared by its calls: order them on the device
+    // the plan's scratch is shared by its calls: order them on the device, whichever host threads make
+    // them (between one call's wait and its record no other may wait)
+    std::lock_guard<std::mutex> lock(p->mu);
     cudaError_t e = cudaStreamWaitEvent(s, p->last, 0);
     if (e != cudaSuccess) return from_cuda(e);
     rms_status st = synth_launch(p, Q, U, nlos, layout, F, pidx, pabs, pphi, s, x);

@@ -21,18 +21,21 @@
 // bytes of a channel row; bulk copies of 256-byte rows were slower, 0.83 against 0.43 ms
 // without F on 262,144 LOS x 360 x 401).  LOS-major cubes come through staging slots of
 // all channels of 8 LOS, one bulk copy per array, which leaves the channel gather to
-// shared memory and gives FP16X3 its row maxima without a second pass; where 8 rows do
-// not fit, the base is not on 16 bytes, or on a last, partial item, the splitters load
-// through registers.
-// 262,144 LOS x 360 x 401 with F: the epilogue (F stores and the peak search) is busy 65%
-// of the time and the splitters 90%; L2-evict-first loads and an evict-last ring keep the
-// ring on chip (0.507 -> 0.478 ms).
+// shared memory; where 8 rows do not fit, the base is not on 16 bytes, on a last, partial
+// item, or with one item per pair, the splitters load through registers.  FP16X3 reads its
+// exponents, a pass of their own before (fold.cu).
+// 262,144 LOS x 360 x 401 with F, channel-major, 0.49 ms: the splitters are busy 98% of the
+// time (bound by the latency of loads whose channels lie a megabyte apart), the epilogue (F
+// stores and the peak search) 78%, the MMAs 62%, most of that at the shared-memory bandwidth
+// of their operands.  LOS-major 0.49 ms: the MMAs 79%, slowed by the staging's traffic.
+// L2-evict-first loads and an evict-last ring keep the ring on chip (0.507 -> 0.478 ms).
 // Every wait is bounded, as in gemm.cu.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <limits.h>
 
 #include <algorithm>
+#include <cstdlib>
 
 #include "rms_internal.h"
 
@@ -180,6 +183,17 @@ __device__ __forceinline__ void chan_walk(const FoldSource &S, const int *list, 
         if (h + 4 < nh) load(h + 4, a);
         if (h + 2 < nh) masked(h + 2, b);
     }
+}
+
+// 64 bytes at a 32-byte aligned address
+__device__ __forceinline__ void load64(const float *p, float (&v)[16])
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        asm volatile("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(v[8 * h]), "=f"(v[8 * h + 1]), "=f"(v[8 * h + 2]), "=f"(v[8 * h + 3]), "=f"(v[8 * h + 4]),
+                       "=f"(v[8 * h + 5]), "=f"(v[8 * h + 6]), "=f"(v[8 * h + 7])
+                     : "l"(p + 8 * h));
 }
 
 // (q + iu) t
@@ -641,25 +655,26 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                     const int64_t at = min(los0 + i, nlos - 1);
                     const bool valid = los0 + i < nlos;
                     const int r0 = 16 * (i >> 3) + (i & 7), sz = (r0 >> 1) & 3;
-                    for (int c = 0; c << P.chunk_log < P.kblocks; ++c) {
-                    const int o_end = 4 * min(P.kblocks, (c + 1) << P.chunk_log);
-                    for (int o = (4 * c << P.chunk_log) + (sw >> 1); o < o_end; o += kNumSplitWarps / 2) {
-                        float q[8], u[8];
-                        float4 t[4];
+                    auto load = [&](int o, float (&q)[8], float (&u)[8]) {
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             const int64_t off = (int64_t)S.list[8 * o + j] * nlos + at;
                             q[j] = load_here<true>(P.src.Q + off);
                             u[j] = load_here<true>(P.src.U + off);
                         }
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) t[j] = __ldg(reinterpret_cast<const float4 *>(T + 8 * o) + j);
-                        uint32_t qh[4], ql[4], uh[4], ul[4];
+                    };
+                    // T of octet o at this LOS, in two loads of 32 bytes: every lane has a row (and a
+                    // cache line per load) of its own
+                    float t[16];
+                    auto load_t = [&](int o) { load64(reinterpret_cast<const float *>(T + 8 * o), t); };
+                    auto work = [&](int o, int next, float (&q)[8], float (&u)[8]) {
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             if (8 * o + j >= P.src.nact || !valid) q[j] = u[j] = 0.f;
-                            rotate(q[j], u[j], j & 1 ? make_float2(t[j >> 1].z, t[j >> 1].w) : make_float2(t[j >> 1].x, t[j >> 1].y));
+                            rotate(q[j], u[j], make_float2(t[2 * j], t[2 * j + 1]));
                         }
+                        load_t(next);
+                        uint32_t qh[4], ql[4], uh[4], ul[4];
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             split_pair_bf16(q[2 * j], q[2 * j + 1], qh[j], ql[j]);
@@ -672,8 +687,25 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                             *reinterpret_cast<uint4 *>(d + kFoldPart) = make_uint4(ql[0], ql[1], ql[2], ql[3]);
                             *reinterpret_cast<uint4 *>(d + kFoldPart + 8 * kFoldRowBytes) = make_uint4(ul[0], ul[1], ul[2], ul[3]);
                         }
-                    }
-                    release(c);
+                    };
+                    // a warp's octets are one to a K block; the next one's values and T are in flight (whole
+                    // 32-byte sectors, two octets at a time, leave no registers for that: 1,048,576 LOS
+                    // learned peak map 5.24 ms, against 5.01 this way and 5.38 with nothing ahead)
+                    constexpr int kStep = kNumSplitWarps / 2;
+                    static_assert(kStep == 4, "one octet of every K block per warp");
+                    for (int c = 0; c << P.chunk_log < P.kblocks; ++c) {
+                        const int o1 = 4 * min(P.kblocks, (c + 1) << P.chunk_log), last = o1 - kStep + (sw >> 1);
+                        float qa[8], ua[8], qb[8], ub[8];
+                        int o = (4 * c << P.chunk_log) + (sw >> 1);
+                        load_t(o);
+                        load(o, qa, ua);
+                        for (; o < o1; o += 2 * kStep) {
+                            if (o + kStep < o1) load(o + kStep, qb, ub);
+                            work(o, min(o + kStep, last), qa, ua);
+                            if (o + 2 * kStep < o1) load(o + 2 * kStep, qa, ua);
+                            if (o + kStep < o1) work(o + kStep, min(o + 2 * kStep, last), qb, ub);
+                        }
+                        release(c);
                     }
                 } else {
                 uint8_t *const dst = tile + row * kFoldRowBytes;
@@ -922,16 +954,21 @@ cudaError_t fused_prepare(rms_plan_s *p, bool window)
 
 // One kernel unless the last round of items over the pairs is too empty (12,000 LOS are 94
 // items on 76 pairs: 69.9 against 64.2 us at 360 channels x 801 phi, but 161 items on two
-// thirds of three rounds 99.0 against 104) or there are few items with many phase tiles,
+// thirds of three rounds 96 against 104) or there are few items with many phase tiles,
 // which the job schedule spreads over more SMs.  Measured with F and the peak map, one
-// kernel against two:
-// 262,144 LOS x 360 x 401 BF16x3 0.474 / 0.636 ms (LOS-major 0.484 / 0.642), 200,003 x
-// 357 x 401 FP16x3 LOS-major 0.535 / 0.612, 400,000 x 800 x 1001 BF16 1.53 / 2.04 ms,
-// 5,000 LOS x 360 x 401 32.6 / 36.1 us.
+// kernel against two: 262,144 LOS x 360 x 401 BF16x3 0.459 / 0.611 ms (LOS-major 0.454 /
+// 0.611), FP16x3 0.590 / 0.741, 200,003 LOS FP16x3 LOS-major 0.470 / 0.583, 400,000 x 800
+// x 1001 BF16 1.41 / 1.99 ms, 5,001 LOS x 360 x 401 34.7 / 42.9 us (timing events included).
 bool fused_wanted(const rms_plan_s &p, int64_t nlos)
 {
     const FoldPlan &f = p.fold;
-    if (f.fused_pairs < 1 || p.contraction != RMS_CONTRACT_AUTO || p.schedule != RMS_SCHEDULE_AUTO || p.l2_budget != 0)
+    // options and knobs of the contraction kernel take a call there
+    static const bool knobs = [] {
+        for (const char *v : {"RMS_GEMM_PAIR", "RMS_GEMM_CTAS", "RMS_L2_BUDGET_MB", "RMS_GROUP_KBLOCKS", "RMS_MAX_TILE_N"})
+            if (std::getenv(v)) return true;
+        return false;
+    }();
+    if (f.fused_pairs < 1 || p.contraction != RMS_CONTRACT_AUTO || p.schedule != RMS_SCHEDULE_AUTO || p.l2_budget != 0 || knobs)
         return false;
     const int64_t nit = (nlos + 2 * kFoldTileLos - 1) / (2 * kFoldTileLos);
     const int64_t rounds = (nit + f.fused_pairs - 1) / f.fused_pairs;

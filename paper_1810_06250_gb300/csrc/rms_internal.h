@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <vector>
 
 #include "../../include/rms.h"
@@ -55,6 +56,7 @@ struct FoldPlan {
 };
 
 struct rms_plan_s {
+    std::mutex mu;                 // queueing a synthesis call
     int device = 0;
     int32_t nchan = 0, nact = 0, nphi = 0, precision = 0;
     double K = 0, lambda0sq = 0, wmax = 0, fwhm_meas = 0, fwhm_est = 0;

@@ -86,3 +86,35 @@ def test_simt_balanced_runs(rms, path, sym, nphi, per_sm, extra, layout):
         want = torch.cat([p[k] for p in parts]).view(torch.int32)
         for g in got:
             assert torch.equal(g[k].view(torch.int32), want), k
+
+
+def test_simt_two_threads_one_plan(rms):
+    """Calls that share blocks between CTAs, on one plan from two host threads and streams: the plan orders them."""
+    import threading
+    nchan, nphi = 12, 64
+    nsm = torch.cuda.get_device_properties(0).multi_processor_count
+    nlos = 256 * nsm + 256 * 40
+    X = torch.randn(2, 2, nchan, nlos, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    out = [[[torch.empty(nlos, dtype=torch.int32, device="cuda"), torch.empty(nlos, device="cuda")] for _ in range(20)] for _ in range(2)]
+    with rms.Plan(np.linspace(120e6, 168e6, nchan), np.linspace(-60.0, 60.0, nphi), "fp32_table") as plan:
+        want = []
+        for t in range(2):
+            want.append([torch.empty(nlos, dtype=torch.int32, device="cuda"), torch.empty(nlos, device="cuda")])
+            plan.synth(X[t, 0], X[t, 1], nlos, "chan", None, *want[t])
+        torch.cuda.synchronize()
+
+        def work(t):
+            s = torch.cuda.Stream()
+            for i, a in out[t]:
+                plan.synth(X[t, 0], X[t, 1], nlos, "chan", None, i, a, stream=s)
+            s.synchronize()
+
+        threads = [threading.Thread(target=work, args=(t,)) for t in range(2)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        plan.sync()
+    for t in range(2):
+        for i, a in out[t]:
+            assert torch.equal(i, want[t][0]) and torch.equal(a, want[t][1])
