@@ -298,12 +298,14 @@ def load_peaks():
         return {}
 
 
-def tensor_roofline(path, useful_flops, kt, timed_s, peaks, traffic, step_ms, hbm_bytes):
+def tensor_roofline(path, useful_flops, kt, timed_s, peaks, traffic, step_ms, hbm_bytes, folded, kernel):
     """Roofline of the contraction kernel (the dominant one): the method's own work,
     8 flop per (LOS, active channel, phi) unit, over the dense BF16 tensor peak.
-    The split precisions issue three 16-bit products per useful flop, so they can
-    reach at most 1/3 of that peak; the issued products are reported beside it."""
-    terms = 1 if path == "bf16" else 3
+    The split precisions issue three 16-bit products per multiply-add, and a phi grid
+    symmetric about zero needs half the multiply-adds (both signs of a depth share
+    theirs), so a split precision can reach at most 1/3, or folded 2/3, of that peak;
+    the issued products are reported beside it."""
+    terms = (1 if path == "bf16" else 3) * (0.5 if folded else 1.0)
     burst, sust = peaks.get("bf16_tflops"), peaks.get("bf16_tflops_sustained")
     kind = "measured"
     if not burst or not sust:
@@ -313,7 +315,7 @@ def tensor_roofline(path, useful_flops, kt, timed_s, peaks, traffic, step_ms, hb
     split_ms, gemm_ms, ncalls = kt
     gemm_launch_ms = gemm_ms / max(1, ncalls)
     achieved = useful_flops / (gemm_launch_ms * 1e-3) / 1e12
-    return {"kernel": "gemm_kernel (tensor-core contraction + fused epilogue)", "bound": "tensor",
+    return {"kernel": kernel, "bound": "tensor", "folded_grid": folded,
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic,
             "traffic_unit": "bytes per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
             "peak_source": "%s %s dense BF16 tensor peak (MEASURED_PEAKS.json %s): the timed region lasted %.2f s, %s"
@@ -330,8 +332,9 @@ def tensor_roofline(path, useful_flops, kt, timed_s, peaks, traffic, step_ms, hb
             "algorithmic": "8 flop per (LOS, active channel, phi) unit (one complex multiply-add); achieved = "
                            "algorithmic flop per launch / the contraction kernel's CUDA-event duration (the "
                            "library's event hook on the launching stream, averaged over the timed launches); "
-                           "FP16 and BF16 share the dense tensor rate; a split precision issues %d 16-bit products "
-                           "per flop, so split_ceiling_frac is its best possible frac" % terms}
+                           "FP16 and BF16 share the dense tensor rate; this path issues %g 16-bit products "
+                           "per flop (3 per multiply-add if split, half the multiply-adds on a grid symmetric "
+                           "about zero), so split_ceiling_frac is its best possible frac" % terms}
 
 
 def measure_cube(args, cfg_name, path, layout, steps, warmup, dev, local, world=1, barrier=None, nlos=None,
@@ -391,16 +394,22 @@ def measure_cube(args, cfg_name, path, layout, steps, warmup, dev, local, world=
     hbm_bytes = L * (8.0 * (nact if layout == "chan" else cfg.nchan) + (0 if peak_only else 8.0 * cfg.nphi) + 12.0)
     full_size = nlos is None and not peak_only
     if tensor_path:
-        traffic = measured_traffic("gemm.cu", "gemm_%s_bf16x3.md" % cfg_name) \
+        # the one-kernel form (pairs, no job panels, no layout kernel to speak of), or the contraction
+        fused = bool(sched["cta_pairs"]) and sched["n_panels"] == 0 and kt[0] < 0.5 * kt[1] and \
+            (not peak_only or kt[0] < 0.02 * kt[1])
+        src, summary = ("fused.cu", "fused_%s_bf16x3.md") if fused else ("gemm.cu", "gemm_%s_bf16x3.md")
+        summary = summary % cfg_name
+        traffic = measured_traffic(src, summary) \
             if (path == "bf16x3" and layout == "chan" and full_size) else None
-        roof = tensor_roofline(path, useful_flops, kt, total_ms * 1e-3, peaks, traffic, avg_launch_ms, hbm_bytes)
+        folded = bool(np.max(np.abs(phi + phi[::-1])) <= 1e-9 * np.max(np.abs(phi)))
+        roof = tensor_roofline(path, useful_flops, kt, total_ms * 1e-3, peaks, traffic, avg_launch_ms, hbm_bytes, folded,
+                               "fused_kernel (split, tensor-core contraction and epilogue)" if fused
+                               else "gemm_kernel (tensor-core contraction + fused epilogue)")
         if traffic is not None:
             # the ncu counters of the same capture (a smaller case of this workload, same kernel source)
-            roof["ncu"] = {"summary": "profiles/gemm_%s_bf16x3.md" % cfg_name,
-                           "tensor_pipe_active_pct": profile_value("gemm.cu", "gemm_%s_bf16x3.md" % cfg_name,
-                                                                   "tensor_pipe_active_pct"),
-                           "dram_throughput_pct": profile_value("gemm.cu", "gemm_%s_bf16x3.md" % cfg_name,
-                                                                "dram_throughput_pct"),
+            roof["ncu"] = {"summary": "profiles/" + summary,
+                           "tensor_pipe_active_pct": profile_value(src, summary, "tensor_pipe_active_pct"),
+                           "dram_throughput_pct": profile_value(src, summary, "dram_throughput_pct"),
                            "hbm_gbs_full_size": traffic / (roof["launch_ms"] * 1e-3) / 1e9}
         roof["schedule"] = dict(sched, note="n_panels 0: each CTA runs every phase tile of its M tile; k > 0: "
                                             "single-tile jobs in k panels of the phase matrix, peaks merged by "
@@ -440,6 +449,8 @@ def measure_cube(args, cfg_name, path, layout, steps, warmup, dev, local, world=
             if (path == "fp32_table" and layout == "chan" and cfg_name == "lofar" and full_size) else None
         roof = {"kernel": "simt_kernel", "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak,
+                # a grid symmetric about zero needs half the multiply-adds
+                "issued_frac": achieved / peak * (0.5 if np.max(np.abs(phi + phi[::-1])) <= 1e-9 * np.max(np.abs(phi)) else 1.0),
                 "traffic": traffic, "traffic_unit": "bytes per launch (ncu dram read + write)",
                 "peak_source": "SMs x 128 FP32 lanes x 2 x max SM clock",
                 "hbm_gbs": hbm_bytes / (avg_launch_ms * 1e-3) / 1e9}
