@@ -515,6 +515,7 @@ fused_kernel(const __grid_constant__ FusedParams P, const __grid_constant__ CUte
                 };
                 for (int c0 = 0; c0 < mine; c0 += 32) {
                     uint32_t v[2][16];
+                    __syncwarp();       // (lanes may have parted over the stores and peaks of the columns before)
                     tmem_ld16x256x4(taddr + c0, v[0]);
                     tmem_ld16x256x4(taddr + (16u << 16) + c0, v[1]);
                     tmem_wait_ld();

@@ -126,10 +126,13 @@ __device__ __forceinline__ void item_coords(const NetGemmParams &P, int64_t it, 
 }
 
 // N accumulator columns of this thread's row, starting at column c0 (fewer before column end).
+// TMEM loads are warp-collective (.sync.aligned), so lanes that parted over the columns before
+// (rows beyond M, unmapped columns, a new maximum) meet here first.
 template <int N>
 __device__ __forceinline__ void load_cols(uint32_t taddr, int c0, int end, float (&v)[N])
 {
     uint32_t r[N / 8][8];
+    __syncwarp();
 #pragma unroll
     for (int j = 0; j < N / 8; ++j)
         if (c0 + 8 * j < end) tmem_ld8(taddr + c0 + 8 * j, r[j]);
@@ -196,17 +199,17 @@ __device__ void epilogue(const NetGemmParams &P, const NSmem &SM, const float *b
         const int rq = lane >> 2, cq = lane & 3;
         for (int c0 = c_lo; c0 < c_hi; c0 += 8) {
             uint32_t v[2][4];
+            __syncwarp();
             tmem_ld16x256(tacc + c0, v[0]);
             tmem_ld16x256(tacc + (16u << 16) + c0, v[1]);
             tmem_wait_ld();
             const int n = n_base + c0 + 2 * cq;
-            if (n >= P.N) continue;                 // N is even, and so are the mapped pairs
-            const int col = P.colmap ? P.colmap[n] : n;
-            if (col < 0) continue;
+            // N is even, and so are the mapped pairs; -1: beyond the gradient, or an image column of no weight
+            const int col = n >= P.N ? -1 : P.colmap ? P.colmap[n] : n;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int64_t row = (int64_t)mt * kTileM + 32 * q + 16 * (i >> 1) + 8 * (i & 1) + rq;
-                if (row < P.M)
+                if (col >= 0 && row < P.M)
                     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(P.outf + row * P.ldf + col),
                                  "f"(__uint_as_float(v[i >> 1][2 * (i & 1)])), "f"(__uint_as_float(v[i >> 1][2 * (i & 1) + 1]))
                                  : "memory");
@@ -397,6 +400,7 @@ __device__ void epilogue(const NetGemmParams &P, const NSmem &SM, const float *b
 #pragma unroll 1
             for (int c0 = g0 & ~7; c0 < g1; c0 += 16) {
                 uint32_t rr[2][8];
+                __syncwarp();
                 tmem_ld8(tacc + c0, rr[0]);
                 if (c0 + 8 < c_hi) tmem_ld8(tacc + c0 + 8, rr[1]);
                 tmem_wait_ld();
