@@ -171,10 +171,11 @@ def _hptr(a, dtype=None, name="array"):
 def _stream(stream):
     if stream is None:
         import torch
-        if torch.cuda.is_initialized():
-            # the current device's current stream as a number: torch.cuda.current_stream() builds an
-            # object around it, 2.7 us of a 13 us call
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        # the current device's current stream as a number: torch.cuda.current_stream() builds an
+        # object around it, 2.7 us of a 13 us call.  The two functions are private to torch.
+        raw, device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+        if raw and device and torch.cuda.is_initialized():
+            return raw(device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
