@@ -57,8 +57,17 @@ constexpr int kTmemCols = 512;
 constexpr int kAccStride = 256;
 constexpr int kHalf = kMaxTileN / 2;              // 104 columns per epilogue thread
 constexpr int kHalfWide = 128;                    // CTA pairs: tiles of up to 256 phase rows
-constexpr int kRegsLaunch = 168, kRegsCtl = 56, kRegsEpi = 224;   // setmaxnreg split of the wide variant
-static_assert(128 * kRegsCtl + 256 * kRegsEpi == kThreads * kRegsLaunch, "register split must fill the launch");
+// setmaxnreg split: the control warpgroup's and an epilogue thread's registers, of kRegsLaunch at launch.
+// The epilogue of a 256-row tile (128 sums) takes all it can; beside that of 208 rows the control warps
+// have 72, which the warp-convergent MMA issuer of a general grid fills: with 56 it spilled (48 bytes
+// stored, 204 loaded; 262,144 LOS x 360 x 401 asymmetric, plain BF16 with F 0.656 -> 0.634 ms).
+// The issuer on one lane (LANE, below) needs no more than 56.
+constexpr int kRegsLaunch = 168;
+constexpr int regs_ctl(int half, bool lane) { return half > 104 || lane ? 56 : 72; }
+constexpr int regs_epi(int half, bool lane) { return half > 104 || lane ? 224 : 216; }
+static_assert(128 * regs_ctl(104, false) + 256 * regs_epi(104, false) == kThreads * kRegsLaunch &&
+                  128 * regs_ctl(104, true) + 256 * regs_epi(104, true) == kThreads * kRegsLaunch,
+              "register split must fill the launch");
 constexpr int kHalfRot = 64;                      // rotating (window) kernel: tile_n <= 128
 constexpr int kEpiCols = 8;                       // staging chunk: 8 columns x 32 rows per warp
 constexpr int kEpiLd = kEpiCols + 1;
@@ -499,8 +508,8 @@ __device__ __forceinline__ void job_of(const GemmParams &P, int64_t nit, int64_t
 // rows in shared memory before the MMA reads them.  PAIR: the two-CTA variant
 // (launched in clusters of two; not combined with ROT).  FOLD: the phi grid is
 // symmetric and a tile holds 64 LOS (see fold.cu): P.nphi is then the number of
-// column pairs (i.e. of +-phi pairs).
-template <int HALF, bool ROT, bool PAIR, bool FOLD>
+// column pairs (i.e. of +-phi pairs).  LANE: the MMA issuer's loop on one lane.
+template <int HALF, bool ROT, bool PAIR, bool FOLD, bool LANE = false>
 __global__ void __launch_bounds__(ROT ? 512 : kThreads, 1)
 gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtensorMap tmB_hi,
             const __grid_constant__ CUtensorMap tmB_lo, const __grid_constant__ CUtensorMap tmA)
@@ -565,7 +574,7 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
     // two epilogue warpgroups at the top of their branches; the shares add up to the
     // launch's 384 x 168 registers (checked on the host before the first launch).
     if (warp < 4) {
-    if constexpr (!ROT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCtl));
+    if constexpr (!ROT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_ctl(HALF, LANE)));
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
@@ -654,14 +663,15 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
         if (PAIR && !leader) {
             // the even CTA's last commit: all MMAs that touch this CTA are complete
             if (lane == 0 && !wait_bounded(smem_u32(S.mma_done), 0, S.abort_flag, P.err, P.timeout_ns)) stop_peer();
-        } else {
+        } else if (!LANE || lane == 0) {
             // -------------------------------------------------------- MMA issuer
             // The warp runs convergent and one elected lane issues: its addresses and
             // descriptors then stay in uniform registers.  With the loop on a single lane
             // the issue, not the tensor pipe, set the pace (peak map only, pairs: 262,144
             // LOS x 360 x 401 BF16x3 0.318 -> 0.303 ms; 400,000 x 800 x 1001 BF16 with
-            // four K blocks per stage 1.23 -> 1.00 ms).
-            const uint32_t one = elect_one();
+            // four K blocks per stage 1.23 -> 1.00 ms).  LANE: the loop on lane 0, for calls
+            // that F's stores bound (launch_gemm).
+            const uint32_t one = LANE ? 1u : elect_one();
             const bool bf = P.mode != MODE_FP16X3;
             const int mrows = PAIR ? 2 * kTileM : kTileM;
             const uint32_t id_full = idesc_f16_m(mrows, P.tile_n, bf), id_last = idesc_f16_m(mrows, P.tile_n_last, bf);
@@ -672,7 +682,7 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
             auto arrived = [&](const uint64_t *bar, uint32_t parity) {
                 const bool in = PAIR ? wait_bounded_cluster(smem_u32(bar), parity, S.abort_flag, P.err, P.timeout_ns)
                                      : wait_bounded(smem_u32(bar), parity, S.abort_flag, P.err, P.timeout_ns);
-                return __all_sync(0xffffffffu, in) != 0;
+                return LANE ? in : __all_sync(0xffffffffu, in) != 0;
             };
             for (int64_t j = it0; j < njobs && ok; j += istride) {
                 int64_t it;
@@ -802,7 +812,7 @@ gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtens
                 }
         }
     } else if (warp >= kEpiWarp0 && warp < kEpiWarp0 + kNumEpiWarps) {
-        if constexpr (!ROT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
+        if constexpr (!ROT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(regs_epi(HALF, LANE)));
         if constexpr (!ROT) {
             // ------------------------------------------------------------ epilogue
             // 16x256b TMEM loads: in each 16-lane block l of the quarter, thread t holds
@@ -1477,9 +1487,10 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
         // launching one with any other register count would leave its epilogue
         // warpgroups waiting for registers, so check the build once
         static const cudaError_t regs_ok = [] {
-            const KernelFn ks[6] = {gemm_kernel<kHalf, false, false, false>,    gemm_kernel<kHalf, false, true, false>,
+            const KernelFn ks[7] = {gemm_kernel<kHalf, false, false, false>,    gemm_kernel<kHalf, false, true, false>,
                                     gemm_kernel<kHalfWide, false, true, false>, gemm_kernel<kHalf, false, false, true>,
-                                    gemm_kernel<kHalf, false, true, true>,      gemm_kernel<kHalfWide, false, true, true>};
+                                    gemm_kernel<kHalf, false, true, true>,      gemm_kernel<kHalfWide, false, true, true>,
+                                    gemm_kernel<kHalf, false, false, false, true>};
             for (const KernelFn k : ks) {
                 cudaFuncAttributes fa;
                 cudaError_t e1 = cudaFuncGetAttributes(&fa, k);
@@ -1591,9 +1602,16 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
         if (e != cudaSuccess) return e;
     } else {
         if (P.tile_n > 2 * kHalf) return cudaErrorInvalidValue;
+        // Plain BF16 with F and a short contraction is bound by F's stores and the operands' traffic, and
+        // operands that the faster warp-convergent issuer demands earlier cost more than they give (general
+        // grids; on one lane against the warp, and one K block per stage on one lane: 262,144 LOS x 360 x 401
+        // 0.607 / 0.634 / 0.605 ms, LOS-major 0.688 / 0.685 / 0.690, 100,000 x 64 x 301 131 / 133 / 135 us).
+        // Long contractions prefer the warp: 100,000 x 1000 x 101 280 / 276 us, 50,000 x 1536 x 401 376 / 362.
+        const bool lane = !fold && mode == MODE_BF16 && o.F && P.kblocks <= 40;
         const CUtensorMap &bhi = fold ? p.fold.tmap_bhi : chan ? p.tmap_bhi : p.tmap_bhi_raw;
         const CUtensorMap &blo = fold ? p.fold.tmap_blo : chan ? p.tmap_blo : p.tmap_blo_raw;
-        auto kern = fold ? gemm_kernel<kHalf, false, false, true> : gemm_kernel<kHalf, false, false, false>;
+        auto kern = fold ? gemm_kernel<kHalf, false, false, true>
+                  : lane ? gemm_kernel<kHalf, false, false, false, true> : gemm_kernel<kHalf, false, false, false>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         kern<<<units, kThreads, smem, s>>>(P, bhi, blo, bhi);   // (the last map is unused here)
