@@ -1471,7 +1471,7 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
         // one K block per stage, 1.02 at two, 1.00 at four).
         for (int c = 4; c > 1; c /= 2)
             if (gemm_stages(P.b_rows, mode, c) >= 3) { P.kbs = c; break; }
-        P.group = (P.group + P.kbs - 1) / P.kbs * P.kbs;
+        // (a group's last stage may hold fewer: its chain of MMAs is what RMS_GROUP_KBLOCKS says)
     }
     P.stages = gemm_stages(P.b_rows, mode, P.kbs);
     if (P.stages < 2) return cudaErrorInvalidConfiguration;
