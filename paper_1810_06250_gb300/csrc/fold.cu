@@ -194,7 +194,60 @@ __global__ void __launch_bounds__(256, 4) fold_split_los_kernel(const FoldSplitP
     }
 }
 
+// The folded image of gathered lines of sight, from an interleaved image (gemm.cu) that holds the same 16-bit parts: one
+// 64-LOS tile and K block per CTA, 8 channels of a LOS per thread.  A row's 64 bytes per 16 channels are contiguous there,
+// where a channel-major cube gives one value of every 32-byte sector to a gathered LOS.
+__global__ void __launch_bounds__(4 * kFoldTileLos) fold_gather_kernel(const uint8_t *src, int32_t src_kblocks,
+                                                                       const int32_t *column, int32_t nact,
+                                                                       const int64_t *rows, const int64_t *count,
+                                                                       int64_t nmax, int32_t parts, uint8_t *dst)
+{
+    const int i = threadIdx.x >> 2, c = threadIdx.x & 3, kb = blockIdx.y;
+    const int64_t n = min(*count, nmax), j = (int64_t)blockIdx.x * kFoldTileLos + i;
+    if ((int64_t)blockIdx.x * kFoldTileLos >= n) return;
+    const int64_t r = rows[min(j, n - 1)];
+    const int ms = (int)(r % kTileM), sws = (ms >> 1) & 3;
+    const uint8_t *const from = src + (size_t)(r / kTileM) * src_kblocks * kBlock + ms * kFoldRowBytes;
+    const int at = 16 * (i >> 3) + (i & 7), sw = (at >> 1) & 3;
+    uint8_t *const to = dst + ((size_t)blockIdx.x * gridDim.y + kb) * kBlock + at * kFoldRowBytes + ((c ^ sw) << 4);
+    for (int part = 0; part < parts; ++part) {
+        uint32_t v[8];                  // (Q, U) of 8 channels
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int a = kb * kKBlock + 8 * c + e;
+            v[e] = 0u;
+            if (a < nact && j < n) {
+                const int ch = column ? __ldg(column + a) : a;
+                v[e] = *reinterpret_cast<const uint32_t *>(from + (size_t)(ch >> 4) * kBlock + part * kFoldPart +
+                                                           ((((ch >> 2) & 3) ^ sws) << 4) + 4 * (ch & 3));
+            }
+        }
+        uint32_t q[4], u[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            q[e] = __byte_perm(v[2 * e], v[2 * e + 1], 0x5410);
+            u[e] = __byte_perm(v[2 * e], v[2 * e + 1], 0x7632);
+        }
+        *reinterpret_cast<uint4 *>(to + part * kFoldPart) = make_uint4(q[0], q[1], q[2], q[3]);
+        *reinterpret_cast<uint4 *>(to + part * kFoldPart + 8 * kFoldRowBytes) = make_uint4(u[0], u[1], u[2], u[3]);
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_fold_gather(const rms_plan_s &p, int layout, const uint8_t *src, const int64_t *rows,
+                               const int64_t *count, int64_t nmax, uint8_t *dst, cudaStream_t s)
+{
+    const bool chan = layout == RMS_CHAN_MAJOR;
+    const int64_t tiles = (nmax + kFoldTileLos - 1) / kFoldTileLos;
+    if (tiles < 1) return cudaSuccess;
+    if (tiles > 0x7fffffff || p.fold.kblocks > 65535) return cudaErrorInvalidValue;
+    // a channel-major image's columns are the active channels, a LOS-major one's all channels
+    fold_gather_kernel<<<dim3((unsigned)tiles, (unsigned)p.fold.kblocks), 4 * kFoldTileLos, 0, s>>>(
+        src, chan ? p.kblocks : p.kblocks_raw, chan ? nullptr : p.d_active, p.nact, rows, count, nmax,
+        p.precision == RMS_BF16 ? 1 : 2, dst);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_fold_exponents(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout,
                                   int8_t *rexp, cudaStream_t s)

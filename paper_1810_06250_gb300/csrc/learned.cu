@@ -13,10 +13,11 @@
 // 0.69 -> 0.37 ms against the split and the rotating contraction, which multiplies in
 // shared memory and serves the longer BF16X3 channel lists).
 //
-// Learned peak map: (1) the network on a BF16 image of the cube, scaled by 1/RMS per
-// row, (2) window synthesis around 2 * proposed bin, (3) for the LOS that fall back
-// (confidence below tau or NaN, window maximum on the window edge or absent) the
-// layout stage and the full-grid contraction on those rows only.
+// Learned peak map: (1) the network on an operand image of the cube, scaled by 1/RMS
+// per row, (2) window synthesis around 2 * proposed bin, from the cube or from that image
+// (window_from_image), (3) for the LOS that fall back (confidence below tau or NaN, window
+// maximum on the window edge or absent) their folded operands, from the image or the
+// cube, and the full-grid contraction on those rows only.
 #include <math.h>
 
 #include <algorithm>
@@ -158,6 +159,22 @@ cudaError_t window_contract(const rms_window_s &w, const uint8_t *img, int64_t n
     go.cmin = w.cmin;
     go.cmax = w.cmax;
     return launch_gemm(*w.sub, go, s);
+}
+
+// Whether the learned peak map's window reads the network's image (hi and lo parts) through the rotating
+// contraction, or the cube once more in one kernel.  The image is there anyway, so the one kernel pays only
+// where the image then keeps its hi parts alone (BF16X3 on grids that fold) and the cube's rows are
+// contiguous (LOS-major), and for calls of at most one item per CTA pair, where the two cost the same and
+// the bits are rms_synth_window's.  Whole call, 360 channels x 401 phi, image / cube, the network's confidence
+// ignored: channel-major BF16X3 8,192 LOS 109 / 111 us, 16,384 135 / 152, 262,144 0.99 / 1.16 ms, 1,048,576
+// 3.65 / 4.33; BF16 3.02 / 3.89, LOS-major 3.22 / 3.65; LOS-major BF16X3 4.10 / 3.56 ms, on an asymmetric
+// grid 4.13 / 4.22 (16,384 LOS 168 / 181 us).
+bool window_from_image(const rms_window_s &w, int64_t nlos, int32_t layout)
+{
+    const int32_t pairs = w.sub->fold.fused_pairs;
+    if (pairs < 1) return true;
+    const bool whole = w.sub->precision == RMS_BF16 || !w.plan->fold.on;      // the image, in any case
+    return nlos > (int64_t)2 * kFoldTileLos * pairs && (layout == RMS_CHAN_MAJOR || whole);
 }
 
 }  // namespace
@@ -310,7 +327,7 @@ rms_status rms_peakmap_learned(rms_window_t w, rms_net_t net, const float *Q, co
     // the fallback rows' image: folded like rms_synth's wherever the plan's grid folds
     const size_t ib_fb = p.fold.on ? up(fold_operand_bytes(p, nlos)) : ib;
     // image | fallback image | h | rscale | bin | conf | centre | widx | wabs | rows | count | peak keys
-    const bool one = w->sub->fold.fused_pairs > 0;
+    const bool one = !window_from_image(*w, nlos, layout);
     const size_t rb = one ? up(fused_ring_bytes(*w->sub, nlos)) : 0;
     const size_t total = ib + ib_fb + hb + 7 * n4 + 2 * n8 + 256 + rb;
     uint8_t *scr = nullptr;
@@ -378,8 +395,13 @@ rms_status rms_peakmap_learned(rms_window_t w, rms_net_t net, const float *Q, co
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
-        e = p.fold.on ? launch_fold_split(p, Q, U, nlos, layout, img_fb, nullptr, s, rows, count)
-                      : launch_image_gather(p, layout, img, rows, count, nlos, img_fb, s);
+        // A folded grid's fallback rows come from a channel-major image that holds all their parts (a LOS there is
+        // one value of every 32-byte sector of the cube: BF16, 1,048,576 LOS, one in ten falling back 3.38 -> 3.02
+        // ms), else from the cube (LOS-major 3.22 against 3.30 ms).
+        e = !p.fold.on ? launch_image_gather(p, layout, img, rows, count, nlos, img_fb, s)
+            : layout == RMS_CHAN_MAJOR && (!one || p.precision == RMS_BF16)
+                ? launch_fold_gather(p, layout, img, rows, count, nlos, img_fb, s)
+                : launch_fold_split(p, Q, U, nlos, layout, img_fb, nullptr, s, rows, count);
     if (e == cudaSuccess) {
         GemmOpts go;
         go.A = img_fb;

@@ -183,6 +183,9 @@ cudaError_t launch_fold_exponents(const rms_plan_s &p, const float *Q, const flo
 cudaError_t launch_fold_split(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout,
                               uint8_t *A, int8_t *rexp, cudaStream_t s, const int64_t *rows = nullptr,
                               const int64_t *count = nullptr);
+// The folded image of rows rows[0 .. *count - 1] of an interleaved image of the same precision (fold.cu)
+cudaError_t launch_fold_gather(const rms_plan_s &p, int layout, const uint8_t *src, const int64_t *rows,
+                               const int64_t *count, int64_t nmax, uint8_t *dst, cudaStream_t s);
 // fused.cu: layout stage and contraction in one kernel, for plans whose K blocks form one
 // accumulation (fused_prepare, at plan creation) and calls of enough LOS (fused_wanted)
 struct FusedRotation {             // window plans: LOS l is multiplied by T[clamp(centre[l], cmin, cmax)][active channel]
