@@ -359,9 +359,16 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
         p->kblocks = (p->nact + kChanPerKBlock - 1) / kChanPerKBlock;
         p->kpad = p->kblocks * kKBlock;
         const bool fp16 = precision == RMS_FP16X3;
-        RMS_TRY(dalloc(&p->d_bhi, (size_t)p->tiles.npad * p->kpad));
-        RMS_TRY(dalloc(&p->d_blo, (size_t)p->tiles.npad * p->kpad));
-        RMS_TRY(launch_phase_bsplit(*p, p->d_dl2, p->d_wact, p->nact, p->kpad, p->d_bhi, p->d_blo, fp16, 0));
+        // The matrices and maps for any grid serve plans that do not fold, windows' rotating
+        // contraction and FP16X3's no-allocation call; a folded BF16 or BF16X3 plan has no kernel
+        // that reads them (rms_plan_get builds them when asked).  1536 channels x 4001 phi: built beside
+        // the folded ones they made a plan of 371 MB where the general form takes 342.
+        const bool general = !p->fold.on || fp16;
+        if (general) {
+            RMS_TRY(dalloc(&p->d_bhi, (size_t)p->tiles.npad * p->kpad));
+            RMS_TRY(dalloc(&p->d_blo, (size_t)p->tiles.npad * p->kpad));
+            RMS_TRY(launch_phase_bsplit(*p, p->d_dl2, p->d_wact, p->nact, p->kpad, p->d_bhi, p->d_blo, fp16, 0));
+        }
         // LOS-major cubes contract over every channel (zero rows where flagged)
         p->kblocks_raw = (nchan + kChanPerKBlock - 1) / kChanPerKBlock;
         p->kpad_raw = p->kblocks_raw * kKBlock;
@@ -370,7 +377,7 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
             if (w[i] != 0.0) kbmask[i / kChanPerKBlock] |= (uint16_t)(1u << (i % kChanPerKBlock));
         RMS_TRY(dalloc(&p->d_kbmask, p->kblocks_raw));
         RMS_TRY(cudaMemcpy(p->d_kbmask, kbmask.data(), p->kblocks_raw * sizeof(uint16_t), cudaMemcpyHostToDevice));
-        if (p->nact == nchan) {
+        if (!general || p->nact == nchan) {
             p->d_bhi_raw = p->d_bhi;
             p->d_blo_raw = p->d_blo;
         } else {
@@ -387,16 +394,17 @@ rms_status plan_create_internal(rms_plan_t *out, const double *axis, int32_t nch
         }
         p->scratch_bytes = (size_t)p->num_sms * (size_t)std::max(p->kblocks, p->kblocks_raw) * kTileM * 128;
         RMS_TRY(cudaMalloc(&p->d_scratch, p->scratch_bytes));
-        if (!encode_b_map(&p->tmap_bhi, p->d_bhi, p->kpad, p->tiles.npad, p->tiles.tile_n) ||
-            !encode_b_map(&p->tmap_blo, p->d_blo, p->kpad, p->tiles.npad, p->tiles.tile_n) ||
-            !encode_b_map(&p->tmap_bhi_raw, p->d_bhi_raw, p->kpad_raw, p->tiles.npad, p->tiles.tile_n) ||
-            !encode_b_map(&p->tmap_blo_raw, p->d_blo_raw, p->kpad_raw, p->tiles.npad, p->tiles.tile_n)) {
+        if (general &&
+            (!encode_b_map(&p->tmap_bhi, p->d_bhi, p->kpad, p->tiles.npad, p->tiles.tile_n) ||
+             !encode_b_map(&p->tmap_blo, p->d_blo, p->kpad, p->tiles.npad, p->tiles.tile_n) ||
+             !encode_b_map(&p->tmap_bhi_raw, p->d_bhi_raw, p->kpad_raw, p->tiles.npad, p->tiles.tile_n) ||
+             !encode_b_map(&p->tmap_blo_raw, p->d_blo_raw, p->kpad_raw, p->tiles.npad, p->tiles.tile_n))) {
             free_plan(p);
             return RMS_ERR_CUDA;
         }
         // half-tile boxes for the two-CTA contraction (tile_n a multiple of 16, so a
         // half is whole 8-row swizzle groups)
-        if (p->tiles.tile_n2 % 16 == 0 && p->tiles.tile_n_last2 % 16 == 0) {
+        if (general && p->tiles.tile_n2 % 16 == 0 && p->tiles.tile_n_last2 % 16 == 0) {
             const int h = p->tiles.tile_n2 / 2;
             p->pair_maps = encode_b_map(&p->tmap2_bhi, p->d_bhi, p->kpad, p->tiles.npad, h) &&
                            encode_b_map(&p->tmap2_blo, p->d_blo, p->kpad, p->tiles.npad, h) &&
@@ -875,6 +883,22 @@ rms_status rms_plan_info(rms_plan_t p, int32_t what, int64_t *value)
     return RMS_OK;
 }
 
+// The phase matrix of the form for any grid, of a plan that keeps none (a folded one).
+static rms_status get_general_matrix(const rms_plan_s &p, bool high, void *dst, size_t n, int64_t bytes)
+{
+    if ((int64_t)n != bytes) return RMS_ERR_INVALID_ARG;
+    DeviceGuard guard(p.device);
+    uint16_t *m = nullptr;              // high part, low part
+    cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&m), 2 * n);
+    uint16_t *const lo = m + n / sizeof(uint16_t);
+    if (e == cudaSuccess)
+        e = launch_phase_bsplit(p, p.d_dl2, p.d_wact, p.nact, p.kpad, m, lo, p.precision == RMS_FP16X3, 0);
+    if (e == cudaSuccess) e = cudaMemcpy(dst, high ? m : lo, n, cudaMemcpyDeviceToHost);
+    cudaFree(m);
+    if (e != cudaSuccess) cudaGetLastError();
+    return from_cuda(e);
+}
+
 rms_status rms_plan_get(rms_plan_t p, int32_t what, void *dst, int64_t bytes)
 {
     if (!p || !dst) return RMS_ERR_INVALID_ARG;
@@ -885,8 +909,12 @@ rms_status rms_plan_get(rms_plan_t p, int32_t what, void *dst, int64_t bytes)
     case RMS_GET_LAMBDA2: src = p->lambda2.data(); n = p->lambda2.size() * sizeof(double); host = true; break;
     case RMS_GET_ACTIVE: src = p->active.data(); n = p->active.size() * sizeof(int32_t); host = true; break;
     case RMS_GET_TABLE: src = p->d_table; n = (size_t)p->nact * p->nphi * sizeof(float2); break;
-    case RMS_GET_B_HI: src = p->d_bhi; n = (size_t)p->tiles.npad * p->kpad * sizeof(uint16_t); break;
-    case RMS_GET_B_LO: src = p->d_blo; n = (size_t)p->tiles.npad * p->kpad * sizeof(uint16_t); break;
+    case RMS_GET_B_HI:
+    case RMS_GET_B_LO:
+        n = (size_t)p->tiles.npad * p->kpad * sizeof(uint16_t);
+        if (n > 0 && !p->d_bhi) return get_general_matrix(*p, what == RMS_GET_B_HI, dst, n, bytes);
+        src = what == RMS_GET_B_HI ? p->d_bhi : p->d_blo;
+        break;
     case RMS_GET_RMSF64: src = p->d_R64; n = (size_t)p->nphi * 2 * sizeof(double); break;
     default: return RMS_ERR_INVALID_ARG;
     }
