@@ -394,9 +394,8 @@ def measure_cube(args, cfg_name, path, layout, steps, warmup, dev, local, world=
     hbm_bytes = L * (8.0 * (nact if layout == "chan" else cfg.nchan) + (0 if peak_only else 8.0 * cfg.nphi) + 12.0)
     full_size = nlos is None and not peak_only
     if tensor_path:
-        # the one-kernel form (pairs, no job panels, no layout kernel to speak of), or the contraction
-        fused = bool(sched["cta_pairs"]) and sched["n_panels"] == 0 and kt[0] < 0.5 * kt[1] and \
-            (not peak_only or kt[0] < 0.02 * kt[1])
+        # the one-kernel form (FP16x3: behind its exponents), or layout stage and contraction
+        fused = sched["kernels_per_step"] == (2 if path == "fp16x3" else 1)
         src, summary = ("fused.cu", "fused_%s_bf16x3.md") if fused else ("gemm.cu", "gemm_%s_bf16x3.md")
         summary = summary % cfg_name
         traffic = measured_traffic(src, summary) \

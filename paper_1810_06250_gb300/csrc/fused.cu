@@ -1053,6 +1053,6 @@ cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, in
     p.last_ctas = 2 * pairs;
     p.last_pair = 1;
     p.last_panels = 0;
-    p.last_kernels = 1;
+    p.last_kernels = rexp ? 2 : 1;      // FP16X3's exponents ran before
     return e;
 }

@@ -1682,6 +1682,6 @@ cudaError_t launch_split_gemm(const rms_plan_s &p, const float *Q, const float *
     go.rexp = rexp;
     go.keys = keys;
     e = launch_gemm(p, go, s);
-    p.last_kernels += 1;   // the split
+    p.last_kernels += p.fold.on && rexp ? 2 : 1;   // the split, on folded grids FP16X3's exponents before it
     return e;
 }
