@@ -582,11 +582,12 @@ static rms_status synth_launch(rms_plan_t p, const float *Q, const float *U, int
             if (rexp) e = launch_fold_exponents(*p, Q, U, nlos, layout, rexp, s);
             if (ev[1]) cudaEventRecord(ev[1], s);
             if (e == cudaSuccess)
-                e = launch_fused(*p, Q, U, nlos, layout, F, pidx, pabs, pphi, x.q, x.u, x.chi, scr, rexp, s);
+                e = launch_fused(*p, Q, U, nlos, layout, F, pidx, pabs, pphi, x.q, x.u, x.chi, scr, rexp, s, nullptr,
+                                 &p->last_call);
         } else {
             e = launch_split_gemm(*p, Q, U, nlos, layout, F, pidx, pabs, pphi, scr,
                               rbytes ? reinterpret_cast<int8_t *>(scr + abytes) : nullptr, s, ev[1], x.q, x.u, x.chi,
-                              reinterpret_cast<unsigned long long *>(scr + abytes + rbytes));
+                              reinterpret_cast<unsigned long long *>(scr + abytes + rbytes), &p->last_call);
         }
         if (ev[2]) {
             if (e == cudaSuccess) e = cudaEventRecord(ev[2], s);
@@ -874,10 +875,16 @@ rms_status rms_plan_info(rms_plan_t p, int32_t what, int64_t *value)
     case RMS_INFO_NPAD: *value = p->tiles.npad; break;
     case RMS_INFO_TILE_N: *value = p->tiles.tile_n; break;
     case RMS_INFO_DEVICE: *value = p->device; break;
-    case RMS_INFO_LAST_CTAS: *value = p->last_ctas; break;
-    case RMS_INFO_LAST_PAIR: *value = p->last_pair; break;
-    case RMS_INFO_LAST_PANELS: *value = p->last_panels; break;
-    case RMS_INFO_LAST_KERNELS: *value = p->last_kernels; break;
+    case RMS_INFO_LAST_CTAS:
+    case RMS_INFO_LAST_PAIR:
+    case RMS_INFO_LAST_PANELS:
+    case RMS_INFO_LAST_KERNELS: {
+        std::lock_guard<std::mutex> lock(p->mu);
+        const CallFacts &f = p->last_call;
+        *value = what == RMS_INFO_LAST_CTAS ? f.ctas : what == RMS_INFO_LAST_PAIR ? f.pair
+               : what == RMS_INFO_LAST_PANELS ? f.panels : f.kernels;
+        break;
+    }
     default: return RMS_ERR_INVALID_ARG;
     }
     return RMS_OK;

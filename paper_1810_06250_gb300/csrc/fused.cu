@@ -986,7 +986,7 @@ size_t fused_ring_bytes(const rms_plan_s &p, int64_t nlos)
 
 cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout, float *F,
                          int32_t *pidx, float *pabs, float *pphi, float *pq, float *pu, float *pchi, uint8_t *ring,
-                         const int8_t *rexp, cudaStream_t s, const FusedRotation *rot)
+                         const int8_t *rexp, cudaStream_t s, const FusedRotation *rot, CallFacts *facts)
 {
     const FoldPlan &f = p.fold;
     const bool chan = layout == RMS_CHAN_MAJOR;
@@ -1050,9 +1050,6 @@ cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, in
     const cudaLaunchConfig_t cfg =
         launch_config(&attr, (unsigned)(2 * pairs), sh.smem, s);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_for(mode, chan, rot != nullptr), P, f.tmap2_bhi, f.tmap2_blo, tmA);
-    p.last_ctas = 2 * pairs;
-    p.last_pair = 1;
-    p.last_panels = 0;
-    p.last_kernels = rexp ? 2 : 1;      // FP16X3's exponents ran before
+    if (facts) *facts = {2 * pairs, 1, 0, rexp ? 2 : 1};       // FP16X3's exponents ran before
     return e;
 }

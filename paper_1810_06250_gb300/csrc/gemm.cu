@@ -1617,12 +1617,9 @@ cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s)
         kern<<<units, kThreads, smem, s>>>(P, bhi, blo, bhi);   // (the last map is unused here)
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    p.last_ctas = pair ? 2 * units : units;
-    p.last_pair = pair ? 1 : 0;
-    p.last_panels = P.jobs_split ? P.npanels : 0;
-    p.last_kernels = 1;
-    if (P.jobs_split && (o.pidx || o.pabs || o.pphi || f_at_peak)) {
-        p.last_kernels = 2;
+    const bool merge = P.jobs_split && (o.pidx || o.pabs || o.pphi || f_at_peak);
+    if (o.facts) *o.facts = {(int32_t)(pair ? 2 * units : units), pair ? 1 : 0, P.jobs_split ? P.npanels : 0, merge ? 2 : 1};
+    if (merge) {
         const int64_t nb = (o.nlos + 255) / 256;
         if (nb > 0x7fffffff) return cudaErrorInvalidValue;
         peak_finalize_kernel<<<(unsigned)nb, 256, 0, s>>>(P.keys, o.nlos, o.count, o.rows, o.F, p.nphi, p.d_phi32,
@@ -1649,7 +1646,7 @@ cudaError_t launch_image_gather(const rms_plan_s &p, int layout, const uint8_t *
 cudaError_t launch_split_gemm(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout,
                               float *F, int32_t *pidx, float *pabs, float *pphi, uint8_t *A, int8_t *rexp,
                               cudaStream_t s, cudaEvent_t ev_mid, float *pq, float *pu, float *pchi,
-                              unsigned long long *keys)
+                              unsigned long long *keys, CallFacts *facts)
 {
     cudaError_t e;
     if (p.fold.on) {
@@ -1681,7 +1678,8 @@ cudaError_t launch_split_gemm(const rms_plan_s &p, const float *Q, const float *
     go.pchi = pchi;
     go.rexp = rexp;
     go.keys = keys;
+    go.facts = facts;
     e = launch_gemm(p, go, s);
-    p.last_kernels += p.fold.on && rexp ? 2 : 1;   // the split, on folded grids FP16X3's exponents before it
+    if (facts) facts->kernels += p.fold.on && rexp ? 2 : 1;   // the split, on folded grids FP16X3's exponents before it
     return e;
 }

@@ -55,8 +55,14 @@ struct FoldPlan {
     CUtensorMap tmap_bhi, tmap_blo, tmap2_bhi, tmap2_blo;
 };
 
+// What a synthesis call ran: persistent CTAs of the contraction, 1 if it ran as CTA pairs, N panels of the split
+// schedule (0: whole schedule), kernels launched.
+struct CallFacts {
+    int32_t ctas = 0, pair = 0, panels = 0, kernels = 0;
+};
+
 struct rms_plan_s {
-    std::mutex mu;                 // queueing a synthesis call
+    std::mutex mu;                 // queueing a synthesis call; its facts
     int device = 0;
     int32_t nchan = 0, nact = 0, nphi = 0, precision = 0;
     double K = 0, lambda0sq = 0, wmax = 0, fwhm_meas = 0, fwhm_est = 0;
@@ -121,10 +127,8 @@ struct rms_plan_s {
     size_t rexp_cap = 0;
     int8_t *d_rexp = nullptr;
 
-    // what the last tensor-core synthesis call ran (rms_plan_info): persistent CTAs of
-    // the contraction, 1 if it ran as CTA pairs, N panels of the split schedule (0:
-    // whole schedule), kernels launched by the call
-    mutable int32_t last_ctas = 0, last_pair = 0, last_panels = 0, last_kernels = 0;
+    // what the last tensor-core synthesis call ran (rms_plan_info), under mu
+    CallFacts last_call;
     // scheduling options (rms_plan_set_option): RMS_CONTRACT_*, L2 budget in bytes (0: default)
     int32_t contraction = 0, schedule = 0;
     int64_t l2_budget = 0;
@@ -198,7 +202,8 @@ bool fused_wanted(const rms_plan_s &p, int64_t nlos);
 size_t fused_ring_bytes(const rms_plan_s &p, int64_t nlos);
 cudaError_t launch_fused(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout, float *F,
                          int32_t *pidx, float *pabs, float *pphi, float *pq, float *pu, float *pchi, uint8_t *ring,
-                         const int8_t *rexp, cudaStream_t s, const FusedRotation *rot = nullptr);
+                         const int8_t *rexp, cudaStream_t s, const FusedRotation *rot = nullptr,
+                         CallFacts *facts = nullptr);
 struct SplitOpts {
     const float *Q = nullptr, *U = nullptr;
     int64_t nlos_src = 0;              // lines of sight in the cube
@@ -230,6 +235,7 @@ struct GemmOpts {
     // optional scratch of nlos 64-bit peak keys: lets the contraction use its split
     // schedule (needed on cubes whose operands do not stay in L2; see gemm.cu)
     unsigned long long *keys = nullptr;
+    CallFacts *facts = nullptr;        // optional, out
 };
 cudaError_t launch_split(const rms_plan_s &p, const SplitOpts &o, cudaStream_t s);
 cudaError_t launch_gemm(const rms_plan_s &p, const GemmOpts &o, cudaStream_t s);
@@ -238,7 +244,8 @@ cudaError_t launch_image_gather(const rms_plan_s &p, int layout, const uint8_t *
 cudaError_t launch_split_gemm(const rms_plan_s &p, const float *Q, const float *U, int64_t nlos, int layout,
                               float *F, int32_t *pidx, float *pabs, float *pphi, uint8_t *A, int8_t *rexp,
                               cudaStream_t s, cudaEvent_t ev_mid = nullptr, float *pq = nullptr,
-                              float *pu = nullptr, float *pchi = nullptr, unsigned long long *keys = nullptr);
+                              float *pu = nullptr, float *pchi = nullptr, unsigned long long *keys = nullptr,
+                              CallFacts *facts = nullptr);
 
 // generate.cu
 cudaError_t launch_generate(const rms_plan_s &p, const rms_source_model &m, int64_t los0, int64_t nlos,
