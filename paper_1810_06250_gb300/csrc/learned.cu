@@ -161,6 +161,30 @@ cudaError_t window_contract(const rms_window_s &w, const uint8_t *img, int64_t n
     return launch_gemm(*w.sub, go, s);
 }
 
+// Whether window synthesis of a cube runs as one kernel (plans that have it): in a single round of items over the CTA
+// pairs always; beyond it, not where an item's few K blocks leave its fixed costs bare (bulk copies of short LOS-major
+// rows; channel-major only after many rounds without F), and not where the second round is mostly empty and the epilogue
+// short (W <= 64; channel-major, and plain BF16, whose two kernels move half the image).  Split and rotating contraction
+// against one kernel, 10 / 100 thousand LOS, BF16X3 (BF16) without F at W 64 unless stated: LOS-major 40 channels 0.91 /
+// 0.75 (0.83 / 0.62), 64 1.00 / 0.95 (0.91 / 0.75), 100 1.00 / 1.40 (0.97 / 1.00), 400 1.19 / 1.81 (0.94 / 1.20), 1536
+// (1.29 / 1.47), W 128 of 40 channels 0.97 / 0.97 (0.93 / 0.88), with F 1.13 / 1.30 (1.08 / 1.13); channel-major 40 channels
+// 1.02 / 0.92 (1.01 / 0.86), W 32 with F 1.06 / 1.13, 100 1.00 / 1.03 (1.00 / 0.98), 400 0.92 / 1.09 (0.90 / 1.05), 13,000
+// LOS of them 0.89, 16,000 1.03, W 128 1.24; 9,728 LOS (one round) 1.00 to 2.3.
+bool window_one_kernel(const rms_window_s &w, int64_t nlos, int32_t layout, bool has_f)
+{
+    const int64_t pairs = w.sub->fold.fused_pairs, nit = (nlos + 2 * kFoldTileLos - 1) / (2 * kFoldTileLos);
+    if (pairs < 1) return false;
+    if (nit <= pairs) return true;
+    const bool bf16 = w.sub->precision == RMS_BF16, narrow = w.width <= 64, sparse = 2 * nit < 3 * pairs;
+    const int32_t nact = w.sub->nact;
+    if (layout == RMS_CHAN_MAJOR) {
+        if (narrow && !has_f && nit > 8 * pairs && nact <= (bf16 ? 112 : 48)) return false;
+        return !(narrow && sparse && nact > 150);
+    }
+    if (narrow ? nact <= 64 : nact <= 48 && !has_f) return false;
+    return !(narrow && sparse && bf16 && nact > 150 && nact <= 448);
+}
+
 // Whether the learned peak map's window reads the network's image (hi and lo parts) through the rotating
 // contraction, or the cube once more in one kernel.  The image is there anyway, so the one kernel pays only
 // where the image then keeps its hi parts alone (BF16X3 on grids that fold) and the cube's rows are
@@ -171,10 +195,9 @@ cudaError_t window_contract(const rms_window_s &w, const uint8_t *img, int64_t n
 // grid 4.13 / 4.22 (16,384 LOS 168 / 181 us).
 bool window_from_image(const rms_window_s &w, int64_t nlos, int32_t layout)
 {
-    const int32_t pairs = w.sub->fold.fused_pairs;
-    if (pairs < 1) return true;
+    if (!window_one_kernel(w, nlos, layout, false)) return true;
     const bool whole = w.sub->precision == RMS_BF16 || !w.plan->fold.on;      // the image, in any case
-    return nlos > (int64_t)2 * kFoldTileLos * pairs && (layout == RMS_CHAN_MAJOR || whole);
+    return nlos > (int64_t)2 * kFoldTileLos * w.sub->fold.fused_pairs && (layout == RMS_CHAN_MAJOR || whole);
 }
 
 }  // namespace
@@ -275,7 +298,7 @@ rms_status rms_synth_window(rms_window_t w, const float *Q, const float *U, int6
     if (!guard.ok) return RMS_ERR_CUDA;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const bool one = w->sub->fold.fused_pairs > 0;      // one kernel (fused.cu), or split and rotating contraction
+    const bool one = window_one_kernel(*w, nlos, layout, F_out != nullptr);      // (fused.cu), or split and rotating contraction
     const size_t ib = one ? fused_ring_bytes(*w->sub, nlos) : split_operand_bytes(p, nlos, layout), xb = (size_t)nlos * 4;
     uint8_t *scr = nullptr;
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&scr), up(ib) + (widx ? 0 : up(xb)), s);
