@@ -36,8 +36,8 @@
  *                                  MWA cube, BF16X3 4.6e-6 at 16 and 6.1e-6 at 32);
  *      RMS_GEMM_CTAS (1..SMs)      persistent CTAs of the contraction;
  *      RMS_HOST_CHUNK (>= 1024)    LOS per chunk of rms_synth_host.
- *    Any of the contraction's five knobs set, a call takes the two-kernel form
- *    (rms_synth below).
+ *    Any of the contraction's five knobs set, a call of rms_synth takes its
+ *    two-kernel form (below).  Window synthesis' one-kernel form takes none of them.
  *  - A plan may be used from several streams and host threads.  Its scratch (device
  *    work areas owned by the plan) is shared, so every synthesis call on a plan
  *    waits on the device for the previous call on that plan (an event recorded
@@ -176,7 +176,7 @@ rms_status rms_rmsf(rms_plan_t plan, float *R_out, double *lambda0sq, double *K,
  * `stream` (cudaMallocAsync / cudaFreeAsync): the cube split into 16-bit hi and
  * lo operands, 8 bytes per (LOS, contraction channel slot; the channels are
  * padded to a multiple of 16 per 128 LOS, or 32 per 64 LOS on a symmetric grid),
- * in the one-kernel form only those of the lines of sight in flight (at most 256
+ * in the one-kernel form only those of the lines of sight in flight (at most 128
  * per SM), and for RMS_FP16X3 one exponent
  * byte per LOS; creating a tensor-core plan sets that pool to keep freed
  * memory reserved.  The FP32 precisions allocate nothing.
@@ -307,12 +307,15 @@ enum {
     RMS_INFO_NPAD = 5,        /* padded rows (2 * nphi rounded up) of the phase matrix */
     RMS_INFO_TILE_N = 6,      /* phase-matrix rows per tensor-core tile */
     RMS_INFO_DEVICE = 7,
-    /* what the last tensor-core rms_synth / rms_synth_peaks / rms_synth_host call ran: */
+    /* what the last tensor-core rms_synth / rms_synth_peaks / rms_synth_host call ran
+       (the learned entry points below leave these as they are): */
     RMS_INFO_LAST_CTAS = 8,   /* persistent CTAs of the contraction kernel */
     RMS_INFO_LAST_PAIR = 9,   /* 1: CTA pairs (two SMs per 256-row MMA), 0: single CTAs */
     RMS_INFO_LAST_PANELS = 10, /* 0: each CTA ran all phase tiles of its lines of sight;
                                   k > 0: single-tile jobs in k panels of the phase matrix */
-    RMS_INFO_LAST_KERNELS = 11 /* kernels the call launched */
+    RMS_INFO_LAST_KERNELS = 11 /* kernels the call launched: 1 in the one-kernel form (RMS_FP16X3 2:
+                                  its exponents run before), else 2 or more (RMS_FP16X3 on a
+                                  symmetric grid 3) */
 };
 rms_status rms_plan_info(rms_plan_t plan, int32_t what, int64_t *value);
 
@@ -337,9 +340,11 @@ rms_status rms_plan_destroy(rms_plan_t plan);
 /* Static English text for a status code (never NULL). */
 const char *rms_status_string(rms_status s);
 
-/* Bounded-wait limit, in nanoseconds, used by the tensor-core kernel's barrier
+/* Bounded-wait limit, in nanoseconds, of the tensor-core kernels' barrier
  * waits (default 2e9).  A kernel whose wait runs out stops, records
- * RMS_ERR_TIMEOUT on the plan and returns. */
+ * RMS_ERR_TIMEOUT on the plan and returns.  The FP32 CUDA-core kernels' waits (a
+ * block's accumulating warps on its copying ones, and back) have a fixed limit of
+ * 20 s, which this call does not change, and end the same way. */
 rms_status rms_plan_set_timeout(rms_plan_t plan, int64_t ns);
 
 /*
@@ -583,7 +588,9 @@ rms_status rms_window_centres(rms_window_t win, const int32_t *bin, int64_t nlos
  * any may be NULL): F_out [nlos][width] complex64; widx [nlos] int32, index in
  * the window of max |F| (lowest on ties, -1 if none finite); wabs [nlos] float,
  * |F| there; wphi [nlos] float, phi there.  Other arguments as rms_synth.
- * Asynchronous; per-call scratch as rms_synth.
+ * Asynchronous; per-call scratch as rms_synth, whose two forms it has too (here
+ * their last bits differ): one kernel for calls of up to about 10,000 LOS and most
+ * larger ones, else the split and a contraction that rotates the operand.
  */
 rms_status rms_synth_window(rms_window_t win, const float *Q, const float *U, int64_t nlos, int32_t layout,
                             const int32_t *centre, float *F_out, int32_t *widx, float *wabs, float *wphi,
@@ -597,11 +604,15 @@ rms_status rms_synth_window(rms_window_t win, const float *Q, const float *U, in
  * or last point, or whose window holds no finite |F|.  Outputs (device, any
  * may be NULL): phi_peak, peak_abs [nlos] floats (as rms_synth; from the
  * window or the full grid); fallback [nlos] int32, 1 where the full grid was
- * used; nfallback: device int64, the number of fallbacks.  net and win must
- * belong to the same plan.  Asynchronous; per-call scratch from the stream-
- * ordered pool: two split operand images (the network's, and one of the fallback
- * rows as rms_synth's two-kernel form has it), the window's ring (rms_synth), 2 x
- * hidden bytes of activations and 44 bytes per LOS.
+ * used; nfallback: device int64, the number of fallbacks.  Full-grid values are
+ * rms_synth's bits; window values are rms_synth_window's up to the precision's
+ * error: larger calls (more than about 10,000 LOS) on channel-major cubes,
+ * asymmetric grids, RMS_BF16 plans or few channels take the window from the
+ * network's operand image instead of the cube.  net and win must belong to the
+ * same plan.  Asynchronous; per-call scratch from the stream-ordered pool: two
+ * split operand images (the network's, and one of the fallback rows as rms_synth's
+ * two-kernel form has it), the window's ring (rms_synth) where it reads the cube,
+ * 2 x hidden bytes of activations and 44 bytes per LOS.
  */
 rms_status rms_peakmap_learned(rms_window_t win, rms_net_t net, const float *Q, const float *U, int64_t nlos,
                                int32_t layout, float tau, float *phi_peak, float *peak_abs, int32_t *fallback,

@@ -114,7 +114,7 @@ bool encode_b_map(CUtensorMap *map, void *base, int kpad, int npad, int tile_n)
 // 64 bytes to a row of the map: a load's requests are whole 128-byte lines.  With rows of
 // kpad columns and 64-byte boxes every request was half a line, and the L2's tag lookups
 // were the busiest unit of the one-kernel form (64 %): 262,144 LOS x 360 x 401 BF16x3 0.520 ->
-// 0.509 ms, 400,000 x 800 x 1001 BF16 1.59 -> 1.54, 160,000 x 1536 x 2001 BF16x3 7.75 -> 7.25.
+// 0.509 ms, 400,000 x 800 x 1001 BF16 1.59 -> 1.54, 160,000 x 1536 x 4001 BF16x3 7.75 -> 7.25.
 bool encode_fold_map(CUtensorMap *map, void *base, const FoldPlan &f, int tile_n)
 {
     constexpr int kRow = kFoldMapRows * kKBlock;

@@ -269,7 +269,8 @@ cudaError_t launch_fold_split(const rms_plan_s &p, const float *Q, const float *
 {
     const int mode = mode_of(p.precision);
     const bool chan = layout == RMS_CHAN_MAJOR;
-    // the image has an even number of 64-LOS tiles: a padding tile is written as zeros
+    // the image has an even number of 64-LOS tiles: a padding tile is zeros channel-major, and stays
+    // unwritten LOS-major (its rows reach no output, and no other row)
     const int64_t pairs = (nlos + kLosPerCta - 1) / kLosPerCta;
     const int64_t nb = chan ? pairs : 2 * pairs;
     if (nb < 1) return cudaSuccess;

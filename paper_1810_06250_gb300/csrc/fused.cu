@@ -2,12 +2,12 @@
 // the contraction): the layout stage runs inside the contraction's CTAs.
 //
 // As two kernels the operand image goes to HBM and back between them, 16 of the
-// 32 bytes per (LOS, active channel) that a call moves besides F.  Here each CTA
+// 24 bytes per (LOS, active channel) that a call moves besides F.  Here each CTA
 // of a pair converts its own next 64 LOS while it contracts the current ones, into
 // one of two slots of a small image ring that stays in L2 (2 tiles per CTA: 58 MB
-// for 360 active channels), and the TMA producer reads the slot once per phase
-// tile.  The MMAs, their order and the scaling are gemm.cu's, so the results are
-// the same bits.
+// for 360 active channels; plain BF16, half as much a channel, see fused_prepare),
+// and the TMA producer reads the slot once per phase tile.  The MMAs, their order
+// and the scaling are gemm.cu's, so the results are the same bits.
 //
 // CTA pairs (cta_group::2), 640 threads per CTA:
 //   warp 0      producer: TMA of the ring slot's operand and of the B hi/lo tiles -> full
@@ -24,11 +24,12 @@
 // shared memory; where 8 rows do not fit, the base is not on 16 bytes, on a last, partial
 // item, or with one item per pair, the splitters load through registers.  FP16X3 reads its
 // exponents, a pass of their own before (fold.cu).
-// 262,144 LOS x 360 x 401 with F, channel-major, 0.49 ms: the splitters are busy 98% of the
-// time (bound by the latency of loads whose channels lie a megabyte apart), the epilogue (F
-// stores and the peak search) 78%, the MMAs 62%, most of that at the shared-memory bandwidth
-// of their operands.  LOS-major 0.49 ms: the MMAs 79%, slowed by the staging's traffic.
-// L2-evict-first loads and an evict-last ring keep the ring on chip (0.507 -> 0.478 ms).
+// 262,144 LOS x 360 x 401 with F: 0.505 ms a call on changing inputs under load, 0.454 ms on
+// repeated ones at boost clocks.  Channel-major the splitters are busy 98% of the time (bound by
+// the latency of loads whose channels lie a megabyte apart), the epilogue (F stores and the
+// peak search) 78%, the MMAs 62%, most of that at the shared-memory bandwidth of their
+// operands; LOS-major (0.455 ms) the MMAs 79%, slowed by the staging's traffic.  L2-evict-first
+// loads and an evict-last ring keep the ring on chip: 6% of the call when they came.
 // Every wait is bounded, as in gemm.cu.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -928,6 +929,16 @@ cudaLaunchConfig_t launch_config(cudaLaunchAttribute *attr, unsigned grid, size_
 
 }  // namespace
 
+// Plans whose K blocks form one accumulation: 16 of 32 channels for the split precisions, any
+// number for plain BF16.  Its ring is 8 KB per K block and slot, 2.4 MB per K block over 76
+// pairs: 61 MB at 800 channels, 117 at 1,536, beyond the 129 MB L2 from 1,700 on.  The form pays to
+// there and, without F, beyond; with F two kernels are up to 12 % faster on longer
+// channel lists (not taken: the one-kernel form is still the faster one on single rounds there,
+// 9,000 LOS x 2500 81 against 94 us).  One kernel against two, ms, channel-major with F / without:
+// 262,144 LOS x 1000 x 401 0.83 / 0.93 and 0.66 / 0.85, x 1536 1.24 / 1.34 and 1.10 / 1.27, x 2000 1.69 /
+// 1.72 and 1.56 / 1.64, x 2600 2.24 / 2.19 and 2.13 / 2.15, 93,568 x 2000 x 1601 1.25 / 1.21 and 1.03 /
+// 1.14, 46,720 x 4000 x 1601 1.26 / 1.12 and 1.15 / 1.24, 262,144 x 1536 x 4001 5.29 / 4.96; LOS-major with F
+// x 1536 1.23 / 1.27, x 2000 1.72 / 1.64, x 2600 2.33 / 2.12.
 cudaError_t fused_prepare(rms_plan_s *p, bool window)
 {
     FoldPlan &f = p->fold;
@@ -955,11 +966,14 @@ cudaError_t fused_prepare(rms_plan_s *p, bool window)
 
 // One kernel unless the last round of items over the pairs is too empty (12,000 LOS are 94
 // items on 76 pairs: 69.9 against 64.2 us at 360 channels x 801 phi, but 161 items on two
-// thirds of three rounds 96 against 104) or there are few items with many phase tiles,
-// which the job schedule spreads over more SMs.  Measured with F and the peak map, one
-// kernel against two: 262,144 LOS x 360 x 401 BF16x3 0.459 / 0.611 ms (LOS-major 0.454 /
-// 0.611), FP16x3 0.590 / 0.741, 200,003 LOS FP16x3 LOS-major 0.470 / 0.583, 400,000 x 800
-// x 1001 BF16 1.41 / 1.99 ms, 5,001 LOS x 360 x 401 34.7 / 42.9 us (timing events included).
+// thirds of three rounds 89 against 97, LOS-major 100 against 95) or there are few items with
+// many phase tiles, which the job schedule spreads over more SMs.  One kernel against two
+// with F and the peak map, repeated inputs at boost clocks: 262,144 LOS x 360 x 401 BF16x3
+// 0.454 / 0.604 ms (LOS-major 0.455 / 0.610), FP16x3 0.583 / 0.730, 200,003 x 357 LOS-major FP16x3
+// 0.466 / 0.581, 400,000 x 800 x 1001 BF16 1.47 / 2.03 ms, 5,001 x 357 x 401 26.7 / 37.1 us; and at
+// the line: 13,900 to 16,000 LOS x 401 0.73 to 0.89 of two kernels' time over 100 to 400 channels and
+// all three precisions, 20,000 (69% of three rounds) 0.78 to 0.98 (1,200 channels BF16 1.00 to 1.04),
+// 100 LOS x 1200 x 401 BF16 1.08 to 1.12 (fewer, longer items: a serial K).
 bool fused_wanted(const rms_plan_s &p, int64_t nlos)
 {
     const FoldPlan &f = p.fold;

@@ -507,15 +507,15 @@ __device__ __forceinline__ void job_of(const GemmParams &P, int64_t nit, int64_t
 // window variant, 512 threads, whose converter warps rotate each stage's A
 // rows in shared memory before the MMA reads them.  PAIR: the two-CTA variant
 // (launched in clusters of two; not combined with ROT).  FOLD: the phi grid is
-// symmetric and a tile holds 64 LOS (see fold.cu): P.nphi is then the number of
-// column pairs (i.e. of +-phi pairs).  LANE: the MMA issuer's loop on one lane.
+// symmetric and a tile holds 64 LOS (see fold.cu): P.ncol is then the number of
+// +-phi pairs, P.nphi still that of the samples.  LANE: the MMA issuer's loop on one lane.
 template <int HALF, bool ROT, bool PAIR, bool FOLD, bool LANE = false>
 __global__ void __launch_bounds__(ROT ? 512 : kThreads, 1)
 gemm_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtensorMap tmB_hi,
             const __grid_constant__ CUtensorMap tmB_lo, const __grid_constant__ CUtensorMap tmA)
 {
     static_assert(!(ROT && PAIR), "the rotating variant is single-CTA");
-    static_assert(!(ROT && FOLD), "windows are not folded");
+    static_assert(!(ROT && FOLD), "windows fold in the one-kernel form only");
     constexpr int kTileLos = FOLD ? kFoldTileLos : kTileM;   // lines of sight per M tile
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);

@@ -7,11 +7,12 @@
 //     T[n][j] = exp(-2i phi_n (lambda_j^2 - lambda_0^2)),
 // so every LOS shares one phase matrix (a plan whose phi grid is the W offsets
 // m D/2) once its data has been multiplied by its own row of T.  T is built in
-// FP64 and stored in FP32.  BF16, and BF16X3 up to 512 channels, multiply on the way
+// FP64 and stored in FP32.  BF16, and BF16X3 up to 512 channels, can multiply on the way
 // into the one-kernel form's ring (fused.cu), whose phase matrix folds the offsets
 // +-m: one pass over the cube and half the products (262,144 LOS x 360 channels x 64:
-// 0.69 -> 0.37 ms against the split and the rotating contraction, which multiplies in
-// shared memory and serves the longer BF16X3 channel lists).
+// 0.69 -> 0.34 ms against the split and the rotating contraction, which multiplies in
+// shared memory and serves the longer BF16X3 channel lists and the calls that the one
+// kernel does not suit, window_one_kernel).
 //
 // Learned peak map: (1) the network on an operand image of the cube, scaled by 1/RMS
 // per row, (2) window synthesis around 2 * proposed bin, from the cube or from that image
