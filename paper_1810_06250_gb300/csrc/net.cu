@@ -146,6 +146,16 @@ __device__ __forceinline__ void load_cols(uint32_t taddr, int c0, int end, float
 
 // The four warps that share a TMEM lane quarter (128 threads, named barrier 1 + q).
 __device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory"); }
+// Whether all four came with ok: they go on, or leave, together.
+__device__ __forceinline__ bool quarter_all(int q, bool ok)
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p, all;\n\tsetp.ne.b32 p, %2, 0;\n\tbar.red.and.pred all, %1, 128, p;\n\tselp.u32 %0, 1, 0, all;\n\t}"
+                 : "=r"(r)
+                 : "r"(1 + q), "r"((uint32_t)ok)
+                 : "memory");
+    return r != 0;
+}
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
@@ -626,7 +636,11 @@ net_gemm_kernel(const __grid_constant__ NetGemmParams P, const __grid_constant__
             int mt, nt, kb0, kb1;
             item_coords(P, it, mt, nt, kb0, kb1);
             const int b = t % P.nbuf;
-            if (!warp_wait(smem_u32(&S.tfull[b]), (tph >> b) & 1, S.abort_flag, P.err, P.timeout_ns)) break;
+            bool ok = warp_wait(smem_u32(&S.tfull[b]), (tph >> b) & 1, S.abort_flag, P.err, P.timeout_ns);
+            // the softmax epilogues meet at barriers of the quarter's four warps, whose waits may end apart: the
+            // accumulator's arrival can race with another role's abort, or with the limit
+            if constexpr (EPI == EPI_SOFTMAX || EPI == EPI_LOSS || EPI == EPI_LOGITS) ok = quarter_all(q, ok);
+            if (!ok) break;
             tph ^= 1u << b;
             tc_fence_after();
             epilogue<EPI>(P, S, bias_s, tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * P.BN), mt, nt, q, h,
